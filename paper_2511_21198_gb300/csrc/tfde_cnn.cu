@@ -4,26 +4,42 @@
 // to (u^{m+1} - u^m) / s.  Not part of the paper: a learned initial guess for
 // its Krylov solves; the FP64 residual test decides what the solver returns.
 //
-// Layout.  Activations are BF16, channels last, 16 channels (zero padded), on
-// a grid with one layer of zero guard points on every side:
+// Layout.  Activations are BF16, 16 channels (zero padded), on a grid with one
+// layer of zero guard points on every side:
 //   slot s = ((z + 1) (n2 + 2) + (y + 1)) R + (x + 1),   R = n1 + 2,
 // so that every 3x3x3 tap is a constant shift of the slot index (dz P + dy R
-// + dx, P = (n2 + 2) R) and the zero padding is the guard data itself.
+// + dx, P = (n2 + 2) R) and the zero padding is the guard data itself.  The
+// two channel halves are separate planes [half][slot][8 channels]: a run of
+// slots of one half is contiguous in memory, so it is staged by ONE bulk copy
+// (an interleaved layout needs a tensor copy with 16-byte rows, whose row rate
+// bounded the convolution), and it lands as K-major core matrices.
 //
-// Forward / input-gradient convolution (tcgen05 implicit GEMM): a tile is 128
-// consecutive slots (M = 128), N = 16 output channels, K = 16 input channels
-// per tap, 27 MMAs per tile.  For each of the 9 (dz, dy) rows one TMA box of
-// 130 slots x 8 channels per channel half is staged (non-swizzled K-major:
-// the two halves are the K-adjacent core matrices); the three dx taps of a
-// row are the same staged rows shifted by 16 bytes.  Warps 0..3 load (the 18
-// boxes of a tile dealt round-robin), warp 4 issues the MMAs into a
-// double-buffered TMEM accumulator, warps 5..8 run the
+// Forward / input-gradient convolution (tcgen05 implicit GEMM): M = 128
+// slots, N = 16 output channels, K = 16 input channels per tap, 27 MMAs per
+// 128 slots.  A tile is NT x 128 consecutive slots; per dz one run of
+// tile + 2 R + 2 slots holds all nine (dy, dx) shifts (three runs per tile),
+// so a slot is staged 3 (1 + (2 R + 2) / tile) times instead of nine; lines
+// too long for two such stages take nine runs of tile + 2 slots.  The taps are
+// shifts of the staged rows by 16 bytes each.  Warp 0 issues the copies, warp
+// 1 the MMAs into double-buffered TMEM accumulators, warps 2..9 run the
 // epilogue (bias, ReLU or ReLU-gradient mask, BF16 store of interior slots, or
-// the FP32 output channel on the plain grid).  Weight gradients and the small
-// element-wise steps run on CUDA cores.
+// the FP32 output channel on the plain grid).
+// Bound: the MMAs, 64 cycles each at this shape whatever N (the 4 KB A operand
+// read from shared memory); without the copies or without the epilogue the
+// time is the same.  Measured on GB300 at 128^3: 107 us per layer (162 us with
+// the nine 16-byte-row tensor copies per 128 slots).
+//
+// Weight gradients: per tap a 16 x 16 matrix summed over all slots, on
+// mma.sync m16n8k16 (tcgen05's smallest M of 64 would leave three quarters of
+// the rows empty); the same staged runs as the convolution serve all 27 taps.
+// One optimiser step of eight 64^3 samples: 2.9 ms, against 25.7 ms with the
+// nine-copy convolution, a CUDA-core weight gradient per tap and 256-slot
+// chunk (477 us per layer, 160 us for the sum of its partials), a one-block
+// max |u| (183 us) and a 16-block bias sum (41 us).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -42,52 +58,76 @@ constexpr int NL = 4;              // layers
 constexpr int NTAP = 27;
 constexpr int WSZ = CH * CH * NTAP;  // weights per layer (FP32 master [co][ci][tap])
 constexpr int PSZ = WSZ + CH;        // + bias
-constexpr int TM = 128;            // slots per tile
-constexpr int BOX = TM + 2;        // staged slots per row
-constexpr int HALF_BYTES = 2176;   // BOX * 16 B rounded up to 128 B
-constexpr int ROW_BYTES = 2 * HALF_BYTES;
-constexpr int STAGE_BYTES = 9 * ROW_BYTES;               // 39168
+constexpr int TM = 128;            // slots per MMA
+constexpr int MAX_NT = 4;          // MMA tiles per staged tile: 1, 2 or 4
 constexpr int STAGES = 2;
 constexpr int W_BYTES = NTAP * 2 * CH * 16;              // 13824: [tap][khalf][co][8 ci]
 constexpr int NUM_BARS = 2 * STAGES + 5;
-constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + W_BYTES + NUM_BARS * 8 + 16;
-constexpr int PRODUCERS = 4;       // warps 0..3 issue the 18 row boxes of a tile round-robin
-constexpr int MMA_WARP = PRODUCERS;
-constexpr int NUM_THREADS = 32 * (PRODUCERS + 1 + 4);   // + MMA warp + 4 epilogue warps
-constexpr uint32_t TMEM_COLS = 32; // 2 x 16 columns
-static_assert(SMEM_BYTES <= 232448, "shared memory budget");
+constexpr int EPI_WARPS = 8;
+constexpr int NUM_THREADS = 32 * (2 + EPI_WARPS);
+constexpr int MAX_SMEM = 232448;
+constexpr int CONV_FIXED_SMEM = 128 + W_BYTES + NUM_BARS * 8 + 16;
+constexpr int WG_WARPS = 9;        // weight gradient: one warp per (dz, dy)
+constexpr int WG_THREADS = 32 * (WG_WARPS + 1);   // + the copy warp
+constexpr int WG_SMEM_FIXED = 128 + 2 * STAGES * 8 + 16;
+constexpr int GSZ = NTAP * 256 + CH;              // one partial: [tap][co][ci], then the bias
+
+// How a tile's input rows are staged: nseg runs of seglen slots per channel
+// half (3 runs, one per dz, or 9, one per (dz, dy)); row r = (dz + 1) 3 +
+// (dy + 1) of the taps starts rowoff[r] slots into a half.
+struct Staging {
+    int nt, tile, nseg, seglen, half_bytes;
+    int rowoff[9];
+};
 
 struct ConvParams {
-    CUtensorMap amap;              // activations [S_total][16] BF16, box {8, 130}
+    const uint8_t* in;             // activations, half 0; half 1 is half_stride bytes on
+    long long half_stride;
+    Staging st;
     const __nv_bfloat16* wts;      // [27][2][16][8] BF16 (B operand layout)
     const float* bias;             // [16] or null
     int relu;                      // apply ReLU after the bias
-    const __nv_bfloat16* mask;     // [S_total][16] or null: multiply by (mask > 0)
-    __nv_bfloat16* out_act;        // [S_total][16] or null
+    const uint8_t* mask;           // activations or null: multiply by (mask > 0)
+    uint8_t* out_act;              // activations or null
     float* out_f32;                // plain grid, channel 0, or null
     int n1, n2, n3;
-    long long R, P, first, ntiles;
+    unsigned R, NY;                // slots per line, lines per plane (n2 + 2)
+    long long P, first;
+    int ntiles;
     int* err;
 };
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     tc::smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(tc::smem_u32(bar))
+                 : "memory");
 }
 
-__device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// The runs of one tile (first slot s0), both halves, into `dst`; the caller
+// has announced 2 nseg seglen 16 bytes on `bar`.
+__device__ __forceinline__ void stage_rows(uint8_t* dst, const uint8_t* in, long long half_stride, const Staging& st,
+                                           long long s0, long long P, unsigned R, uint64_t* bar) {
+    const uint32_t bytes = (uint32_t)st.seglen * 16u;
+    for (int h = 0; h < 2; ++h) {
+        for (int i = 0; i < st.nseg; ++i) {
+            const long long start = st.nseg == 3 ? s0 + (i - 1) * P - (long long)R - 1
+                                                 : s0 + (i / 3 - 1) * P + (i % 3 - 1) * (long long)R - 1;
+            bulk_load(dst + h * st.half_bytes + i * bytes, in + h * half_stride + start * 16, bytes, bar);
+        }
+    }
+}
 
+template <int NT>
 __global__ void __launch_bounds__(NUM_THREADS, 1) conv_kernel(const __grid_constant__ ConvParams p) {
     using namespace tfde::tc;
+    constexpr uint32_t TMEM_COLS = 2 * NT * CH;   // 32, 64 or 128
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* stages = smem;
-    uint8_t* wsm = smem + STAGES * STAGE_BYTES;
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+    const int stage_bytes = 2 * p.st.half_bytes;
+    uint8_t* wsm = smem;
     uint64_t* bars = reinterpret_cast<uint64_t*>(wsm + W_BYTES);
+    uint8_t* stages = wsm + W_BYTES + ((NUM_BARS * 8 + 16 + 15) & ~15);
     uint64_t* full = bars;
     uint64_t* empty = bars + STAGES;
     uint64_t* tfull = bars + 2 * STAGES;
@@ -105,41 +145,31 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) conv_kernel(const __grid_const
     }
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&full[s], PRODUCERS);
+            mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&tfull[b], 1);
-            mbar_init(&tempty[b], 4);
+            mbar_init(&tempty[b], EPI_WARPS);
         }
         mbar_init(mma_done, 1);
         mbar_fence_init();
     }
-    if (warp == MMA_WARP) tmem_alloc(tmem_slot, TMEM_COLS);
+    if (warp == 1) tmem_alloc(tmem_slot, TMEM_COLS);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    const long long total = p.ntiles;
 
-    if (warp < PRODUCERS) {
+    if (warp == 0) {
         if (lane == 0) {
-            const int pw = warp;
             int s = 0;
             uint32_t ph = 0, filled = 0, last_ph = 0;
-            for (long long t = blockIdx.x; t < total; t += gridDim.x) {
+            for (int t = blockIdx.x; t < p.ntiles; t += gridDim.x) {
                 if (!mbar_wait(&empty[s], ph ^ 1u, p.err)) break;
-                uint8_t* st = stages + s * STAGE_BYTES;
-                uint32_t mine = 0;
-                for (int i = pw; i < 18; i += PRODUCERS) mine += BOX * 16u;
-                mbar_expect_tx(&full[s], mine);
-                const long long s0 = p.first + t * TM;
-                for (int i = pw; i < 18; i += PRODUCERS) {
-                    const int r = i >> 1, h = i & 1;
-                    const int dz = r / 3 - 1, dy = r % 3 - 1;
-                    const long long start = s0 - 1 + dz * p.P + dy * p.R;   // >= 0 by the guard planes
-                    tma_load_2d(st + r * ROW_BYTES + h * HALF_BYTES, &p.amap, &full[s], 8 * h, (int)start);
-                }
+                mbar_expect_tx(&full[s], 2u * p.st.nseg * p.st.seglen * 16u);
+                stage_rows(stages + s * stage_bytes, p.in, p.half_stride, p.st, p.first + (long long)t * p.st.tile,
+                           p.P, p.R, &full[s]);
                 filled |= 1u << s;
                 if (ph) last_ph |= 1u << s; else last_ph &= ~(1u << s);
                 if (++s == STAGES) { s = 0; ph ^= 1u; }
@@ -147,29 +177,31 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) conv_kernel(const __grid_const
             for (int i = 0; i < STAGES; ++i)
                 if (filled & (1u << i)) mbar_wait(&full[i], (last_ph >> i) & 1u, p.err, false);
         }
-    } else if (warp == MMA_WARP) {
+    } else if (warp == 1) {
         if (lane == 0) {
             const uint32_t idesc = instr_desc(TM, CH, 0);
             // non-swizzled K-major: LBO = K-adjacent core matrix (channel half), SBO = next 8 rows
-            const uint64_t a0 = smem_desc(smem_u32(stages), HALF_BYTES, 128, 0);
+            const uint64_t a0 = smem_desc(smem_u32(stages), p.st.half_bytes, 128, 0);
             const uint64_t b0 = smem_desc(smem_u32(wsm), 256, 128, 0);
             int s = 0;
             uint32_t ph = 0;
-            long long it = 0;
+            int it = 0;
             bool ok = true;
-            for (long long t = blockIdx.x; t < total && ok; t += gridDim.x, ++it) {
-                const int buf = (int)(it & 1);
+            for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x, ++it) {
+                const int buf = it & 1;
                 const uint32_t use = (uint32_t)(it >> 1);
                 if (!mbar_wait(&tempty[buf], (use & 1u) ^ 1u, p.err)) { ok = false; break; }
                 if (!mbar_wait(&full[s], ph, p.err)) { ok = false; break; }
                 tc_fence_after();
-                const uint64_t as = a0 + (uint64_t)((s * STAGE_BYTES) >> 4);
+                const uint64_t as = a0 + (uint64_t)((s * stage_bytes) >> 4);
 #pragma unroll
-                for (int tap = 0; tap < NTAP; ++tap) {
-                    const int r = tap / 3, dx = tap % 3;   // tap = (dz+1)*9 + (dy+1)*3 + (dx+1)
-                    const uint64_t ad = as + (uint64_t)((r * ROW_BYTES + dx * 16) >> 4);
+                for (int tap = 0; tap < NTAP; ++tap) {   // tap = (dz+1)*9 + (dy+1)*3 + (dx+1)
                     const uint64_t bd = b0 + (uint64_t)((tap * 512) >> 4);
-                    umma_bf16(tmem_base + (uint32_t)(buf * CH), ad, bd, idesc, tap > 0 ? 1u : 0u);
+                    const uint64_t at = as + (uint64_t)(p.st.rowoff[tap / 3] + tap % 3);
+#pragma unroll
+                    for (int m = 0; m < NT; ++m)
+                        umma_bf16(tmem_base + (uint32_t)((buf * NT + m) * CH), at + (uint64_t)(m * TM), bd, idesc,
+                                  tap > 0 ? 1u : 0u);
                 }
                 umma_commit(&empty[s]);
                 umma_commit(&tfull[buf]);
@@ -179,11 +211,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) conv_kernel(const __grid_const
             mbar_wait(mma_done, 0, p.err, false);
         }
     } else {
-        const int q = warp & 3;   // TMEM lane quadrant
-        long long it = 0;
-        const long long plane_slots = p.P;
-        for (long long t = blockIdx.x; t < total; t += gridDim.x, ++it) {
-            const int buf = (int)(it & 1);
+        const int q = warp & 3;             // TMEM lane quadrant
+        const int sub = (warp - 2) >> 2;    // which half of the tile's MMA tiles
+        int it = 0;
+        for (int t = blockIdx.x; t < p.ntiles; t += gridDim.x, ++it) {
+            const int buf = it & 1;
             const uint32_t use = (uint32_t)(it >> 1);
             int ok = 1;
             if (lane == 0) ok = mbar_wait(&tfull[buf], use & 1u, p.err) ? 1 : 0;
@@ -191,107 +223,294 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) conv_kernel(const __grid_const
             if (!ok) break;
             __syncwarp();
             tc_fence_after();
-            uint32_t r[16];
-            tmem_ld16(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * CH), r);
+#pragma unroll 1
+            for (int m = sub; m < NT; m += 2) {
+                const unsigned s = (unsigned)(p.first + (long long)t * p.st.tile) + m * TM + 32 * q + lane;
+                const unsigned line = s / p.R, x1 = s - line * p.R;
+                const unsigned z1 = line / p.NY, y1 = line - z1 * p.NY;
+                const bool interior = x1 >= 1 && x1 <= (unsigned)p.n1 && y1 >= 1 && y1 <= (unsigned)p.n2 && z1 >= 1 &&
+                                      z1 <= (unsigned)p.n3;
+                uint4 mk[2];
+                if (p.mask && interior) {
+                    mk[0] = __ldg(reinterpret_cast<const uint4*>(p.mask + (size_t)s * 16));
+                    mk[1] = __ldg(reinterpret_cast<const uint4*>(p.mask + p.half_stride + (size_t)s * 16));
+                }
+                __syncwarp();
+                uint32_t r[16];
+                tmem_ld16(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)((buf * NT + m) * CH), r);
+                if (!interior) continue;
+                float v[16];
+#pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                    float a = __uint_as_float(r[c]);
+                    if (p.bias) a += __ldg(p.bias + c);
+                    if (p.relu) a = fmaxf(a, 0.f);
+                    v[c] = a;
+                }
+                if (p.mask) {
+                    const __nv_bfloat16* mb = reinterpret_cast<const __nv_bfloat16*>(mk);
+#pragma unroll
+                    for (int c = 0; c < 16; ++c)
+                        if (!(__bfloat162float(mb[c]) > 0.f)) v[c] = 0.f;
+                }
+                if (p.out_act) {
+                    uint4 o[2];
+                    __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(o);
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) h[c] = __floats2bfloat162_rn(v[2 * c], v[2 * c + 1]);
+                    *reinterpret_cast<uint4*>(p.out_act + (size_t)s * 16) = o[0];
+                    *reinterpret_cast<uint4*>(p.out_act + p.half_stride + (size_t)s * 16) = o[1];
+                }
+                if (p.out_f32) p.out_f32[((size_t)(z1 - 1) * p.n2 + (y1 - 1)) * p.n1 + (x1 - 1)] = v[0];
+            }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty[buf]);
-            const long long s = p.first + t * TM + 32 * q + lane;
-            const long long x1 = s % p.R, rem = s / p.R;
-            const long long y1 = rem % (plane_slots / p.R), z1 = rem / (plane_slots / p.R);
-            const bool interior = x1 >= 1 && x1 <= p.n1 && y1 >= 1 && y1 <= p.n2 && z1 >= 1 && z1 <= p.n3;
-            if (!interior) continue;
-            float v[16];
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-                float a = __uint_as_float(r[c]);
-                if (p.bias) a += __ldg(p.bias + c);
-                if (p.relu) a = fmaxf(a, 0.f);
-                v[c] = a;
-            }
-            if (p.mask) {
-                const uint4* mk = reinterpret_cast<const uint4*>(p.mask + s * CH);
-                const uint4 m0 = __ldg(mk), m1 = __ldg(mk + 1);
-                const __nv_bfloat16* mb0 = reinterpret_cast<const __nv_bfloat16*>(&m0);
-                const __nv_bfloat16* mb1 = reinterpret_cast<const __nv_bfloat16*>(&m1);
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    if (!(__bfloat162float(mb0[c]) > 0.f)) v[c] = 0.f;
-                    if (!(__bfloat162float(mb1[c]) > 0.f)) v[8 + c] = 0.f;
-                }
-            }
-            if (p.out_act) {
-                uint4 o0, o1;
-                __nv_bfloat162* h0 = reinterpret_cast<__nv_bfloat162*>(&o0);
-                __nv_bfloat162* h1 = reinterpret_cast<__nv_bfloat162*>(&o1);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    h0[c] = __floats2bfloat162_rn(v[2 * c], v[2 * c + 1]);
-                    h1[c] = __floats2bfloat162_rn(v[8 + 2 * c], v[8 + 2 * c + 1]);
-                }
-                uint4* dst = reinterpret_cast<uint4*>(p.out_act + s * CH);
-                dst[0] = o0;
-                dst[1] = o1;
-            }
-            if (p.out_f32) p.out_f32[((z1 - 1) * p.n2 + (y1 - 1)) * p.n1 + (x1 - 1)] = v[0];
         }
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == MMA_WARP) tmem_dealloc(tmem_base, TMEM_COLS);
+    if (warp == 1) tmem_dealloc(tmem_base, TMEM_COLS);
+}
+
+// ------------------------------------------------------------ weight gradient
+struct WgradParams {
+    const uint8_t* dz;             // gradient w.r.t. the layer's output
+    const uint8_t* in;             // the layer's input activations
+    long long half_stride;
+    Staging st;
+    unsigned R;
+    long long P, first;
+    int ntiles;
+    double* part;                  // [gridDim.x][GSZ]
+    int* err;
+};
+
+__device__ __forceinline__ void ldsm_t4(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// Partial sums over this CTA's tiles of dW[tap][co][ci] = sum_s dZ[s][co]
+// X[s + shift(tap)][ci] and db[co] = sum_s dZ[s][co] (dZ is zero on guard
+// slots).  Warp w < 9 takes the three dx taps of row w: per 16 slots one
+// transposed load of dZ (A, co x slots), three of X (B, slots x ci) and six
+// MMAs; the bias is a seventh MMA of warp 4 against a matrix of ones.  Sums:
+// 16 slots in the tensor core, 128 slots in FP32, and those in pairs of FP32
+// values (two-sum), so that the error does not grow with the grid.
+__global__ void __launch_bounds__(WG_THREADS, 1) wgrad_kernel(const __grid_constant__ WgradParams p) {
+    using namespace tfde::tc;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem);
+    uint64_t* empty = full + STAGES;
+    uint8_t* stages = smem + ((2 * STAGES * 8 + 15) & ~15);
+    const int dz_half = p.st.tile * 16;
+    const int stage_bytes = 2 * p.st.half_bytes + 2 * dz_half;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], WG_WARPS);
+        }
+        mbar_fence_init();
+    }
+    __syncthreads();
+    if (warp == WG_WARPS) {
+        if (lane == 0) {
+            int s = 0;
+            uint32_t ph = 0, filled = 0, last_ph = 0;
+            for (int t = blockIdx.x; t < p.ntiles; t += gridDim.x) {
+                if (!mbar_wait(&empty[s], ph ^ 1u, p.err)) break;
+                const long long s0 = p.first + (long long)t * p.st.tile;
+                uint8_t* st = stages + s * stage_bytes;
+                mbar_expect_tx(&full[s], 2u * (p.st.nseg * p.st.seglen + p.st.tile) * 16u);
+                stage_rows(st, p.in, p.half_stride, p.st, s0, p.P, p.R, &full[s]);
+                for (int h = 0; h < 2; ++h)
+                    bulk_load(st + 2 * p.st.half_bytes + h * dz_half, p.dz + h * p.half_stride + s0 * 16, dz_half,
+                              &full[s]);
+                filled |= 1u << s;
+                if (ph) last_ph |= 1u << s; else last_ph &= ~(1u << s);
+                if (++s == STAGES) { s = 0; ph ^= 1u; }
+            }
+            for (int i = 0; i < STAGES; ++i)
+                if (filled & (1u << i)) mbar_wait(&full[i], (last_ph >> i) & 1u, p.err, false);
+        }
+        return;
+    }
+    float hi[28], lo[28];
+#pragma unroll
+    for (int i = 0; i < 28; ++i) hi[i] = lo[i] = 0.f;
+    // A: matrices (slots 0-7, co 0-7), (0-7, 8-15), (8-15, 0-7), (8-15, 8-15);
+    // B: (slots 0-7, ci 0-7), (8-15, 0-7), (0-7, 8-15), (8-15, 8-15)
+    const int lr = lane & 7, lm = lane >> 3;
+    const uint32_t aoff = (uint32_t)(2 * p.st.half_bytes + (lm & 1) * dz_half + ((lm >> 1) * 8 + lr) * 16);
+    const uint32_t boff = (uint32_t)((lm >> 1) * p.st.half_bytes + ((lm & 1) * 8 + lr + p.st.rowoff[warp]) * 16);
+    const uint32_t one2 = 0x3F803F80u;
+    int s = 0;
+    uint32_t ph = 0;
+    for (int t = blockIdx.x; t < p.ntiles; t += gridDim.x) {
+        int ok = 1;
+        if (lane == 0) ok = mbar_wait(&full[s], ph, p.err) ? 1 : 0;
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok) break;
+        __syncwarp();
+        const uint32_t base = smem_u32(stages + s * stage_bytes);
+        for (int k0 = 0; k0 < p.st.tile; k0 += TM) {
+            float sum[7][4];
+#pragma unroll
+            for (int i = 0; i < 7; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) sum[i][j] = 0.f;
+#pragma unroll 2
+            for (int k = k0; k < k0 + TM; k += 16) {
+                uint32_t a[4];
+                ldsm_t4(base + aoff + (uint32_t)k * 16u, a);
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx) {
+                    uint32_t b[4];
+                    ldsm_t4(base + boff + (uint32_t)(k + dx) * 16u, b);
+                    float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+                    mma_16816(c0, a, b[0], b[1]);
+                    mma_16816(c1, a, b[2], b[3]);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        sum[2 * dx][j] += c0[j];
+                        sum[2 * dx + 1][j] += c1[j];
+                    }
+                }
+                if (warp == 4) {
+                    float c[4] = {0.f, 0.f, 0.f, 0.f};
+                    mma_16816(c, a, one2, one2);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) sum[6][j] += c[j];
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 28; ++i) {
+                const float v = sum[i >> 2][i & 3], h = hi[i] + v, bb = h - hi[i];
+                lo[i] += (hi[i] - (h - bb)) + (v - bb);
+                hi[i] = h;
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[s]);
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
+    }
+    // accumulator (co = lane / 4 (+ 8), ci = 2 (lane % 4) (+ 1) (+ 8))
+    double* out = p.part + (size_t)blockIdx.x * GSZ;
+#pragma unroll
+    for (int i = 0; i < 24; ++i) {
+        const int dx = i >> 3, half = (i >> 2) & 1, j = i & 3;
+        const int co = (lane >> 2) + 8 * (j >> 1), ci = 8 * half + 2 * (lane & 3) + (j & 1);
+        out[(warp * 3 + dx) * 256 + co * 16 + ci] = (double)hi[i] + (double)lo[i];
+    }
+    if (warp == 4 && (lane & 3) == 0)
+        for (int j = 0; j < 4; j += 2)
+            out[NTAP * 256 + (lane >> 2) + 8 * (j >> 1)] = (double)hi[24 + j] + (double)lo[24 + j];
+}
+
+// grad[layer][W co][ci][tap] (and the bias) += the sum of the partials, all layers
+__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const double* __restrict__ part, int nparts,
+                                                           float* __restrict__ grad) {
+    __shared__ double sh[8][33];
+    const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int idx = blockIdx.x * 32 + c;   // (tap, co, ci) or the bias
+    const double* src = part + (size_t)blockIdx.y * nparts * GSZ;
+    double acc = 0.0;
+    if (idx < GSZ)
+        for (int i = g; i < nparts; i += 8) acc += src[(size_t)i * GSZ + idx];
+    sh[g][c] = acc;
+    __syncthreads();
+    if (g == 0 && idx < GSZ) {
+        for (int i = 1; i < 8; ++i) acc += sh[i][c];
+        float* gl = grad + (size_t)blockIdx.y * PSZ;
+        if (idx < NTAP * 256) {
+            const int tap = idx / 256, co = (idx / 16) % 16, ci = idx % 16;
+            gl[(co * CH + ci) * NTAP + tap] += (float)acc;
+        } else {
+            gl[WSZ + idx - NTAP * 256] += (float)acc;
+        }
+    }
 }
 
 // ------------------------------------------------------------ CUDA-core kernels
-__device__ __forceinline__ long long slot_of(long long p, int n1, int n2, long long R, long long P) {
-    const long long x = p % n1, r = p / n1;
-    const long long y = r % n2, z = r / n2;
-    return (z + 1) * P + (y + 1) * R + (x + 1);
+struct Grid {
+    int n1, n2;
+    unsigned R;
+    long long P, half_stride;   // slots per plane; bytes between the channel halves
+};
+__device__ __forceinline__ size_t slot_of(unsigned p, const Grid& g) {
+    const unsigned r = p / (unsigned)g.n1, x = p - r * (unsigned)g.n1;
+    const unsigned z = r / (unsigned)g.n2, y = r - z * (unsigned)g.n2;
+    return (size_t)(z + 1) * g.P + (size_t)((y + 1) * g.R + x + 1);
 }
 
-// max |u| into *out (one block, deterministic)
-__global__ void maxabs_kernel(const double* __restrict__ u, long long N, double* __restrict__ out) {
-    __shared__ double sh[256];
-    double m = 0.0;
-    for (long long i = threadIdx.x; i < N; i += blockDim.x) m = fmax(m, fabs(u[i]));
-    sh[threadIdx.x] = m;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + o]);
-        __syncthreads();
+// max |u| as the bit pattern of a non-negative double (whose order is the
+// integers'), NaNs passed over; *out starts at 0.  Bound by the read of u.
+__global__ void __launch_bounds__(256) maxabs_kernel(const double* __restrict__ u, long long N,
+                                                     unsigned long long* __restrict__ out) {
+    const unsigned long long inf = 0x7ff0000000000000ull;
+    unsigned long long m = 0;
+    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < N; i += gridDim.x * 256LL) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(u[i]) & 0x7fffffffffffffffull;
+        if (b <= inf && b > m) m = b;
     }
-    if (threadIdx.x == 0) out[0] = sh[0] > 0.0 ? sh[0] : 1.0;
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long v = __shfl_xor_sync(0xffffffffu, m, o);
+        m = v > m ? v : m;
+    }
+    __shared__ unsigned long long sh[8];
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < 8; ++i) m = sh[i] > m ? sh[i] : m;
+        if (m) atomicMax(out, m);
+    }
 }
+__device__ __forceinline__ double scale_of(const unsigned long long* bits) {
+    const unsigned long long b = *bits;
+    return b ? __longlong_as_double((long long)b) : 1.0;
+}
+
+struct Coef {
+    float c[9];
+};
 
 // X0[slot] = (u/s, dtF/s, c_0..c_8, d1/s, d2/s, 0...) for every interior grid
 // point; d1 = u - u1 and d2 = u - 2 u1 + u2 are the first and second
 // differences of the time history (zero channels without it)
-__global__ void pack_input_kernel(const double* __restrict__ u, const double* __restrict__ u1,
-                                  const double* __restrict__ u2, const double* __restrict__ dtF,
-                                  const double* __restrict__ scale, const float* __restrict__ coef, int n1, int n2,
-                                  long long N, long long R, long long P, __nv_bfloat16* __restrict__ X) {
-    const double inv = 1.0 / scale[0];
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
+__global__ void __launch_bounds__(256) pack_input_kernel(const double* __restrict__ u, const double* __restrict__ u1,
+                                                         const double* __restrict__ u2, const double* __restrict__ dtF,
+                                                         const unsigned long long* __restrict__ scale, const Coef coef,
+                                                         const Grid g, unsigned N, uint8_t* __restrict__ X) {
+    const double inv = 1.0 / scale_of(scale);
+    for (unsigned p = blockIdx.x * 256u + threadIdx.x; p < N; p += gridDim.x * 256u) {
         float v[16];
-        v[0] = (float)(u[p] * inv);
+        const double up = u[p];
+        v[0] = (float)(up * inv);
         v[1] = dtF ? (float)(dtF[p] * inv) : 0.f;
 #pragma unroll
-        for (int c = 0; c < 9; ++c) v[2 + c] = coef[c];
-        v[11] = u1 ? (float)((u[p] - u1[p]) * inv) : 0.f;
-        v[12] = (u1 && u2) ? (float)((u[p] - 2.0 * u1[p] + u2[p]) * inv) : 0.f;
+        for (int c = 0; c < 9; ++c) v[2 + c] = coef.c[c];
+        v[11] = u1 ? (float)((up - u1[p]) * inv) : 0.f;
+        v[12] = (u1 && u2) ? (float)((up - 2.0 * u1[p] + u2[p]) * inv) : 0.f;
 #pragma unroll
         for (int c = 13; c < 16; ++c) v[c] = 0.f;
-        uint4 o0, o1;
-        __nv_bfloat162* h0 = reinterpret_cast<__nv_bfloat162*>(&o0);
-        __nv_bfloat162* h1 = reinterpret_cast<__nv_bfloat162*>(&o1);
+        uint4 o[2];
+        __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(o);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            h0[c] = __floats2bfloat162_rn(v[2 * c], v[2 * c + 1]);
-            h1[c] = __floats2bfloat162_rn(v[8 + 2 * c], v[8 + 2 * c + 1]);
-        }
-        uint4* dst = reinterpret_cast<uint4*>(X + slot_of(p, n1, n2, R, P) * CH);
-        dst[0] = o0;
-        dst[1] = o1;
+        for (int c = 0; c < 8; ++c) h[c] = __floats2bfloat162_rn(v[2 * c], v[2 * c + 1]);
+        uint8_t* dst = X + slot_of(p, g) * 16;
+        *reinterpret_cast<uint4*>(dst) = o[0];
+        *reinterpret_cast<uint4*>(dst + g.half_stride) = o[1];
     }
 }
 
@@ -306,25 +525,31 @@ __device__ __forceinline__ double guess_base(const double* u, const double* u1, 
 // x0 = base + s * out
 __global__ void guess_kernel(const double* __restrict__ u, const double* __restrict__ u1,
                              const double* __restrict__ u2, const float* __restrict__ out,
-                             const double* __restrict__ scale, long long N, double* __restrict__ x0) {
-    const double s = scale[0];
+                             const unsigned long long* __restrict__ scale, long long N, double* __restrict__ x0) {
+    const double s = scale_of(scale);
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x)
         x0[p] = guess_base(u, u1, u2, p) + s * (double)out[p];
 }
 
-// loss partials and the output gradient: d = out - (u_next - u)/s ; dZ[slot][0] = 2 d / N
-__global__ void loss_grad_kernel(const float* __restrict__ out, const double* __restrict__ u,
-                                 const double* __restrict__ u1, const double* __restrict__ u2,
-                                 const double* __restrict__ un, const double* __restrict__ scale, int n1, int n2,
-                                 long long N, long long R, long long P, __nv_bfloat16* __restrict__ dZ,
-                                 double* __restrict__ part) {
+// loss partials and the output gradient: d = out - (u_next - u)/s ;
+// dZ[slot] = (2 d / N, 0, ..) on every interior slot (both halves, so that the
+// buffer needs no clearing: its guard slots are never written)
+__global__ void __launch_bounds__(256) loss_grad_kernel(const float* __restrict__ out, const double* __restrict__ u,
+                                                        const double* __restrict__ u1, const double* __restrict__ u2,
+                                                        const double* __restrict__ un,
+                                                        const unsigned long long* __restrict__ scale, const Grid g,
+                                                        unsigned N, uint8_t* __restrict__ dZ,
+                                                        double* __restrict__ part) {
     __shared__ double sh[256];
-    const double inv = 1.0 / scale[0];
+    const double inv = 1.0 / scale_of(scale), two_n = 2.0 / (double)N;
     double acc = 0.0;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
+    for (unsigned p = blockIdx.x * 256u + threadIdx.x; p < N; p += gridDim.x * 256u) {
         const double d = (double)out[p] - (un[p] - guess_base(u, u1, u2, p)) * inv;
         acc += d * d;
-        dZ[slot_of(p, n1, n2, R, P) * CH] = __float2bfloat16_rn((float)(2.0 * d / (double)N));
+        uint8_t* dst = dZ + slot_of(p, g) * 16;
+        const unsigned z = __bfloat16_as_ushort(__float2bfloat16_rn((float)(d * two_n)));
+        *reinterpret_cast<uint4*>(dst) = make_uint4(z, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(dst + g.half_stride) = make_uint4(0u, 0u, 0u, 0u);
     }
     sh[threadIdx.x] = acc;
     __syncthreads();
@@ -335,69 +560,19 @@ __global__ void loss_grad_kernel(const float* __restrict__ out, const double* __
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-// Weight-gradient partials of one tap over a chunk of slots:
-//   part[(chunk * 27 + tap) * 256 + co * 16 + ci] = sum_s dZ[s][co] X[s + off][ci]
-// (dZ is zero on guard slots, X is zero there by construction).
-constexpr int WG_CHUNK = 256;
-__global__ __launch_bounds__(256) void wgrad_kernel(const __nv_bfloat16* __restrict__ dZ,
-                                                    const __nv_bfloat16* __restrict__ X, long long first,
-                                                    long long count, long long R, long long P,
-                                                    float* __restrict__ part) {
-    __shared__ float sz[WG_CHUNK][CH + 1];
-    __shared__ float sx[WG_CHUNK][CH + 1];
-    const int tap = blockIdx.y;
-    const long long off = (long long)(tap / 9 - 1) * P + (long long)((tap / 3) % 3 - 1) * R + (tap % 3 - 1);
-    const long long s0 = first + (long long)blockIdx.x * WG_CHUNK;
-    for (int e = threadIdx.x; e < WG_CHUNK * CH; e += 256) {
-        const int i = e / CH, c = e % CH;
-        const long long s = s0 + i;
-        const bool in = s < first + count;
-        sz[i][c] = in ? __bfloat162float(dZ[s * CH + c]) : 0.f;
-        sx[i][c] = in ? __bfloat162float(X[(s + off) * CH + c]) : 0.f;
-    }
-    __syncthreads();
-    const int co = threadIdx.x >> 4, ci = threadIdx.x & 15;
-    float acc = 0.f;
-#pragma unroll 8
-    for (int i = 0; i < WG_CHUNK; ++i) acc = fmaf(sz[i][co], sx[i][ci], acc);
-    part[((long long)blockIdx.x * NTAP + tap) * 256 + threadIdx.x] = acc;
-}
-
-// grad[layer W][co][ci][tap] += sum over chunks; grad bias[co] += sum_s dZ[s][co]
-__global__ void wgrad_reduce_kernel(const float* __restrict__ part, int nchunks, float* __restrict__ gW) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;   // (tap, co, ci)
-    if (idx >= NTAP * 256) return;
-    const int tap = idx / 256, co = (idx / 16) % 16, ci = idx % 16;
-    double acc = 0.0;
-    for (int c = 0; c < nchunks; ++c) acc += part[((long long)c * NTAP + tap) * 256 + co * 16 + ci];
-    gW[(co * CH + ci) * NTAP + tap] += (float)acc;
-}
-
-__global__ void bgrad_kernel(const __nv_bfloat16* __restrict__ dZ, long long first, long long count,
-                             float* __restrict__ gb) {
-    __shared__ float sh[256];
-    const int c = blockIdx.x;
-    float acc = 0.f;
-    for (long long i = threadIdx.x; i < count; i += 256) acc += __bfloat162float(dZ[(first + i) * CH + c]);
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) gb[c] += sh[0];
-}
-
 // Forward weights [27][2][16][8] (B operand: N = co, K = ci) and input-gradient
-// weights (N = ci, K = co, taps mirrored) from the FP32 master [co][ci][27].
-__global__ void pack_weights_kernel(const float* __restrict__ Wm, __nv_bfloat16* __restrict__ fwd,
-                                    __nv_bfloat16* __restrict__ bwd) {
+// weights (N = ci, K = co, taps mirrored) from the FP32 master [co][ci][27];
+// blockIdx.y is the layer.
+__global__ void pack_weights_kernel(const float* __restrict__ prm, __nv_bfloat16* __restrict__ wf,
+                                    __nv_bfloat16* __restrict__ wb) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;   // (tap, h, n, k8)
     if (idx >= NTAP * 256) return;
+    const float* Wm = prm + (size_t)blockIdx.y * PSZ;
+    const size_t at = (size_t)blockIdx.y * NTAP * 256 + idx;
     const int tap = idx / 256, h = (idx / 128) % 2, n = (idx / 8) % 16, k8 = idx % 8;
     const int k = 8 * h + k8;
-    fwd[idx] = __float2bfloat16_rn(Wm[(n * CH + k) * NTAP + tap]);                  // W[co = n][ci = k][tap]
-    bwd[idx] = __float2bfloat16_rn(Wm[(k * CH + n) * NTAP + (NTAP - 1 - tap)]);     // W[co = k][ci = n][-tap]
+    wf[at] = __float2bfloat16_rn(Wm[(n * CH + k) * NTAP + tap]);                  // W[co = n][ci = k][tap]
+    wb[at] = __float2bfloat16_rn(Wm[(k * CH + n) * NTAP + (NTAP - 1 - tap)]);     // W[co = k][ci = n][-tap]
 }
 
 // Adam on all parameters (grads averaged over `count` samples), grads zeroed.
@@ -415,14 +590,15 @@ __global__ void adam_kernel(float* __restrict__ prm, float* __restrict__ grad, f
     grad[i] = 0.f;
 }
 
-bool g_attr = false;
-
 }  // namespace cnn
 }  // namespace tfde
 
 struct tfde_cnn {
     int n[3] = {};
-    long long N = 0, R = 0, P = 0, S_total = 0, first = 0, count = 0, ntiles = 0;
+    long long N = 0, R = 0, P = 0, S_total = 0, first = 0, count = 0;
+    long long half_stride = 0;  // bytes between the channel halves of an activation buffer
+    tfde::cnn::Staging conv_st, wg_st;   // tiles of the convolution and of the weight gradient
+    int conv_tiles = 0, wg_tiles = 0, wg_grid = 0;
     float* prm = nullptr;      // FP32 master parameters, NL * PSZ
     float* grad = nullptr;
     float* adam_m = nullptr;
@@ -431,19 +607,15 @@ struct tfde_cnn {
     int accumulated = 0;
     __nv_bfloat16* wf = nullptr;  // packed forward weights, NL * 27*256
     __nv_bfloat16* wb = nullptr;  // packed input-gradient weights
-    __nv_bfloat16* act[tfde::cnn::NL] = {};  // layer inputs X0..X3 (padded slots)
-    __nv_bfloat16* dz = nullptr;  // gradient buffers (padded slots), two
-    __nv_bfloat16* dz2 = nullptr;
-    float* out = nullptr;         // network output, plain grid
-    float* coef = nullptr;        // 9 input constants (device)
-    double* scale = nullptr;
-    float* wpart = nullptr;
-    double* lpart = nullptr;
+    uint8_t* act[tfde::cnn::NL] = {};  // layer inputs X0..X3 (padded slots, two half planes)
+    uint8_t* dz = nullptr;     // gradient buffers (padded slots), two
+    uint8_t* dz2 = nullptr;
+    float* out = nullptr;      // network output, plain grid
+    unsigned long long* scale = nullptr;   // max |u| (bits of a double; 0: no scaling)
+    double* wpart = nullptr;   // weight-gradient partials [NL][wg_grid][GSZ]
+    double* lpart = nullptr;   // loss partials, then the error flag
     double* lpart_host = nullptr;
-    CUtensorMap amap[tfde::cnn::NL];
-    CUtensorMap dmap[2];
-    int* err = nullptr;
-    int* err_host = nullptr;
+    int* err = nullptr;        // the word after lpart's partials
     bool packed = false;
 };
 
@@ -458,28 +630,49 @@ namespace {
             return set_error(TFDE_ECUDA, std::string(#expr) + ": " + cudaGetErrorString(e__)); \
     } while (0)
 
-int make_act_map(CUtensorMap* m, const __nv_bfloat16* base, long long S_total) {
-    const cuuint64_t dims[2] = {(cuuint64_t)CH, (cuuint64_t)S_total};
-    const cuuint64_t strides[1] = {(cuuint64_t)CH * 2};
-    const cuuint32_t box[2] = {8, (cuuint32_t)BOX};
-    return tc::encode_map(m, base, 2, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE);
-}
-
 int grid1(long long n) {
     long long g = (n + 255) / 256;
     if (g > 152LL * 8) g = 152LL * 8;
     return (int)(g < 1 ? 1 : g);
 }
 
-int conv(tfde_cnn* C, const CUtensorMap& amap, const __nv_bfloat16* w, const float* bias, int relu,
-         const __nv_bfloat16* mask, __nv_bfloat16* out_act, float* out_f32, cudaStream_t s) {
-    if (!g_attr) {
-        CN_TRY(cudaFuncSetAttribute(conv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
-        g_attr = true;
+constexpr int LPART = 1216;   // loss partials (blocks of grid1)
+
+// Tiles of nt x 128 slots, nt as large as leaves every SM a tile; three runs
+// per tile where two stages of them (and `extra` bytes per slot) fit in shared
+// memory, with a smaller tile first, else nine runs.
+Staging staging(long long count, long long R, int fixed_smem, int extra) {
+    Staging st{};
+    auto fits = [&](int nt, int nseg) {
+        const long long tile = nt * (long long)TM, seglen = nseg == 3 ? tile + 2 * R + 2 : tile + 2;
+        return STAGES * (2 * nseg * seglen * 16 + extra * tile) + fixed_smem + 1024 <= MAX_SMEM;
+    };
+    st.nt = MAX_NT;
+    while (st.nt > 1 && count < (long long)st.nt * TM * tc::num_sms()) st.nt /= 2;
+    st.nseg = 3;
+    while (st.nt > 1 && !fits(st.nt, 3)) st.nt /= 2;
+    if (!fits(st.nt, 3)) {
+        st.nseg = 9;
+        st.nt = 2;
     }
+    st.tile = st.nt * TM;
+    st.seglen = (int)(st.nseg == 3 ? st.tile + 2 * R + 2 : st.tile + 2);
+    st.half_bytes = st.nseg * st.seglen * 16;
+    for (int r = 0; r < 9; ++r)
+        st.rowoff[r] = st.nseg == 3 ? (r / 3) * st.seglen + (int)((r % 3) * R) : r * st.seglen;
+    return st;
+}
+
+int conv_smem(const Staging& st) { return CONV_FIXED_SMEM + 16 + STAGES * 2 * st.half_bytes; }
+int wg_smem(const Staging& st) { return WG_SMEM_FIXED + STAGES * (2 * st.half_bytes + 2 * st.tile * 16); }
+
+int conv(tfde_cnn* C, const uint8_t* in, const __nv_bfloat16* w, const float* bias, int relu, const uint8_t* mask,
+         uint8_t* out_act, float* out_f32, cudaStream_t s) {
     ConvParams p;
     std::memset(&p, 0, sizeof(p));
-    p.amap = amap;
+    p.in = in;
+    p.half_stride = C->half_stride;
+    p.st = C->conv_st;
     p.wts = w;
     p.bias = bias;
     p.relu = relu;
@@ -489,14 +682,18 @@ int conv(tfde_cnn* C, const CUtensorMap& amap, const __nv_bfloat16* w, const flo
     p.n1 = C->n[0];
     p.n2 = C->n[1];
     p.n3 = C->n[2];
-    p.R = C->R;
+    p.R = (unsigned)C->R;
+    p.NY = (unsigned)(C->n[1] + 2);
     p.P = C->P;
     p.first = C->first;
-    p.ntiles = C->ntiles;
+    p.ntiles = C->conv_tiles;
     p.err = C->err;
-    long long grid = C->ntiles < tc::num_sms() ? C->ntiles : tc::num_sms();
+    const int grid = std::min(C->conv_tiles, tc::num_sms());
+    const int smem = conv_smem(p.st);
     void* tok = stats_tc_begin(s, TFDE_KIND_CONV);
-    conv_kernel<<<(unsigned)(grid < 1 ? 1 : grid), NUM_THREADS, SMEM_BYTES, s>>>(p);
+    if (p.st.nt == 4) conv_kernel<4><<<grid, NUM_THREADS, smem, s>>>(p);
+    else if (p.st.nt == 2) conv_kernel<2><<<grid, NUM_THREADS, smem, s>>>(p);
+    else conv_kernel<1><<<grid, NUM_THREADS, smem, s>>>(p);
     cudaError_t e = cudaGetLastError();
     // algorithmic: the input activations read once, the output written once
     stats_tc_end(tok, s, TFDE_KIND_CONV, 64.0 * (double)C->N, 2.0 * NTAP * CH * CH * (double)C->N);
@@ -504,43 +701,61 @@ int conv(tfde_cnn* C, const CUtensorMap& amap, const __nv_bfloat16* w, const flo
     return TFDE_OK;
 }
 
+int wgrad(tfde_cnn* C, int layer, const uint8_t* dz, cudaStream_t s) {
+    WgradParams p;
+    std::memset(&p, 0, sizeof(p));
+    p.dz = dz;
+    p.in = C->act[layer];
+    p.half_stride = C->half_stride;
+    p.st = C->wg_st;
+    p.R = (unsigned)C->R;
+    p.P = C->P;
+    p.first = C->first;
+    p.ntiles = C->wg_tiles;
+    p.part = C->wpart + (size_t)layer * C->wg_grid * GSZ;
+    p.err = C->err;
+    stats_count_launch();
+    wgrad_kernel<<<C->wg_grid, WG_THREADS, wg_smem(p.st), s>>>(p);
+    CN_TRY(cudaGetLastError());
+    return TFDE_OK;
+}
+
 int ensure_packed(tfde_cnn* C, cudaStream_t s) {
     if (C->packed) return TFDE_OK;
-    for (int l = 0; l < NL; ++l) {
-        stats_count_launch();
-        pack_weights_kernel<<<(NTAP * 256 + 255) / 256, 256, 0, s>>>(C->prm + (size_t)l * PSZ,
-                                                                        C->wf + (size_t)l * NTAP * 256,
-                                                                        C->wb + (size_t)l * NTAP * 256);
-    }
+    stats_count_launch();
+    pack_weights_kernel<<<dim3(NTAP, NL), 256, 0, s>>>(C->prm, C->wf, C->wb);
     C->packed = true;
     return TFDE_OK;
 }
 
+Grid grid_of(const tfde_cnn* C) { return Grid{C->n[0], C->n[1], (unsigned)C->R, C->P, C->half_stride}; }
+
 // forward pass of (u, dtF, coef) into C->out (plain grid, output channel 0)
 int forward(tfde_cnn* C, const double* u, const double* u1, const double* u2, const double* dtF,
             const double coef[9], cudaStream_t s) {
-    float hc[9];
-    for (int i = 0; i < 9; ++i) hc[i] = (float)coef[i];
-    CN_TRY(cudaMemcpyAsync(C->coef, hc, sizeof(hc), cudaMemcpyHostToDevice, s));
+    Coef hc;
+    for (int i = 0; i < 9; ++i) hc.c[i] = (float)coef[i];
     int st = ensure_packed(C, s);
     if (st) return st;
     stats_count_launch(2);
-    maxabs_kernel<<<1, 256, 0, s>>>(u, C->N, C->scale);
-    pack_input_kernel<<<grid1(C->N), 256, 0, s>>>(u, u1, u2, dtF, C->scale, C->coef, C->n[0], C->n[1], C->N, C->R,
-                                                    C->P, C->act[0]);
+    CN_TRY(cudaMemsetAsync(C->scale, 0, sizeof(*C->scale), s));
+    maxabs_kernel<<<grid1(C->N), 256, 0, s>>>(u, C->N, C->scale);
+    pack_input_kernel<<<grid1(C->N), 256, 0, s>>>(u, u1, u2, dtF, C->scale, hc, grid_of(C), (unsigned)C->N, C->act[0]);
     for (int l = 0; l < NL; ++l) {
         const bool last = l + 1 == NL;
-        if ((st = conv(C, C->amap[l], C->wf + (size_t)l * NTAP * 256, C->prm + (size_t)l * PSZ + WSZ, last ? 0 : 1,
+        if ((st = conv(C, C->act[l], C->wf + (size_t)l * NTAP * 256, C->prm + (size_t)l * PSZ + WSZ, last ? 0 : 1,
                        nullptr, last ? nullptr : C->act[l + 1], last ? C->out : nullptr, s)))
             return st;
     }
     return TFDE_OK;
 }
 
+// Reads the loss partials and the error flag behind them.
 int check(tfde_cnn* C, cudaStream_t s) {
-    CN_TRY(cudaMemcpyAsync(C->err_host, C->err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CN_TRY(cudaMemcpyAsync(C->lpart_host, C->lpart, (LPART + 1) * sizeof(double), cudaMemcpyDeviceToHost, s));
     CN_TRY(cudaStreamSynchronize(s));
-    if (*C->err_host) return set_error(TFDE_ETIMEOUT, "warm-start kernel wait ran out (device error flag set)");
+    if (*reinterpret_cast<const int*>(C->lpart_host + LPART))
+        return set_error(TFDE_ETIMEOUT, "warm-start kernel wait ran out (device error flag set)");
     return TFDE_OK;
 }
 
@@ -560,9 +775,25 @@ int cnn_create(const int n[3], tfde_cnn** out) {
     C->S_total = (long long)(n[2] + 2) * C->P;
     C->first = C->P + C->R + 1;
     C->count = C->S_total - 2 * C->first;   // slots from the first to the last interior point
-    C->ntiles = (C->count + TM - 1) / TM;
-    const size_t act_bytes = (size_t)C->S_total * CH * sizeof(__nv_bfloat16);
-    const int nchunks = (int)((C->count + WG_CHUNK - 1) / WG_CHUNK);
+    if (C->S_total + MAX_NT * TM >= (1LL << 31)) return set_error(TFDE_ENOMEM, "grid too large for the network");
+    // the convolution's and the weight gradient's tiles; a tile may run past
+    // the last interior slot, so every buffer ends in MAX_NT * TM more slots
+    C->conv_st = staging(C->count, C->R, CONV_FIXED_SMEM, 0);
+    C->wg_st = staging(C->count, C->R, WG_SMEM_FIXED, 32);
+    C->conv_tiles = (int)((C->count + C->conv_st.tile - 1) / C->conv_st.tile);
+    C->wg_tiles = (int)((C->count + C->wg_st.tile - 1) / C->wg_st.tile);
+    C->wg_grid = std::min(C->wg_tiles, tc::num_sms());
+    C->half_stride = (C->S_total + MAX_NT * TM) * 16;
+    const size_t act_bytes = 2 * (size_t)C->half_stride;
+    for (auto f : {conv_kernel<1>, conv_kernel<2>, conv_kernel<4>})
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM) != cudaSuccess) {
+            delete C;
+            return set_error(TFDE_ECUDA, "cudaFuncSetAttribute(conv_kernel) failed");
+        }
+    if (cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM) != cudaSuccess) {
+        delete C;
+        return set_error(TFDE_ECUDA, "cudaFuncSetAttribute(wgrad_kernel) failed");
+    }
     bool ok = cudaMalloc((void**)&C->prm, NL * PSZ * sizeof(float)) == cudaSuccess &&
               cudaMalloc((void**)&C->grad, NL * PSZ * sizeof(float)) == cudaSuccess &&
               cudaMalloc((void**)&C->adam_m, NL * PSZ * sizeof(float)) == cudaSuccess &&
@@ -572,37 +803,27 @@ int cnn_create(const int n[3], tfde_cnn** out) {
               cudaMalloc((void**)&C->dz, act_bytes) == cudaSuccess &&
               cudaMalloc((void**)&C->dz2, act_bytes) == cudaSuccess &&
               cudaMalloc((void**)&C->out, C->N * sizeof(float)) == cudaSuccess &&
-              cudaMalloc((void**)&C->coef, 16 * sizeof(float)) == cudaSuccess &&
-              cudaMalloc((void**)&C->scale, sizeof(double)) == cudaSuccess &&
-              cudaMalloc((void**)&C->wpart, (size_t)nchunks * NTAP * 256 * sizeof(float)) == cudaSuccess &&
-              cudaMalloc((void**)&C->lpart, 1216 * sizeof(double)) == cudaSuccess &&
-              cudaMallocHost((void**)&C->lpart_host, 1216 * sizeof(double)) == cudaSuccess &&
-              cudaMalloc((void**)&C->err, sizeof(int)) == cudaSuccess &&
-              cudaMallocHost((void**)&C->err_host, sizeof(int)) == cudaSuccess;
+              cudaMalloc((void**)&C->scale, sizeof(*C->scale)) == cudaSuccess &&
+              cudaMalloc((void**)&C->wpart, (size_t)NL * C->wg_grid * GSZ * sizeof(double)) == cudaSuccess &&
+              cudaMalloc((void**)&C->lpart, (LPART + 1) * sizeof(double)) == cudaSuccess &&
+              cudaMallocHost((void**)&C->lpart_host, (LPART + 1) * sizeof(double)) == cudaSuccess;
     for (int l = 0; l < NL && ok; ++l) ok = cudaMalloc((void**)&C->act[l], act_bytes) == cudaSuccess;
     if (!ok) {
         cnn_destroy(C);
         return set_error(TFDE_ENOMEM, "allocation of the warm-start network workspace failed");
     }
+    C->err = reinterpret_cast<int*>(C->lpart + LPART);
     // guard slots must stay zero: every buffer on the padded grid starts zeroed
     bool z = cudaMemset(C->dz, 0, act_bytes) == cudaSuccess && cudaMemset(C->dz2, 0, act_bytes) == cudaSuccess &&
              cudaMemset(C->prm, 0, NL * PSZ * sizeof(float)) == cudaSuccess &&
              cudaMemset(C->grad, 0, NL * PSZ * sizeof(float)) == cudaSuccess &&
              cudaMemset(C->adam_m, 0, NL * PSZ * sizeof(float)) == cudaSuccess &&
              cudaMemset(C->adam_v, 0, NL * PSZ * sizeof(float)) == cudaSuccess &&
-             cudaMemset(C->err, 0, sizeof(int)) == cudaSuccess;
+             cudaMemset(C->lpart, 0, (LPART + 1) * sizeof(double)) == cudaSuccess;
     for (int l = 0; l < NL && z; ++l) z = cudaMemset(C->act[l], 0, act_bytes) == cudaSuccess;
     if (!z) {
         cnn_destroy(C);
         return set_error(TFDE_ECUDA, "zeroing of the warm-start workspace failed");
-    }
-    int st = TFDE_OK;
-    for (int l = 0; l < NL && !st; ++l) st = make_act_map(&C->amap[l], C->act[l], C->S_total);
-    if (!st) st = make_act_map(&C->dmap[0], C->dz, C->S_total);
-    if (!st) st = make_act_map(&C->dmap[1], C->dz2, C->S_total);
-    if (st) {
-        cnn_destroy(C);
-        return st;
     }
     *out = C;
     return TFDE_OK;
@@ -621,13 +842,10 @@ int cnn_destroy(tfde_cnn* C) {
     cudaFree(C->dz);
     cudaFree(C->dz2);
     cudaFree(C->out);
-    cudaFree(C->coef);
     cudaFree(C->scale);
     cudaFree(C->wpart);
     cudaFree(C->lpart);
     if (C->lpart_host) cudaFreeHost(C->lpart_host);
-    cudaFree(C->err);
-    if (C->err_host) cudaFreeHost(C->err_host);
     delete C;
     return TFDE_OK;
 }
@@ -663,31 +881,22 @@ int cnn_accumulate(tfde_cnn* C, const double* u, const double* u1, const double*
     int st = forward(C, u, u1, u2, dtF, coef, s);
     if (st) return st;
     const int nb = grid1(C->N);
-    stats_count_launch();
-    CN_TRY(cudaMemsetAsync(C->dz, 0, (size_t)C->S_total * CH * sizeof(__nv_bfloat16), s));
-    loss_grad_kernel<<<nb, 256, 0, s>>>(C->out, u, u1, u2, u_next, C->scale, C->n[0], C->n[1], C->N, C->R, C->P,
-                                         C->dz, C->lpart);
-    const int nchunks = (int)((C->count + WG_CHUNK - 1) / WG_CHUNK);
-    __nv_bfloat16* g = C->dz;      // gradient w.r.t. the output of layer l (pre-activation for l < NL - 1 after masking)
-    __nv_bfloat16* g2 = C->dz2;
-    int gm = 0;
+    stats_count_launch(2);
+    loss_grad_kernel<<<nb, 256, 0, s>>>(C->out, u, u1, u2, u_next, C->scale, grid_of(C), (unsigned)C->N, C->dz,
+                                         C->lpart);
+    uint8_t* g = C->dz;      // gradient w.r.t. the output of layer l (pre-activation for l < NL - 1 after masking)
+    uint8_t* g2 = C->dz2;
     for (int l = NL - 1; l >= 0; --l) {
-        float* gW = C->grad + (size_t)l * PSZ;
-        stats_count_launch(3);
-        wgrad_kernel<<<dim3((unsigned)nchunks, NTAP), 256, 0, s>>>(g, C->act[l], C->first, C->count, C->R, C->P,
-                                                                  C->wpart);
-        wgrad_reduce_kernel<<<(NTAP * 256 + 255) / 256, 256, 0, s>>>(C->wpart, nchunks, gW);
-        bgrad_kernel<<<CH, 256, 0, s>>>(g, C->first, C->count, gW + WSZ);
+        if ((st = wgrad(C, l, g, s))) return st;
         if (l > 0) {
             // gradient w.r.t. the input of layer l, masked by the ReLU of layer l - 1
-            if ((st = conv(C, C->dmap[gm], C->wb + (size_t)l * NTAP * 256, nullptr, 0, C->act[l], g2, nullptr, s)))
-                return st;
+            if ((st = conv(C, g, C->wb + (size_t)l * NTAP * 256, nullptr, 0, C->act[l], g2, nullptr, s))) return st;
             std::swap(g, g2);
-            gm ^= 1;
         }
     }
+    wgrad_reduce_kernel<<<dim3((GSZ + 31) / 32, NL), 256, 0, s>>>(C->wpart, C->wg_grid, C->grad);
+    CN_TRY(cudaGetLastError());
     C->accumulated++;
-    CN_TRY(cudaMemcpyAsync(C->lpart_host, C->lpart, nb * sizeof(double), cudaMemcpyDeviceToHost, s));
     if ((st = check(C, s))) return st;
     double acc = 0.0;
     for (int b = 0; b < nb; ++b) acc += C->lpart_host[b];
