@@ -25,6 +25,9 @@
 // 4096 / L complex lines (64 KB in FP64), 256 threads, each pass reads its
 // butterflies into registers, synchronises and writes the reordered results.
 //
+// Short axes take a dense product on CUDA cores instead of the transforms
+// (tfde_line_kernel.cuh; line_limit below says up to which length and why).
+//
 // One launch is one pass along one axis over all lines of the grid:
 //   MODE_TOEPLITZ  out0 = alpha T in0 + beta M in1,  out1 = M in0
 //                  (M = tridiag(1, 6, 1) / 8, the mass stencil; in1 / out1
@@ -34,6 +37,8 @@
 //   MODE_DST       out0 = S in0;
 //   MODE_DST2      out0 = S Lambda^{-1} S in0 along z (the middle of
 //                  Eq. (diag_tau_pre), both z transforms in one pass).
+#include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <complex>
 #include <cstring>
@@ -42,6 +47,7 @@
 
 #include "tfde_fft.h"
 #include "tfde_stats.h"
+#include "tfde_tc.h"
 
 namespace tfde {
 namespace fft {
@@ -479,6 +485,75 @@ int upload_spectrum(const std::vector<long double>& t, int n, int L, Table* out,
     return st;
 }
 
+// The axis lengths up to which a pass takes the dense product of
+// tfde_line_kernel.cuh instead of the transforms, from GB300 times per
+// operator (three passes, 3-D cubes) or preconditioner application (six
+// products), dense against FFT in us:
+//   FP64  unsplit Toeplitz  64: 124 / 238,  96: 478 / 454
+//         split Toeplitz   127: 793 / 926, 191: 4756 / 3912
+//         DST              127: 1482 / 2982, 191: 9191 / 14533 (n^4 against n^3 log n from there)
+//   FP32  unsplit Toeplitz 127: 113 / 188, 255: 1012 / 1179
+//         split Toeplitz   255: 751 / 1178
+//         DST              127: 126 / 387, 255: 1025 / 3032
+// and where the grid does not fill the chip, where the transforms' serial
+// passes count instead of the arithmetic: 511 x 511: 53 / 64 and 68 / 105.
+int line_limit(bool fp64, int form, size_t N) {
+    if (fp64) return form == 0 ? 88 : (form == 1 ? 168 : 232);
+    if (N < (size_t)1 << 19) return 640;
+    return form == 0 ? 288 : (form == 1 ? 384 : 640);
+}
+
+// The dense matrices of the line passes, formed on the device from the
+// problem's own; FP32 ones only where the inner solves run on these passes.
+int line_init(tfde_problem* P, State* F, cudaStream_t s) {
+    const bool fmix = P->prec == TFDE_MIXED && fmix_wanted(P);
+    if (P->prec == TFDE_MIXED && !fmix) return TFDE_OK;   // tensor-core problems: fallback paths only
+    struct Job {
+        LineMatrix* m;
+        const double* src;
+        int n, form;
+        bool fp64;
+    };
+    std::vector<Job> jobs;
+    size_t total = 0;
+    for (int t = 0; t < (fmix ? 2 : 1); ++t) {
+        for (int a = 0; a < 3; ++a) {
+            const int n = P->n[a];
+            const int tform = P->p.kp[a] == P->p.km[a] ? 1 : 0;
+            if (n <= line_limit(t == 0, tform, P->N)) {
+                jobs.push_back({&F->lG[t][a], P->G[a], n, tform, t == 0});
+                if (a == 0)
+                    for (int k = 0; k < 2; ++k) jobs.push_back({&F->lGhat[t][k], P->Ghat[k], n, tform, t == 0});
+            }
+            if (n <= line_limit(t == 0, 2, P->N)) jobs.push_back({&F->lS[t][a], P->S[a], n, 2, t == 0});
+        }
+    }
+    auto bytes = [](Job& j) {
+        LineMatrix& m = *j.m;
+        m.K = j.form ? (j.n + 1) / 2 : j.n;
+        // split rows: half of them sums, half differences, in multiples of 8
+        // and at most LINE_ROWS together; unsplit: multiples of 16
+        m.half = j.form ? std::min(LINE_ROWS / 2, (m.K + 7) / 8 * 8) : 0;
+        m.ld = j.form ? (m.K + m.half - 1) / m.half * 2 * m.half : (j.n + 15) / 16 * 16;
+        if (m.ld > LINE_ROWS) m.ld = (m.ld + LINE_ROWS - 1) / LINE_ROWS * LINE_ROWS;
+        return (size_t)m.K * m.ld * (j.fp64 ? 8 : 4);   // multiples of 32 bytes
+    };
+    for (Job& j : jobs) total += bytes(j);
+    if (jobs.empty()) return TFDE_OK;
+    if (cudaMalloc(&F->line_mem, total) != cudaSuccess) return set_error(TFDE_ENOMEM, "cudaMalloc of line matrices failed");
+    unsigned char* at = static_cast<unsigned char*>(F->line_mem);
+    for (Job& j : jobs) {
+        j.m->m = at;
+        at += bytes(j);
+        const unsigned grid = (unsigned)std::min<size_t>(((size_t)j.m->K * j.m->ld + 255) / 256, 1216);
+        stats_count_launch();
+        if (j.fp64) line_matrix_kernel<double><<<grid, 256, 0, s>>>(j.src, j.n, j.form, *j.m);
+        else line_matrix_kernel<float><<<grid, 256, 0, s>>>(j.src, j.n, j.form, *j.m);
+        if (cudaGetLastError() != cudaSuccess) return set_error(TFDE_ECUDA, "line_matrix_kernel launch failed");
+    }
+    return TFDE_OK;
+}
+
 }  // namespace
 
 bool available(const int n[3]) {
@@ -572,7 +647,7 @@ int init(tfde_problem* P, cudaStream_t s) {
             for (double v : P->lam_tau[a]) lf.push_back((float)v);
         if (int st = dcopy(&F->lamf, lf, s)) return st;
     }
-    return TFDE_OK;
+    return line_init(P, F, s);
 }
 
 void free_state(tfde_problem* P) {
@@ -591,6 +666,7 @@ void free_state(tfde_problem* P) {
     rel(F->Ghat[0]);
     rel(F->Ghat[1]);
     cudaFree(F->lamf);
+    cudaFree(F->line_mem);
     delete F;
     P->fft = nullptr;
 }
@@ -646,9 +722,93 @@ Pass base_pass(const tfde_problem* P, int axis, bool fp64) {
     return p;
 }
 
+// ------------------------------------------------ dense line passes
+constexpr int kLineSmem = 232448;
+
+size_t line_smem(const LinePass& p, int es, int BN, int rows, bool pair) {
+    const int BNS = BN + 16 / es;
+    const size_t lines = (size_t)(pair ? p.n + rows : std::max(p.n, rows)) + (p.in1 ? p.n : 0);
+    return (lines * BNS + (size_t)LINE_STAGES * (64 / es) * rows) * es;
+}
+
+template <typename R, int MODE, int TL, int LT, int RT>
+int launch_line(const LinePass& p, cudaStream_t s) {
+    constexpr int BN = TL * LT;
+    static_assert(256 / TL * RT == LINE_ROWS, "a block's rows");
+    static std::atomic<unsigned long long> ready{0};   // a bit per device
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(ready.load(std::memory_order_relaxed) & bit)) {
+        if (cudaFuncSetAttribute(line_pass_kernel<R, MODE, TL, LT, RT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kLineSmem) != cudaSuccess)
+            return set_error(TFDE_ECUDA, "cudaFuncSetAttribute(line_pass_kernel) failed");
+        ready.fetch_or(bit, std::memory_order_relaxed);
+    }
+    // rows per block: LINE_ROWS, or all of a smaller matrix (a multiple of 16): whole warps
+    const int rows = std::min(p.m.ld, LINE_ROWS);
+    const int gy = (p.m.ld + LINE_ROWS - 1) / LINE_ROWS;
+    const long long blocks = (p.lines + BN - 1) / BN;
+    const double N = (double)p.lines * p.n;
+    const double nio = 2.0 + (p.in1 ? 1.0 : 0.0) + (p.out1 ? 1.0 : 0.0);
+    const double fl = 2.0 * (double)p.m.K * p.n * (double)p.lines;
+    void* tok = stats_tc_begin(s, TFDE_KIND_FFT);
+    line_pass_kernel<R, MODE, TL, LT, RT><<<dim3((unsigned)blocks, (unsigned)gy), rows / RT * TL,
+                                           line_smem(p, sizeof(R), BN, rows, MODE == LINE_DST2), s>>>(p);
+    const cudaError_t e = cudaGetLastError();
+    stats_tc_end(tok, s, TFDE_KIND_FFT, nio * N * sizeof(R), fl * (MODE == LINE_DST2 ? 2.0 : 1.0));
+    if (e != cudaSuccess) return set_error(TFDE_ECUDA, std::string("line_pass_kernel: ") + cudaGetErrorString(e));
+    return TFDE_OK;
+}
+
+// Lines per block: FP32 64, 32 or 16 (8 rows x 4, 2 or 1 lines per thread),
+// the largest that fits and still gives every SM two blocks, so that one's
+// copies run under the other's product; FP64, bound by its pipe (two
+// multiply-adds per clock and SM), always 8 (4 rows x 1 line), for the even
+// spread over the SMs.
+template <typename R, int MODE>
+int line_pass(const LinePass& p, cudaStream_t s) {
+    if constexpr (sizeof(R) == 4) {
+        const int rows = std::min(p.m.ld, LINE_ROWS);
+        auto takes = [&](int BN) {
+            const long long blocks = (p.lines + BN - 1) / BN * ((p.m.ld + LINE_ROWS - 1) / LINE_ROWS);
+            return blocks >= 2 * tc::num_sms() && line_smem(p, 4, BN, rows, MODE == LINE_DST2) <= kLineSmem / 2;
+        };
+        if (takes(64)) return launch_line<R, MODE, 16, 4, 8>(p, s);
+        if (takes(32)) return launch_line<R, MODE, 16, 2, 8>(p, s);
+        return launch_line<R, MODE, 16, 1, 8>(p, s);
+    } else {
+        return launch_line<R, MODE, 8, 1, 4>(p, s);
+    }
+}
+
 template <typename R>
-int toeplitz_pass(const tfde_problem* P, int axis, const Table& T, double alpha, const R* in0, const R* in1,
-                  double beta, R* out0, R* out1, cudaStream_t s) {
+LinePass base_line(const tfde_problem* P, int axis, const LineMatrix& m) {
+    LinePass p;
+    std::memset(&p, 0, sizeof(p));
+    p.m = m;
+    p.n1 = P->n[0];
+    p.n2 = P->n[1];
+    p.n3 = P->n[2];
+    p.axis = axis;
+    p.n = P->n[axis];
+    p.lines = (long long)P->N / P->n[axis];
+    return p;
+}
+
+template <typename R>
+int toeplitz_pass(const tfde_problem* P, int axis, const Table& T, const LineMatrix& m, double alpha, const R* in0,
+                  const R* in1, double beta, R* out0, R* out1, cudaStream_t s) {
+    if (m.K) {
+        LinePass q = base_line<R>(P, axis, m);
+        q.alpha = alpha;
+        q.beta = beta;
+        q.in0 = in0;
+        q.in1 = in1;
+        q.out0 = out0;
+        q.out1 = out1;
+        return line_pass<R, LINE_TOEPLITZ>(q, s);
+    }
     Pass p = base_pass(P, axis, sizeof(R) == 8);
     p.spec = sizeof(R) == 8 ? (const void*)T.d : (const void*)T.f;
     p.alpha = alpha;
@@ -661,14 +821,27 @@ int toeplitz_pass(const tfde_problem* P, int axis, const Table& T, double alpha,
 }
 
 template <typename R>
-int dst_pass(const tfde_problem* P, int axis, const R* in, R* out, bool lambda_pair, cudaStream_t s,
-             bool half_power = false) {
+int dst_pass(const tfde_problem* P, int axis, const R* in, R* out, bool lambda, bool lambda_only, cudaStream_t s,
+             bool half_power) {
     const State* F = static_cast<const State*>(P->fft);
+    const LineMatrix& m = F->lS[sizeof(R) == 8 ? 0 : 1][axis];
+    if (m.K) {
+        LinePass q = base_line<R>(P, axis, m);
+        q.in0 = in;
+        q.out0 = out;
+        if (!lambda) return line_pass<R, LINE_DST>(q, s);
+        q.lam = sizeof(R) == 8 ? (const void*)P->lam : (const void*)F->lamf;
+        q.c0 = P->csum[0];
+        q.c1 = P->csum[1];
+        q.c2 = P->csum[2];
+        q.half_power = half_power ? 1 : 0;
+        return lambda_only ? line_pass<R, LINE_DST>(q, s) : line_pass<R, LINE_DST2>(q, s);
+    }
     Pass p = base_pass(P, axis, sizeof(R) == 8);
     p.spec = sizeof(R) == 8 ? (const void*)F->chirp[axis].d : (const void*)F->chirp[axis].f;
     p.in0 = in;
     p.out0 = out;
-    if (lambda_pair) {
+    if (lambda) {
         p.lam = P->lam;
         p.lamf = F->lamf;
         p.c0 = P->csum[0];
@@ -688,36 +861,56 @@ int apply_A(const tfde_problem* P, int op, const R* x, R* y, R* a, R* w, R* c, R
     const bool rhs = (op & 1) != 0;
     const bool stiff = (op & TFDE_OP_STIFF) != 0;
     const double sg = rhs ? -1.0 : 1.0;
+    const int t = sizeof(R) == 8 ? 0 : 1;
     int st;
     // x: a = Ghat1 x (or sg eta1 B1 x for the stiffness terms alone), w = M1 x
-    if (stiff) st = toeplitz_pass<R>(P, 0, F->G[0], sg, x, nullptr, 0.0, a, w, s);
-    else st = toeplitz_pass<R>(P, 0, F->Ghat[rhs ? 1 : 0], 1.0, x, nullptr, 0.0, a, w, s);
+    if (stiff) st = toeplitz_pass<R>(P, 0, F->G[0], F->lG[t][0], sg, x, nullptr, 0.0, a, w, s);
+    else st = toeplitz_pass<R>(P, 0, F->Ghat[rhs ? 1 : 0], F->lGhat[t][rhs ? 1 : 0], 1.0, x, nullptr, 0.0, a, w, s);
     if (st) return st;
     // 2-D problem: the y pass gives the result (no third axis)
-    if (P->dim2) return toeplitz_pass<R>(P, 1, F->G[1], sg, w, a, 1.0, y, nullptr, s);
+    if (P->dim2) return toeplitz_pass<R>(P, 1, F->G[1], F->lG[t][1], sg, w, a, 1.0, y, nullptr, s);
     // y: c = sg G2 w + M2 a, e = M2 w
-    if ((st = toeplitz_pass<R>(P, 1, F->G[1], sg, w, a, 1.0, c, e, s))) return st;
+    if ((st = toeplitz_pass<R>(P, 1, F->G[1], F->lG[t][1], sg, w, a, 1.0, c, e, s))) return st;
     // z: y = sg G3 e + M3 c
-    return toeplitz_pass<R>(P, 2, F->G[2], sg, e, c, 1.0, y, nullptr, s);
+    return toeplitz_pass<R>(P, 2, F->G[2], F->lG[t][2], sg, e, c, 1.0, y, nullptr, s);
+}
+
+// S_N Lambda^{-1} S_N r (half_power: Lambda^{-1/2}): forward along x (and y),
+// the pair around Lambda along the last axis, and back.  A 2-D problem's pair
+// runs along y where its matrix is dense.  A dense pair is one pass while a
+// block holds every row of its lines, else two (the first divides by Lambda).
+template <typename R>
+int pinv(const tfde_problem* P, const R* r, R* z, R* t1, R* t2, bool half_power, cudaStream_t s) {
+    const State* F = static_cast<const State*>(P->fft);
+    const int t = sizeof(R) == 8 ? 0 : 1;
+    const int last = P->dim2 && F->lS[t][1].K ? 1 : 2;
+    const LineMatrix& m = F->lS[t][last];
+    const bool two = m.K && m.ld > LINE_ROWS;
+    const R* src = r;
+    R* buf[2] = {t1, t2};
+    int b = 0, st;
+    auto step = [&](int axis, bool lam, R* to) {
+        int e = dst_pass<R>(P, axis, src, to, lam, two, s, half_power);
+        src = to;
+        b ^= 1;
+        return e;
+    };
+    for (int a = 0; a < last; ++a)
+        if ((st = step(a, false, buf[b]))) return st;
+    if ((st = step(last, true, buf[b]))) return st;
+    if (two && (st = step(last, false, buf[b]))) return st;
+    for (int a = last - 1; a >= 0; --a)
+        if ((st = step(a, false, a == 0 ? z : buf[b]))) return st;
+    return TFDE_OK;
 }
 
 template <typename R>
 int apply_Pinv(const tfde_problem* P, const R* r, R* z, R* t1, R* t2, cudaStream_t s) {
-    int st;
-    if ((st = dst_pass<R>(P, 0, r, t1, false, s))) return st;
-    if ((st = dst_pass<R>(P, 1, t1, t2, false, s))) return st;
-    if ((st = dst_pass<R>(P, 2, t2, t1, true, s))) return st;   // S_z Lambda^{-1} S_z
-    if ((st = dst_pass<R>(P, 1, t1, t2, false, s))) return st;
-    return dst_pass<R>(P, 0, t2, z, false, s);
+    return pinv<R>(P, r, z, t1, t2, false, s);
 }
 
 int apply_Pinv_half(const tfde_problem* P, const double* r, double* z, double* t1, double* t2, cudaStream_t s) {
-    int st;
-    if ((st = dst_pass<double>(P, 0, r, t1, false, s))) return st;
-    if ((st = dst_pass<double>(P, 1, t1, t2, false, s))) return st;
-    if ((st = dst_pass<double>(P, 2, t2, t1, true, s, true))) return st;   // S_z Lambda^{-1/2} S_z
-    if ((st = dst_pass<double>(P, 1, t1, t2, false, s))) return st;
-    return dst_pass<double>(P, 0, t2, z, false, s);
+    return pinv<double>(P, r, z, t1, t2, true, s);
 }
 
 template int apply_A<double>(const tfde_problem*, int, const double*, double*, double*, double*, double*, double*,

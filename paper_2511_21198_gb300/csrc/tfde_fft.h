@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "tfde_internal.h"
+#include "tfde_line_kernel.cuh"
 
 namespace tfde {
 namespace fft {
@@ -26,6 +27,10 @@ struct State {
     Table pre[3];       // DST phases exp(i pi j^2 / (2(n+1))), j = 1..n
     Table chirp[3];     // spectrum / L of the chirp exp(-i pi m^2 / (2(n+1)))
     double dst_scale[3] = {0, 0, 0};
+    // dense per-axis matrices of the line passes, FP64 [0] and FP32 [1]; an
+    // empty one (K = 0) leaves the axis to the FFT passes
+    LineMatrix lG[2][3], lGhat[2][2], lS[2][3];
+    void* line_mem = nullptr;   // their storage, one allocation
     float* lamf = nullptr;   // the mass and tau eigenvalues of every axis in FP32 (as tfde_problem::lam)
 };
 
