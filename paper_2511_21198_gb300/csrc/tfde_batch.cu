@@ -21,6 +21,7 @@
 #include "tfde_mixed.h"
 #include "tfde_stats.h"
 #include "tfde_chain.cuh"
+#include "tfde_gs.cuh"
 
 namespace tfde {
 
@@ -72,15 +73,7 @@ __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16& hi, __nv_bflo
     lo = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
 
-struct KSum {
-    float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float v) {
-        const float y = v - c;
-        const float t = s + y;
-        c = (t - s) - y;
-        s = t;
-    }
-};
+using gs::KSum;
 
 __device__ __forceinline__ double block_sum(double v) {
     __shared__ double sh[kBT / 32];
@@ -95,6 +88,7 @@ __device__ __forceinline__ double block_sum(double v) {
     return t;
 }
 
+static_assert(kBT == gs::kThreads, "block width of the Gram-Schmidt sweeps");
 // The chunk of block b: problem bi[b], elements [bo[b], min(bo[b] + kCH, N)).
 #define BK_PROLOGUE                                        \
     const int inst = bi[blockIdx.x];                       \
@@ -118,31 +112,13 @@ __global__ __launch_bounds__(kBT) void bk_scale64to32(const BVec* __restrict__ v
 }
 
 // <V_{m0+j}, V_jw>, j < mc (<= 8), per block into part[(m0 + j) * NB + b]
-__global__ __launch_bounds__(kBT) void bk_multidot(const BVec* __restrict__ vt, const int* __restrict__ bi,
-                                                  const long long* __restrict__ bo, const int* __restrict__ act,
-                                                  int m0, int mc, int jw, double* __restrict__ part) {
-    const int inst = bi[blockIdx.x];
-    const bool on = act[inst] != 0;
-    KSum k[8];
-    if (on) {
-        const BVec& v = vt[inst];
-        const long long e0 = bo[blockIdx.x];
-        const long long e1 = e0 + kCH < v.N ? e0 + kCH : v.N;
-        const float* w = v.V + (long long)jw * v.N;
-        for (long long e = e0 + threadIdx.x; e < e1; e += kBT) {
-            const float we = w[e];
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (j < mc) k[j].add(v.V[(long long)(m0 + j) * v.N + e] * we);
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        if (j < mc) {
-            const double t = block_sum((double)k[j].s - (double)k[j].c);
-            if (threadIdx.x == 0) part[(long long)(m0 + j) * gridDim.x + blockIdx.x] = t;
-        }
-    }
+__global__ __launch_bounds__(kBT, 2) void bk_multidot(const BVec* __restrict__ vt, const int* __restrict__ bi,
+                                                     const long long* __restrict__ bo, const int* __restrict__ act,
+                                                     int m0, int mc, int jw, double* __restrict__ part) {
+    BK_PROLOGUE
+    const long long N = v.N;
+    gs::dots(v.V, N, m0, mc, v.V + (long long)jw * N, e0, e1, true,
+             [&](int j, double sum) { part[(long long)j * gridDim.x + blockIdx.x] = sum; });
 }
 
 // out[i * ostride + ooff + j] = sum over problem i's blocks of part[(p0 + j) * NB + b], j < m
@@ -151,6 +127,7 @@ __global__ void bk_reduce(const double* __restrict__ part, int NB, const int* __
     const int inst = blockIdx.x, j = blockIdx.y;
     if (!act[inst]) return;
     double acc = 0.0;
+#pragma unroll 8
     for (int b = bstart[inst] + threadIdx.x; b < bstart[inst + 1]; b += 32) acc += part[(long long)(p0 + j) * NB + b];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -165,12 +142,17 @@ __global__ __launch_bounds__(kBT) void bk_multiaxpy(const BVec* __restrict__ vt,
     __shared__ float hs[64];
     for (int j = threadIdx.x; j < m; j += blockDim.x) hs[j] = (float)coef[inst * kHS + coff + j];
     __syncthreads();
-    float* w = jt >= 0 ? v.V + (long long)jt * v.N : v.x32;
-    for (long long e = e0 + threadIdx.x; e < e1; e += kBT) {
-        float acc = w[e];
-        for (int j = 0; j < m; ++j) acc = fmaf(-hs[j], v.V[(long long)j * v.N + e], acc);
-        w[e] = acc;
-    }
+    const float* V = v.V;
+    const long long N = v.N;
+    float* w = jt >= 0 ? v.V + (long long)jt * N : v.x32;
+    gs::sweep(
+        e0, e1, true,
+        [&](long long i) {
+            float4 wi = *reinterpret_cast<const float4*>(w + i);
+            gs::update4(wi, V, N, hs, m, i);
+            *reinterpret_cast<float4*>(w + i) = wi;
+        },
+        [&](long long i) { w[i] = gs::update1(w[i], V, N, hs, m, i); });
 }
 
 // V_jw *= sc ; split into (ph, pl)
@@ -396,39 +378,20 @@ __global__ __launch_bounds__(kBT) void bkp_direction(const BVec* __restrict__ vt
 // from *jd (device), the new vector is the fixed per-problem W.
 // Block partial sums of <V_{m0+t}, W> for t < min(8, j + 1 - m0), or (ww) of
 // <W, W> into row R + 1.
-__global__ __launch_bounds__(kBT) void bkg_dots(const BVec* __restrict__ vt, const int* __restrict__ bi,
+__global__ __launch_bounds__(kBT, 2) void bkg_dots(const BVec* __restrict__ vt, const int* __restrict__ bi,
                                                const long long* __restrict__ bo, const int* __restrict__ act,
                                                int m0, const int* __restrict__ jd, int R, int ww,
                                                double* __restrict__ part) {
-    const int inst = bi[blockIdx.x];
     const int j = *jd;
     const int mc = ww ? 1 : min(8, j + 1 - m0);
     if (mc <= 0) return;
-    const bool on = act[inst] != 0;
-    KSum k[8];
-    if (on) {
-        const BVec& v = vt[inst];
-        const long long e0 = bo[blockIdx.x];
-        const long long e1 = e0 + kCH < v.N ? e0 + kCH : v.N;
-        for (long long e = e0 + threadIdx.x; e < e1; e += kBT) {
-            const float we = v.W[e];
-            if (ww) {
-                k[0].add(we * we);
-                continue;
-            }
-#pragma unroll
-            for (int t = 0; t < 8; ++t)
-                if (t < mc) k[t].add(v.V[(long long)(m0 + t) * v.N + e] * we);
-        }
-    }
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        if (t < mc) {
-            const double sum = block_sum((double)k[t].s - (double)k[t].c);
-            const int row = ww ? R + 1 : m0 + t;
-            if (threadIdx.x == 0) part[(long long)row * gridDim.x + blockIdx.x] = sum;
-        }
-    }
+    BK_PROLOGUE
+    if (ww)
+        gs::update_norm(nullptr, 4, nullptr, 0, v.W, e0, e1, true,
+                        [&](double sum) { part[(long long)(R + 1) * gridDim.x + blockIdx.x] = sum; });
+    else
+        gs::dots(v.V, v.N, m0, mc, v.W, e0, e1, true,
+                 [&](int t, double sum) { part[(long long)t * gridDim.x + blockIdx.x] = sum; });
 }
 
 // out[i * ostride + ooff + t] = sum over problem i's blocks, t <= j (rows
@@ -440,6 +403,7 @@ __global__ void bkg_reduce(const double* __restrict__ part, int NB, const int* _
     if (!act[inst] || t > (ww ? 0 : *jd)) return;
     const int row = ww ? R + 1 : t;
     double acc = 0.0;
+#pragma unroll 8
     for (int b = bstart[inst] + threadIdx.x; b < bstart[inst + 1]; b += 32) acc += part[(long long)row * NB + b];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -449,9 +413,8 @@ __global__ void bkg_reduce(const double* __restrict__ part, int NB, const int* _
 // The second Gram-Schmidt pass's projections fused with the first pass's
 // update: W -= sum_{t <= j} coef[i * kHS + coff + t] V_t over the block's
 // chunk, then the block partial sums of <V_t, W> (t <= j) of the updated
-// chunk into rows t of part (each thread re-reads the elements it wrote):
-// the arithmetic of a plain multi-axpy followed by bkg_dots.
-__global__ __launch_bounds__(kBT) void bkg_axpy_dots(const BVec* __restrict__ vt, const int* __restrict__ bi,
+// chunk into rows t of part.
+__global__ __launch_bounds__(kBT, 2) void bkg_axpy_dots(const BVec* __restrict__ vt, const int* __restrict__ bi,
                                                     const long long* __restrict__ bo, const int* __restrict__ act,
                                                     const int* __restrict__ jd, const double* __restrict__ coef,
                                                     int coff, double* __restrict__ part) {
@@ -460,28 +423,8 @@ __global__ __launch_bounds__(kBT) void bkg_axpy_dots(const BVec* __restrict__ vt
     __shared__ float hs[64];
     for (int t = threadIdx.x; t < m; t += blockDim.x) hs[t] = (float)coef[inst * kHS + coff + t];
     __syncthreads();
-    for (long long e = e0 + threadIdx.x; e < e1; e += kBT) {
-        float acc = v.W[e];
-        for (int t = 0; t < m; ++t) acc = fmaf(-hs[t], v.V[(long long)t * v.N + e], acc);
-        v.W[e] = acc;
-    }
-    for (int m0 = 0; m0 < m; m0 += 8) {
-        const int mc = min(8, m - m0);
-        KSum k[8];
-        for (long long e = e0 + threadIdx.x; e < e1; e += kBT) {
-            const float we = v.W[e];
-#pragma unroll
-            for (int t = 0; t < 8; ++t)
-                if (t < mc) k[t].add(v.V[(long long)(m0 + t) * v.N + e] * we);
-        }
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            if (t < mc) {
-                const double sum = block_sum((double)k[t].s - (double)k[t].c);
-                if (threadIdx.x == 0) part[(long long)(m0 + t) * gridDim.x + blockIdx.x] = sum;
-            }
-        }
-    }
+    gs::update_dots(v.V, v.N, hs, m, v.W, e0, e1, true,
+                    [&](int t, double sum) { part[(long long)t * gridDim.x + blockIdx.x] = sum; });
 }
 
 // The second pass's update fused with ||W||^2: W -= sum_{t <= j} coef V_t and
@@ -495,15 +438,8 @@ __global__ __launch_bounds__(kBT) void bkg_axpy_ww(const BVec* __restrict__ vt, 
     __shared__ float hs[64];
     for (int t = threadIdx.x; t < m; t += blockDim.x) hs[t] = (float)coef[inst * kHS + coff + t];
     __syncthreads();
-    KSum k;
-    for (long long e = e0 + threadIdx.x; e < e1; e += kBT) {
-        float acc = v.W[e];
-        for (int t = 0; t < m; ++t) acc = fmaf(-hs[t], v.V[(long long)t * v.N + e], acc);
-        v.W[e] = acc;
-        k.add(acc * acc);
-    }
-    const double sum = block_sum((double)k.s - (double)k.c);
-    if (threadIdx.x == 0) part[(long long)(R + 1) * gridDim.x + blockIdx.x] = sum;
+    gs::update_norm(v.V, v.N, hs, m, v.W, e0, e1, true,
+                    [&](double sum) { part[(long long)(R + 1) * gridDim.x + blockIdx.x] = sum; });
 }
 
 // V_{j+1} = W sc and its split planes (ph, pl)

@@ -7,6 +7,7 @@
 
 #include "tfde_internal.h"
 #include "tfde_stats.h"
+#include "tfde_gs.cuh"
 #include "tfde_mixed.h"
 #include "tfde_pow2conv.cuh"
 
@@ -14,22 +15,14 @@ namespace tfde {
 namespace {
 
 constexpr int kT = 256;
+static_assert(kT == gs::kThreads, "block width of the Gram-Schmidt sweeps");
 
 __device__ __forceinline__ void split(float v, __nv_bfloat16& hi, __nv_bfloat16& lo) {
     hi = __float2bfloat16_rn(v);
     lo = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
 
-// Kahan-compensated FP32 accumulation.
-struct KSum {
-    float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float v) {
-        const float y = v - c;
-        const float t = s + y;
-        c = (t - s) - y;
-        s = t;
-    }
-};
+using gs::KSum;
 
 __device__ __forceinline__ double block_sum64(double v) {
     __shared__ double sh[kT / 32];
@@ -474,41 +467,46 @@ __global__ void widen32_kernel(long long N, const float* __restrict__ v, double 
 // coef[0] = num[0] / den[0]  (device-side scalar, no host round trip)
 __global__ void ratio_kernel(const double* num, const double* den, double* coef) { coef[0] = num[0] / den[0]; }
 
-// Up to C dot products <V_j, w>, j = m0 .. m0 + mc - 1, per block into part[j * nblk + b].
-template <int C>
+// The block's share of N elements for the Gram-Schmidt sweeps (a multiple of 4
+// elements per block), and whether the vectors can be read four at a time.
+__device__ __forceinline__ void chunk4(long long N, long long& lo, long long& hi) {
+    const long long per = ((N + gridDim.x - 1) / gridDim.x + 3) / 4 * 4;
+    lo = min((long long)blockIdx.x * per, N);
+    hi = min(lo + per, N);
+}
+__device__ __forceinline__ bool aligned4(const float* V, long long ldv, const float* w) {
+    return ldv % 4 == 0 && ((reinterpret_cast<uintptr_t>(V) | reinterpret_cast<uintptr_t>(w)) & 15) == 0;
+}
+
+// Up to 8 dot products <V_j, w>, j = m0 .. m0 + mc - 1, per block into part[j * nblk + b].
 __global__ __launch_bounds__(kT) void multidot32_kernel(long long N, int m0, int mc, const float* __restrict__ V,
                                                         long long ldv, const float* __restrict__ w,
                                                         double* __restrict__ part) {
     long long lo, hi;
-    chunk(N, lo, hi);
-    KSum k[C];
-    for (long long i = lo + threadIdx.x; i < hi; i += kT) {
-        const float wi = w[i];
-#pragma unroll
-        for (int j = 0; j < C; ++j)
-            if (j < mc) k[j].add(V[(long long)(m0 + j) * ldv + i] * wi);
-    }
-#pragma unroll
-    for (int j = 0; j < C; ++j) {
-        if (j < mc) {
-            const double t = block_sum64((double)k[j].s - (double)k[j].c);
-            if (threadIdx.x == 0) part[(long long)(m0 + j) * gridDim.x + blockIdx.x] = t;
-        }
-    }
+    chunk4(N, lo, hi);
+    gs::dots(V, ldv, m0, mc, w, lo, hi, aligned4(V, ldv, w),
+             [&](int j, double sum) { part[(long long)j * gridDim.x + blockIdx.x] = sum; });
 }
 
 // w -= sum_{j < m} h[j] V_j   (h: FP64 coefficients on the device, m <= 128)
-__global__ void multiaxpy32_kernel(long long N, int m, const float* __restrict__ V, long long ldv,
-                                   const double* __restrict__ h, float* __restrict__ w) {
+__global__ __launch_bounds__(kT) void multiaxpy32_kernel(long long N, int m, const float* __restrict__ V,
+                                                         long long ldv, const double* __restrict__ h,
+                                                         float* __restrict__ w) {
     __shared__ float hs[128];
     for (int j = threadIdx.x; j < m; j += blockDim.x) hs[j] = (float)h[j];
     __syncthreads();
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        float acc = w[i];
-        for (int j = 0; j < m; ++j)
-            if (hs[j] != 0.f) acc = fmaf(-hs[j], V[(long long)j * ldv + i], acc);
-        w[i] = acc;
-    }
+    // trailing zero coefficients belong to vectors that may never have been written
+    while (m > 0 && hs[m - 1] == 0.f) --m;
+    long long lo, hi;
+    chunk4(N, lo, hi);
+    gs::sweep(
+        lo, hi, aligned4(V, ldv, w),
+        [&](long long i) {
+            float4 wi = *reinterpret_cast<const float4*>(w + i);
+            gs::update4(wi, V, ldv, hs, m, i);
+            *reinterpret_cast<float4*>(w + i) = wi;
+        },
+        [&](long long i) { w[i] = gs::update1(w[i], V, ldv, hs, m, i); });
 }
 
 // out = sc * in ; (h, l) = split(out)   (in == out allowed)
@@ -627,30 +625,17 @@ __global__ void pcg_fold_dev_kernel(long long N4, CombineArgs a, float4* __restr
 // kernel takes the step index from gctl, so one step is the body of the loop.
 
 // the first m = j + 1 inner products <V_i, w>, 8 basis vectors per sweep of w
-__global__ __launch_bounds__(kT) void gm_multidot_kernel(long long N, const float* __restrict__ V, long long ldv,
-                                                         const float* __restrict__ w, double* __restrict__ part,
-                                                         const int* gctl) {
+__global__ __launch_bounds__(kT, 2) void gm_multidot_kernel(long long N, const float* __restrict__ V, long long ldv,
+                                                            const float* __restrict__ w, double* __restrict__ part,
+                                                            const int* gctl) {
     if (gctl[1]) return;
     const int m = gctl[0] + 1;
     long long lo, hi;
-    chunk(N, lo, hi);
-    for (int m0 = 0; m0 < m; m0 += 8) {
-        const int mc = m - m0 < 8 ? m - m0 : 8;
-        KSum k[8];
-        for (long long i = lo + threadIdx.x; i < hi; i += kT) {
-            const float wi = w[i];
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (j < mc) k[j].add(V[(long long)(m0 + j) * ldv + i] * wi);
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if (j < mc) {
-                const double t = block_sum64((double)k[j].s - (double)k[j].c);
-                if (threadIdx.x == 0) part[(long long)(m0 + j) * gridDim.x + blockIdx.x] = t;
-            }
-        }
-    }
+    chunk4(N, lo, hi);
+    const bool vec = aligned4(V, ldv, w);
+    for (int m0 = 0; m0 < m; m0 += gs::kWidth)
+        gs::dots(V, ldv, m0, min(m - m0, gs::kWidth), w, lo, hi, vec,
+                 [&](int j, double sum) { part[(long long)j * gridDim.x + blockIdx.x] = sum; });
 }
 
 // out[j] = sum of the block partials of result j, j < m (m = mfix, or the
@@ -662,6 +647,7 @@ __global__ void gm_reduce_kernel(const double* __restrict__ part, int nblk, doub
     const int j = blockIdx.x;
     if (j >= m) return;
     double acc = 0.0;
+#pragma unroll 8
     for (int b = threadIdx.x; b < nblk; b += 32) acc += part[(long long)j * nblk + b];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -670,48 +656,25 @@ __global__ void gm_reduce_kernel(const double* __restrict__ part, int nblk, doub
 
 // The second Gram-Schmidt pass's projections fused with the first pass's
 // update: w -= sum_{i <= j} h[i] V_i over the block's chunk, then the first
-// m = j + 1 inner products <V_i, w> of the updated chunk (each thread re-reads
-// the elements it wrote), 8 basis vectors per sweep; the same arithmetic as
-// a plain multi-axpy followed by gm_multidot_kernel.
-__global__ __launch_bounds__(kT) void gm_axpy_dot_kernel(long long N, const float* __restrict__ V, long long ldv,
-                                                         const double* __restrict__ h, float* __restrict__ w,
-                                                         double* __restrict__ part, const int* gctl) {
+// m = j + 1 inner products <V_i, w> of the updated chunk.
+__global__ __launch_bounds__(kT, 2) void gm_axpy_dot_kernel(long long N, const float* __restrict__ V, long long ldv,
+                                                            const double* __restrict__ h, float* w,
+                                                            double* __restrict__ part, const int* gctl) {
     if (gctl[1]) return;
     const int m = gctl[0] + 1;
     __shared__ float hs[128];
     for (int j = threadIdx.x; j < m; j += blockDim.x) hs[j] = (float)h[j];
     __syncthreads();
     long long lo, hi;
-    chunk(N, lo, hi);
-    for (long long i = lo + threadIdx.x; i < hi; i += kT) {
-        float acc = w[i];
-        for (int j = 0; j < m; ++j) acc = fmaf(-hs[j], V[(long long)j * ldv + i], acc);
-        w[i] = acc;
-    }
-    for (int m0 = 0; m0 < m; m0 += 8) {
-        const int mc = m - m0 < 8 ? m - m0 : 8;
-        KSum k[8];
-        for (long long i = lo + threadIdx.x; i < hi; i += kT) {
-            const float wi = w[i];
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (j < mc) k[j].add(V[(long long)(m0 + j) * ldv + i] * wi);
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if (j < mc) {
-                const double t = block_sum64((double)k[j].s - (double)k[j].c);
-                if (threadIdx.x == 0) part[(long long)(m0 + j) * gridDim.x + blockIdx.x] = t;
-            }
-        }
-    }
+    chunk4(N, lo, hi);
+    gs::update_dots(V, ldv, hs, m, w, lo, hi, aligned4(V, ldv, w),
+                    [&](int j, double sum) { part[(long long)j * gridDim.x + blockIdx.x] = sum; });
 }
 
 // The second pass's update fused with ||w||^2: w -= sum_{i <= j} h[i] V_i over
-// the block's chunk and the block's partial sum of the updated w^2 (the
-// arithmetic of a plain multi-axpy followed by gm_dot_kernel).
+// the block's chunk and the block's partial sum of the updated w^2.
 __global__ __launch_bounds__(kT) void gm_axpy_norm_kernel(long long N, const float* __restrict__ V, long long ldv,
-                                                          const double* __restrict__ h, float* __restrict__ w,
+                                                          const double* __restrict__ h, float* w,
                                                           double* __restrict__ part, const int* gctl) {
     if (gctl[1]) return;
     const int m = gctl[0] + 1;
@@ -719,27 +682,17 @@ __global__ __launch_bounds__(kT) void gm_axpy_norm_kernel(long long N, const flo
     for (int j = threadIdx.x; j < m; j += blockDim.x) hs[j] = (float)h[j];
     __syncthreads();
     long long lo, hi;
-    chunk(N, lo, hi);
-    KSum k;
-    for (long long i = lo + threadIdx.x; i < hi; i += kT) {
-        float acc = w[i];
-        for (int j = 0; j < m; ++j) acc = fmaf(-hs[j], V[(long long)j * ldv + i], acc);
-        w[i] = acc;
-        k.add(acc * acc);
-    }
-    const double t = block_sum64((double)k.s - (double)k.c);
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
+    chunk4(N, lo, hi);
+    gs::update_norm(V, ldv, hs, m, w, lo, hi, aligned4(V, ldv, w), [&](double sum) { part[blockIdx.x] = sum; });
 }
 
-__global__ __launch_bounds__(kT) void gm_dot_kernel(long long N, const float* __restrict__ a, double* __restrict__ part,
+__global__ __launch_bounds__(kT) void gm_dot_kernel(long long N, const float* a, double* __restrict__ part,
                                                     const int* gctl) {
     if (gctl[1]) return;
     long long lo, hi;
-    chunk(N, lo, hi);
-    KSum k;
-    for (long long i = lo + threadIdx.x; i < hi; i += kT) k.add(a[i] * a[i]);
-    const double t = block_sum64((double)k.s - (double)k.c);
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
+    chunk4(N, lo, hi);
+    gs::update_norm(nullptr, 4, nullptr, 0, const_cast<float*>(a), lo, hi, aligned4(a, 4, a),
+                    [&](double sum) { part[blockIdx.x] = sum; });
 }
 
 // Column j of the Hessenberg matrix (h + h2 from the two Gram-Schmidt
@@ -831,11 +784,15 @@ __global__ void gm_solve_kernel(const double* gs, const int* gctl, double* ny, i
     for (int i = 0; i < maxm; ++i) ny[i] = i < k ? -y[i] : 0.0;
 }
 
+// Blocks of the Gram-Schmidt sweeps: two per SM (their register limit), so that
+// there are few partial sums to add, but not more than the partials' rows hold.
+static int gs_blocks(int nblk) { return nblk < 304 ? nblk : 304; }
 void launch_gm_step(size_t N, const float* V, float* w, double* part, int nblk, double* hbuf, double* h2buf,
                     double* wwbuf, double* gs, int* gctl, cudaGraphConditionalHandle hc, float* Vout,
                     __nv_bfloat16* ph, __nv_bfloat16* pl, int maxm, cudaStream_t s) {
     stats_count_launch(7);
     const long long n = (long long)N;
+    nblk = gs_blocks(nblk);
     // CGS2: <V, w>; w -= V h and <V, w> again (one pass over the block's chunk);
     // w -= V h2 and ||w||^2 (one pass)
     gm_multidot_kernel<<<nblk, kT, 0, s>>>(n, V, n, w, part, gctl);
@@ -853,6 +810,7 @@ void launch_gm_start(size_t N, const float* w, double* part, int nblk, double* w
                      int maxsteps, double ptheta, float* V0, __nv_bfloat16* ph, __nv_bfloat16* pl, cudaStream_t s) {
     stats_count_launch(4);
     const long long n = (long long)N;
+    nblk = gs_blocks(nblk);
     // gctl[1] = 0 here (set by the caller's reset) so that the dot and reduce run
     gm_dot_kernel<<<nblk, kT, 0, s>>>(n, w, part, gctl);
     gm_reduce_kernel<<<1, 32, 0, s>>>(part, nblk, wwbuf, 1, gctl);
@@ -1041,7 +999,7 @@ void launch_multidot32(size_t N, int m, const float* V, size_t ldv, const float*
     for (int m0 = 0; m0 < m; m0 += 8) {
         const int mc = (m - m0) < 8 ? (m - m0) : 8;
         stats_count_launch();
-        multidot32_kernel<8><<<nblk, kT, 0, s>>>((long long)N, m0, mc, V, (long long)ldv, w, part);
+        multidot32_kernel<<<nblk, kT, 0, s>>>((long long)N, m0, mc, V, (long long)ldv, w, part);
     }
 }
 void launch_multiaxpy32(size_t N, int m, const float* V, size_t ldv, const double* h, float* w, cudaStream_t s) {

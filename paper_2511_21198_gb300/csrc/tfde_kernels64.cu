@@ -318,6 +318,7 @@ __global__ void reduce_finish_kernel(const double* __restrict__ part, int nblk, 
     const int j = blockIdx.x;
     if (j >= m) return;
     double acc = 0.0;
+#pragma unroll 8
     for (int b = threadIdx.x; b < nblk; b += 32) acc += part[(long long)j * nblk + b];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
