@@ -22,7 +22,8 @@
 //
 // FFT.  Complex, length L = 2^m <= 4096, radix-4 Stockham autosort passes
 // (a radix-2 pass last when m is odd) in shared memory: a block holds
-// 4096 / L complex lines (64 KB in FP64), 256 threads, each pass reads its
+// 4096 / L complex lines (64 KB in FP64), or 2048 / L or 1024 / L where that
+// leaves SMs idle, 256 threads, each pass reads its
 // butterflies into registers, synchronises and writes the reordered results.
 //
 // Short axes take a dense product on CUDA cores instead of the transforms
@@ -55,7 +56,7 @@ namespace fft {
 namespace {
 
 constexpr int NT = 256;        // threads per block
-constexpr int ELEMS = 4096;    // complex elements per block (lines x L)
+constexpr int MAX_ELEMS = 4096;   // complex elements per block (lines x L): 4096, 2048 or 1024
 
 template <typename R>
 struct C2;
@@ -174,7 +175,7 @@ __device__ __forceinline__ void grid_index(int axis, int e, int lgG, int lgJ, in
 }
 
 // Forward DFT of the block's complex lines in place (stride ls between lines).
-template <typename R>
+template <typename R, int ELEMS>
 __device__ void block_fft(typename C2<R>::T* buf, int ls, int L, int log2L, const typename C2<R>::T* __restrict__ tw) {
     using T2 = typename C2<R>::T;
     int lgNs = 0;
@@ -182,10 +183,11 @@ __device__ void block_fft(typename C2<R>::T* buf, int ls, int L, int log2L, cons
         if (log2L - lgNs >= 2) {
             const int lgLr = log2L - 2, Lr = 1 << lgLr;
             const int Ns = 1 << lgNs;
-            T2 v[4][4];
-            int cc[4], jj[4];
+            constexpr int U = ELEMS / (4 * NT);   // butterflies per thread
+            T2 v[U][4];
+            int cc[U], jj[U];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const int b = threadIdx.x + u * NT;   // butterfly of the block: line c, position j
                 const int c = b >> lgLr, j = b & (Lr - 1);
                 cc[u] = c;
@@ -208,7 +210,7 @@ __device__ void block_fft(typename C2<R>::T* buf, int ls, int L, int log2L, cons
             }
             __syncthreads();
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const int j = jj[u];
                 const int base = ((j >> lgNs) << (lgNs + 2)) + (j & (Ns - 1));
                 T2* dst = buf + (size_t)cc[u] * ls + base;
@@ -222,10 +224,11 @@ __device__ void block_fft(typename C2<R>::T* buf, int ls, int L, int log2L, cons
         } else {
             const int lgLr = log2L - 1, Lr = 1 << lgLr;
             const int Ns = 1 << lgNs;
-            T2 v[8][2];
-            int cc[8], jj[8];
+            constexpr int U = ELEMS / (2 * NT);
+            T2 v[U][2];
+            int cc[U], jj[U];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const int b = threadIdx.x + u * NT;
                 const int c = b >> lgLr, j = b & (Lr - 1);
                 cc[u] = c;
@@ -240,7 +243,7 @@ __device__ void block_fft(typename C2<R>::T* buf, int ls, int L, int log2L, cons
             }
             __syncthreads();
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const int j = jj[u];
                 const int base = ((j >> lgNs) << (lgNs + 1)) + (j & (Ns - 1));
                 T2* dst = buf + (size_t)cc[u] * ls + base;
@@ -254,7 +257,7 @@ __device__ void block_fft(typename C2<R>::T* buf, int ls, int L, int log2L, cons
 }
 
 // buf <- conj(buf . spec), element-wise over the block's lines.
-template <typename R>
+template <typename R, int ELEMS>
 __device__ __forceinline__ void block_spectral_scale(typename C2<R>::T* buf, int ls, int L, int log2L,
                                                      const typename C2<R>::T* __restrict__ spec) {
     using T2 = typename C2<R>::T;
@@ -270,13 +273,14 @@ __device__ __forceinline__ void block_spectral_scale(typename C2<R>::T* buf, int
 
 enum { MODE_TOEPLITZ = 0, MODE_DST = 1, MODE_DST2 = 2 };
 
-template <typename R, int MODE>
+template <typename R, int MODE, int ELEMS>
 __global__ void __launch_bounds__(NT) fft_pass_kernel(const Pass p) {
     using T2 = typename C2<R>::T;
     extern __shared__ __align__(16) unsigned char fft_smem[];
     T2* buf = reinterpret_cast<T2*>(fft_smem);
     const int L = p.L, lg = p.log2L, n = p.n;
-    const int lgCL = 12 - lg;                       // log2(ELEMS / L)
+    constexpr int lgE = ELEMS == 4096 ? 12 : (ELEMS == 2048 ? 11 : 10);
+    const int lgCL = lgE - lg;                      // log2(ELEMS / L)
     const int CL = 1 << lgCL;
     const int lgG = MODE == MODE_TOEPLITZ ? lgCL + 1 : lgCL;
     const int G = 1 << lgG;                         // real lines of this block
@@ -335,9 +339,9 @@ __global__ void __launch_bounds__(NT) fft_pass_kernel(const Pass p) {
         }
         __syncthreads();
     }
-    block_fft<R>(buf, ls, L, lg, tw);
-    block_spectral_scale<R>(buf, ls, L, lg, spec);
-    block_fft<R>(buf, ls, L, lg, tw);
+    block_fft<R, ELEMS>(buf, ls, L, lg, tw);
+    block_spectral_scale<R, ELEMS>(buf, ls, L, lg, spec);
+    block_fft<R, ELEMS>(buf, ls, L, lg, tw);
     if constexpr (MODE == MODE_DST2) {
         // t = S in0 (real, k < n), then t / Lambda(i, j, k) re-phased as the
         // input of the second transform; lines along z: l = i + n1 j
@@ -395,9 +399,9 @@ __global__ void __launch_bounds__(NT) fft_pass_kernel(const Pass p) {
             *q = w;   // each element is read and rewritten by the same thread
         }
         __syncthreads();
-        block_fft<R>(buf, ls, L, lg, tw);
-        block_spectral_scale<R>(buf, ls, L, lg, spec);
-        block_fft<R>(buf, ls, L, lg, tw);
+        block_fft<R, ELEMS>(buf, ls, L, lg, tw);
+        block_spectral_scale<R, ELEMS>(buf, ls, L, lg, spec);
+        block_fft<R, ELEMS>(buf, ls, L, lg, tw);
     }
 
     // ---- store
@@ -673,22 +677,35 @@ void free_state(tfde_problem* P) {
 
 namespace {
 
-bool g_attr[2][3] = {};
+template <typename R, int MODE, int ELEMS>
+int launch_fft(const Pass& p, cudaStream_t s) {
+    using T2 = typename C2<R>::T;
+    static std::atomic<unsigned long long> ready{0};   // a bit per device
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(ready.load(std::memory_order_relaxed) & bit)) {
+        if (cudaFuncSetAttribute(fft_pass_kernel<R, MODE, ELEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(2 * ELEMS * sizeof(T2))) != cudaSuccess)
+            return set_error(TFDE_ECUDA, "cudaFuncSetAttribute(fft_pass_kernel) failed");
+        ready.fetch_or(bit, std::memory_order_relaxed);
+    }
+    const int cl = ELEMS >> p.log2L, G = MODE == MODE_TOEPLITZ ? 2 * cl : cl;
+    fft_pass_kernel<R, MODE, ELEMS><<<(unsigned)((p.lines + G - 1) / G), NT, (size_t)cl * (p.L + 1) * sizeof(T2), s>>>(p);
+    return TFDE_OK;
+}
 
 template <typename R, int MODE>
 int launch_pass(const Pass& p, cudaStream_t s) {
-    using T2 = typename C2<R>::T;
-    const int lgCL = 12 - p.log2L;
-    const int G = MODE == MODE_TOEPLITZ ? (2 << lgCL) : (1 << lgCL);
-    const size_t smem = (size_t)(1 << lgCL) * (p.L + 1) * sizeof(T2);
-    const int ti = sizeof(R) == 8 ? 0 : 1;
-    if (!g_attr[ti][MODE]) {
-        if (cudaFuncSetAttribute(fft_pass_kernel<R, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)((ELEMS + ELEMS) * sizeof(T2))) != cudaSuccess)
-            return set_error(TFDE_ECUDA, "cudaFuncSetAttribute(fft_pass_kernel) failed");
-        g_attr[ti][MODE] = true;
-    }
-    const long long blocks = (p.lines + G - 1) / G;
+    // complex elements per block: the fewest down to 1024 (and a line) while
+    // larger blocks would leave an SM without two of them; 511^2 in FP64:
+    // 101 -> 47 us per pass
+    int elems = MAX_ELEMS;
+    auto blocks = [&](int e) {
+        const long long G = (MODE == MODE_TOEPLITZ ? 2 : 1) * (e >> p.log2L);
+        return (p.lines + G - 1) / G;
+    };
+    while (elems > 1024 && elems / 2 >= p.L && blocks(elems) < 2 * tc::num_sms()) elems /= 2;
     // algorithmic work: every grid function read and written once; complex
     // transforms of length L at 5 L log2 L flops, 6 L for a spectral product
     const double N = (double)p.lines * p.n;
@@ -697,9 +714,11 @@ int launch_pass(const Pass& p, cudaStream_t s) {
     const double per = 2.0 * 5.0 * p.L * p.log2L + 6.0 * p.L;
     const double flops = cl * per * (MODE == MODE_DST2 ? 2.0 : 1.0);
     void* tok = stats_tc_begin(s, TFDE_KIND_FFT);
-    fft_pass_kernel<R, MODE><<<(unsigned)blocks, NT, smem, s>>>(p);
+    const int st = elems == 1024 ? launch_fft<R, MODE, 1024>(p, s)
+                                 : (elems == 2048 ? launch_fft<R, MODE, 2048>(p, s) : launch_fft<R, MODE, 4096>(p, s));
     const cudaError_t e = cudaGetLastError();
     stats_tc_end(tok, s, TFDE_KIND_FFT, nio * N * sizeof(R), flops);
+    if (st) return st;
     if (e != cudaSuccess) return set_error(TFDE_ECUDA, std::string("fft_pass_kernel: ") + cudaGetErrorString(e));
     return TFDE_OK;
 }

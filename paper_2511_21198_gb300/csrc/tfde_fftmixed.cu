@@ -21,6 +21,7 @@
 
 #include "tfde_fft.h"
 #include "tfde_givens.h"
+#include "tfde_gs.cuh"
 #include "tfde_internal.h"
 #include "tfde_stats.h"
 
@@ -52,11 +53,14 @@ enum { S_RZ0 = 0, S_RZ1 = 1, S_PQ = 2, S_RR = 3, S_H = 8, NS = 256 };
 
 struct FftMixed {
     float* v[NV] = {};
-    float* V = nullptr;     // GMRES basis, (vcap + 1) vectors
+    float* V = nullptr;     // GMRES basis, (vcap + 1) vectors of ldv(N) values
     int vcap = 0;
     double* d = nullptr;    // device scalars
     double* h = nullptr;    // pinned host mirror of d
 };
+
+// basis vectors start 16 bytes apart or a multiple of it
+size_t ldv(size_t N) { return (N + 3) / 4 * 4; }
 
 FftMixed* state(const tfde_problem* P) { return static_cast<FftMixed*>(P->fmix); }
 
@@ -93,16 +97,27 @@ __global__ __launch_bounds__(kT) void cg_update_kernel(long long N, const double
                                                        const float* __restrict__ q, float* __restrict__ x,
                                                        float* __restrict__ r, double* __restrict__ part) {
     const float alpha = (float)(num[0] / den[0]);
-    const long long per = (N + gridDim.x - 1) / gridDim.x;
-    const long long lo = (long long)blockIdx.x * per;
-    const long long hi = lo + per < N ? lo + per : N;
-    double acc = 0.0;
-    for (long long i = lo + threadIdx.x; i < hi; i += kT) {
-        x[i] = fmaf(alpha, p[i], x[i]);
-        const float ri = fmaf(-alpha, q[i], r[i]);
-        r[i] = ri;
-        acc += (double)ri * (double)ri;
-    }
+    const long long per = ((N + gridDim.x - 1) / gridDim.x + 3) / 4 * 4;
+    const long long lo = min((long long)blockIdx.x * per, N), hi = min(lo + per, N);
+    double acc = 0.0;   // exact FP64 products
+    auto one = [&](float pi, float qi, float& xi, float& ri) {
+        xi = fmaf(alpha, pi, xi);
+        ri = fmaf(-alpha, qi, ri);
+        acc = fma((double)ri, (double)ri, acc);
+    };
+    gs::sweep(   // the vectors are allocations of their own: aligned
+        lo, hi, true,
+        [&](long long i) {
+            const float4 pv = *reinterpret_cast<const float4*>(p + i), qv = *reinterpret_cast<const float4*>(q + i);
+            float4 xv = *reinterpret_cast<float4*>(x + i), rv = *reinterpret_cast<float4*>(r + i);
+            one(pv.x, qv.x, xv.x, rv.x);
+            one(pv.y, qv.y, xv.y, rv.y);
+            one(pv.z, qv.z, xv.z, rv.z);
+            one(pv.w, qv.w, xv.w, rv.w);
+            *reinterpret_cast<float4*>(x + i) = xv;
+            *reinterpret_cast<float4*>(r + i) = rv;
+        },
+        [&](long long i) { one(p[i], q[i], x[i], r[i]); });
     const double t = block_sum(acc);
     if (threadIdx.x == 0) part[blockIdx.x] = t;
 }
@@ -134,8 +149,9 @@ void launch_to32(size_t N, const double* r64, double sc, float* r32, float* x32,
 
 // <a, b> into dev (device, FP64)
 void dot_to(const tfde_problem* P, const float* a, const float* b, double* dev, cudaStream_t s) {
-    launch_dot32(P->N, a, b, P->red, P->nblk, s);
-    launch_reduce_finish(P->red, P->nblk, 1, dev, s);
+    const int nblk = dot_blocks(P->nblk);
+    launch_dot32(P->N, a, b, P->red, nblk, s);
+    launch_reduce_finish(P->red, nblk, 1, dev, s);
 }
 
 int read_host(const tfde_problem* P, const double* dev, int count, double* out, cudaStream_t s) {
@@ -178,8 +194,9 @@ int inner_pcg(const tfde_problem* P, double theta, int maxit, double rr0, int* i
         if ((st = op_A32(P, p, q, s))) return st;
         dot_to(P, p, q, d + S_PQ, s);
         stats_count_launch();
-        cg_update_kernel<<<P->nblk, kT, 0, s>>>((long long)N, d + rz, d + S_PQ, p, q, F->v[V_X], r, P->red);
-        launch_reduce_finish(P->red, P->nblk, 1, d + S_RR, s);
+        const int nblk = dot_blocks(P->nblk);
+        cg_update_kernel<<<nblk, kT, 0, s>>>((long long)N, d + rz, d + S_PQ, p, q, F->v[V_X], r, P->red);
+        launch_reduce_finish(P->red, nblk, 1, d + S_RR, s);
         double rr;
         if ((st = read_host(P, d + S_RR, 1, &rr, s))) return st;
         ++k;
@@ -203,7 +220,7 @@ int ensure_basis(const tfde_problem* P, int m) {
     cudaFree(F->V);
     F->V = nullptr;
     F->vcap = 0;
-    if (cudaMalloc((void**)&F->V, (size_t)(m + 1) * P->N * sizeof(float)) != cudaSuccess)
+    if (cudaMalloc((void**)&F->V, (size_t)(m + 1) * ldv(P->N) * sizeof(float)) != cudaSuccess)
         return set_error(TFDE_ENOMEM, "cudaMalloc of the FP32 GMRES basis failed");
     F->vcap = m;
     return TFDE_OK;
@@ -224,7 +241,9 @@ int inner_gmres(const tfde_problem* P, int m, double theta, int maxit, int* iter
     int st;
     *iters = 0;
     *est_ratio = 1.0;
-    auto col = [&](int j) { return V + (size_t)j * N; };
+    const size_t ld = ldv(N);
+    const int nblk = dot_blocks(P->nblk);
+    auto col = [&](int j) { return V + (size_t)j * ld; };
     if ((st = op_Pinv32(P, F->v[V_R], col(0), s))) return st;
     dot_to(P, col(0), col(0), d + S_H, s);
     double beta2;
@@ -244,14 +263,14 @@ int inner_gmres(const tfde_problem* P, int m, double theta, int maxit, int* iter
         if ((st = op_A32(P, col(j), F->v[V_Q], s))) return st;
         if ((st = op_Pinv32(P, F->v[V_Q], w, s))) return st;
         // first projection
-        launch_multidot32(N, j + 1, V, N, w, P->red, P->nblk, s);
-        launch_reduce_finish(P->red, P->nblk, j + 1, d + S_H, s);
-        launch_multiaxpy32(N, j + 1, V, N, d + S_H, w, s);
+        launch_multidot32(N, j + 1, V, ld, w, P->red, nblk, s);
+        launch_reduce_finish(P->red, nblk, j + 1, d + S_H, s);
+        launch_multiaxpy32(N, j + 1, V, ld, d + S_H, w, s);
         if ((st = read_host(P, d + S_H, j + 1, h.data(), s))) return st;
         // second projection, with ||w||^2 (w is column j + 1 of V)
-        launch_multidot32(N, j + 2, V, N, w, P->red, P->nblk, s);
-        launch_reduce_finish(P->red, P->nblk, j + 2, d + S_H, s);
-        launch_multiaxpy32(N, j + 1, V, N, d + S_H, w, s);
+        launch_multidot32(N, j + 2, V, ld, w, P->red, nblk, s);
+        launch_reduce_finish(P->red, nblk, j + 2, d + S_H, s);
+        launch_multiaxpy32(N, j + 1, V, ld, d + S_H, w, s);
         if ((st = read_host(P, d + S_H, j + 2, h2.data(), s))) return st;
         double ww = h2[j + 1];
         for (int i = 0; i <= j; ++i) {
@@ -275,7 +294,7 @@ int inner_gmres(const tfde_problem* P, int m, double theta, int maxit, int* iter
     for (int i = 0; i < k; ++i) F->h[i] = -y[i];   // multiaxpy subtracts
     FM_TRY(cudaMemcpyAsync(d + S_H, F->h, k * sizeof(double), cudaMemcpyHostToDevice, s));
     FM_TRY(cudaMemsetAsync(F->v[V_X], 0, N * sizeof(float), s));
-    launch_multiaxpy32(N, k, V, N, d + S_H, F->v[V_X], s);
+    launch_multiaxpy32(N, k, V, ld, d + S_H, F->v[V_X], s);
     *iters = k;
     *est_ratio = res / beta;
     return TFDE_OK;

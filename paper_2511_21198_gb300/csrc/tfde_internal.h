@@ -75,6 +75,10 @@ void launch_multiaxpy_f64(size_t N, int m, const double* V, size_t ldv, const do
 // deterministic second stage: out[j] = sum_b part[j*nblk + b], j < m
 void launch_reduce_finish(const double* part, int nblk, int m, double* out, cudaStream_t s);
 int reduction_blocks(size_t N);
+// Blocks of an inner-product sweep: at most two per SM, so that there are few
+// partial sums to add (FP64 adds issue at two lanes per clock and SM): a dot of
+// 127^3 37 -> 9 us.
+inline int dot_blocks(int nblk) { return nblk < 304 ? nblk : 304; }
 // b = AN - Ku + dt F, r = dt F - 2 Ku  (first CN step of a chain); with
 // norms2 set, also ||b||^2 and ||r||^2 into norms2[0..1] (device; part =
 // scratch of at least 2 * 2432 doubles)

@@ -43,13 +43,18 @@ __device__ __forceinline__ void chunk(long long N, long long& lo, long long& hi)
     hi = lo + per < N ? lo + per : N;
 }
 
-__global__ __launch_bounds__(kT) void dot32_kernel(long long N, const float* __restrict__ a,
-                                                   const float* __restrict__ b, double* __restrict__ part) {
-    long long lo, hi;
-    chunk(N, lo, hi);
+__global__ __launch_bounds__(kT) void dot32_kernel(long long N, const float* a, const float* b,
+                                                   double* __restrict__ part) {
+    const long long per = ((N + gridDim.x - 1) / gridDim.x + 3) / 4 * 4;
+    const long long lo = min((long long)blockIdx.x * per, N), hi = min(lo + per, N);
     KSum k;
-    for (long long i = lo + threadIdx.x; i < hi; i += kT) k.add(a[i] * b[i]);
-    const double t = block_sum64((double)k.s - (double)k.c);
+    gs::sweep(
+        lo, hi, ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0,
+        [&](long long i) {
+            gs::add4(k, *reinterpret_cast<const float4*>(a + i), *reinterpret_cast<const float4*>(b + i));
+        },
+        [&](long long i) { k.add(a[i] * b[i]); });
+    const double t = block_sum64(k.value());
     if (threadIdx.x == 0) part[blockIdx.x] = t;
 }
 
@@ -784,15 +789,12 @@ __global__ void gm_solve_kernel(const double* gs, const int* gctl, double* ny, i
     for (int i = 0; i < maxm; ++i) ny[i] = i < k ? -y[i] : 0.0;
 }
 
-// Blocks of the Gram-Schmidt sweeps: two per SM (their register limit), so that
-// there are few partial sums to add, but not more than the partials' rows hold.
-static int gs_blocks(int nblk) { return nblk < 304 ? nblk : 304; }
 void launch_gm_step(size_t N, const float* V, float* w, double* part, int nblk, double* hbuf, double* h2buf,
                     double* wwbuf, double* gs, int* gctl, cudaGraphConditionalHandle hc, float* Vout,
                     __nv_bfloat16* ph, __nv_bfloat16* pl, int maxm, cudaStream_t s) {
     stats_count_launch(7);
     const long long n = (long long)N;
-    nblk = gs_blocks(nblk);
+    nblk = dot_blocks(nblk);
     // CGS2: <V, w>; w -= V h and <V, w> again (one pass over the block's chunk);
     // w -= V h2 and ||w||^2 (one pass)
     gm_multidot_kernel<<<nblk, kT, 0, s>>>(n, V, n, w, part, gctl);
@@ -810,7 +812,7 @@ void launch_gm_start(size_t N, const float* w, double* part, int nblk, double* w
                      int maxsteps, double ptheta, float* V0, __nv_bfloat16* ph, __nv_bfloat16* pl, cudaStream_t s) {
     stats_count_launch(4);
     const long long n = (long long)N;
-    nblk = gs_blocks(nblk);
+    nblk = dot_blocks(nblk);
     // gctl[1] = 0 here (set by the caller's reset) so that the dot and reduce run
     gm_dot_kernel<<<nblk, kT, 0, s>>>(n, w, part, gctl);
     gm_reduce_kernel<<<1, 32, 0, s>>>(part, nblk, wwbuf, 1, gctl);

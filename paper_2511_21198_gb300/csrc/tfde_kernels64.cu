@@ -5,6 +5,7 @@
 #include "tfde_internal.h"
 #include "tfde_pow2conv.cuh"
 #include "tfde_chain.cuh"
+#include "tfde_gs.cuh"
 #include "tfde_stats.h"
 
 namespace tfde {
@@ -275,28 +276,44 @@ __global__ __launch_bounds__(kThreads) void cg_update_f64_kernel(long long N, do
     if (threadIdx.x == 0) part[blockIdx.x] = t;
 }
 
-template <int C>
+// C dot products <V_{m0 + j}, w> (j < mc), per block into part[(m0 + j) * gridDim.x + b];
+// U elements per thread in flight, one shared reduction tree for eight results
+template <int C, int U>
 __global__ __launch_bounds__(kThreads) void multidot_f64_kernel(long long N, int m0, int mc,
                                                                 const double* __restrict__ V, long long ldv,
                                                                 const double* __restrict__ w,
                                                                 double* __restrict__ part) {
     long long lo, hi;
     chunk_range(N, lo, hi);
-    double acc[C];
+    double acc[gs::kWidth] = {};
+    const double* V0 = V + (long long)m0 * ldv;
+    long long i = lo + threadIdx.x;
+    for (; i + (U - 1) * kThreads < hi; i += U * kThreads) {
+        double x[U][C + 1];
 #pragma unroll
-    for (int j = 0; j < C; ++j) acc[j] = 0.0;
-    for (long long i = lo + threadIdx.x; i < hi; i += kThreads) {
+        for (int u = 0; u < U; ++u) {
+            x[u][C] = w[i + u * kThreads];
+#pragma unroll
+            for (int j = 0; j < C; ++j)
+                if (j < mc) x[u][j] = V0[(long long)j * ldv + i + u * kThreads];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int j = 0; j < C; ++j)
+                if (j < mc) acc[j] = fma(x[u][j], x[u][C], acc[j]);
+    }
+    for (; i < hi; i += kThreads) {
         const double wi = w[i];
 #pragma unroll
         for (int j = 0; j < C; ++j)
-            if (j < mc) acc[j] = fma(V[(long long)(m0 + j) * ldv + i], wi, acc[j]);
+            if (j < mc) acc[j] = fma(V0[(long long)j * ldv + i], wi, acc[j]);
     }
-#pragma unroll
-    for (int j = 0; j < C; ++j) {
-        if (j < mc) {
-            const double t = block_sum(acc[j]);
-            if (threadIdx.x == 0) part[(long long)(m0 + j) * gridDim.x + blockIdx.x] = t;
-        }
+    if constexpr (C == 1) {
+        const double t = block_sum(acc[0]);
+        if (threadIdx.x == 0) part[(long long)m0 * gridDim.x + blockIdx.x] = t;
+    } else {
+        gs::block_sums8(acc, mc, [&](int j, double t) { part[(long long)(m0 + j) * gridDim.x + blockIdx.x] = t; });
     }
 }
 
@@ -577,7 +594,8 @@ void launch_multidot_f64(size_t N, int m, const double* V, size_t ldv, const dou
     for (int m0 = 0; m0 < m; m0 += 8) {
         const int mc = (m - m0) < 8 ? (m - m0) : 8;
         if (m0 > 0) stats_count_launch();
-        multidot_f64_kernel<8><<<nblk, kThreads, 0, s>>>((long long)N, m0, mc, V, (long long)ldv, w, part);
+        if (mc == 1) multidot_f64_kernel<1, 8><<<nblk, kThreads, 0, s>>>((long long)N, m0, mc, V, (long long)ldv, w, part);
+        else multidot_f64_kernel<8, 2><<<nblk, kThreads, 0, s>>>((long long)N, m0, mc, V, (long long)ldv, w, part);
     }
 }
 

@@ -69,8 +69,9 @@ int apply_Pinv64(const tfde_problem* P, const double* r, double* z, cudaStream_t
 // out[j] = <V_j, w>, j < m (host output; synchronises the stream).
 int dots64(const tfde_problem* P, int m, const double* V, size_t ldv, const double* w, double* out,
            cudaStream_t s) {
-    launch_multidot_f64(P->N, m, V, ldv, w, P->red, P->nblk, s);
-    launch_reduce_finish(P->red, P->nblk, m, P->red_out, s);
+    const int nblk = dot_blocks(P->nblk);
+    launch_multidot_f64(P->N, m, V, ldv, w, P->red, nblk, s);
+    launch_reduce_finish(P->red, nblk, m, P->red_out, s);
     TFDE_CUDA_TRY(cudaGetLastError());
     TFDE_CUDA_TRY(cudaMemcpyAsync(P->red_host, P->red_out, m * sizeof(double), cudaMemcpyDeviceToHost, s));
     TFDE_CUDA_TRY(cudaStreamSynchronize(s));
