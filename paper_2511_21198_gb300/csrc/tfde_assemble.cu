@@ -8,6 +8,7 @@
 #include <string>
 
 #include "tfde_fft.h"
+#include "tfde_pcgloop.h"
 #include "tfde_internal.h"
 
 namespace tfde {
@@ -331,6 +332,7 @@ int destroy_problem(tfde_problem* P) {
     cudaDeviceSynchronize();
     mixed_free(P);
     fmix_free(P);
+    pcg_loop_free(P);
     fft::free_state(P);
     for (auto& g : P->Ghat) cudaFree(g);
     for (int a = 0; a < 3; ++a) {

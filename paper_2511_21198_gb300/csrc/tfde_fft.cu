@@ -114,6 +114,7 @@ struct Pass {
     const float* lamf;  // the same in FP32 (the FP32 passes form Lambda in FP32)
     double c0, c1, c2;  // MODE_DST2: eta_a (k+ + k-)
     int half_power;     // MODE_DST2: divide by Lambda^{1/2} instead of Lambda (P^{-1/2})
+    const int* skip;    // optional: no work when *skip != 0
 };
 
 __device__ __forceinline__ long long axis_stride(const Pass& p) {
@@ -277,6 +278,7 @@ template <typename R, int MODE, int ELEMS>
 __global__ void __launch_bounds__(NT) fft_pass_kernel(const Pass p) {
     using T2 = typename C2<R>::T;
     extern __shared__ __align__(16) unsigned char fft_smem[];
+    if (p.skip && *p.skip) return;
     T2* buf = reinterpret_cast<T2*>(fft_smem);
     const int L = p.L, lg = p.log2L, n = p.n;
     constexpr int lgE = ELEMS == 4096 ? 12 : (ELEMS == 2048 ? 11 : 10);
@@ -841,13 +843,14 @@ int toeplitz_pass(const tfde_problem* P, int axis, const Table& T, const LineMat
 
 template <typename R>
 int dst_pass(const tfde_problem* P, int axis, const R* in, R* out, bool lambda, bool lambda_only, cudaStream_t s,
-             bool half_power) {
+             bool half_power, const int* skip) {
     const State* F = static_cast<const State*>(P->fft);
     const LineMatrix& m = F->lS[sizeof(R) == 8 ? 0 : 1][axis];
     if (m.K) {
         LinePass q = base_line<R>(P, axis, m);
         q.in0 = in;
         q.out0 = out;
+        q.skip = skip;
         if (!lambda) return line_pass<R, LINE_DST>(q, s);
         q.lam = sizeof(R) == 8 ? (const void*)P->lam : (const void*)F->lamf;
         q.c0 = P->csum[0];
@@ -860,6 +863,7 @@ int dst_pass(const tfde_problem* P, int axis, const R* in, R* out, bool lambda, 
     p.spec = sizeof(R) == 8 ? (const void*)F->chirp[axis].d : (const void*)F->chirp[axis].f;
     p.in0 = in;
     p.out0 = out;
+    p.skip = skip;
     if (lambda) {
         p.lam = P->lam;
         p.lamf = F->lamf;
@@ -894,22 +898,38 @@ int apply_A(const tfde_problem* P, int op, const R* x, R* y, R* a, R* w, R* c, R
     return toeplitz_pass<R>(P, 2, F->G[2], F->lG[t][2], sg, e, c, 1.0, y, nullptr, s);
 }
 
+// The axis of the preconditioner's pair, and whether the pair is two launches.
+template <typename R>
+int pair_axis(const tfde_problem* P) {
+    const State* F = static_cast<const State*>(P->fft);
+    return P->dim2 && F->lS[sizeof(R) == 8 ? 0 : 1][1].K ? 1 : 2;
+}
+template <typename R>
+bool pair_split(const tfde_problem* P) {
+    const LineMatrix& m = static_cast<const State*>(P->fft)->lS[sizeof(R) == 8 ? 0 : 1][pair_axis<R>(P)];
+    return m.K && m.ld > LINE_ROWS;
+}
+int operator_launches(const tfde_problem* P) { return P->dim2 ? 2 : 3; }
+template <typename R>
+int preconditioner_launches(const tfde_problem* P) {
+    return 2 * pair_axis<R>(P) + (pair_split<R>(P) ? 2 : 1);
+}
+template int preconditioner_launches<double>(const tfde_problem*);
+template int preconditioner_launches<float>(const tfde_problem*);
+
 // S_N Lambda^{-1} S_N r (half_power: Lambda^{-1/2}): forward along x (and y),
 // the pair around Lambda along the last axis, and back.  A 2-D problem's pair
 // runs along y where its matrix is dense.  A dense pair is one pass while a
 // block holds every row of its lines, else two (the first divides by Lambda).
 template <typename R>
-int pinv(const tfde_problem* P, const R* r, R* z, R* t1, R* t2, bool half_power, cudaStream_t s) {
-    const State* F = static_cast<const State*>(P->fft);
-    const int t = sizeof(R) == 8 ? 0 : 1;
-    const int last = P->dim2 && F->lS[t][1].K ? 1 : 2;
-    const LineMatrix& m = F->lS[t][last];
-    const bool two = m.K && m.ld > LINE_ROWS;
+int pinv(const tfde_problem* P, const R* r, R* z, R* t1, R* t2, bool half_power, cudaStream_t s, const int* skip) {
+    const int last = pair_axis<R>(P);
+    const bool two = pair_split<R>(P);
     const R* src = r;
     R* buf[2] = {t1, t2};
     int b = 0, st;
     auto step = [&](int axis, bool lam, R* to) {
-        int e = dst_pass<R>(P, axis, src, to, lam, two, s, half_power);
+        int e = dst_pass<R>(P, axis, src, to, lam, two, s, half_power, skip);
         src = to;
         b ^= 1;
         return e;
@@ -924,20 +944,21 @@ int pinv(const tfde_problem* P, const R* r, R* z, R* t1, R* t2, bool half_power,
 }
 
 template <typename R>
-int apply_Pinv(const tfde_problem* P, const R* r, R* z, R* t1, R* t2, cudaStream_t s) {
-    return pinv<R>(P, r, z, t1, t2, false, s);
+int apply_Pinv(const tfde_problem* P, const R* r, R* z, R* t1, R* t2, cudaStream_t s, const int* skip) {
+    return pinv<R>(P, r, z, t1, t2, false, s, skip);
 }
 
 int apply_Pinv_half(const tfde_problem* P, const double* r, double* z, double* t1, double* t2, cudaStream_t s) {
-    return pinv<double>(P, r, z, t1, t2, true, s);
+    return pinv<double>(P, r, z, t1, t2, true, s, nullptr);
 }
 
 template int apply_A<double>(const tfde_problem*, int, const double*, double*, double*, double*, double*, double*,
                              cudaStream_t);
 template int apply_A<float>(const tfde_problem*, int, const float*, float*, float*, float*, float*, float*,
                             cudaStream_t);
-template int apply_Pinv<double>(const tfde_problem*, const double*, double*, double*, double*, cudaStream_t);
-template int apply_Pinv<float>(const tfde_problem*, const float*, float*, float*, float*, cudaStream_t);
+template int apply_Pinv<double>(const tfde_problem*, const double*, double*, double*, double*, cudaStream_t,
+                                const int*);
+template int apply_Pinv<float>(const tfde_problem*, const float*, float*, float*, float*, cudaStream_t, const int*);
 
 }  // namespace fft
 }  // namespace tfde

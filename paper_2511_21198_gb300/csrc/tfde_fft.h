@@ -45,8 +45,13 @@ void free_state(tfde_problem* P);
 template <typename R>
 int apply_A(const tfde_problem* P, int op, const R* x, R* y, R* a, R* w, R* c, R* e, cudaStream_t s);
 // z = S_N Lambda^{-1} S_N r: five passes (the z pair fused); t1, t2 workspace.
+// With skip set, a launch that finds *skip != 0 does no work (device-side loops).
 template <typename R>
-int apply_Pinv(const tfde_problem* P, const R* r, R* z, R* t1, R* t2, cudaStream_t s);
+int apply_Pinv(const tfde_problem* P, const R* r, R* z, R* t1, R* t2, cudaStream_t s, const int* skip = nullptr);
+// kernel launches of one application
+int operator_launches(const tfde_problem* P);
+template <typename R>
+int preconditioner_launches(const tfde_problem* P);
 
 // z = P^{-1/2} r = S_N Lambda^{-1/2} S_N r (FP64): the symmetric square root
 // of the preconditioner's inverse, from the same diagonalisation.

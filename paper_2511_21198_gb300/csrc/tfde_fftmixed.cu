@@ -11,10 +11,11 @@
 // applied by the FP32 FFT DST-I passes.  The inner operator carries FP32
 // rounding only (about 1e-7 relative per product against the split-BF16
 // contraction's 2^-16), so one sweep reaches further: the inner floor is
-// 1e-5.  Inner products accumulate in FP64; the CG coefficients alpha and
-// beta are formed on the device and the host reads one scalar per PCG
-// iteration (its stopping test) and two per Arnoldi step (the Hessenberg
-// column, whose Givens rotations run on the host as in the FP64 PGMRES).
+// 1e-5.  Inner products accumulate in FP64.  The inner iterations run as one
+// CUDA graph per sweep with the stop test on the device (PCG: tfde_pcgloop.cu;
+// GMRES: build_cycle below, restart lengths up to GS_MAXM); with per-launch
+// timing on, or without such a graph, the host drives them and reads one scalar
+// per PCG iteration and two projections per Arnoldi step.
 #include <chrono>
 #include <cmath>
 #include <vector>
@@ -23,16 +24,14 @@
 #include "tfde_givens.h"
 #include "tfde_gs.cuh"
 #include "tfde_internal.h"
+#include "tfde_mixed.h"
+#include "tfde_pcgloop.h"
 #include "tfde_stats.h"
 
 namespace tfde {
 
 int pcg64(const tfde_problem*, const double*, double*, double, int, tfde_info*, cudaStream_t, bool);
 int pgmres64(tfde_problem*, const double*, double*, int, double, int, tfde_info*, cudaStream_t, bool);
-void launch_dot32(size_t N, const float* a, const float* b, double* part, int nblk, cudaStream_t s);
-void launch_multidot32(size_t N, int m, const float* V, size_t ldv, const float* w, double* part, int nblk,
-                       cudaStream_t s);
-void launch_multiaxpy32(size_t N, int m, const float* V, size_t ldv, const double* h, float* w, cudaStream_t s);
 void launch_add32to64(size_t N, double sc, const float* d, double* x, cudaStream_t s);
 void launch_widen32(size_t N, const float* v, double sc, double* y, cudaStream_t s);
 
@@ -50,6 +49,9 @@ constexpr int kMaxRestart = 120;   // GMRES columns: the reduction scratch holds
 enum { V_R, V_Z, V_P, V_Q, V_X, V_A, V_W, V_C, V_E, NV };
 // device scalars
 enum { S_RZ0 = 0, S_RZ1 = 1, S_PQ = 2, S_RR = 3, S_H = 8, NS = 256 };
+// the device-side GMRES cycle's: both projections, ||w||^2, -y
+enum { S_GH = 8, S_GH2 = S_GH + GS_MAXM, S_GWW = S_GH2 + GS_MAXM, S_GY = S_GWW + 1 };
+static_assert(S_GY + GS_MAXM <= NS, "device scalars of the GMRES cycle");
 
 struct FftMixed {
     float* v[NV] = {};
@@ -57,6 +59,14 @@ struct FftMixed {
     int vcap = 0;
     double* d = nullptr;    // device scalars
     double* h = nullptr;    // pinned host mirror of d
+    // device-side GMRES cycle: the least-squares state, the control words
+    // behind it, and the graph for one restart length
+    double* gm_state = nullptr;
+    cudaGraph_t gm_graph = nullptr;
+    cudaGraphExec_t gm_exec = nullptr;
+    int gm_restart = 0;
+    bool gm_failed = false;
+    int* gm_ctl() const { return reinterpret_cast<int*>(gm_state + GS_WORDS); }
 };
 
 // basis vectors start 16 bytes apart or a multiple of it
@@ -186,6 +196,16 @@ int inner_pcg(const tfde_problem* P, double theta, int maxit, double rr0, int* i
     *iters = 0;
     *reached = 1.0;
     if (!(rr0 > 0.0)) return TFDE_OK;
+    PcgLoopResult loop;
+    const PcgLoopVectors<float> vec{r, z, p, q, {F->v[V_A], F->v[V_W], F->v[V_C], F->v[V_E]}};
+    if ((st = pcg_loop<float>(P, vec, F->v[V_X], theta * theta * rr0, maxit, &loop, s))) return st;
+    if (loop.ran) {
+        if (loop.bad == PCGLOOP_NAN_PAP || loop.bad == PCGLOOP_NAN_RR)
+            return set_error(TFDE_ENAN, "non-finite inner residual");
+        *iters = loop.iters;   // <p, A p> <= 0 ends the sweep: the refinement's stall test decides
+        if (loop.iters > 0) *reached = std::sqrt(loop.rr / rr0);
+        return TFDE_OK;
+    }
     if ((st = op_Pinv32(P, r, p, s))) return st;   // p_0 = z_0 = P^{-1} r_0
     dot_to(P, r, p, d + S_RZ0, s);
     int rz = S_RZ0;
@@ -217,12 +237,105 @@ int inner_pcg(const tfde_problem* P, double theta, int maxit, double rr0, int* i
 int ensure_basis(const tfde_problem* P, int m) {
     FftMixed* F = state(P);
     if (F->vcap >= m) return TFDE_OK;
+    F->gm_restart = 0;   // a graph built before holds the old basis
     cudaFree(F->V);
     F->V = nullptr;
     F->vcap = 0;
     if (cudaMalloc((void**)&F->V, (size_t)(m + 1) * ldv(P->N) * sizeof(float)) != cudaSuccess)
         return set_error(TFDE_ENOMEM, "cudaMalloc of the FP32 GMRES basis failed");
     F->vcap = m;
+    return TFDE_OK;
+}
+
+// The cycle's Arnoldi steps as one graph (a WHILE node; one step per pass of
+// its body): operator on the fixed vector V_P, preconditioner into V_Z, then
+// the Gram-Schmidt sweeps, Givens update, stop test and normalisation of
+// launch_gm_step, which also writes the next V_P.  Built for one restart
+// length; a failure leaves the host-driven cycle in use.
+int build_cycle(const tfde_problem* P, int m, cudaStream_t s) {
+    FftMixed* F = state(P);
+    if (F->gm_failed || m > GS_MAXM || (F->gm_exec && F->gm_restart == m)) return TFDE_OK;
+    if (F->gm_exec) {
+        cudaGraphExecDestroy(F->gm_exec);
+        cudaGraphDestroy(F->gm_graph);
+        F->gm_exec = nullptr;
+        F->gm_graph = nullptr;
+    }
+    if (!F->gm_state) FM_TRY(cudaMalloc((void**)&F->gm_state, GS_WORDS * sizeof(double) + 4 * sizeof(int)));
+    // once outside the capture: the passes' launch attributes are set on first use
+    int st = op_A32(P, F->v[V_P], F->v[V_Q], s);
+    if (!st) st = op_Pinv32(P, F->v[V_Q], F->v[V_Z], s);
+    if (st) return st;
+    cudaGraphConditionalHandle h{};
+    cudaGraphNodeParams cp = {};
+    cudaGraphNode_t node;
+    bool ok = cudaGraphCreate(&F->gm_graph, 0) == cudaSuccess;
+    if (ok) ok = cudaGraphConditionalHandleCreate(&h, F->gm_graph, 1, cudaGraphCondAssignDefault) == cudaSuccess;
+    if (ok) {
+        cp.type = cudaGraphNodeTypeConditional;
+        cp.conditional.handle = h;
+        cp.conditional.type = cudaGraphCondTypeWhile;
+        cp.conditional.size = 1;
+        ok = cudaGraphAddNode(&node, F->gm_graph, nullptr, nullptr, 0, &cp) == cudaSuccess;
+    }
+    const cudaStream_t c = capture_stream();   // the caller's may be the legacy default stream
+    if (ok)
+        ok = cudaStreamBeginCaptureToGraph(c, cp.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                           cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+    if (ok) {
+        stats_set_capturing(true);
+        st = op_A32(P, F->v[V_P], F->v[V_Q], c);
+        if (!st) st = op_Pinv32(P, F->v[V_Q], F->v[V_Z], c);
+        double* d = F->d;
+        if (!st)
+            launch_gm_step(P->N, F->V, ldv(P->N), F->v[V_Z], P->red, P->nblk, d + S_GH, d + S_GH2, d + S_GWW,
+                           F->gm_state, F->gm_ctl(), h, nullptr, nullptr, F->v[V_P], m + 1, c);
+        stats_set_capturing(false);
+        cudaGraph_t out = nullptr;
+        const cudaError_t e = cudaStreamEndCapture(c, &out);
+        ok = st == TFDE_OK && e == cudaSuccess;
+    }
+    if (ok) ok = cudaGraphInstantiate(&F->gm_exec, F->gm_graph, 0) == cudaSuccess;
+    if (!ok) {
+        cudaGetLastError();
+        if (F->gm_graph) cudaGraphDestroy(F->gm_graph);
+        F->gm_graph = nullptr;
+        F->gm_exec = nullptr;
+        F->gm_failed = true;
+        set_error(TFDE_OK, "");
+        return TFDE_OK;
+    }
+    F->gm_restart = m;
+    return TFDE_OK;
+}
+
+// inner_gmres (below) with the Arnoldi steps in the device-side loop: one host
+// read per cycle instead of two per step.
+int inner_gmres_loop(const tfde_problem* P, int m, double theta, int maxit, int* iters, double* est_ratio,
+                     cudaStream_t s) {
+    FftMixed* F = state(P);
+    const size_t N = P->N;
+    double* d = F->d;
+    int* ctl = F->gm_ctl();
+    FM_TRY(cudaMemsetAsync(ctl, 0, 4 * sizeof(int), s));
+    if (int st = op_Pinv32(P, F->v[V_R], F->v[V_Z], s)) return st;
+    launch_gm_start(N, F->v[V_Z], P->red, P->nblk, d + S_GWW, F->gm_state, ctl, m < maxit ? m : maxit, theta, F->V,
+                    nullptr, nullptr, F->v[V_P], s);
+    FM_TRY(cudaGraphLaunch(F->gm_exec, s));
+    launch_gm_solve(F->gm_state, ctl, d + S_GY, m, s);
+    FM_TRY(cudaMemsetAsync(F->v[V_X], 0, N * sizeof(float), s));
+    launch_multiaxpy32(N, m, F->V, ldv(N), d + S_GY, F->v[V_X], s);   // d = V y
+    FM_TRY(cudaMemcpyAsync(F->h, F->gm_state, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
+    FM_TRY(cudaMemcpyAsync(F->h + 2, ctl, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    FM_TRY(cudaStreamSynchronize(s));
+    const int* hc = reinterpret_cast<const int*>(F->h + 2);
+    const double beta = F->h[GS_BETA], est = F->h[GS_EST];
+    if (hc[3] || !std::isfinite(beta))
+        return set_error(TFDE_ENAN, "non-finite preconditioned residual or Arnoldi vector");
+    *iters = hc[0];
+    *est_ratio = beta > 0.0 ? est / beta : 1.0;
+    stats_count_launch((unsigned)(hc[0] > 0 ? hc[0] : 1) *
+                       (8u + (unsigned)fft::operator_launches(P) + (unsigned)fft::preconditioner_launches<float>(P)));
     return TFDE_OK;
 }
 
@@ -241,6 +354,10 @@ int inner_gmres(const tfde_problem* P, int m, double theta, int maxit, int* iter
     int st;
     *iters = 0;
     *est_ratio = 1.0;
+    if (!stats_timing() && maxit > 0) {
+        if ((st = build_cycle(P, m, s))) return st;
+        if (F->gm_exec && F->gm_restart == m) return inner_gmres_loop(P, m, theta, maxit, iters, est_ratio, s);
+    }
     const size_t ld = ldv(N);
     const int nblk = dot_blocks(P->nblk);
     auto col = [&](int j) { return V + (size_t)j * ld; };
@@ -362,6 +479,9 @@ int fmix_init(tfde_problem* P, cudaStream_t s) {
 void fmix_free(tfde_problem* P) {
     FftMixed* F = state(P);
     if (!F) return;
+    if (F->gm_exec) cudaGraphExecDestroy(F->gm_exec);
+    if (F->gm_graph) cudaGraphDestroy(F->gm_graph);
+    cudaFree(F->gm_state);
     for (float* v : F->v) cudaFree(v);
     cudaFree(F->V);
     cudaFree(F->d);

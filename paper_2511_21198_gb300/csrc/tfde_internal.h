@@ -146,6 +146,7 @@ struct tfde_problem {
 
     void* mixed = nullptr;  // mixed-precision state (tensor-core path)
     void* fft = nullptr;    // FFT tables of the FFT-embedded passes (tfde_fft.h), null: dense FP64
+    mutable void* pcg_loop[2] = {nullptr, nullptr};   // device-side PCG loops, FP64 and FP32 (tfde_pcgloop.cu)
     void* fmix = nullptr;   // mixed-precision state on the FFT passes (tfde_fftmixed.cu)
 
     // host copies of a tfde_cn_advance_host step (out == null otherwise): the

@@ -744,18 +744,19 @@ __global__ void gm_givens_kernel(double* gs, const double* h, const double* h2, 
     cudaGraphSetConditional(hc, done ? 0u : 1u);
 }
 
-// V_j (j = the steps done) = w / ||w|| and its split planes, the next
-// operator input
+// V_j (j = the steps done) = w / ||w|| and the next operator input: its split
+// planes, or (next) a copy at a fixed address
 __global__ void gm_scale_basis_kernel(long long N, const float* __restrict__ w, float* V, long long ldv,
                                       const double* gs, const int* gctl, __nv_bfloat16* __restrict__ h,
-                                      __nv_bfloat16* __restrict__ l) {
+                                      __nv_bfloat16* __restrict__ l, float* __restrict__ next) {
     if (gctl[1]) return;
     const float sc = (float)gs[GS_INV];
     float* out = V + (long long)gctl[0] * ldv;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
         const float v = w[i] * sc;
         out[i] = v;
-        split(v, h[i], l[i]);
+        if (next) next[i] = v;
+        else split(v, h[i], l[i]);
     }
 }
 
@@ -789,27 +790,26 @@ __global__ void gm_solve_kernel(const double* gs, const int* gctl, double* ny, i
     for (int i = 0; i < maxm; ++i) ny[i] = i < k ? -y[i] : 0.0;
 }
 
-void launch_gm_step(size_t N, const float* V, float* w, double* part, int nblk, double* hbuf, double* h2buf,
-                    double* wwbuf, double* gs, int* gctl, cudaGraphConditionalHandle hc, float* Vout,
-                    __nv_bfloat16* ph, __nv_bfloat16* pl, int maxm, cudaStream_t s) {
-    stats_count_launch(7);
-    const long long n = (long long)N;
+void launch_gm_step(size_t N, const float* V, size_t ldv, float* w, double* part, int nblk, double* hbuf,
+                    double* h2buf, double* wwbuf, double* gs, int* gctl, cudaGraphConditionalHandle hc,
+                    __nv_bfloat16* ph, __nv_bfloat16* pl, float* next, int maxm, cudaStream_t s) {
+    stats_count_launch(8);
+    const long long n = (long long)N, ld = (long long)ldv;
     nblk = dot_blocks(nblk);
     // CGS2: <V, w>; w -= V h and <V, w> again (one pass over the block's chunk);
     // w -= V h2 and ||w||^2 (one pass)
-    gm_multidot_kernel<<<nblk, kT, 0, s>>>(n, V, n, w, part, gctl);
+    gm_multidot_kernel<<<nblk, kT, 0, s>>>(n, V, ld, w, part, gctl);
     gm_reduce_kernel<<<maxm, 32, 0, s>>>(part, nblk, hbuf, 0, gctl);
-    gm_axpy_dot_kernel<<<nblk, kT, 0, s>>>(n, V, n, hbuf, w, part, gctl);
+    gm_axpy_dot_kernel<<<nblk, kT, 0, s>>>(n, V, ld, hbuf, w, part, gctl);
     gm_reduce_kernel<<<maxm, 32, 0, s>>>(part, nblk, h2buf, 0, gctl);
-    gm_axpy_norm_kernel<<<nblk, kT, 0, s>>>(n, V, n, h2buf, w, part, gctl);
+    gm_axpy_norm_kernel<<<nblk, kT, 0, s>>>(n, V, ld, h2buf, w, part, gctl);
     gm_reduce_kernel<<<1, 32, 0, s>>>(part, nblk, wwbuf, 1, gctl);
     gm_givens_kernel<<<1, 1, 0, s>>>(gs, hbuf, h2buf, wwbuf, gctl, hc);
-    (void)Vout;
-    stats_count_launch();
-    gm_scale_basis_kernel<<<grid_for(n), kT, 0, s>>>(n, w, const_cast<float*>(V), n, gs, gctl, ph, pl);
+    gm_scale_basis_kernel<<<grid_for(n), kT, 0, s>>>(n, w, const_cast<float*>(V), ld, gs, gctl, ph, pl, next);
 }
 void launch_gm_start(size_t N, const float* w, double* part, int nblk, double* wwbuf, double* gs, int* gctl,
-                     int maxsteps, double ptheta, float* V0, __nv_bfloat16* ph, __nv_bfloat16* pl, cudaStream_t s) {
+                     int maxsteps, double ptheta, float* V0, __nv_bfloat16* ph, __nv_bfloat16* pl, float* next,
+                     cudaStream_t s) {
     stats_count_launch(4);
     const long long n = (long long)N;
     nblk = dot_blocks(nblk);
@@ -817,7 +817,7 @@ void launch_gm_start(size_t N, const float* w, double* part, int nblk, double* w
     gm_dot_kernel<<<nblk, kT, 0, s>>>(n, w, part, gctl);
     gm_reduce_kernel<<<1, 32, 0, s>>>(part, nblk, wwbuf, 1, gctl);
     gm_start_kernel<<<1, 1, 0, s>>>(gs, wwbuf, gctl, maxsteps, ptheta);
-    gm_scale_basis_kernel<<<grid_for(n), kT, 0, s>>>(n, w, V0, n, gs, gctl, ph, pl);
+    gm_scale_basis_kernel<<<grid_for(n), kT, 0, s>>>(n, w, V0, n, gs, gctl, ph, pl, next);
 }
 void launch_gm_solve(const double* gs, const int* gctl, double* ny, int maxm, cudaStream_t s) {
     stats_count_launch();

@@ -42,6 +42,7 @@ struct LinePass {
     const void* lam;              // [mass x | y | z | tau x | y | z] (double or float) or null
     double c0, c1, c2;            // eta_a (k+ + k-)
     int half_power;               // divide by Lambda^{1/2} instead of Lambda
+    const int* skip;              // optional: no work when *skip != 0
 };
 
 constexpr int LINE_ROWS = 128;    // matrix rows per block of the grid
@@ -126,6 +127,7 @@ __global__ void __launch_bounds__(256, LT >= 4 ? 2 : 3) line_pass_kernel(const _
     constexpr int KC = line_chunk<R>();
     constexpr int Q = 16 / sizeof(R);
     extern __shared__ __align__(16) unsigned char line_smem[];
+    if (p.skip && *p.skip) return;
     const int n = p.n, K = p.m.K, half = p.m.half, ld = p.m.ld;
     const int rows = blockDim.x / TL * RT;                   // matrix rows of this block
     const int row0 = blockIdx.y * LINE_ROWS;

@@ -877,8 +877,8 @@ int build_gmres_graph_spec(const tfde_problem* P, int restart, cudaStream_t s) {
             const int* skip = M->gm_ctl + 1;
             int st = spec_matvec(P, nullptr, M->f[F_Z], nullptr, s, skip, true);   // w = Lambda^{-1} A~ v_j
             if (!st)
-                launch_gm_step(N, M->V32, M->f[F_Z], P->red, P->nblk, M->gm + GM_H, M->gm + GM_H2, M->gm + GM_WW,
-                               M->gm_state, M->gm_ctl, h, nullptr, M->hi[PL_P], M->lo[PL_P], restart + 1, s);
+                launch_gm_step(N, M->V32, N, M->f[F_Z], P->red, P->nblk, M->gm + GM_H, M->gm + GM_H2, M->gm + GM_WW,
+                               M->gm_state, M->gm_ctl, h, M->hi[PL_P], M->lo[PL_P], nullptr, restart + 1, s);
             stats_set_capturing(false);
             cudaGraph_t out = nullptr;
             const cudaError_t e = cudaStreamEndCapture(s, &out);
@@ -926,7 +926,7 @@ int inner_gmres_spec(const tfde_problem* P, int restart, double ptheta, int maxi
         MX_TRY(cudaMemsetAsync(M->gm_ctl, 0, 4 * sizeof(int), s));
         const int maxsteps = restart < maxit ? restart : maxit;
         launch_gm_start(N, M->f[F_Z], P->red, P->nblk, g + GM_WW, M->gm_state, M->gm_ctl, maxsteps, ptheta, V,
-                        M->hi[PL_P], M->lo[PL_P], s);
+                        M->hi[PL_P], M->lo[PL_P], nullptr, s);
         MX_TRY(cudaGraphLaunch(M->gms_exec, s));
         ++M->graph_launches;
         launch_gm_solve(M->gm_state, M->gm_ctl, g + GM_Y, restart, s);
@@ -1097,8 +1097,8 @@ int build_gmres_graph(const tfde_problem* P, int restart, cudaStream_t s) {
             int st = fast_matvec(P, TFDE_OP_A, nullptr, s, PL_R, nullptr, nullptr, skip);
             if (!st) st = fast_precond(P, M->f[F_Z], s, nullptr, nullptr, skip);
             if (!st)
-                launch_gm_step(N, M->V32, M->f[F_Z], P->red, P->nblk, M->gm + GM_H, M->gm + GM_H2, M->gm + GM_WW,
-                               M->gm_state, M->gm_ctl, h, nullptr, M->hi[PL_P], M->lo[PL_P], restart + 1, s);
+                launch_gm_step(N, M->V32, N, M->f[F_Z], P->red, P->nblk, M->gm + GM_H, M->gm + GM_H2, M->gm + GM_WW,
+                               M->gm_state, M->gm_ctl, h, M->hi[PL_P], M->lo[PL_P], nullptr, restart + 1, s);
             stats_set_capturing(false);
             cudaGraph_t out = nullptr;
             const cudaError_t e = cudaStreamEndCapture(s, &out);
@@ -1134,7 +1134,7 @@ int inner_gmres_graph(const tfde_problem* P, int restart, double ptheta, int max
     if (st) return st;
     const int maxsteps = restart < maxit ? restart : maxit;
     launch_gm_start(N, M->f[F_Z], P->red, P->nblk, M->gm + GM_WW, M->gm_state, M->gm_ctl, maxsteps, ptheta, M->V32,
-                    M->hi[PL_P], M->lo[PL_P], s);
+                    M->hi[PL_P], M->lo[PL_P], nullptr, s);
     MX_TRY(cudaGraphLaunch(M->gm_exec, s));
     ++M->graph_launches;
     launch_gm_solve(M->gm_state, M->gm_ctl, M->gm + GM_Y, restart, s);

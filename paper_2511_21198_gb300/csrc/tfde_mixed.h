@@ -68,12 +68,15 @@ enum { GS_BETA = 0, GS_EST = 1, GS_INV = 2, GS_THR = 3, GS_G = 8, GS_CS = GS_G +
 // one Arnoldi step on w (the preconditioner's output): CGS2 against V_0..V_j,
 // ||w||, the Givens update and stop test (loop condition hc), V_{j+1} = w/||w||
 // with its split planes; every count and address from the control words
-void launch_gm_step(size_t N, const float* V, float* w, double* part, int nblk, double* hbuf, double* h2buf,
-                    double* wwbuf, double* gs, int* gctl, cudaGraphConditionalHandle hc, float* Vout,
-                    __nv_bfloat16* ph, __nv_bfloat16* pl, int maxm, cudaStream_t s);
-// cycle start on w = P^{-1} r: beta, g = beta e_1, V_0 = w / beta and its planes
+// (V_i at V + i ldv; the next operator input goes to the split planes, or with
+// `next` as FP32 to that fixed address)
+void launch_gm_step(size_t N, const float* V, size_t ldv, float* w, double* part, int nblk, double* hbuf,
+                    double* h2buf, double* wwbuf, double* gs, int* gctl, cudaGraphConditionalHandle hc,
+                    __nv_bfloat16* ph, __nv_bfloat16* pl, float* next, int maxm, cudaStream_t s);
+// cycle start on w = P^{-1} r: beta, g = beta e_1, V_0 = w / beta and the next operator input
 void launch_gm_start(size_t N, const float* w, double* part, int nblk, double* wwbuf, double* gs, int* gctl,
-                     int maxsteps, double ptheta, float* V0, __nv_bfloat16* ph, __nv_bfloat16* pl, cudaStream_t s);
+                     int maxsteps, double ptheta, float* V0, __nv_bfloat16* ph, __nv_bfloat16* pl, float* next,
+                     cudaStream_t s);
 // ny = -y of the cycle's least-squares problem (zero beyond the steps done)
 void launch_gm_solve(const double* gs, const int* gctl, double* ny, int maxm, cudaStream_t s);
 // c64 = sc * d32; x64 += c64

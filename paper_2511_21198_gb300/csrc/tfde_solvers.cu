@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "tfde_fft.h"
+#include "tfde_pcgloop.h"
 #include "tfde_internal.h"
 #include "tfde_givens.h"
 
@@ -127,6 +128,38 @@ int true_residual(const tfde_problem* P, const double* b, const double* x, doubl
     return TFDE_OK;
 }
 
+// pcg64's iterations in the device-side loop (tfde_pcgloop.cu): the recursive
+// residual (W_R) runs down to the target, the true one decides, and the loop
+// restarts from it when the two have parted.  *looped = false: no such loop.
+int pcg64_looped(const tfde_problem* P, const double* b, double* x, double target, int maxit, tfde_info* loc,
+                 double* nr, int* status, bool* looped, cudaStream_t s) {
+    double* const* w = P->w;
+    using T = tfde_problem;
+    const PcgLoopVectors<double> v{w[T::W_R], w[T::W_Z], w[T::W_P], w[T::W_Q],
+                                   {w[T::W_A], w[T::W_W], w[T::W_C], w[T::W_E]}};
+    *status = TFDE_ENOCONV;
+    while (loc->iters < maxit) {
+        PcgLoopResult res;
+        int st = pcg_loop<double>(P, v, x, target * target, maxit - loc->iters, &res, s);
+        if (st) return st;
+        if (!res.ran) return TFDE_OK;
+        *looped = true;
+        loc->iters += res.iters;
+        if (res.bad) {
+            *status = res.bad == PCGLOOP_BREAKDOWN ? set_error(TFDE_EBREAKDOWN, "PCG breakdown: p.Ap <= 0")
+                                                   : set_error(TFDE_ENAN, res.bad == PCGLOOP_NAN_PAP ? "non-finite p.Ap"
+                                                                                                     : "non-finite residual");
+            return TFDE_OK;
+        }
+        if ((st = true_residual(P, b, x, w[T::W_R], nr, s))) return st;
+        if (*nr <= target) {
+            *status = TFDE_OK;
+            return TFDE_OK;
+        }
+    }
+    return TFDE_OK;
+}
+
 }  // namespace
 
 // Preconditioned CG (Sec. 3.1) in FP64, true-residual stopping test.
@@ -164,6 +197,14 @@ int pcg64(const tfde_problem* P, const double* b, double* x, double tol, int max
     } else if (nr <= tol * nb) {
         status = TFDE_OK;
         loc.relres = nr / nb;
+    } else if (bool looped = false; (st = pcg64_looped(P, b, x, tol * nb, maxit, &loc, &nr, &status, &looped, s))) {
+        return st;
+    } else if (looped) {
+        if (status == TFDE_OK) loc.relres = nr / nb;
+        if (status == TFDE_ENOCONV) {
+            loc.relres = nr / nb;
+            set_error(TFDE_ENOCONV, "PCG reached maxit");
+        }
     } else {
         if ((st = apply_Pinv64(P, r, z, s))) return st;
         TFDE_CUDA_TRY(cudaMemcpyAsync(p, z, P->N * sizeof(double), cudaMemcpyDeviceToDevice, s));
@@ -249,7 +290,7 @@ int pgmres64(tfde_problem* P, const double* b, double* x, int restart, double to
     loc.relres0 = nr / nb;
     double ratio = 1.0;  // observed (true relres) / (preconditioned relres)
     int status = TFDE_ENOCONV;
-    std::vector<double> h(restart + 2), h2(restart + 2), y;
+    std::vector<double> h(restart + 2), y;
     double* hdev = P->red_out + 128;
     while (true) {
         if (!std::isfinite(nr)) { status = set_error(TFDE_ENAN, "non-finite residual"); break; }
@@ -274,16 +315,22 @@ int pgmres64(tfde_problem* P, const double* b, double* x, int restart, double to
             double* w = V + (size_t)(j + 1) * N;
             if ((st = apply_A64(P, TFDE_OP_A, vj, q, s))) return st;
             if ((st = apply_Pinv64(P, q, w, s))) return st;
-            // CGS2: two rounds of h = V^T w, w -= V h
-            if ((st = dots64(P, j + 1, V, N, w, h.data(), s))) return st;
-            TFDE_CUDA_TRY(cudaMemcpyAsync(hdev, h.data(), (j + 1) * sizeof(double), cudaMemcpyHostToDevice, s));
-            launch_multiaxpy_f64(N, j + 1, V, N, hdev, w, s);
-            if ((st = dots64(P, j + 1, V, N, w, h2.data(), s))) return st;
-            TFDE_CUDA_TRY(cudaMemcpyAsync(hdev, h2.data(), (j + 1) * sizeof(double), cudaMemcpyHostToDevice, s));
-            launch_multiaxpy_f64(N, j + 1, V, N, hdev, w, s);
-            for (int i = 0; i <= j; ++i) h[i] += h2[i];
-            double ww;
-            if ((st = dot(P, w, w, &ww, s))) return st;
+            // CGS2: two rounds of h = V^T w, w -= V h, the coefficients on the
+            // device (slots 0.., 64.. of red_out, restart <= 64), ||w||^2 behind
+            // them: one host read per step
+            const int nblk = dot_blocks(P->nblk);
+            for (int pass = 0; pass < 2; ++pass) {
+                launch_multidot_f64(N, j + 1, V, N, w, P->red, nblk, s);
+                launch_reduce_finish(P->red, nblk, j + 1, P->red_out + 64 * pass, s);
+                launch_multiaxpy_f64(N, j + 1, V, N, P->red_out + 64 * pass, w, s);
+            }
+            launch_multidot_f64(N, 1, w, 0, w, P->red, nblk, s);
+            launch_reduce_finish(P->red, nblk, 1, hdev, s);
+            TFDE_CUDA_TRY(cudaGetLastError());
+            TFDE_CUDA_TRY(cudaMemcpyAsync(P->red_host, P->red_out, 129 * sizeof(double), cudaMemcpyDeviceToHost, s));
+            TFDE_CUDA_TRY(cudaStreamSynchronize(s));
+            for (int i = 0; i <= j; ++i) h[i] = P->red_host[i] + P->red_host[64 + i];
+            const double ww = P->red_host[128];
             const double hn = std::sqrt(ww);
             h[j + 1] = hn;
             if (!std::isfinite(hn)) { status = set_error(TFDE_ENAN, "non-finite Arnoldi vector"); break; }
