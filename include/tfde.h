@@ -450,7 +450,8 @@ int tfde_batch_cn_advance(tfde_batch* batch, double* const* u, const double* con
  * and 3/4 of the SMs) and the depth of the operand ring (2 .. 4 stages of
  * 48 KB, or 2 of 96 KB), per launch class.  A class is the kernel instance
  * (grouped, operand layout, output mode), the stage size, the rows n of the
- * contraction (0 for grouped launches) and the number of 128 x 256 tiles.
+ * contraction (0 for grouped launches) and the number of tiles (128 rows x 256,
+ * 128 or 64 lines, by the size of the launch).
  *
  * tfde_tune records the launches of one operator and one preconditioner
  * application of a TFDE_MIXED problem on the tensor-core path, times each
@@ -475,7 +476,7 @@ typedef struct {
     int out_mode;     /* 0 FP32, 1 split planes, 2 direction update, 3 hi plane */
     int stage_bytes;  /* ring stage size of the class                            */
     int n;            /* rows of the contraction (0 for grouped launches)        */
-    long long tiles;  /* 128 x 256 tiles of the launch                           */
+    long long tiles;  /* tiles of the launch                                      */
     int grid;         /* chosen persistent CTAs                                  */
     int stages;       /* chosen ring stages                                      */
     float us;         /* measured microseconds per launch with the choice        */

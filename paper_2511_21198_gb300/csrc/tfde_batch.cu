@@ -717,6 +717,7 @@ struct tfde_batch {
     long long pcg_graph_launches = 0;
     long long* d_gstart = nullptr;  // [3][count + 1]
     long long gtotal[3] = {};
+    int bn[3] = {256, 256, 256};   // lines per tile of the grouped passes along each axis
     // vector kernels: per-problem pointers and the block table
     tfde::BVec* d_vt = nullptr;
     tfde::BVec* h_vt = nullptr;
@@ -848,7 +849,7 @@ int free_batch(tfde_batch* B) {
 
 int grouped(tfde_batch* B, const tc::Params* d, int axis, int out_mode, double bytes, double flops, cudaStream_t s) {
     return tc::launch_grouped(d, B->d_gstart + (size_t)axis * (B->count + 1), B->count, B->gtotal[axis],
-                              axis == 0 ? 1 : 0, out_mode, B->d_act, B->d_err, s, bytes, flops);
+                              axis == 0 ? 1 : 0, out_mode, B->bn[axis], B->d_act, B->d_err, s, bytes, flops);
 }
 
 // v_j (split planes PL_P of every active problem) -> PL_R = A v_j
@@ -1318,6 +1319,17 @@ int batch_create(const tfde_params* params, int count, int restart, cudaStream_t
         free_batch(B);
         return set_error(code, what);
     };
+    // one tile width per axis for the grouped launches (and the problems' own)
+    for (int a = 0; a < 3; ++a) {
+        long long wide = 0;
+        for (tfde_problem* P : B->P) wide += tc::wide_tiles(P->n, a);
+        B->bn[a] = tc::tile_lines(wide);
+    }
+    for (tfde_problem* P : B->P)
+        if ((st = mixed_set_tiles(P, B->bn))) {
+            free_batch(B);
+            return st;
+        }
     // grouped descriptors
     const size_t C = count, PS = sizeof(tc::Params);
     std::vector<tc::Params> mv(5 * C), pc(5 * C), pcl((size_t)(restart + 1) * C);
@@ -1375,7 +1387,7 @@ int batch_create(const tfde_params* params, int count, int restart, cudaStream_t
         }
         for (int a = 0; a < 3; ++a) {
             tc::Params g;
-            tc::set_geometry(g, P->n, a);
+            tc::set_geometry(g, P->n, a, B->bn[a]);
             gstart[a * (C + 1) + i + 1] = gstart[a * (C + 1) + i] + g.ntiles * g.mhalves;
         }
     }

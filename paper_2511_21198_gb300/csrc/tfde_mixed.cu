@@ -73,7 +73,7 @@ void gemm_params(const tfde_problem* P, int axis, const SegSpec* segs, int nseg,
                  float* out_f32, int out_plane, bool lam_scale, tc::Params& prm, double* bytes, double* flops) {
     MixedState* M = mixed(P);
     std::memset(&prm, 0, sizeof(prm));
-    tc::set_geometry(prm, P->n, axis);
+    tc::set_geometry(prm, P->n, axis, M->bn[axis]);
     // tensor maps: merged boxes where the allocation allows one copy per operand
     // (hi/lo operator pair; hi/lo plane pair with, on y/z, all line blocks)
     int na = 0, nb = 0;
@@ -257,7 +257,7 @@ int fast_matvec(const tfde_problem* P, int op, float* q32, cudaStream_t s, int o
     for (int g = 0; g < 2; ++g) {
         M->gemm_launches++;
         st = tc::launch_grouped(M->pair_d + 2 * g, M->pair_gstart + 3 * g, 2, M->pair_total[g], g == 0 ? 1 : 0,
-                                tc::OUT_HILO, nullptr, M->err, s, M->pair_bytes[g], M->pair_flops[g], skip);
+                                tc::OUT_HILO, M->bn[g == 0 ? 0 : 1], nullptr, M->err, s, M->pair_bytes[g], M->pair_flops[g], skip);
         if (st) return st;
     }
     return run_passes(P, ps + 4, 1, q32, s, dot_vec, dot_out, skip);
@@ -1277,6 +1277,22 @@ int spec_pass_descriptors(const tfde_problem* P, int kind, float* out_f32, tc::P
     return 3;
 }
 
+// The lines per tile along each axis, and the input maps whose boxes follow
+// them (before any pass or graph of the problem uses them).
+int mixed_set_tiles(const tfde_problem* P, const int bn[3]) {
+    MixedState* M = mixed(P);
+    for (int a = 0; a < 3; ++a) M->bn[a] = bn[a];
+    for (int pl = 0; pl < NPL; ++pl)
+        for (int a = 0; a < 3; ++a) {
+            int st = tc::make_map_B(&M->bmap_hi[pl][a], M->hi[pl], P->n, a, bn[a]);
+            if (!st) st = tc::make_map_B(&M->bmap_lo[pl][a], M->lo[pl], P->n, a, bn[a]);
+            if (st) return st;
+            M->bmap2_rank[pl][a] = tc::make_map_B_pair(&M->bmap2[pl][a], M->hi[pl], P->n, a, bn[a]);
+            M->bmap1_rank[pl][a] = tc::make_map_B_pair(&M->bmap1[pl][a], M->hi[pl], P->n, a, bn[a], 1);
+        }
+    return TFDE_OK;
+}
+
 int mixed_prepare_gmres(const tfde_problem* P, int restart) { return ensure_v32(P, restart); }
 
 namespace {
@@ -1404,15 +1420,16 @@ int mixed_init(tfde_problem* P, cudaStream_t s) {
         M->lo[pl] = M->hi[pl] + N;
         MX_TRY(cudaMemsetAsync(M->hi[pl], 0, 2 * N * sizeof(__nv_bfloat16), s));
         for (int a = 0; a < 3; ++a) {
-            int st = tc::make_map_B(&M->bmap_hi[pl][a], M->hi[pl], P->n, a);
-            if (!st) st = tc::make_map_B(&M->bmap_lo[pl][a], M->lo[pl], P->n, a);
-            if (st) return st;
-            M->bmap2_rank[pl][a] = tc::make_map_B_pair(&M->bmap2[pl][a], M->hi[pl], P->n, a);
-            M->bmap1_rank[pl][a] = tc::make_map_B_pair(&M->bmap1[pl][a], M->hi[pl], P->n, a, 1);
+            int st;
             if ((st = tc::make_out_map(&M->omap_hi[pl][a], M->hi[pl], P->n, a, false)) ||
                 (st = tc::make_out_map_pair(&M->omap_hl[pl][a], M->hi[pl], P->n, a)))
                 return st;
         }
+    }
+    {
+        int bn[3];
+        for (int a = 0; a < 3; ++a) bn[a] = tc::tile_lines(tc::wide_tiles(P->n, a));
+        if (int st = mixed_set_tiles(P, bn)) return st;
     }
     for (int v = 0; v < NF; ++v) {
         MX_TRY(cudaMalloc((void**)&M->f[v], N * sizeof(float)));

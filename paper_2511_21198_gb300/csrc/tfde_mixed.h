@@ -143,6 +143,7 @@ struct MixedState {
     __nv_bfloat16* lo[NPL] = {};
     CUtensorMap bmap_hi[NPL][3];
     CUtensorMap bmap_lo[NPL][3];
+    int bn[3] = {256, 256, 256};   // lines per tile of the passes along each axis (the planes' boxes)
     CUtensorMap bmap2[NPL][3];     // both planes (and on y/z all four 64-line blocks) in one box
     int bmap2_rank[NPL][3] = {};   // 3 (x), 5 (y/z), 0 = not available
     CUtensorMap bmap1[NPL][3];     // the hi plane alone, same box otherwise
@@ -239,6 +240,7 @@ int spec_pass_descriptors(const tfde_problem* P, int kind, float* out_f32, tc::P
                           double* flops, const float* dot_vec = nullptr, double* dot_out = nullptr);
 // Allocate the FP32 GMRES basis (restart + 1 vectors) and Hessenberg scratch.
 int mixed_prepare_gmres(const tfde_problem* P, int restart);
+int mixed_set_tiles(const tfde_problem* P, const int bn[3]);
 
 int oz_init(tfde_problem* P, const std::vector<double> etaB[3], cudaStream_t s);
 void oz_free(MixedState* M);

@@ -79,15 +79,15 @@ int make_map_A(CUtensorMap* m, const __nv_bfloat16* base, int n) {
 }
 
 // Vector plane viewed along `axis` -> B operand of the split contraction
-// (k-blocks of SK, 128B swizzle): x axis K-major box {SK, BN}; y / z axes
+// (k-blocks of SK, 128B swizzle): x axis K-major box {SK, bn}; y / z axes
 // MN-major box {64 lines, SK, 1}.
-int make_map_B(CUtensorMap* m, const __nv_bfloat16* base, const int n[3], int axis) {
+int make_map_B(CUtensorMap* m, const __nv_bfloat16* base, const int n[3], int axis, int bn) {
     const cuuint64_t n1 = n[0], n2 = n[1], n3 = n[2];
     if (n[0] % 8) return set_error(TFDE_EUNSUPPORTED, "tensor-core path needs n1 multiple of 8");
     if (axis == 0) {
         const cuuint64_t dims[2] = {n1, n2 * n3};
         const cuuint64_t strides[1] = {n1 * 2};
-        const cuuint32_t box[2] = {(cuuint32_t)SK, (cuuint32_t)BN};
+        const cuuint32_t box[2] = {(cuuint32_t)SK, (cuuint32_t)bn};
         return encode(m, base, 2, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
     }
     cuuint64_t C, K, P;
@@ -111,26 +111,26 @@ int make_map_B_box(CUtensorMap* m, const __nv_bfloat16* base, const int n[3], in
 }
 
 // Both planes of a split pair (hi at base, lo at base + N) along `axis` as one
-// tensor: x axis 3-D (k, line, plane) with box {SK, BN, planes}; y / z axes,
-// when the contiguous line extent C is a multiple of BN, 5-D (line in block,
-// k, block, outer plane, hi/lo) with box {64, SK, BN / 64, 1, planes}, so that
+// tensor: x axis 3-D (k, line, plane) with box {SK, bn, planes}; y / z axes,
+// when the contiguous line extent C is a multiple of bn, 5-D (line in block,
+// k, block, outer plane, hi/lo) with box {64, SK, bn / 64, 1, planes}, so that
 // a single copy fills the whole B stage in the layout of the per-plane boxes.
 // Returns the rank, or 0 when no merged map applies.
-int make_map_B_pair(CUtensorMap* m, const __nv_bfloat16* base, const int n[3], int axis, int planes) {
+int make_map_B_pair(CUtensorMap* m, const __nv_bfloat16* base, const int n[3], int axis, int bn, int planes) {
     const cuuint64_t n1 = n[0], n2 = n[1], n3 = n[2], N = n1 * n2 * n3;
     if (axis == 0) {
         const cuuint64_t dims[3] = {n1, n2 * n3, 2};
         const cuuint64_t strides[2] = {n1 * 2, N * 2};
-        const cuuint32_t box[3] = {(cuuint32_t)SK, (cuuint32_t)BN, (cuuint32_t)planes};
+        const cuuint32_t box[3] = {(cuuint32_t)SK, (cuuint32_t)bn, (cuuint32_t)planes};
         return encode(m, base, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B) == TFDE_OK ? 3 : 0;
     }
     cuuint64_t C, K, P;
     if (axis == 1) { C = n1; K = n2; P = n3; }
     else { C = n1 * n2; K = n3; P = 1; }
-    if (C % BN != 0) return 0;
+    if (C % bn != 0) return 0;
     const cuuint64_t dims[5] = {64, K, C / 64, P, 2};
     const cuuint64_t strides[4] = {C * 2, 128, C * K * 2, N * 2};
-    const cuuint32_t box[5] = {64, (cuuint32_t)SK, (cuuint32_t)(BN / 64), 1, (cuuint32_t)planes};
+    const cuuint32_t box[5] = {64, (cuuint32_t)SK, (cuuint32_t)(bn / 64), 1, (cuuint32_t)planes};
     if (encode(m, base, 5, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B) != TFDE_OK) {
         set_error(TFDE_OK, "");
         return 0;
@@ -192,13 +192,14 @@ void set_ring(Params& P) {
         if (P.seg[g].nb > nb) nb = P.seg[g].nb;
     }
     P.stage_b_off = na * A_TILE_BYTES;
-    P.stage_bytes = P.stage_b_off + nb * B_TILE_BYTES;
+    P.stage_bytes = P.stage_b_off + nb * P.bn * SK * 2;
     const int ns = RING_BYTES / P.stage_bytes;
     P.nstages = ns < MAX_STAGES ? ns : MAX_STAGES;
 }
 
 // Fill the geometry fields of Params for a contraction along `axis`.
-void set_geometry(Params& P, const int n[3], int axis) {
+void set_geometry(Params& P, const int n[3], int axis, int bn) {
+    P.bn = bn;
     const long long n1 = n[0], n2 = n[1], n3 = n[2];
     P.n = n[axis];
     P.mhalves = (n[axis] + BM - 1) / BM;
@@ -206,7 +207,7 @@ void set_geometry(Params& P, const int n[3], int axis) {
     if (axis == 0) {
         P.b_kmajor = 1;
         P.lines = n2 * n3;
-        P.ntiles = (P.lines + BN - 1) / BN;
+        P.ntiles = (P.lines + bn - 1) / bn;
         P.C = 0; P.nbc = 1; P.P = 1; P.nblocks = 0; P.plane = 0;
     } else {
         P.b_kmajor = 0;
@@ -214,10 +215,37 @@ void set_geometry(Params& P, const int n[3], int axis) {
         else { P.C = (int)(n1 * n2); P.P = 1; }
         P.nbc = (P.C + 63) / 64;
         P.nblocks = (long long)P.nbc * P.P;
-        P.ntiles = (P.nblocks + (BN / 64) - 1) / (BN / 64);
+        P.ntiles = (P.nblocks + (bn / 64) - 1) / (bn / 64);
         P.lines = (long long)P.C * P.P;
         P.plane = (long long)P.C * n[axis];
     }
+}
+
+long long wide_tiles(const int n[3], int axis) {
+    Params p;
+    set_geometry(p, n, axis, BN);
+    return p.ntiles * p.mhalves;
+}
+
+// The width with the least rounds of tiles over the SMs x cost of a tile (its
+// epilogue runs 32 x 32 chunks in turn; about a tenth of a 256-line tile does
+// not shrink with it).  Measured on GB300, 256 lines against the choice: 40 x
+// 32 x 24 (6 tiles; 64 lines) 13.7 -> 11.3 ms per 8 steps, 128^3 (64 tiles; 128
+// lines) 36.2 -> 33.2 ms per 10 steps (64 lines: 33.8), 256^3 (512 tiles in
+// 3.4 rounds; 128 lines) 56.1 -> 55.7; 192^3 (288 tiles; 256 lines stay) 19.4
+// against 19.6 ms with 128.
+int tile_lines(long long wide) {
+    const long long sms = num_sms();
+    int best = 0;
+    long long least = 0;
+    for (const int bn : {256, 128, 64}) {
+        const long long tiles = wide * (256 / bn), cost = (tiles + sms - 1) / sms * (bn == 256 ? 40 : (bn == 128 ? 22 : 13));
+        if (!best || cost < least) {
+            best = bn;
+            least = cost;
+        }
+    }
+    return best;
 }
 
 bool attr_done = false;
@@ -353,8 +381,8 @@ TuneKey tune_key_single(const Params& P) {
     return TuneKey{0, P.b_kmajor, P.out_mode, P.stage_bytes, P.n, P.ntiles * P.mhalves};
 }
 
-TuneKey tune_key_grouped(int b_kmajor, int out_mode, long long total) {
-    return TuneKey{1, b_kmajor, out_mode, MAXA * A_TILE_BYTES + MAXB * B_TILE_BYTES, 0, total};
+TuneKey tune_key_grouped(int b_kmajor, int out_mode, int stage_bytes, long long total) {
+    return TuneKey{1, b_kmajor, out_mode, stage_bytes, 0, total};
 }
 
 void tune_put(const TuneKey& k, const TuneVal& v) {
@@ -429,7 +457,7 @@ int launch(const Params& P0, cudaStream_t s, double bytes, double flops) {
 }
 
 int launch_grouped(const Params* groups, const long long* gstart, int ngroups, long long total, int b_kmajor,
-                   int out_mode, const int* gactive, int* err, cudaStream_t s, double bytes, double flops,
+                   int out_mode, int bn, const int* gactive, int* err, cudaStream_t s, double bytes, double flops,
                    const int* skip) {
     if (int st = set_attrs()) return st;
     if (out_mode == OUT_HI || out_mode == OUT_XPAY)
@@ -441,15 +469,16 @@ int launch_grouped(const Params* groups, const long long* gstart, int ngroups, l
     p0.mhalves = 1;
     // the largest stage any group may need: two operator terms, two planes
     p0.stage_b_off = MAXA * A_TILE_BYTES;
-    p0.stage_bytes = p0.stage_b_off + MAXB * B_TILE_BYTES;
+    p0.bn = bn;
+    p0.stage_bytes = p0.stage_b_off + MAXB * bn * SK * 2;
     p0.b_kmajor = b_kmajor;
     p0.out_mode = out_mode;
     p0.err = err;
     p0.skip = skip;
     long long grid;
-    choose(tune_key_grouped(b_kmajor, out_mode, total), total, stage_capacity(p0.stage_bytes), &grid, &p0.nstages);
+    choose(tune_key_grouped(b_kmajor, out_mode, p0.stage_bytes, total), total, stage_capacity(p0.stage_bytes), &grid, &p0.nstages);
     if (g_recording)
-        g_rec.push_back(Rec{tune_key_grouped(b_kmajor, out_mode, total), p0, groups, gstart, ngroups, total, gactive});
+        g_rec.push_back(Rec{tune_key_grouped(b_kmajor, out_mode, p0.stage_bytes, total), p0, groups, gstart, ngroups, total, gactive});
     void* tok = stats_tc_begin(s, TFDE_KIND_SPLIT);
     launch_instance<true>(b_kmajor, out_mode, (unsigned)grid, s, p0, groups, gstart, ngroups, gactive);
     cudaError_t e = cudaGetLastError();

@@ -25,27 +25,33 @@ int make_out_map(CUtensorMap* m, const void* base, const int n[3], int axis, boo
 // the split-plane pair (hi at base, lo N elements after it) as one output tensor
 int make_out_map_pair(CUtensorMap* m, const void* base, const int n[3], int axis);
 void set_ring(Params& P);
-int make_map_B(CUtensorMap* m, const __nv_bfloat16* base, const int n[3], int axis);
+// bn: lines per tile (256, 128 or 64) in the next two and set_geometry
+int make_map_B(CUtensorMap* m, const __nv_bfloat16* base, const int n[3], int axis, int bn);
 int make_map_B_box(CUtensorMap* m, const __nv_bfloat16* base, const int n[3], int axis, int box_lines);
 // planes: 2 (hi and lo in one box) or 1 (the hi plane alone)
-int make_map_B_pair(CUtensorMap* m, const __nv_bfloat16* base, const int n[3], int axis, int planes = 2);
-void set_geometry(Params& P, const int n[3], int axis);
+int make_map_B_pair(CUtensorMap* m, const __nv_bfloat16* base, const int n[3], int axis, int bn, int planes = 2);
+void set_geometry(Params& P, const int n[3], int axis, int bn);
+// Tiles of 256 lines of one launch over a grid along `axis`, and the lines per
+// tile for a launch of that many.
+long long wide_tiles(const int n[3], int axis);
+int tile_lines(long long wide);
 int launch(const Params& P, cudaStream_t s, double bytes, double flops);
 // One persistent launch over the tiles of `ngroups` contractions along the same
 // axis (descriptors and tile offsets gstart[0..ngroups] in device memory,
 // total = gstart[ngroups]); groups with gactive[g] == 0 are skipped.  All
-// groups share the layout b_kmajor and the output mode out_mode.
+// groups share the layout b_kmajor, the output mode out_mode and the lines per
+// tile bn.
 // Bounded-wait self-test (tfde_selftest_wait).
 int wait_selftest(long long limit_ns, int* tmem_freed, cudaStream_t s);
 int launch_grouped(const Params* groups, const long long* gstart, int ngroups, long long total, int b_kmajor,
-                   int out_mode, const int* gactive, int* err, cudaStream_t s, double bytes, double flops,
+                   int out_mode, int bn, const int* gactive, int* err, cudaStream_t s, double bytes, double flops,
                    const int* skip = nullptr);
 
 // Launch parameters chosen by the autotuner (tfde_tune, tfde_batch_tune):
 // the number of persistent CTAs and of ring stages, per launch class.  A
 // class is the kernel instance (grouped, operand layout, output mode), the
 // stage size, the rows n of the contraction (0 for grouped launches) and the
-// number of 128 x 256 tiles of the launch.
+// number of tiles of the launch (128 rows x 256, 128 or 64 lines).
 struct TuneKey {
     int grouped, kmajor, out_mode, stage_bytes, n;
     long long tiles;
@@ -58,7 +64,7 @@ struct TuneVal {
 void tune_force(int grid, int stages);
 // The class of a single launch with descriptor P (after set_ring) / of a grouped launch.
 TuneKey tune_key_single(const Params& P);
-TuneKey tune_key_grouped(int b_kmajor, int out_mode, long long total);
+TuneKey tune_key_grouped(int b_kmajor, int out_mode, int stage_bytes, long long total);
 int stage_capacity(int stage_bytes);
 void tune_put(const TuneKey& k, const TuneVal& v);
 int tune_count();

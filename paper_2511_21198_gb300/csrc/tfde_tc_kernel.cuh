@@ -9,7 +9,8 @@
 // Eq. (linear_sys) / Eq. (diag_tau_pre) with the line batch as the GEMM N
 // dimension.
 //
-// Design (one CTA per SM, persistent over tiles of 128 rows x 256 lines):
+// Design (one CTA per SM, persistent over tiles of 128 rows x 256 lines; 128 or
+// 64 lines where 256 would leave SMs without a tile, Params::bn):
 //   warps 0..2  TMA producers: A tiles [128 x 64] (K-major, 128B swizzle; the
 //               hi and lo terms of a split operator in one 3-D box) and B
 //               tiles [64 x 256] (x axis: K-major 128B swizzle; y/z axes:
@@ -39,7 +40,7 @@ namespace tfde {
 namespace tc {
 
 constexpr int BM = 128;
-constexpr int BN = 256;
+constexpr int BN = 256;            // lines per tile at most
 constexpr int BK = 32;             // k-block of the exact-slice contraction's operator maps (tfde_oz.cu)
 constexpr int SK = 64;             // k-block of this contraction: 128-byte rows of 64 BF16
 constexpr int MAXA = 2;
@@ -102,7 +103,8 @@ struct Params {
     long long lines;     // valid lines (K-major case)
     int C, nbc, P;       // MN-major: contiguous line extent per plane, 64-blocks per plane, planes
     long long nblocks;   // MN-major: nbc * P
-    long long ntiles;    // line tiles of BN
+    int bn;              // lines per tile: 256, 128 or 64
+    long long ntiles;    // line tiles of bn
     int n1;              // K-major output: Y[l * n1 + m]
     long long plane;     // MN-major output plane stride (C * n)
     int out_mode;
@@ -245,7 +247,7 @@ __device__ __forceinline__ int find_group(const long long* __restrict__ gstart, 
 // same axis) whose descriptors sit in global memory; tile t belongs to group
 // g with gstart[g] <= t < gstart[g+1], and groups with gactive[g] == 0 are
 // skipped by all three roles alike.  p0 then carries only the common fields
-// (err, the ring geometry) and ntiles = gstart[ngroups], mhalves = 1.  KM
+// (err, bn, the ring geometry) and ntiles = gstart[ngroups], mhalves = 1.  KM
 // (= Params::b_kmajor) and OM (= Params::out_mode) are compile-time so that
 // each instance carries one straight-line epilogue.
 template <bool GROUPED, int KM, int OM>
@@ -268,6 +270,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     const int lane = threadIdx.x & 31;
     const int nst = p0.nstages;
     const int sbytes = p0.stage_bytes;
+    const int bn = p0.bn;
+    const uint32_t btile = (uint32_t)(bn * SK * 2);   // bytes of one B plane of a stage
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < MAX_STAGES; ++s) {
@@ -282,6 +286,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         mbar_fence_init();
     }
     if (warp == MMA_WARP) tmem_alloc(tmem_slot, TMEM_COLS);
+    if (!GROUPED && threadIdx.x < 3) {   // the descriptors, before the first copy or store needs them
+        const CUtensorMap* om = OM == OUT_HI ? &p0.omap_hi : (OM == OUT_HILO ? &p0.omap_hl : &p0.omap_f32);
+        const CUtensorMap* m = threadIdx.x == 0 ? &p0.amaps[0] : (threadIdx.x == 1 ? &p0.bmaps[0] : om);
+        asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -324,10 +333,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     // merged boxes: one copy for all A terms and one for both B planes
                     const int na_box = S.amap2 >= 0 ? 1 : S.na;
                     const uint32_t abytes = S.amap2 >= 0 ? (uint32_t)(S.na * A_TILE_BYTES) : (uint32_t)A_TILE_BYTES;
-                    const int bbox = S.bmap2 >= 0 ? 1 : (b_kmajor ? 1 : BN / 64);
+                    const int bbox = S.bmap2 >= 0 ? 1 : (b_kmajor ? 1 : bn / 64);
                     const int nb_box = S.bmap2 >= 0 ? 1 : S.nb * bbox;
-                    const uint32_t bbytes = S.bmap2 >= 0 ? (uint32_t)(S.nb * B_TILE_BYTES)
-                                                         : (b_kmajor ? (uint32_t)B_TILE_BYTES : (uint32_t)(64 * SK * 2));
+                    const uint32_t bbytes = S.bmap2 >= 0 ? S.nb * btile
+                                                         : (b_kmajor ? btile : (uint32_t)(64 * SK * 2));
                     uint32_t mine = 0;
                     for (int i = pw; i < na_box + nb_box; i += PRODUCERS) mine += i < na_box ? abytes : bbytes;
                     for (int kb = 0; kb < S.nkb; ++kb) {
@@ -345,9 +354,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                             if (S.bmap2 >= 0) {
                                 uint8_t* dstb = st + boff;
                                 if (p.b_rank == 3) {
-                                    tma_load_3d(dstb, &p.bmaps[S.bmap2], &full[s], kb * SK, (int)(tile * BN), 0);
+                                    tma_load_3d(dstb, &p.bmaps[S.bmap2], &full[s], kb * SK, (int)(tile * bn), 0);
                                 } else {
-                                    const long long gb = tile * (BN / 64);
+                                    const long long gb = tile * (bn / 64);
                                     tma_load_5d(dstb, &p.bmaps[S.bmap2], &full[s], 0, kb * SK, (int)(gb % p.nbc),
                                                 (int)(gb / p.nbc), 0);
                                 }
@@ -355,11 +364,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                             }
                             const int jb = i - na_box;   // B box index in the per-plane enumeration
                             const int b = jb / bbox, blk = jb % bbox;
-                            uint8_t* dst = st + boff + b * B_TILE_BYTES;
+                            uint8_t* dst = st + boff + b * btile;
                             if (b_kmajor) {
-                                tma_load_2d(dst, &p.bmaps[S.bmap[b]], &full[s], kb * SK, (int)(tile * BN));
+                                tma_load_2d(dst, &p.bmaps[S.bmap[b]], &full[s], kb * SK, (int)(tile * bn));
                             } else {
-                                const long long gb = tile * (BN / 64) + blk;
+                                const long long gb = tile * (bn / 64) + blk;
                                 const int pl = (int)(gb / p.nbc);
                                 const int c0 = (int)(gb % p.nbc) * 64;
                                 tma_load_3d(dst + blk * (64 * SK * 2), &p.bmaps[S.bmap[b]], &full[s], c0, kb * SK, pl);
@@ -378,7 +387,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     } else if (warp == MMA_WARP) {
         if (lane == 0) {
             // ------------------------------------------------ MMA issuer
-            const uint32_t idesc = instr_desc(BM, BN, b_kmajor ? 0 : 1);
+            const uint32_t idesc = instr_desc(BM, bn, b_kmajor ? 0 : 1);
             // descriptor templates at stage 0 (128-byte swizzle, 8-row groups
             // 1024 bytes apart; MN-major B: 64-line blocks 64 x SK x 2 bytes
             // apart); in-smem offsets are added to the start-address field
@@ -415,7 +424,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                         const uint64_t bd_s = b_desc0 + (uint64_t)((s * sbytes) >> 4);
                         for (int pr = 0; pr < S.npair; ++pr) {
                             const uint64_t ad_p = ad_s + (uint64_t)((S.pa[pr] * A_TILE_BYTES) >> 4);
-                            const uint64_t bd_p = bd_s + (uint64_t)((S.pb[pr] * B_TILE_BYTES) >> 4);
+                            const uint64_t bd_p = bd_s + (uint64_t)((S.pb[pr] * btile) >> 4);
 #pragma unroll
                             for (int k16 = 0; k16 < SK / 16; ++k16) {
                                 const uint32_t acc = (sg == 0 && kb == 0 && pr == 0 && k16 == 0) ? 0u : 1u;
@@ -437,7 +446,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         // ---------------------------------------------------- epilogue warps
         const int ew = warp - EPI_WARP0;
         const int q = warp & 3;               // TMEM lane quadrant this warp may access
-        const int half = ew >> 2;             // which 128 of the 256 columns
+        const int half = ew >> 2;             // which half of the tile's columns
         uint8_t* slot = epi + ew * EPI_SLOT_BYTES;
         // the hi-plane output (one 2 KB chunk) alternates between the two
         // halves of the slot, so that a chunk is converted while the previous
@@ -494,18 +503,18 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 ra = __ldg(p.lam_ra + m);
                 rb = __ldg(p.lam_rb + m);
             }
-            for (int cc = 0; cc < BN / 2; cc += 32) {
-                const int c0 = half * (BN / 2) + cc;
+            for (int cc = 0; cc < bn / 2; cc += 32) {
+                const int c0 = half * (bn / 2) + cc;
                 // chunk position: x axis -> lines line0 .. line0 + 31 (Y[line * n1 + m]);
                 // y / z axes -> plane pl, columns cx .. cx + 31 (Y[pl * plane + m * C + c])
                 long long line0 = 0, gb = 0;
                 int pl = 0, cx = 0, ncol;
                 if (b_kmajor) {
-                    line0 = tile * BN + c0;
+                    line0 = tile * bn + c0;
                     const long long rem = p.lines - line0;
                     ncol = rem >= 32 ? 32 : (rem > 0 ? (int)rem : 0);
                 } else {
-                    gb = tile * (BN / 64) + c0 / 64;
+                    gb = tile * (bn / 64) + c0 / 64;
                     pl = (int)(gb / p.nbc);
                     cx = (int)(gb % p.nbc) * 64 + (c0 & 63);
                     const int rem = p.C - cx;
