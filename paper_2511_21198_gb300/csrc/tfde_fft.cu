@@ -774,9 +774,17 @@ int launch_line(const LinePass& p, cudaStream_t s) {
     const double nio = 2.0 + (p.in1 ? 1.0 : 0.0) + (p.out1 ? 1.0 : 0.0);
     const double fl = 2.0 * (double)p.m.K * p.n * (double)p.lines;
     void* tok = stats_tc_begin(s, TFDE_KIND_FFT);
-    line_pass_kernel<R, MODE, TL, LT, RT><<<dim3((unsigned)blocks, (unsigned)gy), rows / RT * TL,
-                                           line_smem(p, sizeof(R), BN, rows, MODE == LINE_DST2), s>>>(p);
-    const cudaError_t e = cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks, (unsigned)gy);
+    cfg.blockDim = dim3((unsigned)(rows / RT * TL));
+    cfg.dynamicSmemBytes = line_smem(p, sizeof(R), BN, rows, MODE == LINE_DST2);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, line_pass_kernel<R, MODE, TL, LT, RT>, p);
     stats_tc_end(tok, s, TFDE_KIND_FFT, nio * N * sizeof(R), fl * (MODE == LINE_DST2 ? 2.0 : 1.0));
     if (e != cudaSuccess) return set_error(TFDE_ECUDA, std::string("line_pass_kernel: ") + cudaGetErrorString(e));
     return TFDE_OK;
@@ -785,8 +793,11 @@ int launch_line(const LinePass& p, cudaStream_t s) {
 // Lines per block: FP32 64, 32 or 16 (8 rows x 4, 2 or 1 lines per thread),
 // the largest that fits and still gives every SM two blocks, so that one's
 // copies run under the other's product; FP64, bound by its pipe (two
-// multiply-adds per clock and SM), always 8 (4 rows x 1 line), for the even
-// spread over the SMs.
+// multiply-adds per clock and SM), 8 (4 rows x 1 line per thread), or 4 (2 x 1)
+// where the SMs would get few blocks of 8: the fullest one decides (4096 lines
+// are 3.4 blocks of 8 per SM, 6.7 of 4; preconditioner at 64^3 140 -> 119 us).
+// The Toeplitz passes, with their stencils' neighbours to fetch, gain only
+// below one block per SM (64^3: 124 us with 8, 128 with 4).
 template <typename R, int MODE>
 int line_pass(const LinePass& p, cudaStream_t s) {
     if constexpr (sizeof(R) == 4) {
@@ -799,6 +810,8 @@ int line_pass(const LinePass& p, cudaStream_t s) {
         if (takes(32)) return launch_line<R, MODE, 16, 2, 8>(p, s);
         return launch_line<R, MODE, 16, 1, 8>(p, s);
     } else {
+        const long long blocks = (p.lines + 7) / 8 * ((p.m.ld + LINE_ROWS - 1) / LINE_ROWS);
+        if (blocks < (MODE == LINE_TOEPLITZ ? 1 : 6) * tc::num_sms()) return launch_line<R, MODE, 4, 1, 2>(p, s);
         return launch_line<R, MODE, 8, 1, 4>(p, s);
     }
 }

@@ -127,7 +127,6 @@ __global__ void __launch_bounds__(256, LT >= 4 ? 2 : 3) line_pass_kernel(const _
     constexpr int KC = line_chunk<R>();
     constexpr int Q = 16 / sizeof(R);
     extern __shared__ __align__(16) unsigned char line_smem[];
-    if (p.skip && *p.skip) return;
     const int n = p.n, K = p.m.K, half = p.m.half, ld = p.m.ld;
     const int rows = blockDim.x / TL * RT;                   // matrix rows of this block
     const int row0 = blockIdx.y * LINE_ROWS;
@@ -196,11 +195,23 @@ __global__ void __launch_bounds__(256, LT >= 4 ? 2 : 3) line_pass_kernel(const _
             }
         });
     };
+    // launched with programmatic stream serialisation: the first matrix chunks
+    // are on their way before the previous kernel has ended; its results are
+    // read only after the wait
+    for (int c = 0; c < LINE_STAGES - 1; ++c) fetch(c);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // (a long matrix streams from L2 through the whole product: the next
+    // launch's first chunks would only get in its way, 511^2: 13.0 against 12.7 ms)
+    if (K <= 256) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (p.skip && *reinterpret_cast<const volatile int*>(p.skip)) {
+        line_wait<0>();
+        return;
+    }
     fetch_lines(X, in0);
     line_commit();
     if (MODE == LINE_TOEPLITZ && in1) fetch_lines(Z, in1);
-    for (int c = 0; c < LINE_STAGES - 1; ++c) fetch(c);   // the first carries Z too
-    line_wait<LINE_STAGES - 1>();
+    line_commit();
+    line_wait<1>();   // the lines; the second operand's are waited for below
     __syncthreads();
 
     if (MODE == LINE_TOEPLITZ && out1) {
