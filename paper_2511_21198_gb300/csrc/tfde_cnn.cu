@@ -24,15 +24,20 @@
 // 1 the MMAs into double-buffered TMEM accumulators, warps 2..9 run the
 // epilogue (bias, ReLU or ReLU-gradient mask, BF16 store of interior slots, or
 // the FP32 output channel on the plain grid).
-// Bound: the MMAs, 64 cycles each at this shape whatever N (the 4 KB A operand
-// read from shared memory); without the copies or without the epilogue the
-// time is the same.  Measured on GB300 at 128^3: 107 us per layer (162 us with
-// the nine 16-byte-row tensor copies per 128 slots).
+// Bound: the chain of 27 MMAs on one accumulator, about 256 cycles from one to
+// the next (the time per layer is the same with N = 32, with M = 64, or with
+// the operands exchanged, and without the copies or the epilogue).  So what
+// counts is how many accumulators an SM has in flight: a CTA's NT = 4 tiles
+// take the taps in turn, and two CTAs share an SM, which their memory allows
+// because the ring holds planes (one dz of a tile, four of them) instead of
+// whole tiles.  Measured on GB300 at 128^3: 107 us per layer with one CTA and
+// two whole tiles, 75 us with two CTAs (162 us with nine 16-byte-row tensor
+// copies per 128 slots).
 //
 // Weight gradients: per tap a 16 x 16 matrix summed over all slots, on
 // mma.sync m16n8k16 (tcgen05's smallest M of 64 would leave three quarters of
 // the rows empty); the same staged runs as the convolution serve all 27 taps.
-// One optimiser step of eight 64^3 samples: 2.9 ms, against 25.7 ms with the
+// One optimiser step of eight 64^3 samples: 2.7 ms, against 25.7 ms with the
 // nine-copy convolution, a CUDA-core weight gradient per tap and 256-slot
 // chunk (477 us per layer, 160 us for the sum of its partials), a one-block
 // max |u| (183 us) and a 16-block bias sum (41 us).
@@ -62,7 +67,8 @@ constexpr int TM = 128;            // slots per MMA
 constexpr int MAX_NT = 4;          // MMA tiles per staged tile: 1, 2 or 4
 constexpr int STAGES = 2;
 constexpr int W_BYTES = NTAP * 2 * CH * 16;              // 13824: [tap][khalf][co][8 ci]
-constexpr int NUM_BARS = 2 * STAGES + 5;
+constexpr int PLANES = 4;          // convolution: input planes (one dz of a tile) in the ring
+constexpr int NUM_BARS = 2 * PLANES + 5;
 constexpr int EPI_WARPS = 8;
 constexpr int NUM_THREADS = 32 * (2 + EPI_WARPS);
 constexpr int MAX_SMEM = 232448;
@@ -74,9 +80,10 @@ constexpr int GSZ = NTAP * 256 + CH;              // one partial: [tap][co][ci],
 
 // How a tile's input rows are staged: nseg runs of seglen slots per channel
 // half (3 runs, one per dz, or 9, one per (dz, dy)); row r = (dz + 1) 3 +
-// (dy + 1) of the taps starts rowoff[r] slots into a half.
+// (dy + 1) of the taps starts rowoff[r] slots into a half.  A plane is a
+// third of it: plane_bytes per half, its row (dy + 1) rowoff[dy + 1] slots in.
 struct Staging {
-    int nt, tile, nseg, seglen, half_bytes;
+    int nt, tile, nseg, seglen, half_bytes, plane_bytes;
     int rowoff[9];
 };
 
@@ -104,35 +111,35 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                  : "memory");
 }
 
-// The runs of one tile (first slot s0), both halves, into `dst`; the caller
-// has announced 2 nseg seglen 16 bytes on `bar`.
-__device__ __forceinline__ void stage_rows(uint8_t* dst, const uint8_t* in, long long half_stride, const Staging& st,
-                                           long long s0, long long P, unsigned R, uint64_t* bar) {
+// The runs of plane dz (0, 1, 2 for dz = -1, 0, 1) of the tile from slot s0,
+// both halves half_bytes apart, into `dst`; the caller has announced their
+// bytes on `bar`.
+__device__ __forceinline__ void stage_plane(uint8_t* dst, int half_bytes, const uint8_t* in, long long half_stride,
+                                            const Staging& st, long long s0, int dz, long long P, unsigned R,
+                                            uint64_t* bar) {
     const uint32_t bytes = (uint32_t)st.seglen * 16u;
-    for (int h = 0; h < 2; ++h) {
-        for (int i = 0; i < st.nseg; ++i) {
-            const long long start = st.nseg == 3 ? s0 + (i - 1) * P - (long long)R - 1
-                                                 : s0 + (i / 3 - 1) * P + (i % 3 - 1) * (long long)R - 1;
-            bulk_load(dst + h * st.half_bytes + i * bytes, in + h * half_stride + start * 16, bytes, bar);
-        }
-    }
+    const long long first = s0 + (dz - 1) * P - (long long)R - 1;
+    for (int h = 0; h < 2; ++h)
+        for (int i = 0; i < st.nseg / 3; ++i)
+            bulk_load(dst + h * half_bytes + i * bytes, in + h * half_stride + (first + i * (long long)R) * 16, bytes,
+                      bar);
 }
 
 template <int NT>
-__global__ void __launch_bounds__(NUM_THREADS, 1) conv_kernel(const __grid_constant__ ConvParams p) {
+__global__ void __launch_bounds__(NUM_THREADS, 2) conv_kernel(const __grid_constant__ ConvParams p) {
     using namespace tfde::tc;
     constexpr uint32_t TMEM_COLS = 2 * NT * CH;   // 32, 64 or 128
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
-    const int stage_bytes = 2 * p.st.half_bytes;
+    const int pbytes = 2 * p.st.plane_bytes;   // both halves of a plane
     uint8_t* wsm = smem;
     uint64_t* bars = reinterpret_cast<uint64_t*>(wsm + W_BYTES);
-    uint8_t* stages = wsm + W_BYTES + ((NUM_BARS * 8 + 16 + 15) & ~15);
+    uint8_t* ring = wsm + W_BYTES + ((NUM_BARS * 8 + 16 + 15) & ~15);
     uint64_t* full = bars;
-    uint64_t* empty = bars + STAGES;
-    uint64_t* tfull = bars + 2 * STAGES;
-    uint64_t* tempty = bars + 2 * STAGES + 2;
-    uint64_t* mma_done = bars + 2 * STAGES + 4;
+    uint64_t* empty = bars + PLANES;
+    uint64_t* tfull = bars + 2 * PLANES;
+    uint64_t* tempty = bars + 2 * PLANES + 2;
+    uint64_t* mma_done = bars + 2 * PLANES + 4;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + NUM_BARS);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -144,7 +151,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) conv_kernel(const __grid_const
         fence_proxy_async_smem();
     }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (int s = 0; s < PLANES; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
@@ -165,23 +172,26 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) conv_kernel(const __grid_const
         if (lane == 0) {
             int s = 0;
             uint32_t ph = 0, filled = 0, last_ph = 0;
-            for (int t = blockIdx.x; t < p.ntiles; t += gridDim.x) {
-                if (!mbar_wait(&empty[s], ph ^ 1u, p.err)) break;
-                mbar_expect_tx(&full[s], 2u * p.st.nseg * p.st.seglen * 16u);
-                stage_rows(stages + s * stage_bytes, p.in, p.half_stride, p.st, p.first + (long long)t * p.st.tile,
-                           p.P, p.R, &full[s]);
-                filled |= 1u << s;
-                if (ph) last_ph |= 1u << s; else last_ph &= ~(1u << s);
-                if (++s == STAGES) { s = 0; ph ^= 1u; }
+            bool ok = true;
+            for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
+                for (int dz = 0; dz < 3; ++dz) {
+                    if (!mbar_wait(&empty[s], ph ^ 1u, p.err)) { ok = false; break; }
+                    mbar_expect_tx(&full[s], 2u * (uint32_t)p.st.plane_bytes);
+                    stage_plane(ring + s * pbytes, p.st.plane_bytes, p.in, p.half_stride, p.st,
+                                p.first + (long long)t * p.st.tile, dz, p.P, p.R, &full[s]);
+                    filled |= 1u << s;
+                    if (ph) last_ph |= 1u << s; else last_ph &= ~(1u << s);
+                    if (++s == PLANES) { s = 0; ph ^= 1u; }
+                }
             }
-            for (int i = 0; i < STAGES; ++i)
+            for (int i = 0; i < PLANES; ++i)
                 if (filled & (1u << i)) mbar_wait(&full[i], (last_ph >> i) & 1u, p.err, false);
         }
     } else if (warp == 1) {
         if (lane == 0) {
             const uint32_t idesc = instr_desc(TM, CH, 0);
             // non-swizzled K-major: LBO = K-adjacent core matrix (channel half), SBO = next 8 rows
-            const uint64_t a0 = smem_desc(smem_u32(stages), p.st.half_bytes, 128, 0);
+            const uint64_t a0 = smem_desc(smem_u32(ring), p.st.plane_bytes, 128, 0);
             const uint64_t b0 = smem_desc(smem_u32(wsm), 256, 128, 0);
             int s = 0;
             uint32_t ph = 0;
@@ -191,21 +201,23 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) conv_kernel(const __grid_const
                 const int buf = it & 1;
                 const uint32_t use = (uint32_t)(it >> 1);
                 if (!mbar_wait(&tempty[buf], (use & 1u) ^ 1u, p.err)) { ok = false; break; }
-                if (!mbar_wait(&full[s], ph, p.err)) { ok = false; break; }
-                tc_fence_after();
-                const uint64_t as = a0 + (uint64_t)((s * stage_bytes) >> 4);
+                for (int dz = 0; dz < 3; ++dz) {
+                    if (!mbar_wait(&full[s], ph, p.err)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint64_t as = a0 + (uint64_t)((s * pbytes) >> 4);
 #pragma unroll
-                for (int tap = 0; tap < NTAP; ++tap) {   // tap = (dz+1)*9 + (dy+1)*3 + (dx+1)
-                    const uint64_t bd = b0 + (uint64_t)((tap * 512) >> 4);
-                    const uint64_t at = as + (uint64_t)(p.st.rowoff[tap / 3] + tap % 3);
+                    for (int k = 0; k < 9; ++k) {   // tap = 9 dz + k, k = (dy+1)*3 + (dx+1)
+                        const uint64_t bd = b0 + (uint64_t)(((dz * 9 + k) * 512) >> 4);
+                        const uint64_t at = as + (uint64_t)(p.st.rowoff[k / 3] + k % 3);
 #pragma unroll
-                    for (int m = 0; m < NT; ++m)
-                        umma_bf16(tmem_base + (uint32_t)((buf * NT + m) * CH), at + (uint64_t)(m * TM), bd, idesc,
-                                  tap > 0 ? 1u : 0u);
+                        for (int m = 0; m < NT; ++m)
+                            umma_bf16(tmem_base + (uint32_t)((buf * NT + m) * CH), at + (uint64_t)(m * TM), bd, idesc,
+                                      dz + k > 0 ? 1u : 0u);
+                    }
+                    umma_commit(&empty[s]);
+                    if (++s == PLANES) { s = 0; ph ^= 1u; }
                 }
-                umma_commit(&empty[s]);
-                umma_commit(&tfull[buf]);
-                if (++s == STAGES) { s = 0; ph ^= 1u; }
+                if (ok) umma_commit(&tfull[buf]);
             }
             umma_commit(mma_done);
             mbar_wait(mma_done, 0, p.err, false);
@@ -333,7 +345,9 @@ __global__ void __launch_bounds__(WG_THREADS, 1) wgrad_kernel(const __grid_const
                 const long long s0 = p.first + (long long)t * p.st.tile;
                 uint8_t* st = stages + s * stage_bytes;
                 mbar_expect_tx(&full[s], 2u * (p.st.nseg * p.st.seglen + p.st.tile) * 16u);
-                stage_rows(st, p.in, p.half_stride, p.st, s0, p.P, p.R, &full[s]);
+                for (int dz = 0; dz < 3; ++dz)
+                    stage_plane(st + dz * p.st.plane_bytes, p.st.half_bytes, p.in, p.half_stride, p.st, s0, dz, p.P, p.R,
+                                &full[s]);
                 for (int h = 0; h < 2; ++h)
                     bulk_load(st + 2 * p.st.half_bytes + h * dz_half, p.dz + h * p.half_stride + s0 * 16, dz_half,
                               &full[s]);
@@ -638,32 +652,33 @@ int grid1(long long n) {
 
 constexpr int LPART = 1216;   // loss partials (blocks of grid1)
 
-// Tiles of nt x 128 slots, nt as large as leaves every SM a tile; three runs
-// per tile where two stages of them (and `extra` bytes per slot) fit in shared
-// memory, with a smaller tile first, else nine runs.
-Staging staging(long long count, long long R, int fixed_smem, int extra) {
+// Tiles of nt x 128 slots, nt as large as leaves every SM a tile and smem(st)
+// in `limit`, with three runs per tile (one per dz) where a tile of 128 slots
+// fits so, else nine of two blocks.
+template <typename F>
+Staging staging(long long count, long long R, int limit, F smem) {
     Staging st{};
-    auto fits = [&](int nt, int nseg) {
-        const long long tile = nt * (long long)TM, seglen = nseg == 3 ? tile + 2 * R + 2 : tile + 2;
-        return STAGES * (2 * nseg * seglen * 16 + extra * tile) + fixed_smem + 1024 <= MAX_SMEM;
+    auto make = [&](int nt, int nseg) {
+        st.nt = nt;
+        st.tile = nt * TM;
+        st.nseg = nseg;
+        st.seglen = (int)(nseg == 3 ? st.tile + 2 * R + 2 : st.tile + 2);
+        st.plane_bytes = nseg / 3 * st.seglen * 16;
+        st.half_bytes = 3 * st.plane_bytes;
+        return smem(st) <= limit;
     };
-    st.nt = MAX_NT;
-    while (st.nt > 1 && count < (long long)st.nt * TM * tc::num_sms()) st.nt /= 2;
-    st.nseg = 3;
-    while (st.nt > 1 && !fits(st.nt, 3)) st.nt /= 2;
-    if (!fits(st.nt, 3)) {
-        st.nseg = 9;
-        st.nt = 2;
-    }
-    st.tile = st.nt * TM;
-    st.seglen = (int)(st.nseg == 3 ? st.tile + 2 * R + 2 : st.tile + 2);
-    st.half_bytes = st.nseg * st.seglen * 16;
+    int nt = MAX_NT;
+    while (nt > 1 && count < (long long)nt * TM * tc::num_sms()) nt /= 2;
+    while (nt > 1 && !make(nt, 3)) nt /= 2;
+    if (R > (1 << 20) || !make(nt, 3)) make(2, 9);
     for (int r = 0; r < 9; ++r)
         st.rowoff[r] = st.nseg == 3 ? (r / 3) * st.seglen + (int)((r % 3) * R) : r * st.seglen;
     return st;
 }
 
-int conv_smem(const Staging& st) { return CONV_FIXED_SMEM + 16 + STAGES * 2 * st.half_bytes; }
+// Two CTAs per SM share its 228 KB (1 KB of it reserved per CTA).
+constexpr int CONV_SMEM_LIMIT = 116736 - 1024;
+int conv_smem(const Staging& st) { return CONV_FIXED_SMEM + 16 + PLANES * 2 * st.plane_bytes; }
 int wg_smem(const Staging& st) { return WG_SMEM_FIXED + STAGES * (2 * st.half_bytes + 2 * st.tile * 16); }
 
 int conv(tfde_cnn* C, const uint8_t* in, const __nv_bfloat16* w, const float* bias, int relu, const uint8_t* mask,
@@ -688,7 +703,7 @@ int conv(tfde_cnn* C, const uint8_t* in, const __nv_bfloat16* w, const float* bi
     p.first = C->first;
     p.ntiles = C->conv_tiles;
     p.err = C->err;
-    const int grid = std::min(C->conv_tiles, tc::num_sms());
+    const int grid = std::min(C->conv_tiles, 2 * tc::num_sms());
     const int smem = conv_smem(p.st);
     void* tok = stats_tc_begin(s, TFDE_KIND_CONV);
     if (p.st.nt == 4) conv_kernel<4><<<grid, NUM_THREADS, smem, s>>>(p);
@@ -778,8 +793,8 @@ int cnn_create(const int n[3], tfde_cnn** out) {
     if (C->S_total + MAX_NT * TM >= (1LL << 31)) return set_error(TFDE_ENOMEM, "grid too large for the network");
     // the convolution's and the weight gradient's tiles; a tile may run past
     // the last interior slot, so every buffer ends in MAX_NT * TM more slots
-    C->conv_st = staging(C->count, C->R, CONV_FIXED_SMEM, 0);
-    C->wg_st = staging(C->count, C->R, WG_SMEM_FIXED, 32);
+    C->conv_st = staging(C->count, C->R, CONV_SMEM_LIMIT, conv_smem);
+    C->wg_st = staging(C->count, C->R, MAX_SMEM, wg_smem);
     C->conv_tiles = (int)((C->count + C->conv_st.tile - 1) / C->conv_st.tile);
     C->wg_tiles = (int)((C->count + C->wg_st.tile - 1) / C->wg_st.tile);
     C->wg_grid = std::min(C->wg_tiles, tc::num_sms());
