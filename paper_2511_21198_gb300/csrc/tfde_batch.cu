@@ -35,7 +35,8 @@ int pgmres64(tfde_problem*, const double*, double*, int, double, int, tfde_info*
 namespace {
 
 constexpr int kBT = 256;       // threads per block of the vector kernels
-constexpr int kCH = 4096;      // elements per block chunk
+constexpr int kCH = 4096;      // elements per block chunk at least, and at most: the sweeps
+constexpr int kMaxCH = 16384;  // end in a block reduction, so chunks grow while blocks are plenty
 constexpr int kHS = 192;       // per-problem Hessenberg stride: H (64) | H2 (64) | -y (64)
 constexpr int kSS = 16;        // per-problem scalar stride
 constexpr int kStreams = 8;    // stream pool of the per-problem work
@@ -66,6 +67,10 @@ struct BVec {
     unsigned nc4;        // n1 n2 / 4
     int n3;
     const double* norms; // ||b||^2, ||r_0||^2 of the problem's last cn_prepare
+    int chunk;           // elements per block of the vector kernels
+    int nblk;            // this problem's blocks
+    long long b0;        // the first of them
+    unsigned* ticket;    // counts its blocks (gs::last_block)
 };
 
 __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16& hi, __nv_bfloat16& lo) {
@@ -89,13 +94,13 @@ __device__ __forceinline__ double block_sum(double v) {
 }
 
 static_assert(kBT == gs::kThreads, "block width of the Gram-Schmidt sweeps");
-// The chunk of block b: problem bi[b], elements [bo[b], min(bo[b] + kCH, N)).
+// The chunk of block b: problem bi[b], elements [bo[b], min(bo[b] + chunk, N)).
 #define BK_PROLOGUE                                        \
     const int inst = bi[blockIdx.x];                       \
     if (!act[inst]) return;                                \
     const BVec& v = vt[inst];                              \
     const long long e0 = bo[blockIdx.x];                   \
-    const long long e1 = e0 + kCH < v.N ? e0 + kCH : v.N;
+    const long long e1 = e0 + v.chunk < v.N ? e0 + v.chunk : v.N;
 
 // r32 = r64 * sc ; split into (rh, rl) ; x32 = 0
 __global__ __launch_bounds__(kBT) void bk_scale64to32(const BVec* __restrict__ vt, const int* __restrict__ bi,
@@ -190,7 +195,7 @@ __global__ __launch_bounds__(kBT) void bk_add32to64(const BVec* __restrict__ vt,
 // where the tau preconditioner is the diagonal Lambda (Eq. (diag_tau_pre)):
 // per problem r~ = S_N r (r32), p (p32 and its split planes), x~ (x32),
 // q = S_N A S_N p (W); the scalars in the problem's slots.  Elements go four
-// at a time (a chunk holds whole groups: N and kCH are multiples of 4).
+// at a time (a chunk holds whole groups: N and the chunks are multiples of 4).
 __device__ __forceinline__ float4 bk_lam4(const BVec& v, unsigned e4) {
     const unsigned k = e4 / v.nc4, c4 = e4 - k * v.nc4;
     const float ra = __ldg(v.lam + k), rb = __ldg(v.lam + v.n3 + k);
@@ -376,70 +381,67 @@ __global__ __launch_bounds__(kBT) void bkp_direction(const BVec* __restrict__ vt
 
 // ---- the same steps for the graph-captured cycle: the step index j comes
 // from *jd (device), the new vector is the fixed per-problem W.
-// Block partial sums of <V_{m0+t}, W> for t < min(8, j + 1 - m0), or (ww) of
-// <W, W> into row R + 1.
+// <V_t, W>, t <= j: partial sums per block, and the last block of a problem
+// sums them into h[i * kHS + t].
 __global__ __launch_bounds__(kBT, 2) void bkg_dots(const BVec* __restrict__ vt, const int* __restrict__ bi,
                                                const long long* __restrict__ bo, const int* __restrict__ act,
-                                               int m0, const int* __restrict__ jd, int R, int ww,
-                                               double* __restrict__ part) {
-    const int j = *jd;
-    const int mc = ww ? 1 : min(8, j + 1 - m0);
-    if (mc <= 0) return;
+                                               const int* __restrict__ jd, double* part, double* h) {
     BK_PROLOGUE
-    if (ww)
-        gs::update_norm(nullptr, 4, nullptr, 0, v.W, e0, e1, true,
-                        [&](double sum) { part[(long long)(R + 1) * gridDim.x + blockIdx.x] = sum; });
-    else
-        gs::dots(v.V, v.N, m0, mc, v.W, e0, e1, true,
+    const int m = *jd + 1;
+    for (int m0 = 0; m0 < m; m0 += gs::kWidth)
+        gs::dots(v.V, v.N, m0, min(m - m0, gs::kWidth), v.W, e0, e1, true,
                  [&](int t, double sum) { part[(long long)t * gridDim.x + blockIdx.x] = sum; });
-}
-
-// out[i * ostride + ooff + t] = sum over problem i's blocks, t <= j (rows
-// 0 .. j), or (ww) row R + 1 into out[i * ostride + ooff]
-__global__ void bkg_reduce(const double* __restrict__ part, int NB, const int* __restrict__ bstart,
-                           const int* __restrict__ act, const int* __restrict__ jd, int R, int ww,
-                           double* __restrict__ out, int ostride, int ooff) {
-    const int inst = blockIdx.x, t = blockIdx.y;
-    if (!act[inst] || t > (ww ? 0 : *jd)) return;
-    const int row = ww ? R + 1 : t;
-    double acc = 0.0;
-#pragma unroll 8
-    for (int b = bstart[inst] + threadIdx.x; b < bstart[inst + 1]; b += 32) acc += part[(long long)row * NB + b];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if (threadIdx.x == 0) out[inst * ostride + ooff + t] = acc;
+    if (gs::last_block(v.ticket, v.nblk))
+        gs::sum_partials(part + v.b0, gridDim.x, v.nblk, m, [&](int t, double sum) { h[inst * kHS + t] = sum; });
 }
 
 // The second Gram-Schmidt pass's projections fused with the first pass's
 // update: W -= sum_{t <= j} coef[i * kHS + coff + t] V_t over the block's
-// chunk, then the block partial sums of <V_t, W> (t <= j) of the updated
-// chunk into rows t of part.
+// chunk, then <V_t, W> (t <= j) of the updated chunk, summed over the problem's
+// blocks into h[i * kHS + ooff + t].
 __global__ __launch_bounds__(kBT, 2) void bkg_axpy_dots(const BVec* __restrict__ vt, const int* __restrict__ bi,
                                                     const long long* __restrict__ bo, const int* __restrict__ act,
-                                                    const int* __restrict__ jd, const double* __restrict__ coef,
-                                                    int coff, double* __restrict__ part) {
+                                                    const int* __restrict__ jd, double* h, int coff, int ooff,
+                                                    double* part) {
     BK_PROLOGUE
     const int m = *jd + 1;
     __shared__ float hs[64];
-    for (int t = threadIdx.x; t < m; t += blockDim.x) hs[t] = (float)coef[inst * kHS + coff + t];
+    for (int t = threadIdx.x; t < m; t += blockDim.x) hs[t] = (float)h[inst * kHS + coff + t];
     __syncthreads();
     gs::update_dots(v.V, v.N, hs, m, v.W, e0, e1, true,
                     [&](int t, double sum) { part[(long long)t * gridDim.x + blockIdx.x] = sum; });
+    if (gs::last_block(v.ticket, v.nblk))
+        gs::sum_partials(part + v.b0, gridDim.x, v.nblk, m,
+                         [&](int t, double sum) { h[inst * kHS + ooff + t] = sum; });
 }
 
+// Arnoldi step j of problem i's least-squares problem (below)
+__device__ __forceinline__ void givens_step(int i, int R, int j, double* __restrict__ gs,
+                                            const double* __restrict__ h, double* __restrict__ s,
+                                            const double* __restrict__ theta, int* __restrict__ act,
+                                            int* __restrict__ its, double* __restrict__ est, int* __restrict__ cnt,
+                                            int* __restrict__ bad);
+
 // The second pass's update fused with ||W||^2: W -= sum_{t <= j} coef V_t and
-// the block partial sum of the updated W^2 into row R + 1 of part.
+// the sum of the updated W^2; a problem's last block closes its Arnoldi step
+// (givens_step, the count of problems still in the cycle into cnt[j + 1]).
 __global__ __launch_bounds__(kBT) void bkg_axpy_ww(const BVec* __restrict__ vt, const int* __restrict__ bi,
-                                                  const long long* __restrict__ bo, const int* __restrict__ act,
-                                                  const int* __restrict__ jd, const double* __restrict__ coef,
-                                                  int coff, int R, double* __restrict__ part) {
+                                                  const long long* __restrict__ bo, const int* act,
+                                                  const int* __restrict__ jd, const double* __restrict__ h, int coff,
+                                                  int R, double* part, double* gsv, double* s,
+                                                  const double* __restrict__ theta, int* act_out, int* its,
+                                                  double* est, int* cnt, int* bad) {
     BK_PROLOGUE
-    const int m = *jd + 1;
+    const int j = *jd, m = j + 1;
     __shared__ float hs[64];
-    for (int t = threadIdx.x; t < m; t += blockDim.x) hs[t] = (float)coef[inst * kHS + coff + t];
+    for (int t = threadIdx.x; t < m; t += blockDim.x) hs[t] = (float)h[inst * kHS + coff + t];
     __syncthreads();
-    gs::update_norm(v.V, v.N, hs, m, v.W, e0, e1, true,
-                    [&](double sum) { part[(long long)(R + 1) * gridDim.x + blockIdx.x] = sum; });
+    gs::update_norm(v.V, v.N, hs, m, v.W, e0, e1, true, [&](double sum) { part[blockIdx.x] = sum; });
+    if (gs::last_block(v.ticket, v.nblk))
+        gs::sum_partials(part + v.b0, gridDim.x, v.nblk, 1, [&](int, double sum) {
+            s[inst * kSS + S_WW] = sum;
+            givens_step(inst, R, j, gsv, h, s, theta, act_out, its, est, cnt + m, bad);
+        });
 }
 
 // V_{j+1} = W sc and its split planes (ph, pl)
@@ -492,17 +494,6 @@ __global__ void bk_cycle_start(int C, int R, double* __restrict__ gs, double* __
     }
 }
 
-// Arnoldi step j: column j of the Hessenberg matrix (the two CGS projections
-// summed, ||w|| from S_WW) rotated into the least-squares state, the new
-// rotation, the residual estimate |g_{j+1}|; the problem leaves the cycle
-// when that estimate reaches theta beta, else V_{j+1} gets the scale 1/||w||.
-// *cnt counts the problems still in the cycle.
-__device__ __forceinline__ void givens_step(int i, int R, int j, double* __restrict__ gs,
-                                            const double* __restrict__ h, double* __restrict__ s,
-                                            const double* __restrict__ theta, int* __restrict__ act,
-                                            int* __restrict__ its, double* __restrict__ est, int* __restrict__ cnt,
-                                            int* __restrict__ bad);
-
 __global__ void bk_givens(int C, int R, int j, double* __restrict__ gs, const double* __restrict__ h,
                           double* __restrict__ s, const double* __restrict__ theta, int* __restrict__ act,
                           int* __restrict__ its, double* __restrict__ est, int* __restrict__ cnt,
@@ -510,17 +501,6 @@ __global__ void bk_givens(int C, int R, int j, double* __restrict__ gs, const do
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= C || !act[i]) return;
     givens_step(i, R, j, gs, h, s, theta, act, its, est, cnt, bad);
-}
-
-// the same with j = *jd, the count into cnt[j + 1]
-__global__ void bkg_givens(int C, int R, const int* __restrict__ jd, double* __restrict__ gs,
-                           const double* __restrict__ h, double* __restrict__ s, const double* __restrict__ theta,
-                           int* __restrict__ act, int* __restrict__ its, double* __restrict__ est,
-                           int* __restrict__ cnt, int* __restrict__ bad) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= C || !act[i]) return;
-    const int j = *jd;
-    givens_step(i, R, j, gs, h, s, theta, act, its, est, cnt + j + 1, bad);
 }
 
 // the loop condition of the graph-captured cycle: another step while a
@@ -531,6 +511,11 @@ __global__ void bkg_next(int* __restrict__ jd, const int* __restrict__ cnt, int 
     cudaGraphSetConditional(hc, (cnt[j] > 0 && j < R) ? 1u : 0u);
 }
 
+// Arnoldi step j: column j of the Hessenberg matrix (the two CGS projections
+// summed, ||w|| from S_WW) rotated into the least-squares state, the new
+// rotation, the residual estimate |g_{j+1}|; the problem leaves the cycle
+// when that estimate reaches theta beta, else V_{j+1} gets the scale 1/||w||.
+// *cnt counts the problems still in the cycle.
 __device__ __forceinline__ void givens_step(int i, int R, int j, double* __restrict__ gs,
                                             const double* __restrict__ h, double* __restrict__ s,
                                             const double* __restrict__ theta, int* __restrict__ act,
@@ -746,6 +731,7 @@ struct tfde_batch {
     int* d_cnt = nullptr;           // max(restart, kPcgMaxIt) + 1
     int* h_cnt = nullptr;
     int* d_bad = nullptr;
+    unsigned* d_ticket = nullptr;  // blocks of each problem done with a sweep
     int* h_bad = nullptr;
     std::vector<cudaEvent_t> cnt_ev;   // max(restart, kPcgMaxIt) + 1
     cudaStream_t aux[tfde::kStreams] = {};
@@ -835,6 +821,7 @@ int free_batch(tfde_batch* B) {
     cudaFree(B->d_cnt);
     if (B->h_cnt) cudaFreeHost(B->h_cnt);
     cudaFree(B->d_bad);
+    cudaFree(B->d_ticket);
     if (B->h_bad) cudaFreeHost(B->h_bad);
     for (cudaEvent_t e : B->cnt_ev)
         if (e) cudaEventDestroy(e);
@@ -951,19 +938,12 @@ int build_cycle_graph(tfde_batch* B, cudaStream_t s) {
                 st = grouped(B, B->d_sop + (size_t)a * C, a, tc::OUT_SUM, B->sop_bytes[a], B->sop_flops[a], s);
             if (!st) st = grouped(B, B->d_sopzw, 2, tc::OUT_SUM, B->sop_bytes[2], B->sop_flops[2], s);
             if (!st) {   // CGS2: <V, W>; W -= V h and <V, W> again (one pass); W -= V h2 and ||W||^2 (one pass)
-                for (int m0 = 0; m0 < R; m0 += 8)
-                    bkg_dots<<<B->NB, kBT, 0, s>>>(B->d_vt, B->d_bi, B->d_bo, B->d_act, m0, B->d_j, R, 0, B->d_part);
-                bkg_reduce<<<dim3((unsigned)C, (unsigned)R), 32, 0, s>>>(B->d_part, B->NB, B->d_bstart, B->d_act,
-                                                                         B->d_j, R, 0, B->d_h, kHS, 0);
-                bkg_axpy_dots<<<B->NB, kBT, 0, s>>>(B->d_vt, B->d_bi, B->d_bo, B->d_act, B->d_j, B->d_h, 0, B->d_part);
-                bkg_reduce<<<dim3((unsigned)C, (unsigned)R), 32, 0, s>>>(B->d_part, B->NB, B->d_bstart, B->d_act,
-                                                                         B->d_j, R, 0, B->d_h, kHS, 64);
+                bkg_dots<<<B->NB, kBT, 0, s>>>(B->d_vt, B->d_bi, B->d_bo, B->d_act, B->d_j, B->d_part, B->d_h);
+                bkg_axpy_dots<<<B->NB, kBT, 0, s>>>(B->d_vt, B->d_bi, B->d_bo, B->d_act, B->d_j, B->d_h, 0, 64,
+                                                    B->d_part);
                 bkg_axpy_ww<<<B->NB, kBT, 0, s>>>(B->d_vt, B->d_bi, B->d_bo, B->d_act, B->d_j, B->d_h, 64, R,
-                                                  B->d_part);
-                bkg_reduce<<<dim3((unsigned)C, 1u), 32, 0, s>>>(B->d_part, B->NB, B->d_bstart, B->d_act, B->d_j, R,
-                                                               1, B->d_s, kSS, S_WW);
-                bkg_givens<<<gb, 64, 0, s>>>(C, R, B->d_j, B->d_gs, B->d_h, B->d_s, B->d_theta, B->d_act, B->d_its,
-                                             B->d_est, B->d_cnt, B->d_bad);
+                                                  B->d_part, B->d_gs, B->d_s, B->d_theta, B->d_act, B->d_its,
+                                                  B->d_est, B->d_cnt, B->d_bad);
                 bkg_scale_split<<<B->NB, kBT, 0, s>>>(B->d_vt, B->d_bi, B->d_bo, B->d_act, B->d_j, B->d_s);
                 bkg_next<<<1, 1, 0, s>>>(B->d_j, B->d_cnt, R, h);
             }
@@ -987,9 +967,8 @@ int build_cycle_graph(tfde_batch* B, cudaStream_t s) {
     return TFDE_OK;
 }
 
-// launches of one captured step: 3 grouped + ceil(R / 8) + 1 (first projections)
-// + 4 (fused second pass and norm with their reductions) + 3 (Givens, scale, loop)
-unsigned cycle_step_launches(int R) { return 3u + (unsigned)((R + 7) / 8 + 1) + 4u + 3u; }
+// launches of one captured step: 3 grouped, 3 Gram-Schmidt sweeps, scale, loop
+constexpr unsigned kCycleStepLaunches = 8;
 
 // The batched PCG iteration of every symmetric problem as the body of a while
 // node: the operator's three grouped passes (<p, q> per problem), the update,
@@ -1168,7 +1147,7 @@ int batch_cycle(tfde_batch* B, const std::vector<int>& outer, const std::vector<
     if (*B->h_bad) return set_error(TFDE_ENAN, "non-finite value in a batched GMRES cycle");
     int kmax = 0;
     for (int i = 0; i < C; ++i) kmax = std::max(kmax, outer[i] ? B->h_its[i] : 0);
-    if (graph && B->cyc_exec) stats_count_launch((unsigned)(kmax > 0 ? kmax : 1) * cycle_step_launches(R));
+    if (graph && B->cyc_exec) stats_count_launch((unsigned)(kmax > 0 ? kmax : 1) * kCycleStepLaunches);
     kmax = 0;
     for (int i = 0; i < C; ++i) {
         its[i] = outer[i] ? B->h_its[i] : 0;
@@ -1406,12 +1385,16 @@ int batch_create(const tfde_params* params, int count, int restart, cudaStream_t
     // block table
     std::vector<int> bstart(C + 1, 0), bi;
     std::vector<long long> bo;
+    long long points = 0;
+    for (tfde_problem* P : B->P) points += (long long)P->N;
+    int chunk = kCH;   // at least eight blocks per SM
+    while (chunk < kMaxCH && points / (2 * chunk) >= 8LL * tc::num_sms()) chunk *= 2;
     for (size_t i = 0; i < C; ++i) {
         const long long N = (long long)B->P[i]->N;
-        const long long nb = (N + kCH - 1) / kCH;
+        const long long nb = (N + chunk - 1) / chunk;
         for (long long b = 0; b < nb; ++b) {
             bi.push_back((int)i);
-            bo.push_back(b * kCH);
+            bo.push_back(b * chunk);
         }
         bstart[i + 1] = bstart[i] + (int)nb;
     }
@@ -1437,6 +1420,8 @@ int batch_create(const tfde_params* params, int count, int restart, cudaStream_t
         cudaMallocHost((void**)&B->h_est, C * sizeof(double)) != cudaSuccess ||
         cudaMalloc((void**)&B->d_cnt, (size_t)(ncnt + 1) * sizeof(int)) != cudaSuccess ||
         cudaMallocHost((void**)&B->h_cnt, (size_t)(ncnt + 1) * sizeof(int)) != cudaSuccess ||
+        cudaMalloc((void**)&B->d_ticket, C * sizeof(unsigned)) != cudaSuccess ||
+        cudaMemsetAsync(B->d_ticket, 0, C * sizeof(unsigned), s) != cudaSuccess ||
         cudaMalloc((void**)&B->d_bad, sizeof(int)) != cudaSuccess ||
         cudaMallocHost((void**)&B->h_bad, sizeof(int)) != cudaSuccess)
         return fail(TFDE_ENOMEM, "allocation of the batch workspace failed");
@@ -1466,6 +1451,10 @@ int batch_create(const tfde_params* params, int count, int restart, cudaStream_t
         v.nc4 = (unsigned)((long long)P->n[0] * P->n[1] / 4);
         v.n3 = P->n[2];
         v.norms = P->red_out + kNormsSlot;
+        v.chunk = chunk;
+        v.nblk = bstart[i + 1] - bstart[i];
+        v.b0 = bstart[i];
+        v.ticket = B->d_ticket + i;
     }
     // the batched PCG's descriptors (the z pass adds <p, q> into the problem's S_PQ)
     std::vector<tc::Params> sfp(3 * C), sopq(C);

@@ -49,8 +49,8 @@ constexpr int kMaxRestart = 120;   // GMRES columns: the reduction scratch holds
 enum { V_R, V_Z, V_P, V_Q, V_X, V_A, V_W, V_C, V_E, NV };
 // device scalars
 enum { S_RZ0 = 0, S_RZ1 = 1, S_PQ = 2, S_RR = 3, S_H = 8, NS = 256 };
-// the device-side GMRES cycle's: both projections, ||w||^2, -y
-enum { S_GH = 8, S_GH2 = S_GH + GS_MAXM, S_GWW = S_GH2 + GS_MAXM, S_GY = S_GWW + 1 };
+// the device-side GMRES cycle's: both projections, -y
+enum { S_GH = 8, S_GH2 = S_GH + GS_MAXM, S_GY = S_GH2 + GS_MAXM };
 static_assert(S_GY + GS_MAXM <= NS, "device scalars of the GMRES cycle");
 
 struct FftMixed {
@@ -288,8 +288,8 @@ int build_cycle(const tfde_problem* P, int m, cudaStream_t s) {
         if (!st) st = op_Pinv32(P, F->v[V_Q], F->v[V_Z], c);
         double* d = F->d;
         if (!st)
-            launch_gm_step(P->N, F->V, ldv(P->N), F->v[V_Z], P->red, P->nblk, d + S_GH, d + S_GH2, d + S_GWW,
-                           F->gm_state, F->gm_ctl(), h, nullptr, nullptr, F->v[V_P], m + 1, c);
+            launch_gm_step(P->N, F->V, ldv(P->N), F->v[V_Z], P->red, P->nblk, d + S_GH, d + S_GH2,
+                           F->gm_state, F->gm_ctl(), h, nullptr, nullptr, F->v[V_P], c);
         stats_set_capturing(false);
         cudaGraph_t out = nullptr;
         const cudaError_t e = cudaStreamEndCapture(c, &out);
@@ -319,7 +319,7 @@ int inner_gmres_loop(const tfde_problem* P, int m, double theta, int maxit, int*
     int* ctl = F->gm_ctl();
     FM_TRY(cudaMemsetAsync(ctl, 0, 4 * sizeof(int), s));
     if (int st = op_Pinv32(P, F->v[V_R], F->v[V_Z], s)) return st;
-    launch_gm_start(N, F->v[V_Z], P->red, P->nblk, d + S_GWW, F->gm_state, ctl, m < maxit ? m : maxit, theta, F->V,
+    launch_gm_start(N, F->v[V_Z], P->red, P->nblk, F->gm_state, ctl, m < maxit ? m : maxit, theta, F->V,
                     nullptr, nullptr, F->v[V_P], s);
     FM_TRY(cudaGraphLaunch(F->gm_exec, s));
     launch_gm_solve(F->gm_state, ctl, d + S_GY, m, s);
@@ -335,7 +335,7 @@ int inner_gmres_loop(const tfde_problem* P, int m, double theta, int maxit, int*
     *iters = hc[0];
     *est_ratio = beta > 0.0 ? est / beta : 1.0;
     stats_count_launch((unsigned)(hc[0] > 0 ? hc[0] : 1) *
-                       (8u + (unsigned)fft::operator_launches(P) + (unsigned)fft::preconditioner_launches<float>(P)));
+                       ((unsigned)kGmStepLaunches + (unsigned)fft::operator_launches(P) + (unsigned)fft::preconditioner_launches<float>(P)));
     return TFDE_OK;
 }
 

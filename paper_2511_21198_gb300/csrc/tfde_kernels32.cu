@@ -629,10 +629,11 @@ __global__ void pcg_fold_dev_kernel(long long N4, CombineArgs a, float4* __restr
 // step's vector w is the fixed FP32 vector the preconditioner writes; every
 // kernel takes the step index from gctl, so one step is the body of the loop.
 
-// the first m = j + 1 inner products <V_i, w>, 8 basis vectors per sweep of w
+// the first m = j + 1 inner products <V_i, w>, 8 basis vectors per sweep of w;
+// their sums into h
 __global__ __launch_bounds__(kT, 2) void gm_multidot_kernel(long long N, const float* __restrict__ V, long long ldv,
-                                                            const float* __restrict__ w, double* __restrict__ part,
-                                                            const int* gctl) {
+                                                            const float* __restrict__ w, double* part, double* h,
+                                                            unsigned* ticket, const int* gctl) {
     if (gctl[1]) return;
     const int m = gctl[0] + 1;
     long long lo, hi;
@@ -641,30 +642,15 @@ __global__ __launch_bounds__(kT, 2) void gm_multidot_kernel(long long N, const f
     for (int m0 = 0; m0 < m; m0 += gs::kWidth)
         gs::dots(V, ldv, m0, min(m - m0, gs::kWidth), w, lo, hi, vec,
                  [&](int j, double sum) { part[(long long)j * gridDim.x + blockIdx.x] = sum; });
-}
-
-// out[j] = sum of the block partials of result j, j < m (m = mfix, or the
-// step's j + 1 when mfix == 0); one warp per result in a fixed order
-__global__ void gm_reduce_kernel(const double* __restrict__ part, int nblk, double* __restrict__ out, int mfix,
-                                 const int* gctl) {
-    if (gctl[1]) return;
-    const int m = mfix > 0 ? mfix : gctl[0] + 1;
-    const int j = blockIdx.x;
-    if (j >= m) return;
-    double acc = 0.0;
-#pragma unroll 8
-    for (int b = threadIdx.x; b < nblk; b += 32) acc += part[(long long)j * nblk + b];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if (threadIdx.x == 0) out[j] = acc;
+    if (gs::last_block(ticket, gridDim.x)) gs::sum_partials(part, gridDim.x, gridDim.x, m, [&](int j, double sum) { h[j] = sum; });
 }
 
 // The second Gram-Schmidt pass's projections fused with the first pass's
 // update: w -= sum_{i <= j} h[i] V_i over the block's chunk, then the first
-// m = j + 1 inner products <V_i, w> of the updated chunk.
+// m = j + 1 inner products <V_i, w> of the updated chunk; their sums into h2.
 __global__ __launch_bounds__(kT, 2) void gm_axpy_dot_kernel(long long N, const float* __restrict__ V, long long ldv,
-                                                            const double* __restrict__ h, float* w,
-                                                            double* __restrict__ part, const int* gctl) {
+                                                            const double* __restrict__ h, float* w, double* part,
+                                                            double* h2, unsigned* ticket, const int* gctl) {
     if (gctl[1]) return;
     const int m = gctl[0] + 1;
     __shared__ float hs[128];
@@ -674,21 +660,7 @@ __global__ __launch_bounds__(kT, 2) void gm_axpy_dot_kernel(long long N, const f
     chunk4(N, lo, hi);
     gs::update_dots(V, ldv, hs, m, w, lo, hi, aligned4(V, ldv, w),
                     [&](int j, double sum) { part[(long long)j * gridDim.x + blockIdx.x] = sum; });
-}
-
-// The second pass's update fused with ||w||^2: w -= sum_{i <= j} h[i] V_i over
-// the block's chunk and the block's partial sum of the updated w^2.
-__global__ __launch_bounds__(kT) void gm_axpy_norm_kernel(long long N, const float* __restrict__ V, long long ldv,
-                                                          const double* __restrict__ h, float* w,
-                                                          double* __restrict__ part, const int* gctl) {
-    if (gctl[1]) return;
-    const int m = gctl[0] + 1;
-    __shared__ float hs[128];
-    for (int j = threadIdx.x; j < m; j += blockDim.x) hs[j] = (float)h[j];
-    __syncthreads();
-    long long lo, hi;
-    chunk4(N, lo, hi);
-    gs::update_norm(V, ldv, hs, m, w, lo, hi, aligned4(V, ldv, w), [&](double sum) { part[blockIdx.x] = sum; });
+    if (gs::last_block(ticket, gridDim.x)) gs::sum_partials(part, gridDim.x, gridDim.x, m, [&](int j, double sum) { h2[j] = sum; });
 }
 
 __global__ __launch_bounds__(kT) void gm_dot_kernel(long long N, const float* a, double* __restrict__ part,
@@ -700,48 +672,72 @@ __global__ __launch_bounds__(kT) void gm_dot_kernel(long long N, const float* a,
                     [&](double sum) { part[blockIdx.x] = sum; });
 }
 
-// Column j of the Hessenberg matrix (h + h2 from the two Gram-Schmidt
-// passes, ||w|| below the diagonal) rotated by the previous Givens
-// rotations, the new rotation, the residual estimate |g_{j+1}| (Sec. 3.2 left
-// preconditioned GMRES), the stop test and the loop condition.
-__global__ void gm_givens_kernel(double* gs, const double* h, const double* h2, const double* ww, int* gctl,
-                                 cudaGraphConditionalHandle hc) {
+// The second pass's update fused with ||w||^2: w -= sum_{i <= j} h2[i] V_i
+// over the block's chunk and the block's partial sum of the updated w^2.  The
+// last block closes the step: column j of the Hessenberg matrix (h + h2 from
+// the two Gram-Schmidt passes, ||w|| below the diagonal) rotated by the
+// previous Givens rotations, the new rotation, the residual estimate
+// |g_{j+1}| (Sec. 3.2 left preconditioned GMRES), the stop test and the loop
+// condition.  The rotations are a serial chain, so their operands are staged
+// in shared memory first.
+__global__ __launch_bounds__(kT) void gm_axpy_norm_kernel(long long N, const float* __restrict__ V, long long ldv,
+                                                          const double* __restrict__ h, const double* __restrict__ h2,
+                                                          float* w, double* part, unsigned* ticket, double* gs,
+                                                          int* gctl, cudaGraphConditionalHandle hc) {
     if (gctl[1]) {   // the loop ends whenever its condition kernel runs on a finished cycle
-        cudaGraphSetConditional(hc, 0u);
+        if (blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(hc, 0u);
         return;
     }
-    const int j = gctl[0];
+    const int j = gctl[0], m = j + 1;
+    __shared__ float hs[128];
+    for (int i = threadIdx.x; i < m; i += blockDim.x) hs[i] = (float)h2[i];
+    __syncthreads();
+    long long lo, hi;
+    chunk4(N, lo, hi);
+    gs::update_norm(V, ldv, hs, m, w, lo, hi, aligned4(V, ldv, w), [&](double sum) { part[blockIdx.x] = sum; });
+    if (!gs::last_block(ticket, gridDim.x)) return;
+    __shared__ double R[GS_MAXM + 2], cs[GS_MAXM], sn[GS_MAXM];
     double* g = gs + GS_G;
-    double* cs = gs + GS_CS;
-    double* sn = gs + GS_SN;
-    double* R = gs + GS_R + (long long)j * GS_LD;   // column j, entries 0..j+1
-    for (int i = 0; i <= j; ++i) R[i] = h[i] + h2[i];
-    const double hn = sqrt(*ww);
-    R[j + 1] = hn;
-    for (int i = 0; i < j; ++i) {
-        const double t = cs[i] * R[i] + sn[i] * R[i + 1];
-        R[i + 1] = -sn[i] * R[i] + cs[i] * R[i + 1];
-        R[i] = t;
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+        R[i] = h[i] + h2[i];
+        if (i < j) {
+            cs[i] = gs[GS_CS + i];
+            sn[i] = gs[GS_SN + i];
+        }
     }
-    const double den = hypot(R[j], R[j + 1]);
-    cs[j] = den > 0.0 ? R[j] / den : 1.0;
-    sn[j] = den > 0.0 ? R[j + 1] / den : 0.0;
-    R[j] = den;
-    R[j + 1] = 0.0;
-    g[j + 1] = -sn[j] * g[j];
-    g[j] = cs[j] * g[j];
-    const double est = fabs(g[j + 1]);
-    gs[GS_EST] = est;
-    gs[GS_INV] = 1.0 / hn;
-    const int k = j + 1;
-    gctl[0] = k;
-    int done = (est <= gs[GS_THR] || hn == 0.0 || k >= gctl[2]) ? 1 : 0;
-    if (!isfinite(hn) || !isfinite(est)) {
-        gctl[3] = 1;
-        done = 1;
+    gs::sum_partials(part, gridDim.x, gridDim.x, 1, [&](int, double sum) { R[m] = sqrt(sum); });
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const double hn = R[m], gj = g[j], thr = gs[GS_THR];
+        const int maxsteps = gctl[2];
+        double r = R[0];
+        for (int i = 0; i < j; ++i) {
+            const double next = R[i + 1];
+            R[i] = cs[i] * r + sn[i] * next;
+            r = -sn[i] * r + cs[i] * next;
+        }
+        const double den = hypot(r, hn);
+        const double c = den > 0.0 ? r / den : 1.0, q = den > 0.0 ? hn / den : 0.0;
+        R[j] = den;
+        R[m] = 0.0;
+        gs[GS_CS + j] = c;
+        gs[GS_SN + j] = q;
+        g[m] = -q * gj;
+        g[j] = c * gj;
+        const double est = fabs(q * gj);
+        gs[GS_EST] = est;
+        gs[GS_INV] = 1.0 / hn;
+        gctl[0] = m;
+        int done = (est <= thr || hn == 0.0 || m >= maxsteps) ? 1 : 0;
+        if (!isfinite(hn) || !isfinite(est)) {
+            gctl[3] = 1;
+            done = 1;
+        }
+        gctl[1] = done;
+        cudaGraphSetConditional(hc, done ? 0u : 1u);
     }
-    gctl[1] = done;
-    cudaGraphSetConditional(hc, done ? 0u : 1u);
+    __syncthreads();
+    for (int i = threadIdx.x; i <= m; i += blockDim.x) gs[GS_R + (long long)j * GS_LD + i] = R[i];
 }
 
 // V_j (j = the steps done) = w / ||w|| and the next operator input: its split
@@ -760,13 +756,17 @@ __global__ void gm_scale_basis_kernel(long long N, const float* __restrict__ w, 
     }
 }
 
-// cycle start: beta = ||P^{-1} r|| (from the reduced dot), g = beta e_1, the
-// stop target ptheta beta, control words
-__global__ void gm_start_kernel(double* gs, const double* ww, int* gctl, int maxsteps, double ptheta) {
-    const double beta = sqrt(*ww);
+// cycle start (one warp): beta = ||P^{-1} r|| from the dot's partial sums,
+// g = beta e_1, the stop target ptheta beta, control words
+__global__ void gm_start_kernel(double* gs, const double* part, int nblk, int* gctl, int maxsteps, double ptheta) {
+    double ww = 0.0;
+    gs::sum_partials(part, nblk, nblk, 1, [&](int, double sum) { ww = sum; });
+    if (threadIdx.x) return;
+    const double beta = sqrt(ww);
     gs[GS_BETA] = beta;
     gs[GS_EST] = beta;
     gs[GS_INV] = 1.0 / beta;
+    gs[GS_TICKET] = 0.0;
     gs[GS_THR] = ptheta * beta;
     for (int i = 0; i <= GS_MAXM; ++i) gs[GS_G + i] = 0.0;
     gs[GS_G] = beta;
@@ -791,32 +791,28 @@ __global__ void gm_solve_kernel(const double* gs, const int* gctl, double* ny, i
 }
 
 void launch_gm_step(size_t N, const float* V, size_t ldv, float* w, double* part, int nblk, double* hbuf,
-                    double* h2buf, double* wwbuf, double* gs, int* gctl, cudaGraphConditionalHandle hc,
-                    __nv_bfloat16* ph, __nv_bfloat16* pl, float* next, int maxm, cudaStream_t s) {
-    stats_count_launch(8);
+                    double* h2buf, double* gs, int* gctl, cudaGraphConditionalHandle hc,
+                    __nv_bfloat16* ph, __nv_bfloat16* pl, float* next, cudaStream_t s) {
+    stats_count_launch(kGmStepLaunches);
     const long long n = (long long)N, ld = (long long)ldv;
     nblk = dot_blocks(nblk);
+    unsigned* ticket = reinterpret_cast<unsigned*>(gs + GS_TICKET);
     // CGS2: <V, w>; w -= V h and <V, w> again (one pass over the block's chunk);
     // w -= V h2 and ||w||^2 (one pass)
-    gm_multidot_kernel<<<nblk, kT, 0, s>>>(n, V, ld, w, part, gctl);
-    gm_reduce_kernel<<<maxm, 32, 0, s>>>(part, nblk, hbuf, 0, gctl);
-    gm_axpy_dot_kernel<<<nblk, kT, 0, s>>>(n, V, ld, hbuf, w, part, gctl);
-    gm_reduce_kernel<<<maxm, 32, 0, s>>>(part, nblk, h2buf, 0, gctl);
-    gm_axpy_norm_kernel<<<nblk, kT, 0, s>>>(n, V, ld, h2buf, w, part, gctl);
-    gm_reduce_kernel<<<1, 32, 0, s>>>(part, nblk, wwbuf, 1, gctl);
-    gm_givens_kernel<<<1, 1, 0, s>>>(gs, hbuf, h2buf, wwbuf, gctl, hc);
+    gm_multidot_kernel<<<nblk, kT, 0, s>>>(n, V, ld, w, part, hbuf, ticket, gctl);
+    gm_axpy_dot_kernel<<<nblk, kT, 0, s>>>(n, V, ld, hbuf, w, part, h2buf, ticket, gctl);
+    gm_axpy_norm_kernel<<<nblk, kT, 0, s>>>(n, V, ld, hbuf, h2buf, w, part, ticket, gs, gctl, hc);
     gm_scale_basis_kernel<<<grid_for(n), kT, 0, s>>>(n, w, const_cast<float*>(V), ld, gs, gctl, ph, pl, next);
 }
-void launch_gm_start(size_t N, const float* w, double* part, int nblk, double* wwbuf, double* gs, int* gctl,
+void launch_gm_start(size_t N, const float* w, double* part, int nblk, double* gs, int* gctl,
                      int maxsteps, double ptheta, float* V0, __nv_bfloat16* ph, __nv_bfloat16* pl, float* next,
                      cudaStream_t s) {
-    stats_count_launch(4);
+    stats_count_launch(3);
     const long long n = (long long)N;
     nblk = dot_blocks(nblk);
-    // gctl[1] = 0 here (set by the caller's reset) so that the dot and reduce run
+    // gctl[1] = 0 here (set by the caller's reset) so that the dot runs
     gm_dot_kernel<<<nblk, kT, 0, s>>>(n, w, part, gctl);
-    gm_reduce_kernel<<<1, 32, 0, s>>>(part, nblk, wwbuf, 1, gctl);
-    gm_start_kernel<<<1, 1, 0, s>>>(gs, wwbuf, gctl, maxsteps, ptheta);
+    gm_start_kernel<<<1, 32, 0, s>>>(gs, part, nblk, gctl, maxsteps, ptheta);
     gm_scale_basis_kernel<<<grid_for(n), kT, 0, s>>>(n, w, V0, n, gs, gctl, ph, pl, next);
 }
 void launch_gm_solve(const double* gs, const int* gctl, double* ny, int maxm, cudaStream_t s) {

@@ -877,8 +877,8 @@ int build_gmres_graph_spec(const tfde_problem* P, int restart, cudaStream_t s) {
             const int* skip = M->gm_ctl + 1;
             int st = spec_matvec(P, nullptr, M->f[F_Z], nullptr, s, skip, true);   // w = Lambda^{-1} A~ v_j
             if (!st)
-                launch_gm_step(N, M->V32, N, M->f[F_Z], P->red, P->nblk, M->gm + GM_H, M->gm + GM_H2, M->gm + GM_WW,
-                               M->gm_state, M->gm_ctl, h, M->hi[PL_P], M->lo[PL_P], nullptr, restart + 1, s);
+                launch_gm_step(N, M->V32, N, M->f[F_Z], P->red, P->nblk, M->gm + GM_H, M->gm + GM_H2,
+                               M->gm_state, M->gm_ctl, h, M->hi[PL_P], M->lo[PL_P], nullptr, s);
             stats_set_capturing(false);
             cudaGraph_t out = nullptr;
             const cudaError_t e = cudaStreamEndCapture(s, &out);
@@ -925,7 +925,7 @@ int inner_gmres_spec(const tfde_problem* P, int restart, double ptheta, int maxi
     if (M->device_loop && !stats_timing() && maxit > 0 && M->gms_exec && M->gms_graph_restart == restart) {
         MX_TRY(cudaMemsetAsync(M->gm_ctl, 0, 4 * sizeof(int), s));
         const int maxsteps = restart < maxit ? restart : maxit;
-        launch_gm_start(N, M->f[F_Z], P->red, P->nblk, g + GM_WW, M->gm_state, M->gm_ctl, maxsteps, ptheta, V,
+        launch_gm_start(N, M->f[F_Z], P->red, P->nblk, M->gm_state, M->gm_ctl, maxsteps, ptheta, V,
                         M->hi[PL_P], M->lo[PL_P], nullptr, s);
         MX_TRY(cudaGraphLaunch(M->gms_exec, s));
         ++M->graph_launches;
@@ -935,7 +935,7 @@ int inner_gmres_spec(const tfde_problem* P, int restart, double ptheta, int maxi
         MX_TRY(cudaMemcpyAsync(P->red_host, M->gm_state, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
         MX_TRY(cudaStreamSynchronize(s));
         k = M->gm_ctl_host[0];
-        stats_count_launch((unsigned)(k > 0 ? k : 1) * 11u);   // the graph's launches, 11 per step
+        stats_count_launch((unsigned)(k > 0 ? k : 1) * (3u + kGmStepLaunches));   // the graph's launches
         const double beta = P->red_host[GS_BETA], est = P->red_host[GS_EST];
         if (M->gm_ctl_host[3] || !std::isfinite(beta))
             return set_error(TFDE_ENAN, "non-finite preconditioned residual or Arnoldi vector");
@@ -1097,8 +1097,8 @@ int build_gmres_graph(const tfde_problem* P, int restart, cudaStream_t s) {
             int st = fast_matvec(P, TFDE_OP_A, nullptr, s, PL_R, nullptr, nullptr, skip);
             if (!st) st = fast_precond(P, M->f[F_Z], s, nullptr, nullptr, skip);
             if (!st)
-                launch_gm_step(N, M->V32, N, M->f[F_Z], P->red, P->nblk, M->gm + GM_H, M->gm + GM_H2, M->gm + GM_WW,
-                               M->gm_state, M->gm_ctl, h, M->hi[PL_P], M->lo[PL_P], nullptr, restart + 1, s);
+                launch_gm_step(N, M->V32, N, M->f[F_Z], P->red, P->nblk, M->gm + GM_H, M->gm + GM_H2,
+                               M->gm_state, M->gm_ctl, h, M->hi[PL_P], M->lo[PL_P], nullptr, s);
             stats_set_capturing(false);
             cudaGraph_t out = nullptr;
             const cudaError_t e = cudaStreamEndCapture(s, &out);
@@ -1133,7 +1133,7 @@ int inner_gmres_graph(const tfde_problem* P, int restart, double ptheta, int max
     int st = fast_precond(P, M->f[F_Z], s);   // w = P^{-1} r
     if (st) return st;
     const int maxsteps = restart < maxit ? restart : maxit;
-    launch_gm_start(N, M->f[F_Z], P->red, P->nblk, M->gm + GM_WW, M->gm_state, M->gm_ctl, maxsteps, ptheta, M->V32,
+    launch_gm_start(N, M->f[F_Z], P->red, P->nblk, M->gm_state, M->gm_ctl, maxsteps, ptheta, M->V32,
                     M->hi[PL_P], M->lo[PL_P], nullptr, s);
     MX_TRY(cudaGraphLaunch(M->gm_exec, s));
     ++M->graph_launches;
@@ -1143,7 +1143,7 @@ int inner_gmres_graph(const tfde_problem* P, int restart, double ptheta, int max
     MX_TRY(cudaMemcpyAsync(P->red_host, M->gm_state, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
     MX_TRY(cudaStreamSynchronize(s));
     const int k = M->gm_ctl_host[0];
-    stats_count_launch((unsigned)(k > 0 ? k : 1) * 17u);   // the graph's launches, 17 per step
+    stats_count_launch((unsigned)(k > 0 ? k : 1) * (9u + kGmStepLaunches));   // the graph's launches
     const double beta = P->red_host[GS_BETA], est = P->red_host[GS_EST];
     if (M->gm_ctl_host[3] || !std::isfinite(beta))
         return set_error(TFDE_ENAN, "non-finite preconditioned residual or Arnoldi vector");

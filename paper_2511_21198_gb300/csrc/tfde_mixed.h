@@ -63,18 +63,19 @@ void launch_pcg_fold_dev(size_t N, const float* const* p, const double* const* a
 // most GS_MAXM Arnoldi steps per cycle
 constexpr int GS_MAXM = 64;
 constexpr int GS_LD = GS_MAXM + 2;   // leading dimension of a Hessenberg column
-enum { GS_BETA = 0, GS_EST = 1, GS_INV = 2, GS_THR = 3, GS_G = 8, GS_CS = GS_G + GS_MAXM + 1,
+enum { GS_BETA = 0, GS_EST = 1, GS_INV = 2, GS_THR = 3, GS_TICKET = 4, GS_G = 8, GS_CS = GS_G + GS_MAXM + 1,
        GS_SN = GS_CS + GS_MAXM, GS_R = GS_SN + GS_MAXM, GS_WORDS = GS_R + GS_LD * GS_MAXM };
+constexpr int kGmStepLaunches = 4;
 // one Arnoldi step on w (the preconditioner's output): CGS2 against V_0..V_j,
 // ||w||, the Givens update and stop test (loop condition hc), V_{j+1} = w/||w||
 // with its split planes; every count and address from the control words
 // (V_i at V + i ldv; the next operator input goes to the split planes, or with
 // `next` as FP32 to that fixed address)
 void launch_gm_step(size_t N, const float* V, size_t ldv, float* w, double* part, int nblk, double* hbuf,
-                    double* h2buf, double* wwbuf, double* gs, int* gctl, cudaGraphConditionalHandle hc,
-                    __nv_bfloat16* ph, __nv_bfloat16* pl, float* next, int maxm, cudaStream_t s);
+                    double* h2buf, double* gs, int* gctl, cudaGraphConditionalHandle hc,
+                    __nv_bfloat16* ph, __nv_bfloat16* pl, float* next, cudaStream_t s);
 // cycle start on w = P^{-1} r: beta, g = beta e_1, V_0 = w / beta and the next operator input
-void launch_gm_start(size_t N, const float* w, double* part, int nblk, double* wwbuf, double* gs, int* gctl,
+void launch_gm_start(size_t N, const float* w, double* part, int nblk, double* gs, int* gctl,
                      int maxsteps, double ptheta, float* V0, __nv_bfloat16* ph, __nv_bfloat16* pl, float* next,
                      cudaStream_t s);
 // ny = -y of the cycle's least-squares problem (zero beyond the steps done)
