@@ -834,9 +834,10 @@ int free_batch(tfde_batch* B) {
     return TFDE_OK;
 }
 
-int grouped(tfde_batch* B, const tc::Params* d, int axis, int out_mode, double bytes, double flops, cudaStream_t s) {
+int grouped(tfde_batch* B, const tc::Params* d, int axis, int out_mode, double bytes, double flops, cudaStream_t s,
+            int ep = 0) {
     return tc::launch_grouped(d, B->d_gstart + (size_t)axis * (B->count + 1), B->count, B->gtotal[axis],
-                              axis == 0 ? 1 : 0, out_mode, B->bn[axis], B->d_act, B->d_err, s, bytes, flops);
+                              axis == 0 ? 1 : 0, out_mode, ep, B->bn[axis], B->d_act, B->d_err, s, bytes, flops);
 }
 
 // v_j (split planes PL_P of every active problem) -> PL_R = A v_j
@@ -864,7 +865,7 @@ int grouped_precond(tfde_batch* B, int j, cudaStream_t s) {
 int grouped_spec_start(tfde_batch* B, cudaStream_t s) {
     for (int a = 0; a < 3; ++a) {
         int st = grouped(B, B->d_sfw + (size_t)a * B->count, a, a < 2 ? tc::OUT_HILO : tc::OUT_SUM, B->sfw_bytes[a],
-                         B->sfw_flops[a], s);
+                         B->sfw_flops[a], s, a < 2 ? 0 : tc::EP_DIV);
         if (st) return st;
     }
     return TFDE_OK;
@@ -876,7 +877,8 @@ int grouped_spec_step(tfde_batch* B, int j, cudaStream_t s) {
         int st = grouped(B, B->d_sop + (size_t)a * B->count, a, tc::OUT_SUM, B->sop_bytes[a], B->sop_flops[a], s);
         if (st) return st;
     }
-    return grouped(B, B->d_sopz + (size_t)j * B->count, 2, tc::OUT_SUM, B->sop_bytes[2], B->sop_flops[2], s);
+    return grouped(B, B->d_sopz + (size_t)j * B->count, 2, tc::OUT_SUM, B->sop_bytes[2], B->sop_flops[2], s,
+                   tc::EP_DIV);
 }
 
 // eigenbasis: x32 = S_N x32 for the problems with act set (planes PL_T1 -> PL_T2 -> PL_R -> x32)
@@ -936,7 +938,8 @@ int build_cycle_graph(tfde_batch* B, cudaStream_t s) {
             int st = TFDE_OK;
             for (int a = 0; a < 2 && !st; ++a)
                 st = grouped(B, B->d_sop + (size_t)a * C, a, tc::OUT_SUM, B->sop_bytes[a], B->sop_flops[a], s);
-            if (!st) st = grouped(B, B->d_sopzw, 2, tc::OUT_SUM, B->sop_bytes[2], B->sop_flops[2], s);
+            if (!st) st = grouped(B, B->d_sopzw, 2, tc::OUT_SUM, B->sop_bytes[2], B->sop_flops[2], s,
+                   tc::EP_DIV);
             if (!st) {   // CGS2: <V, W>; W -= V h and <V, W> again (one pass); W -= V h2 and ||W||^2 (one pass)
                 bkg_dots<<<B->NB, kBT, 0, s>>>(B->d_vt, B->d_bi, B->d_bo, B->d_act, B->d_j, B->d_part, B->d_h);
                 bkg_axpy_dots<<<B->NB, kBT, 0, s>>>(B->d_vt, B->d_bi, B->d_bo, B->d_act, B->d_j, B->d_h, 0, 64,
@@ -1011,7 +1014,7 @@ int build_pcg_graph(tfde_batch* B) {
             int st = TFDE_OK;
             for (int a = 0; a < 2 && !st; ++a)
                 st = grouped(B, B->d_sop + (size_t)a * C, a, tc::OUT_SUM, B->sop_bytes[a], B->sop_flops[a], s);
-            if (!st) st = grouped(B, B->d_sopq, 2, tc::OUT_SUM, B->sopq_bytes, B->sopq_flops, s);
+            if (!st) st = grouped(B, B->d_sopq, 2, tc::OUT_SUM, B->sopq_bytes, B->sopq_flops, s, tc::EP_DOT);
             if (!st) {
                 bkp_update<<<B->NB, kBT, 0, s>>>(B->d_vt, B->d_bi, B->d_bo, B->d_act, B->d_s);
                 bkpg_stop<<<gb, 64, 0, s>>>(C, B->d_j, kPcgMaxIt, B->d_s, B->d_theta, B->d_act, B->d_its, B->d_est,
@@ -1220,7 +1223,8 @@ int batch_pcg(tfde_batch* B, const std::vector<int>& outer, const std::vector<do
         for (int a = 0; a < 2; ++a)
             if ((st = grouped(B, B->d_sop + (size_t)a * C, a, tc::OUT_SUM, B->sop_bytes[a], B->sop_flops[a], s)))
                 return st;
-        if ((st = grouped(B, B->d_sopq, 2, tc::OUT_SUM, B->sopq_bytes, B->sopq_flops, s))) return st;
+        if ((st = grouped(B, B->d_sopq, 2, tc::OUT_SUM, B->sopq_bytes, B->sopq_flops, s, tc::EP_DOT)))
+            return st;
         vec_launch_count();
         bkp_update<<<B->NB, kBT, 0, s>>>(B->d_vt, B->d_bi, B->d_bo, B->d_act, B->d_s);
         vec_launch_count();

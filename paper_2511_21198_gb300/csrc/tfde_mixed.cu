@@ -257,7 +257,7 @@ int fast_matvec(const tfde_problem* P, int op, float* q32, cudaStream_t s, int o
     for (int g = 0; g < 2; ++g) {
         M->gemm_launches++;
         st = tc::launch_grouped(M->pair_d + 2 * g, M->pair_gstart + 3 * g, 2, M->pair_total[g], g == 0 ? 1 : 0,
-                                tc::OUT_HILO, M->bn[g == 0 ? 0 : 1], nullptr, M->err, s, M->pair_bytes[g], M->pair_flops[g], skip);
+                                tc::OUT_HILO, 0, M->bn[g == 0 ? 0 : 1], nullptr, M->err, s, M->pair_bytes[g], M->pair_flops[g], skip);
         if (st) return st;
     }
     return run_passes(P, ps + 4, 1, q32, s, dot_vec, dot_out, skip);

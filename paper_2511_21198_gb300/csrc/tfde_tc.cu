@@ -250,9 +250,9 @@ int tile_lines(long long wide) {
 
 bool attr_done = false;
 
-template <bool G, int KM, int OM>
+template <bool G, int KM, int OM, int EP = 0>
 bool set_attr_one() {
-    return cudaFuncSetAttribute(axis_gemm_kernel<G, KM, OM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(axis_gemm_kernel<G, KM, OM, EP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 SMEM_BYTES) == cudaSuccess;
 }
 
@@ -265,7 +265,9 @@ int set_attrs() {
                         set_attr_one<false, 0, OUT_XPAY>() && set_attr_one<false, 1, OUT_XPAY>() &&
                         set_attr_one<false, 0, OUT_HI>() && set_attr_one<false, 1, OUT_HI>() &&
                         set_attr_one<false, 0, OUT_SUM>() && set_attr_one<false, 1, OUT_SUM>() &&
-                        set_attr_one<true, 0, OUT_SUM>() && set_attr_one<true, 1, OUT_SUM>();
+                        set_attr_one<true, 0, OUT_SUM>() && set_attr_one<true, 1, OUT_SUM>() &&
+                        set_attr_one<false, 0, OUT_SUM, EP_DOT>() && set_attr_one<false, 0, OUT_SUM, EP_DIV>() &&
+                        set_attr_one<true, 0, OUT_SUM, EP_DOT>() && set_attr_one<true, 0, OUT_SUM, EP_DIV>();
         if (!ok) return set_error(TFDE_ECUDA, "cudaFuncSetAttribute(smem) failed");
         attr_done = true;
     }
@@ -276,7 +278,7 @@ int set_attrs() {
 // initialisation, TMEM allocation) may start while the previous kernel on the
 // stream drains; the kernel waits for that kernel's completion
 // (griddepcontrol.wait) before its first global memory access.
-template <bool G, int KM, int OM>
+template <bool G, int KM, int OM, int EP = 0>
 void launch_one(unsigned grid, cudaStream_t s, const Params& p0, const Params* groups, const long long* gstart,
                 int ngroups, const int* gactive) {
     cudaLaunchConfig_t cfg = {};
@@ -289,15 +291,18 @@ void launch_one(unsigned grid, cudaStream_t s, const Params& p0, const Params* g
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, axis_gemm_kernel<G, KM, OM>, p0, groups, gstart, ngroups, gactive);
+    cudaLaunchKernelEx(&cfg, axis_gemm_kernel<G, KM, OM, EP>, p0, groups, gstart, ngroups, gactive);
 }
 
-// The kernel instance for (layout, output mode).
+// The kernel instance for (layout, output mode, and what an OUT_SUM pass on y / z
+// does besides the addend: a dot product or the division by Lambda, never both).
 template <bool G>
-void launch_instance(int kmajor, int out_mode, unsigned grid, cudaStream_t s, const Params& p0, const Params* groups,
+void launch_instance(int kmajor, int out_mode, int ep, unsigned grid, cudaStream_t s, const Params& p0, const Params* groups,
                      const long long* gstart, int ngroups, const int* gactive) {
     if (out_mode == OUT_SUM) {   // the eigenbasis passes: single and grouped (the batched solver)
         if (kmajor) launch_one<G, 1, OUT_SUM>(grid, s, p0, groups, gstart, ngroups, gactive);
+        else if (ep == EP_DOT) launch_one<G, 0, OUT_SUM, EP_DOT>(grid, s, p0, groups, gstart, ngroups, gactive);
+        else if (ep == EP_DIV) launch_one<G, 0, OUT_SUM, EP_DIV>(grid, s, p0, groups, gstart, ngroups, gactive);
         else launch_one<G, 0, OUT_SUM>(grid, s, p0, groups, gstart, ngroups, gactive);
         return;
     }
@@ -336,6 +341,7 @@ struct Rec {
     int ngroups;
     long long total;
     const int* gactive;
+    int ep;
 };
 bool g_recording = false;
 std::vector<Rec> g_rec;
@@ -370,6 +376,10 @@ void choose(const TuneKey& k, long long total, int cap, long long* grid, int* st
 void tune_force(int grid, int stages) {
     g_force_grid = grid;
     g_force_stages = stages;
+}
+
+int sum_part(const Params& P) {
+    return P.out_mode != OUT_SUM || P.b_kmajor ? 0 : (P.dot_vec ? EP_DOT : (P.lam_ra ? EP_DIV : 0));
 }
 
 int stage_capacity(int stage_bytes) {
@@ -444,12 +454,13 @@ int launch(const Params& P0, cudaStream_t s, double bytes, double flops) {
     if (int st = set_attrs()) return st;
     Params P = P0;
     set_ring(P);
+    const int ep = sum_part(P);
     const long long total = P.ntiles * P.mhalves;
     long long grid;
     choose(tune_key_single(P), total, stage_capacity(P.stage_bytes), &grid, &P.nstages);
-    if (g_recording) g_rec.push_back(Rec{tune_key_single(P), P, nullptr, nullptr, 0, total, nullptr});
+    if (g_recording) g_rec.push_back(Rec{tune_key_single(P), P, nullptr, nullptr, 0, total, nullptr, ep});
     void* tok = stats_tc_begin(s, TFDE_KIND_SPLIT);
-    launch_instance<false>(P.b_kmajor, P.out_mode, (unsigned)grid, s, P, nullptr, nullptr, 0, nullptr);
+    launch_instance<false>(P.b_kmajor, P.out_mode, ep, (unsigned)grid, s, P, nullptr, nullptr, 0, nullptr);
     cudaError_t e = cudaGetLastError();
     stats_tc_end(tok, s, TFDE_KIND_SPLIT, bytes, flops);
     if (e != cudaSuccess) return set_error(TFDE_ECUDA, std::string("axis_gemm_kernel launch: ") + cudaGetErrorString(e));
@@ -457,8 +468,8 @@ int launch(const Params& P0, cudaStream_t s, double bytes, double flops) {
 }
 
 int launch_grouped(const Params* groups, const long long* gstart, int ngroups, long long total, int b_kmajor,
-                   int out_mode, int bn, const int* gactive, int* err, cudaStream_t s, double bytes, double flops,
-                   const int* skip) {
+                   int out_mode, int ep, int bn, const int* gactive, int* err, cudaStream_t s, double bytes,
+                   double flops, const int* skip) {
     if (int st = set_attrs()) return st;
     if (out_mode == OUT_HI || out_mode == OUT_XPAY)
         return set_error(TFDE_EUNSUPPORTED, "grouped axis_gemm_kernel: split, FP32 or eigenbasis output only");   // no such instances
@@ -478,9 +489,9 @@ int launch_grouped(const Params* groups, const long long* gstart, int ngroups, l
     long long grid;
     choose(tune_key_grouped(b_kmajor, out_mode, p0.stage_bytes, total), total, stage_capacity(p0.stage_bytes), &grid, &p0.nstages);
     if (g_recording)
-        g_rec.push_back(Rec{tune_key_grouped(b_kmajor, out_mode, p0.stage_bytes, total), p0, groups, gstart, ngroups, total, gactive});
+        g_rec.push_back(Rec{tune_key_grouped(b_kmajor, out_mode, p0.stage_bytes, total), p0, groups, gstart, ngroups, total, gactive, ep});
     void* tok = stats_tc_begin(s, TFDE_KIND_SPLIT);
-    launch_instance<true>(b_kmajor, out_mode, (unsigned)grid, s, p0, groups, gstart, ngroups, gactive);
+    launch_instance<true>(b_kmajor, out_mode, ep, (unsigned)grid, s, p0, groups, gstart, ngroups, gactive);
     cudaError_t e = cudaGetLastError();
     stats_tc_end(tok, s, TFDE_KIND_SPLIT, bytes, flops);
     if (e != cudaSuccess)
@@ -547,10 +558,10 @@ int tune_recorded(int reps, cudaStream_t s) {
             P.nstages = cand[c].second;
             auto go = [&]() {
                 if (r.key.grouped)
-                    launch_instance<true>(r.key.kmajor, r.key.out_mode, (unsigned)grid, s, P, r.groups, r.gstart,
+                    launch_instance<true>(r.key.kmajor, r.key.out_mode, r.ep, (unsigned)grid, s, P, r.groups, r.gstart,
                                           r.ngroups, r.gactive);
                 else
-                    launch_instance<false>(P.b_kmajor, P.out_mode, (unsigned)grid, s, P, nullptr, nullptr, 0, nullptr);
+                    launch_instance<false>(P.b_kmajor, P.out_mode, r.ep, (unsigned)grid, s, P, nullptr, nullptr, 0, nullptr);
             };
             go();
             cudaEventRecord(e0, s);

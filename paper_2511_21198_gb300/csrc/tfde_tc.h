@@ -44,8 +44,11 @@ int launch(const Params& P, cudaStream_t s, double bytes, double flops);
 // Bounded-wait self-test (tfde_selftest_wait).
 int wait_selftest(long long limit_ns, int* tmem_freed, cudaStream_t s);
 int launch_grouped(const Params* groups, const long long* gstart, int ngroups, long long total, int b_kmajor,
-                   int out_mode, int bn, const int* gactive, int* err, cudaStream_t s, double bytes, double flops,
-                   const int* skip = nullptr);
+                   int out_mode, int ep, int bn, const int* gactive, int* err, cudaStream_t s, double bytes,
+                   double flops, const int* skip = nullptr);
+// EP_DOT, EP_DIV or 0: the epilogue part of a launch with descriptor P (the same
+// for every group of a grouped one)
+int sum_part(const Params& P);
 
 // Launch parameters chosen by the autotuner (tfde_tune, tfde_batch_tune):
 // the number of persistent CTAs and of ring stages, per launch class.  A

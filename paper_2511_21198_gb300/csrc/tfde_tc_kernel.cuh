@@ -85,6 +85,7 @@ struct Segment {
 // by pass (the operator in the sine-transform eigenbasis); on the z axis
 // with lam_ra set, the result is divided by Lambda (the preconditioned
 // operator of left-preconditioned GMRES).
+enum { EP_DOT = 1, EP_DIV = 2 };   // OUT_SUM on y / z: dot_vec set, lam_ra set
 enum { OUT_F32 = 0, OUT_HILO = 1, OUT_XPAY = 2, OUT_HI = 3, OUT_SUM = 4 };
 
 struct Params {
@@ -249,8 +250,9 @@ __device__ __forceinline__ int find_group(const long long* __restrict__ gstart, 
 // skipped by all three roles alike.  p0 then carries only the common fields
 // (err, bn, the ring geometry) and ntiles = gstart[ngroups], mhalves = 1.  KM
 // (= Params::b_kmajor) and OM (= Params::out_mode) are compile-time so that
-// each instance carries one straight-line epilogue.
-template <bool GROUPED, int KM, int OM>
+// each instance carries one straight-line epilogue; so is EP, what a y / z pass
+// of OUT_SUM does besides the addend (EP_DOT, EP_DIV).
+template <bool GROUPED, int KM, int OM, int EP = 0>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
     axis_gemm_kernel(const __grid_constant__ Params p0, const Params* __restrict__ groups,
                      const long long* __restrict__ gstart, int ngroups, const int* __restrict__ gactive) {
@@ -466,6 +468,38 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             if (lane == 0 && dot_dst) atomicAdd(dot_dst, t);
             da = DotAcc();
         };
+        // OUT_SUM on y / z.  Bound: the latency of a chunk's global operands, two
+        // chunks per warp and tile at 128^3 (x pass without operands 8.5 us, y 15,
+        // z 16; y / z together 17.5 -> 15.5 us with the following and with Lambda's
+        // factors read once per chunk and row instead of per access; batch of 64
+        // uneven problems 155 -> 147 ms).  The addend and the dot vector are read
+        // coalesced (lane l: rows 4i + l / 8, columns 4 (l % 8) .. + 3, a
+        // 128-byte row segment per 8 lanes).  Each register is loaded for the
+        // warp's next chunk as soon as this chunk has used it, so that the
+        // loads run under the next chunk's accumulator read.
+        float4 ad4[8], w4[8];
+        struct Operands {
+            const float *ad, *w;   // of row mrow0 + l / 8, or null
+            long long step;        // four rows
+            int rows;              // rows from there to the last
+        };
+        auto operands = [&](const Params& p, long long tile, int mh, int cc) -> Operands {
+            const int c0 = half * (bn / 2) + cc;
+            const long long gb = tile * (bn / 64) + c0 / 64;
+            const unsigned pl = (unsigned)gb / (unsigned)p.nbc;   // nblocks < 2^31
+            const int cx = (int)((unsigned)gb - pl * (unsigned)p.nbc) * 64 + (c0 & 63) + (lane & 7) * 4;
+            const int row = mh * BM + 32 * q + (lane >> 3);
+            const long long at = (long long)pl * p.plane + (long long)row * p.C + cx;
+            const bool in = gb < p.nblocks && cx < p.C;
+            return Operands{in && p.addend ? p.addend + at : nullptr, (EP & EP_DOT) && in ? p.dot_vec + at : nullptr,
+                            4LL * p.C, p.n - row};
+        };
+        auto fetch = [&](const Operands& o, int i) {
+            const bool in = 4 * i < o.rows;
+            ad4[i] = o.ad && in ? __ldg(reinterpret_cast<const float4*>(o.ad + i * o.step)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr ((EP & EP_DOT) != 0)
+                w4[i] = o.w && in ? __ldg(reinterpret_cast<const float4*>(o.w + i * o.step)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
         float xp_beta = 0.f;                  // OUT_XPAY coefficient
         if constexpr (OM == OUT_XPAY) {
             if (p0.xp_den) xp_beta = (float)(__ldg(p0.xp_num) / __ldg(p0.xp_den));
@@ -486,14 +520,21 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             }
             const int buf = (int)(it & 1);
             const uint32_t use = (uint32_t)(it >> 1);
+            const long long tile = lt / p.mhalves;
+            const int mh = (int)(lt % p.mhalves);
+            if constexpr (OM == OUT_SUM && KM == 0) {
+                if (GROUPED || it == 0) {
+                    const Operands o = operands(p, tile, mh, 0);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) fetch(o, i);
+                }
+            }
             int ok = 1;
             if (lane == 0) ok = mbar_wait(&tfull[buf], use & 1u, err) ? 1 : 0;
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) break;  // warp-uniform: the TMEM loads below are .sync.aligned
             __syncwarp();
             tc_fence_after();
-            const long long tile = lt / p.mhalves;
-            const int mh = (int)(lt % p.mhalves);
             const int mrow0 = mh * BM + 32 * q;   // first row of this warp's quadrant
             const int m = mrow0 + lane;           // this thread's row
             const bool mval = m < p.n;
@@ -524,8 +565,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                 const long long gbase = b_kmajor ? line0 * p.n1 + m : (long long)pl * p.plane + (long long)m * p.C + cx;
                 const long long gstep = b_kmajor ? (long long)p.n1 : 1LL;
                 if constexpr (OM == OUT_SUM) {
-                    const bool use_w = p.dot_vec != nullptr;
-                    const bool use_ad = p.addend != nullptr;
                     if constexpr (KM != 0) {
                         // x axis (no addend or dot vector): the column factor
                         // of this lane's line, broadcast by shuffles
@@ -544,30 +583,26 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                                     __shfl_sync(0xffffffffu, csl, 16 * hf + j) * (p.alpha * __uint_as_float(r[j]));
                         }
                     } else {
-                        // y / z axes: the chunk's addend and dot vector are read
-                        // coalesced (lane l: rows 4i + l / 8, columns 4 (l % 8)
-                        // .. + 3, a 128-byte row segment per 8 lanes), issued
-                        // before the accumulator read; the accumulator goes
-                        // through the slot from its row layout to that one
+                        // y / z axes: the accumulator goes through the slot from
+                        // its row layout to the operands' (Operands above)
                         const int rr = lane >> 3, c4 = (lane & 7) * 4;
                         const bool cval = c4 < ncol;
-                        const long long cbase = (long long)pl * p.plane + cx + c4;
-                        float4 ad4[8], w4[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int row = mrow0 + 4 * i + rr;   // the warp's first row + 4 i + l / 8
-                            const bool ok = cval && row < p.n;
-                            const long long g = cbase + (long long)row * p.C;
-                            ad4[i] = (use_ad && ok) ? __ldg(reinterpret_cast<const float4*>(p.addend + g))
-                                                    : make_float4(0.f, 0.f, 0.f, 0.f);
-                            w4[i] = (use_w && ok) ? __ldg(reinterpret_cast<const float4*>(p.dot_vec + g))
-                                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-                        }
+                        Operands next{nullptr, nullptr, 0, 0};   // of the chunk after this one
+                        if (cc + 32 < bn / 2) next = operands(p, tile, mh, cc + 32);
+                        else if (!GROUPED && t + gridDim.x < total)
+                            next = operands(p, (t + gridDim.x) / p.mhalves, (int)((t + gridDim.x) % p.mhalves), 0);
                         float4 cs4 = make_float4(1.f, 1.f, 1.f, 1.f);
                         if (p.col_scale && cval)
                             cs4 = __ldg(reinterpret_cast<const float4*>(p.col_scale + (long long)pl * p.C + cx + c4));
-                        // optional Lambda^{-1} (z pass: rows k, columns i + n1 j)
-                        const bool ldiv = p.lam_ra != nullptr;
+                        // Lambda^{-1} (z pass: rows k, columns i + n1 j): the column
+                        // factors of this lane; the rows' sit in ra and rb by lane
+                        float4 lu4 = make_float4(1.f, 1.f, 1.f, 1.f), lv4 = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if constexpr ((EP & EP_DIV) != 0) {
+                            if (cval) {
+                                lu4 = __ldg(reinterpret_cast<const float4*>(p.lam_U + cx + c4));
+                                lv4 = __ldg(reinterpret_cast<const float4*>(p.lam_V + cx + c4));
+                            }
+                        }
                         if (pending && lane == 0) bulk_wait_read0();
                         __syncwarp();
 #pragma unroll
@@ -594,26 +629,23 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                             t.y = fmaf(cs4.y, t.y, ad4[i].y);
                             t.z = fmaf(cs4.z, t.z, ad4[i].z);
                             t.w = fmaf(cs4.w, t.w, ad4[i].w);
-                            if (ldiv) {
-                                const float a = grow < p.n ? __ldg(p.lam_ra + grow) : 1.f;
-                                const float b = grow < p.n ? __ldg(p.lam_rb + grow) : 0.f;
-                                float4 lu4 = make_float4(1.f, 1.f, 1.f, 1.f), lv4 = make_float4(0.f, 0.f, 0.f, 0.f);
-                                if (cval) {   // the column factors (L1-resident after the first row)
-                                    lu4 = __ldg(reinterpret_cast<const float4*>(p.lam_U + cx + c4));
-                                    lv4 = __ldg(reinterpret_cast<const float4*>(p.lam_V + cx + c4));
-                                }
+                            if constexpr ((EP & EP_DIV) != 0) {   // rows past the last: a = 1, b = 0
+                                const float a = __shfl_sync(0xffffffffu, ra, row), b = __shfl_sync(0xffffffffu, rb, row);
                                 t.x = __fdividef(t.x, fmaf(a, lu4.x, b * lv4.x));
                                 t.y = __fdividef(t.y, fmaf(a, lu4.y, b * lv4.y));
                                 t.z = __fdividef(t.z, fmaf(a, lu4.z, b * lv4.z));
                                 t.w = __fdividef(t.w, fmaf(a, lu4.w, b * lv4.w));
                             }
                             *e = t;
-                            dacc = fmaf(t.x, w4[i].x, dacc);   // w = 0 beyond ncol and below row n
-                            dacc = fmaf(t.y, w4[i].y, dacc);
-                            dacc = fmaf(t.z, w4[i].z, dacc);
-                            dacc = fmaf(t.w, w4[i].w, dacc);
+                            if constexpr ((EP & EP_DOT) != 0) {
+                                dacc = fmaf(t.x, w4[i].x, dacc);   // w = 0 beyond ncol and below row n
+                                dacc = fmaf(t.y, w4[i].y, dacc);
+                                dacc = fmaf(t.z, w4[i].z, dacc);
+                                dacc = fmaf(t.w, w4[i].w, dacc);
+                            }
+                            fetch(next, i);
                         }
-                        if (use_w) da.add(dacc);
+                        if constexpr ((EP & EP_DOT) != 0) da.add(dacc);
                     }
                     if (ncol == 0) continue;   // warp-uniform
                     fence_proxy_async_smem();
