@@ -392,16 +392,24 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             const uint32_t use = (uint32_t)(it / nbuf);
             ++it;
             const uint32_t dbase = tmem_base + (uint32_t)(buf * (TMEM_COLS / 2));
+            const long long tile = lt / p.mhalves;
+            const int mh = (int)(lt % p.mhalves);
+            const int m = mh * BM + 32 * q + lane;
+            const bool mvalid = m < p.n;
+            if (!p.b_kmajor && p.addend && mvalid && tile < p.nblocks) {
+                // this thread's 16 addend values (a plane's last block may be narrower), towards L2
+                // while the products run
+                const int pl = (int)(tile / p.nbc), cb = (int)(tile % p.nbc) * 64 + part * EPI_COLS;
+                if (cb < p.C)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(p.addend + (long long)pl * p.plane +
+                                                                  (long long)m * p.C + cb));
+            }
             int ok = 1;
             if (lane == 0) ok = mbar_wait(&tfull[buf], use & 1u, err) ? 1 : 0;
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) break;
             __syncwarp();
             tc_fence_after();
-            const long long tile = lt / p.mhalves;
-            const int mh = (int)(lt % p.mhalves);
-            const int m = mh * BM + 32 * q + lane;
-            const bool mvalid = m < p.n;
             const int es = mvalid ? __ldg(p.row_exp + m) : 0;
             // Up to six slices the accumulators of this thread's row and EPI_COLS
             // columns are read diagonal by diagonal (8 columns per TMEM load) and
@@ -482,11 +490,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 #pragma unroll
                 for (int h8 = 0; h8 < EPI_COLS; h8 += 8) {
                     for (int d = 0; d < S; ++d) {
+                        // (the integer pipe is the longest chain of a tile) one 32 x 32
+                        // + 64-bit multiply-add each: 2^35 = 2^7 2^28 for
+                        // the leading diagonal (|a_0| 2^7 < 2^31), 2^28 at most after it
+                        const int lead = d == 0 && D > 0 ? 7 : 0, w = 1 << (7 * (D - d) - lead);
                         uint32_t r[8];
                         tmem_ld8(trow + (uint32_t)(d * BN + h8), r);
 #pragma unroll
                         for (int j = 0; j < 8; ++j)
-                            I[h8 + j] = I[h8 + j] * 128 + (long long)__float2int_rn(__uint_as_float(r[j]));
+                            I[h8 + j] += (long long)(__float2int_rn(__uint_as_float(r[j])) << lead) * (long long)w;
                     }
                 }
                 tc_fence_before();
@@ -516,11 +528,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
                     // in int64; above, floor(I / 2^8) keeps at least 54 significant bits,
                     // so the rounded double moves by at most one ulp
                     emit(cc, [&](int j, int el) {
-                        long long av[7];
+                        int a[7];
 #pragma unroll
-                        for (int d = 0; d < 7; ++d) av[d] = __float2int_rn(__uint_as_float(r[d][j]));
-                        const long long h = ((av[0] * 128 + av[1]) * 128 + av[2]) * 128 + av[3];
-                        const long long l = (av[4] * 128 + av[5]) * 128 + av[6];
+                        for (int d = 0; d < 7; ++d) a[d] = __float2int_rn(__uint_as_float(r[d][j]));
+                        const long long h = (long long)a[0] * (1 << 21) + (long long)a[1] * (1 << 14) +
+                                            (long long)a[2] * (1 << 7) + a[3];
+                        const long long l = (long long)a[4] * (1 << 14) + (long long)a[5] * (1 << 7) + a[6];
                         const bool big = h >= (1LL << 40) || h <= -(1LL << 40);
                         const long long v = big ? h * (1LL << 13) + (l >> 8) : h * (1LL << 21) + l;
                         return i64_ldexp(p.value_sign < 0 ? -v : v, sh + el + (big ? 8 : 0));
