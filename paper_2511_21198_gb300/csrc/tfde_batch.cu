@@ -78,6 +78,21 @@ __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16& hi, __nv_bflo
     lo = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
 
+// the split planes of the four elements from e (a multiple of 4)
+__device__ __forceinline__ void split4(const float4 z, __nv_bfloat16* hi, __nv_bfloat16* lo, long long e) {
+    __align__(8) __nv_bfloat16 h[4], l[4];
+    split_bf16(z.x, h[0], l[0]);
+    split_bf16(z.y, h[1], l[1]);
+    split_bf16(z.z, h[2], l[2]);
+    split_bf16(z.w, h[3], l[3]);
+    *reinterpret_cast<uint2*>(hi + e) = *reinterpret_cast<const uint2*>(h);
+    *reinterpret_cast<uint2*>(lo + e) = *reinterpret_cast<const uint2*>(l);
+}
+__device__ __forceinline__ float4 scaled4(const float* v, long long e, float f) {
+    const float4 x = *reinterpret_cast<const float4*>(v + e);
+    return make_float4(x.x * f, x.y * f, x.z * f, x.w * f);
+}
+
 using gs::KSum;
 
 __device__ __forceinline__ double block_sum(double v) {
@@ -108,11 +123,13 @@ __global__ __launch_bounds__(kBT) void bk_scale64to32(const BVec* __restrict__ v
                                                      const double* __restrict__ sc) {
     BK_PROLOGUE
     const double f = sc[inst * kSS + S_SC32];
-    for (long long e = e0 + threadIdx.x; e < e1; e += kBT) {
-        const float x = (float)(v.r64[e] * f);
-        v.r32[e] = x;
-        split_bf16(x, v.rh[e], v.rl[e]);
-        v.x32[e] = 0.f;
+    for (long long e = e0 + 4 * threadIdx.x; e < e1; e += 4 * kBT) {
+        const double2 a = *reinterpret_cast<const double2*>(v.r64 + e);
+        const double2 b = *reinterpret_cast<const double2*>(v.r64 + e + 2);
+        const float4 x = make_float4((float)(a.x * f), (float)(a.y * f), (float)(b.x * f), (float)(b.y * f));
+        *reinterpret_cast<float4*>(v.r32 + e) = x;
+        split4(x, v.rh, v.rl, e);
+        *reinterpret_cast<float4*>(v.x32 + e) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
 
@@ -167,10 +184,10 @@ __global__ __launch_bounds__(kBT) void bk_scale_split(const BVec* __restrict__ v
     BK_PROLOGUE
     const float f = (float)sc[inst * kSS + S_SPLIT];
     float* w = v.V + (long long)jw * v.N;
-    for (long long e = e0 + threadIdx.x; e < e1; e += kBT) {
-        const float x = w[e] * f;
-        w[e] = x;
-        split_bf16(x, v.ph[e], v.pl[e]);
+    for (long long e = e0 + 4 * threadIdx.x; e < e1; e += 4 * kBT) {
+        const float4 x = scaled4(w, e, f);
+        *reinterpret_cast<float4*>(w + e) = x;
+        split4(x, v.ph, v.pl, e);
     }
 }
 
@@ -179,7 +196,8 @@ __global__ __launch_bounds__(kBT) void bk_scale_split(const BVec* __restrict__ v
 __global__ __launch_bounds__(kBT) void bk_split_x32(const BVec* __restrict__ vt, const int* __restrict__ bi,
                                                    const long long* __restrict__ bo, const int* __restrict__ act) {
     BK_PROLOGUE
-    for (long long e = e0 + threadIdx.x; e < e1; e += kBT) split_bf16(v.x32[e], v.th[e], v.tl[e]);
+    for (long long e = e0 + 4 * threadIdx.x; e < e1; e += 4 * kBT)
+        split4(*reinterpret_cast<const float4*>(v.x32 + e), v.th, v.tl, e);
 }
 
 // x64 += sc * x32
@@ -203,12 +221,6 @@ __device__ __forceinline__ float4 bk_lam4(const BVec& v, unsigned e4) {
     const float4 w = __ldg(reinterpret_cast<const float4*>(v.lam + 2 * v.n3) + v.nc4 + c4);
     return make_float4(fmaf(ra, u.x, rb * w.x), fmaf(ra, u.y, rb * w.y), fmaf(ra, u.z, rb * w.z),
                        fmaf(ra, u.w, rb * w.w));
-}
-__device__ __forceinline__ void split4(const float4 z, __nv_bfloat16* hi, __nv_bfloat16* lo, long long e) {
-    split_bf16(z.x, hi[e], lo[e]);
-    split_bf16(z.y, hi[e + 1], lo[e + 1]);
-    split_bf16(z.z, hi[e + 2], lo[e + 2]);
-    split_bf16(z.w, hi[e + 3], lo[e + 3]);
 }
 __device__ __forceinline__ void ksum4(KSum& k, float4 a, float4 b) {
     k.add(a.x * b.x);
@@ -451,10 +463,10 @@ __global__ __launch_bounds__(kBT) void bkg_scale_split(const BVec* __restrict__ 
     BK_PROLOGUE
     const float f = (float)sc[inst * kSS + S_SPLIT];
     float* w = v.V + (long long)(*jd + 1) * v.N;
-    for (long long e = e0 + threadIdx.x; e < e1; e += kBT) {
-        const float x = v.W[e] * f;
-        w[e] = x;
-        split_bf16(x, v.ph[e], v.pl[e]);
+    for (long long e = e0 + 4 * threadIdx.x; e < e1; e += 4 * kBT) {
+        const float4 x = scaled4(v.W, e, f);
+        *reinterpret_cast<float4*>(w + e) = x;
+        split4(x, v.ph, v.pl, e);
     }
 }
 

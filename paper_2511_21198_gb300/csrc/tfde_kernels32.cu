@@ -748,7 +748,27 @@ __global__ void gm_scale_basis_kernel(long long N, const float* __restrict__ w, 
     if (gctl[1]) return;
     const float sc = (float)gs[GS_INV];
     float* out = V + (long long)gctl[0] * ldv;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+    const long long first = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    auto ptr = [](const void* p) { return reinterpret_cast<uintptr_t>(p); };
+    const bool vec = ((ptr(out) | ptr(w) | ptr(next)) & 15) == 0 && ((ptr(h) | ptr(l)) & 7) == 0;
+    const long long done = vec ? N / 4 * 4 : 0;
+    for (long long i = 4 * first; i < done; i += 4 * step) {
+        float4 v = *reinterpret_cast<const float4*>(w + i);
+        v = make_float4(v.x * sc, v.y * sc, v.z * sc, v.w * sc);
+        *reinterpret_cast<float4*>(out + i) = v;
+        if (next) {
+            *reinterpret_cast<float4*>(next + i) = v;
+        } else {
+            __align__(8) __nv_bfloat16 a[4], b[4];
+            split(v.x, a[0], b[0]);
+            split(v.y, a[1], b[1]);
+            split(v.z, a[2], b[2]);
+            split(v.w, a[3], b[3]);
+            *reinterpret_cast<uint2*>(h + i) = *reinterpret_cast<const uint2*>(a);
+            *reinterpret_cast<uint2*>(l + i) = *reinterpret_cast<const uint2*>(b);
+        }
+    }
+    for (long long i = done + first; i < N; i += step) {
         const float v = w[i] * sc;
         out[i] = v;
         if (next) next[i] = v;
@@ -776,18 +796,25 @@ __global__ void gm_start_kernel(double* gs, const double* part, int nblk, int* g
     gctl[3] = isfinite(beta) ? 0 : 1;
 }
 
-// -y (the least-squares solution R y = g over the steps done), zero beyond
-__global__ void gm_solve_kernel(const double* gs, const int* gctl, double* ny, int maxm) {
-    const int k = gctl[0];
-    const double* g = gs + GS_G;
+// -y (the least-squares solution R y = g over the steps done), zero beyond.
+// Thread r keeps row r's right-hand side; column i's entries are fetched while
+// the column before it is eliminated (one thread with a serial chain of global
+// loads took 5.6 us at 40 x 32 x 24 and 8.9 us at 128^3).
+__global__ void __launch_bounds__(GS_MAXM) gm_solve_kernel(const double* gs, const int* gctl, double* ny, int maxm) {
+    __shared__ double y;
+    const int k = gctl[0], r = threadIdx.x;
     const double* R = gs + GS_R;
-    double y[GS_MAXM];
+    double t = r < k ? gs[GS_G + r] : 0.0, out = 0.0;
+    double a = r < k ? R[(long long)(k - 1) * GS_LD + r] : 0.0;
     for (int i = k - 1; i >= 0; --i) {
-        double t = g[i];
-        for (int j = i + 1; j < k; ++j) t -= R[(long long)j * GS_LD + i] * y[j];
-        y[i] = t / R[(long long)i * GS_LD + i];
+        const double next = i > 0 && r < i ? R[(long long)(i - 1) * GS_LD + r] : 0.0;
+        if (r == i) y = out = t / a;
+        __syncthreads();
+        if (r < i) t -= a * y;
+        __syncthreads();
+        a = next;
     }
-    for (int i = 0; i < maxm; ++i) ny[i] = i < k ? -y[i] : 0.0;
+    if (r < maxm) ny[r] = -out;
 }
 
 void launch_gm_step(size_t N, const float* V, size_t ldv, float* w, double* part, int nblk, double* hbuf,
@@ -817,7 +844,7 @@ void launch_gm_start(size_t N, const float* w, double* part, int nblk, double* g
 }
 void launch_gm_solve(const double* gs, const int* gctl, double* ny, int maxm, cudaStream_t s) {
     stats_count_launch();
-    gm_solve_kernel<<<1, 1, 0, s>>>(gs, gctl, ny, maxm);
+    gm_solve_kernel<<<1, GS_MAXM, 0, s>>>(gs, gctl, ny, maxm);
 }
 
 namespace {
