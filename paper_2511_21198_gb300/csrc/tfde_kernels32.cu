@@ -9,6 +9,7 @@
 #include "tfde_stats.h"
 #include "tfde_gs.cuh"
 #include "tfde_mixed.h"
+#include "tfde_pdl.cuh"
 #include "tfde_pow2conv.cuh"
 
 namespace tfde {
@@ -632,8 +633,9 @@ __global__ void pcg_fold_dev_kernel(long long N4, CombineArgs a, float4* __restr
 // the first m = j + 1 inner products <V_i, w>, 8 basis vectors per sweep of w;
 // their sums into h
 __global__ __launch_bounds__(kT, 2) void gm_multidot_kernel(long long N, const float* __restrict__ V, long long ldv,
-                                                            const float* __restrict__ w, double* part, double* h,
+                                                            const float* w, double* part, double* h,
                                                             unsigned* ticket, const int* gctl) {
+    pdl_begin();
     if (gctl[1]) return;
     const int m = gctl[0] + 1;
     long long lo, hi;
@@ -649,8 +651,9 @@ __global__ __launch_bounds__(kT, 2) void gm_multidot_kernel(long long N, const f
 // update: w -= sum_{i <= j} h[i] V_i over the block's chunk, then the first
 // m = j + 1 inner products <V_i, w> of the updated chunk; their sums into h2.
 __global__ __launch_bounds__(kT, 2) void gm_axpy_dot_kernel(long long N, const float* __restrict__ V, long long ldv,
-                                                            const double* __restrict__ h, float* w, double* part,
+                                                            const double* h, float* w, double* part,
                                                             double* h2, unsigned* ticket, const int* gctl) {
+    pdl_begin();
     if (gctl[1]) return;
     const int m = gctl[0] + 1;
     __shared__ float hs[128];
@@ -681,9 +684,10 @@ __global__ __launch_bounds__(kT) void gm_dot_kernel(long long N, const float* a,
 // condition.  The rotations are a serial chain, so their operands are staged
 // in shared memory first.
 __global__ __launch_bounds__(kT) void gm_axpy_norm_kernel(long long N, const float* __restrict__ V, long long ldv,
-                                                          const double* __restrict__ h, const double* __restrict__ h2,
+                                                          const double* h, const double* h2,
                                                           float* w, double* part, unsigned* ticket, double* gs,
                                                           int* gctl, cudaGraphConditionalHandle hc) {
+    pdl_begin();
     if (gctl[1]) {   // the loop ends whenever its condition kernel runs on a finished cycle
         if (blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(hc, 0u);
         return;
@@ -716,17 +720,15 @@ __global__ __launch_bounds__(kT) void gm_axpy_norm_kernel(long long N, const flo
             R[i] = cs[i] * r + sn[i] * next;
             r = -sn[i] * r + cs[i] * next;
         }
-        const double den = hypot(r, hn);
-        const double c = den > 0.0 ? r / den : 1.0, q = den > 0.0 ? hn / den : 0.0;
+        const double den = sqrt(fma(r, r, hn * hn)), inv = 1.0 / den;   // r, hn at most the unit vector's image
+        const double c = den > 0.0 ? r * inv : 1.0, q = den > 0.0 ? hn * inv : 0.0;
         R[j] = den;
-        R[m] = 0.0;
         gs[GS_CS + j] = c;
         gs[GS_SN + j] = q;
         g[m] = -q * gj;
         g[j] = c * gj;
         const double est = fabs(q * gj);
         gs[GS_EST] = est;
-        gs[GS_INV] = 1.0 / hn;
         gctl[0] = m;
         int done = (est <= thr || hn == 0.0 || m >= maxsteps) ? 1 : 0;
         if (!isfinite(hn) || !isfinite(est)) {
@@ -735,16 +737,19 @@ __global__ __launch_bounds__(kT) void gm_axpy_norm_kernel(long long N, const flo
         }
         gctl[1] = done;
         cudaGraphSetConditional(hc, done ? 0u : 1u);
+    } else if (threadIdx.x == 32) {   // a warp of its own: the division runs beside the rotations
+        gs[GS_INV] = 1.0 / R[m];
     }
     __syncthreads();
-    for (int i = threadIdx.x; i <= m; i += blockDim.x) gs[GS_R + (long long)j * GS_LD + i] = R[i];
+    for (int i = threadIdx.x; i <= m; i += blockDim.x) gs[GS_R + (long long)j * GS_LD + i] = i < m ? R[i] : 0.0;
 }
 
 // V_j (j = the steps done) = w / ||w|| and the next operator input: its split
 // planes, or (next) a copy at a fixed address
-__global__ void gm_scale_basis_kernel(long long N, const float* __restrict__ w, float* V, long long ldv,
+__global__ void gm_scale_basis_kernel(long long N, const float* w, float* V, long long ldv,
                                       const double* gs, const int* gctl, __nv_bfloat16* __restrict__ h,
                                       __nv_bfloat16* __restrict__ l, float* __restrict__ next) {
+    pdl_begin();
     if (gctl[1]) return;
     const float sc = (float)gs[GS_INV];
     float* out = V + (long long)gctl[0] * ldv;
@@ -824,12 +829,13 @@ void launch_gm_step(size_t N, const float* V, size_t ldv, float* w, double* part
     const long long n = (long long)N, ld = (long long)ldv;
     nblk = dot_blocks(nblk);
     unsigned* ticket = reinterpret_cast<unsigned*>(gs + GS_TICKET);
+    const bool early = nblk <= kPdlBlocks;
     // CGS2: <V, w>; w -= V h and <V, w> again (one pass over the block's chunk);
     // w -= V h2 and ||w||^2 (one pass)
-    gm_multidot_kernel<<<nblk, kT, 0, s>>>(n, V, ld, w, part, hbuf, ticket, gctl);
-    gm_axpy_dot_kernel<<<nblk, kT, 0, s>>>(n, V, ld, hbuf, w, part, h2buf, ticket, gctl);
-    gm_axpy_norm_kernel<<<nblk, kT, 0, s>>>(n, V, ld, hbuf, h2buf, w, part, ticket, gs, gctl, hc);
-    gm_scale_basis_kernel<<<grid_for(n), kT, 0, s>>>(n, w, const_cast<float*>(V), ld, gs, gctl, ph, pl, next);
+    launch_pdl(early, gm_multidot_kernel, nblk, kT, s, n, V, ld, w, part, hbuf, ticket, gctl);
+    launch_pdl(early, gm_axpy_dot_kernel, nblk, kT, s, n, V, ld, hbuf, w, part, h2buf, ticket, gctl);
+    launch_pdl(early, gm_axpy_norm_kernel, nblk, kT, s, n, V, ld, hbuf, h2buf, w, part, ticket, gs, gctl, hc);
+    launch_pdl(early, gm_scale_basis_kernel, grid_for(n), kT, s, n, w, const_cast<float*>(V), ld, gs, gctl, ph, pl, next);
 }
 void launch_gm_start(size_t N, const float* w, double* part, int nblk, double* gs, int* gctl,
                      int maxsteps, double ptheta, float* V0, __nv_bfloat16* ph, __nv_bfloat16* pl, float* next,

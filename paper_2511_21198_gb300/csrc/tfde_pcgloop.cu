@@ -12,6 +12,7 @@
 #include "tfde_gs.cuh"
 #include "tfde_internal.h"
 #include "tfde_pcgloop.h"
+#include "tfde_pdl.cuh"
 #include "tfde_stats.h"
 
 namespace tfde {
@@ -55,6 +56,7 @@ __device__ __forceinline__ void block_range(long long N, long long& lo, long lon
 template <typename R>
 __global__ void __launch_bounds__(kT) dot_kernel(long long N, const R* a, const R* b, double* __restrict__ part,
                                                  const int* ctl) {
+    pdl_begin();
     if (ctl[cDone]) return;
     long long lo, hi;
     block_range<R>(N, lo, hi);
@@ -78,13 +80,15 @@ __global__ void __launch_bounds__(kT) dot_kernel(long long N, const R* a, const 
 }
 
 // <r, z> of the start
-__global__ void first_kernel(const double* __restrict__ part, int nblk, double* S) {
+__global__ void first_kernel(const double* part, int nblk, double* S) {
+    pdl_begin();
     const double t = warp_partials(part, nblk);
     if (threadIdx.x == 0) S[kRZ] = t;
 }
 
 // <p, A p>: alpha, or the end of the loop before anything is updated
-__global__ void alpha_kernel(const double* __restrict__ part, int nblk, double* S, int* ctl) {
+__global__ void alpha_kernel(const double* part, int nblk, double* S, int* ctl) {
+    pdl_begin();
     const double pq = warp_partials(part, nblk);
     if (threadIdx.x) return;
     S[kAlpha] = S[kRZ] / pq;
@@ -94,9 +98,10 @@ __global__ void alpha_kernel(const double* __restrict__ part, int nblk, double* 
 
 // x += alpha p; r -= alpha q; partial sums of r.r (FP64 products and sums)
 template <typename R>
-__global__ void __launch_bounds__(kT) update_kernel(long long N, const double* __restrict__ S, const R* __restrict__ p,
+__global__ void __launch_bounds__(kT) update_kernel(long long N, const double* S, const R* __restrict__ p,
                                                     const R* __restrict__ q, R* const* xp, R* __restrict__ r,
                                                     double* __restrict__ part, const int* ctl) {
+    pdl_begin();
     if (ctl[cBad]) return;
     R* __restrict__ x = *xp;
     const R alpha = (R)S[kAlpha];
@@ -141,8 +146,8 @@ __global__ void __launch_bounds__(kT) update_kernel(long long N, const double* _
 }
 
 // the stop test and the loop condition
-__global__ void stop_kernel(const double* __restrict__ part, int nblk, double* S, int* ctl,
-                            cudaGraphConditionalHandle h) {
+__global__ void stop_kernel(const double* part, int nblk, double* S, int* ctl, cudaGraphConditionalHandle h) {
+    pdl_begin();
     const double rr = warp_partials(part, nblk);
     if (threadIdx.x) return;
     int done = 1;
@@ -157,7 +162,8 @@ __global__ void stop_kernel(const double* __restrict__ part, int nblk, double* S
 }
 
 // <r, z>: beta
-__global__ void beta_kernel(const double* __restrict__ part, int nblk, double* S, const int* ctl) {
+__global__ void beta_kernel(const double* part, int nblk, double* S, const int* ctl) {
+    pdl_begin();
     if (ctl[cDone]) return;
     const double t = warp_partials(part, nblk);
     if (threadIdx.x) return;
@@ -167,8 +173,9 @@ __global__ void beta_kernel(const double* __restrict__ part, int nblk, double* S
 
 // p = z + beta p
 template <typename R>
-__global__ void __launch_bounds__(kT) direction_kernel(long long N, const double* __restrict__ S,
+__global__ void __launch_bounds__(kT) direction_kernel(long long N, const double* S,
                                                        const R* __restrict__ z, R* __restrict__ p, const int* ctl) {
+    pdl_begin();
     if (ctl[cDone]) return;
     const R beta = (R)S[kBeta];
     long long lo, hi;
@@ -225,6 +232,7 @@ int build(const tfde_problem* P, Loop* L, const PcgLoopVectors<R>& v, cudaStream
             return set_error(TFDE_ENOMEM, "allocation of the PCG loop's scalars failed");
     }
     const int nblk = dot_blocks(P->nblk);
+    const bool early = nblk <= kPdlBlocks;
     // once outside the capture: the passes' launch attributes are set on first use
     int st = fft::apply_A<R>(P, TFDE_OP_A, v.p, v.q, v.t[0], v.t[1], v.t[2], v.t[3], s);
     if (!st) st = fft::apply_Pinv<R>(P, v.r, v.z, v.t[0], v.t[2], s);
@@ -252,14 +260,14 @@ int build(const tfde_problem* P, Loop* L, const PcgLoopVectors<R>& v, cudaStream
         double* S = L->S;
         int* ctl = L->ctl();
         st = fft::apply_A<R>(P, TFDE_OP_A, v.p, v.q, v.t[0], v.t[1], v.t[2], v.t[3], c);
-        dot_kernel<R><<<nblk, kT, 0, c>>>(N, v.p, v.q, part, ctl);
-        alpha_kernel<<<1, 32, 0, c>>>(part, nblk, S, ctl);
-        update_kernel<R><<<nblk, kT, 0, c>>>(N, S, v.p, v.q, reinterpret_cast<R* const*>(L->xp()), v.r, part, ctl);
-        stop_kernel<<<1, 32, 0, c>>>(part, nblk, S, ctl, h);
+        launch_pdl(early, dot_kernel<R>, nblk, kT, c, N, v.p, v.q, part, ctl);
+        launch_pdl(early, alpha_kernel, 1, 32, c, part, nblk, S, ctl);
+        launch_pdl(early, update_kernel<R>, nblk, kT, c, N, S, v.p, v.q, reinterpret_cast<R* const*>(L->xp()), v.r, part, ctl);
+        launch_pdl(early, stop_kernel, 1, 32, c, part, nblk, S, ctl, h);
         if (!st) st = fft::apply_Pinv<R>(P, v.r, v.z, v.t[0], v.t[2], c, ctl + cDone);
-        dot_kernel<R><<<nblk, kT, 0, c>>>(N, v.r, v.z, part, ctl);
-        beta_kernel<<<1, 32, 0, c>>>(part, nblk, S, ctl);
-        direction_kernel<R><<<grid_for(P->N), kT, 0, c>>>(N, S, v.z, v.p, ctl);
+        launch_pdl(early, dot_kernel<R>, nblk, kT, c, N, v.r, v.z, part, ctl);
+        launch_pdl(early, beta_kernel, 1, 32, c, part, nblk, S, ctl);
+        launch_pdl(early, direction_kernel<R>, grid_for(P->N), kT, c, N, S, v.z, v.p, ctl);
         stats_set_capturing(false);
         cudaGraph_t out = nullptr;
         const cudaError_t e = cudaStreamEndCapture(c, &out);
