@@ -50,6 +50,7 @@
 #include <string>
 #include <vector>
 
+#include "tfde_pdl.cuh"
 #include "tfde_pow2conv.cuh"
 #include "tfde_internal.h"
 #include "tfde_stats.h"
@@ -170,6 +171,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 2) conv_kernel(const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    // the weights above were packed before the previous kernel began; the
+    // activations are its output
+    pdl_begin();
 
     if (warp == 0) {
         if (lane == 0) {
@@ -349,6 +353,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1) wgrad_kernel(const __grid_const
         mbar_fence_init();
     }
     __syncthreads();
+    pdl_begin();
     if (warp == WG_WARPS) {
         if (lane == 0) {
             int s = 0;
@@ -756,10 +761,10 @@ int conv(tfde_cnn* C, const uint8_t* in, const __nv_bfloat16* w, const float* bi
     const int grid = std::min(C->conv_tiles, 2 * tc::num_sms());
     const int smem = conv_smem(p.st);
     void* tok = stats_tc_begin(s, TFDE_KIND_CONV);
-    if (p.st.nt == 4) conv_kernel<4><<<grid, NUM_THREADS, smem, s>>>(p);
-    else if (p.st.nt == 2) conv_kernel<2><<<grid, NUM_THREADS, smem, s>>>(p);
-    else conv_kernel<1><<<grid, NUM_THREADS, smem, s>>>(p);
-    cudaError_t e = cudaGetLastError();
+    // launched early: a block's set-up (weights, barriers, TMEM) runs as soon as
+    // one of the previous kernel's blocks leaves its SM
+    auto* kernel = p.st.nt == 4 ? conv_kernel<4> : (p.st.nt == 2 ? conv_kernel<2> : conv_kernel<1>);
+    const cudaError_t e = launch_pdl_smem(true, kernel, grid, NUM_THREADS, smem, s, p);
     // algorithmic: the input activations read once, the output written once
     stats_tc_end(tok, s, TFDE_KIND_CONV, 64.0 * (double)C->N, 2.0 * NTAP * CH * CH * (double)C->N);
     if (e != cudaSuccess) return set_error(TFDE_ECUDA, std::string("conv_kernel launch: ") + cudaGetErrorString(e));
@@ -780,8 +785,7 @@ int wgrad(tfde_cnn* C, int layer, const uint8_t* dz, cudaStream_t s) {
     p.part = C->wpart + (size_t)layer * C->wg_grid * GSZ;
     p.err = C->err;
     stats_count_launch();
-    wgrad_kernel<<<C->wg_grid, WG_THREADS, wg_smem(p.st), s>>>(p);
-    CN_TRY(cudaGetLastError());
+    CN_TRY(launch_pdl_smem(true, wgrad_kernel, C->wg_grid, WG_THREADS, wg_smem(p.st), s, p));
     return TFDE_OK;
 }
 

@@ -24,17 +24,23 @@ __device__ __forceinline__ void pdl_begin() {
 constexpr int kPdlBlocks = 152;   // of a sweep over the grid's points: one per SM
 
 template <typename... P, typename... A>
-inline void launch_pdl(bool early, void (*kernel)(P...), int grid, int block, cudaStream_t s, A&&... args) {
+inline cudaError_t launch_pdl_smem(bool early, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s,
+                                   A&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = early ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, kernel, P(std::forward<A>(args))...);
+    return cudaLaunchKernelEx(&cfg, kernel, P(std::forward<A>(args))...);
+}
+template <typename... P, typename... A>
+inline void launch_pdl(bool early, void (*kernel)(P...), int grid, int block, cudaStream_t s, A&&... args) {
+    launch_pdl_smem(early, kernel, grid, block, 0, s, std::forward<A>(args)...);
 }
 
 }  // namespace tfde
