@@ -32,12 +32,14 @@
 // because the ring holds planes (one dz of a tile, four of them) instead of
 // whole tiles.  Measured on GB300 at 128^3: 107 us per layer with one CTA and
 // two whole tiles, 75 us with two CTAs (162 us with nine 16-byte-row tensor
-// copies per 128 slots).
+// copies per 128 slots).  Nine MMAs per 128 slots with the three dx taps side by
+// side (N = 48, added up from neighbouring rows in the epilogue) took 85 us: the
+// epilogue then reads three times the columns.
 //
 // Weight gradients: per tap a 16 x 16 matrix summed over all slots, on
 // mma.sync m16n8k16 (tcgen05's smallest M of 64 would leave three quarters of
 // the rows empty); the same staged runs as the convolution serve all 27 taps.
-// One optimiser step of eight 64^3 samples: 2.6 ms, against 25.7 ms with the
+// One optimiser step of eight 64^3 samples: 2.3 ms, against 25.7 ms with the
 // nine-copy convolution, a CUDA-core weight gradient per tap and 256-slot
 // chunk (477 us per layer, 160 us for the sum of its partials), a one-block
 // max |u| (183 us) and a 16-block bias sum (41 us).
@@ -762,7 +764,8 @@ int conv(tfde_cnn* C, const uint8_t* in, const __nv_bfloat16* w, const float* bi
     const int smem = conv_smem(p.st);
     void* tok = stats_tc_begin(s, TFDE_KIND_CONV);
     // launched early: a block's set-up (weights, barriers, TMEM) runs as soon as
-    // one of the previous kernel's blocks leaves its SM
+    // one of the previous kernel's blocks leaves its SM (with the weight gradient's:
+    // one optimiser step of eight 64^3 samples 2.56 -> 2.28 ms)
     auto* kernel = p.st.nt == 4 ? conv_kernel<4> : (p.st.nt == 2 ? conv_kernel<2> : conv_kernel<1>);
     const cudaError_t e = launch_pdl_smem(true, kernel, grid, NUM_THREADS, smem, s, p);
     // algorithmic: the input activations read once, the output written once
