@@ -32,9 +32,9 @@
 // because the ring holds planes (one dz of a tile, four of them) instead of
 // whole tiles.  Measured on GB300 at 128^3: 107 us per layer with one CTA and
 // two whole tiles, 75 us with two CTAs (162 us with nine 16-byte-row tensor
-// copies per 128 slots).  Nine MMAs per 128 slots with the three dx taps side by
-// side (N = 48, added up from neighbouring rows in the epilogue) took 85 us: the
-// epilogue then reads three times the columns.
+// copies per 128 slots); the tcgen05 pipe is then 83 % active (96^3).  Nine MMAs
+// per 128 slots with the three dx taps side by side (N = 48, added up from
+// neighbouring rows in the epilogue) took 85 us.
 //
 // Weight gradients: per tap a 16 x 16 matrix summed over all slots, on
 // mma.sync m16n8k16 (tcgen05's smallest M of 64 would leave three quarters of
