@@ -792,7 +792,10 @@ int launch_line(const LinePass& p, cudaStream_t s) {
 
 // Lines per block: FP32 64, 32 or 16 (8 rows x 4, 2 or 1 lines per thread),
 // the largest that fits and still gives every SM two blocks, so that one's
-// copies run under the other's product; FP64, bound by its pipe (two
+// copies run under the other's product, or 8 (4 rows x 1) where blocks of 16
+// would leave half of the SMs idle (4 steps: 255^2 6.79 -> 6.10 ms, 100 x 90 4.72 ->
+// 4.39, 15 x 16 x 17 3.23 -> 3.04; with 128 blocks of 16 the doubled matrix
+// traffic costs more: 511^2 11.9 against 13.7 ms); FP64, bound by its pipe (two
 // multiply-adds per clock and SM), 8 (4 rows x 1 line per thread), or 4 (2 x 1)
 // where the SMs would get few blocks of 8: the fullest one decides (4096 lines
 // are 3.4 blocks of 8 per SM, 6.7 of 4; preconditioner at 64^3 140 -> 119 us).
@@ -808,6 +811,8 @@ int line_pass(const LinePass& p, cudaStream_t s) {
         };
         if (takes(64)) return launch_line<R, MODE, 16, 4, 8>(p, s);
         if (takes(32)) return launch_line<R, MODE, 16, 2, 8>(p, s);
+        const long long blocks = (p.lines + 15) / 16 * ((p.m.ld + LINE_ROWS - 1) / LINE_ROWS);
+        if (2 * blocks <= tc::num_sms()) return launch_line<R, MODE, 8, 1, 4>(p, s);
         return launch_line<R, MODE, 16, 1, 8>(p, s);
     } else {
         const long long blocks = (p.lines + 7) / 8 * ((p.m.ld + LINE_ROWS - 1) / LINE_ROWS);
