@@ -293,6 +293,7 @@ int assemble_problem(const tfde_params* params, int precision, cudaStream_t s, t
     if (cudaMallocHost((void**)&P->red_host, 256 * sizeof(double)) != cudaSuccess)
         return fail(set_error(TFDE_ENOMEM, "cudaMallocHost failed"));
     if ((st = fft::init(P, s))) return fail(st);
+    if (precision == TFDE_FP64 && P->symmetric && P->fft && (st = pcg_loop_reserve<double>(P))) return fail(st);
     if (P->dim2 && !P->fft) return fail(set_error(TFDE_EUNSUPPORTED, "2-D problems need n_a <= 2048"));
     if (precision == TFDE_MIXED) {
         // the tensor-core contraction where the grid suits it, else FP32 FFT

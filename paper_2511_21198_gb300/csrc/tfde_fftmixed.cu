@@ -261,7 +261,6 @@ int build_cycle(const tfde_problem* P, int m, cudaStream_t s) {
         F->gm_exec = nullptr;
         F->gm_graph = nullptr;
     }
-    if (!F->gm_state) FM_TRY(cudaMalloc((void**)&F->gm_state, GS_WORDS * sizeof(double) + 4 * sizeof(int)));
     // once outside the capture: the passes' launch attributes are set on first use
     int st = op_A32(P, F->v[V_P], F->v[V_Q], s);
     if (!st) st = op_Pinv32(P, F->v[V_Q], F->v[V_Z], s);
@@ -472,6 +471,10 @@ int fmix_init(tfde_problem* P, cudaStream_t s) {
     FM_TRY(cudaMalloc((void**)&F->d, NS * sizeof(double)));
     FM_TRY(cudaMemsetAsync(F->d, 0, NS * sizeof(double), s));
     FM_TRY(cudaMallocHost((void**)&F->h, NS * sizeof(double)));
+    // the device-side loops' state
+    FM_TRY(cudaMalloc((void**)&F->gm_state, GS_WORDS * sizeof(double) + 4 * sizeof(int)));
+    if (P->symmetric)
+        if (int st = pcg_loop_reserve<float>(P)) return st;
     // the basis of the default restart length (20) up front, larger ones on demand
     return ensure_basis(P, 20);
 }

@@ -223,14 +223,34 @@ int grid_for(size_t N) {
     return (int)(g > 304 * 4 ? 304 * 4 : (g < 1 ? 1 : g));
 }
 
+void release(Loop* L) {
+    if (L->exec) cudaGraphExecDestroy(L->exec);
+    if (L->graph) cudaGraphDestroy(L->graph);
+    cudaFree(L->S);
+    if (L->host) cudaFreeHost(L->host);
+    delete L;
+}
+
+// The problem's loop with both of its buffers, or null (no memory for them).
+template <typename R>
+Loop* loop_of(const tfde_problem* P) {
+    void*& slot = P->pcg_loop[sizeof(R) == 8 ? 0 : 1];
+    if (!slot) {
+        Loop* L = new Loop();
+        if (cudaMalloc((void**)&L->S, kWords * sizeof(double)) != cudaSuccess ||
+            cudaMallocHost((void**)&L->host, kWords * sizeof(double)) != cudaSuccess) {
+            cudaGetLastError();
+            release(L);
+            return nullptr;
+        }
+        slot = L;
+    }
+    return static_cast<Loop*>(slot);
+}
+
 template <typename R>
 int build(const tfde_problem* P, Loop* L, const PcgLoopVectors<R>& v, cudaStream_t s) {
     if (L->exec || L->failed) return TFDE_OK;
-    if (!L->S) {
-        if (cudaMalloc((void**)&L->S, kWords * sizeof(double)) != cudaSuccess ||
-            cudaMallocHost((void**)&L->host, kWords * sizeof(double)) != cudaSuccess)
-            return set_error(TFDE_ENOMEM, "allocation of the PCG loop's scalars failed");
-    }
     const int nblk = dot_blocks(P->nblk);
     const bool early = nblk <= kPdlBlocks;
     // once outside the capture: the passes' launch attributes are set on first use
@@ -288,12 +308,19 @@ int build(const tfde_problem* P, Loop* L, const PcgLoopVectors<R>& v, cudaStream
 }  // namespace
 
 template <typename R>
+int pcg_loop_reserve(const tfde_problem* P) {
+    return loop_of<R>(P) ? TFDE_OK : set_error(TFDE_ENOMEM, "allocation of the PCG loop's scalars failed");
+}
+template int pcg_loop_reserve<double>(const tfde_problem*);
+template int pcg_loop_reserve<float>(const tfde_problem*);
+
+template <typename R>
 int pcg_loop(const tfde_problem* P, const PcgLoopVectors<R>& v, R* x, double thr, int maxit, PcgLoopResult* res,
              cudaStream_t s) {
     res->ran = false;
     if (!P->fft || stats_timing() || maxit < 1) return TFDE_OK;
-    Loop*& L = reinterpret_cast<Loop*&>(P->pcg_loop[sizeof(R) == 8 ? 0 : 1]);
-    if (!L) L = new Loop();
+    Loop* L = loop_of<R>(P);   // there since assembly, but for a mixed solve's FP64 fallback
+    if (!L) return TFDE_OK;
     if (int st = build<R>(P, L, v, s)) return st;
     if (!L->exec) return TFDE_OK;
     const int nblk = dot_blocks(P->nblk);
@@ -323,13 +350,7 @@ template int pcg_loop<float>(const tfde_problem*, const PcgLoopVectors<float>&, 
 
 void pcg_loop_free(tfde_problem* P) {
     for (void*& slot : P->pcg_loop) {
-        Loop* L = static_cast<Loop*>(slot);
-        if (!L) continue;
-        if (L->exec) cudaGraphExecDestroy(L->exec);
-        if (L->graph) cudaGraphDestroy(L->graph);
-        cudaFree(L->S);
-        if (L->host) cudaFreeHost(L->host);
-        delete L;
+        if (slot) release(static_cast<Loop*>(slot));
         slot = nullptr;
     }
 }

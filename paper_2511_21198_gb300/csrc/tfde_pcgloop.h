@@ -16,11 +16,14 @@ struct PcgLoopVectors {
 // updated) or not positive (nothing updated), <r, r> not finite
 enum { PCGLOOP_OK = 0, PCGLOOP_NAN_PAP = 1, PCGLOOP_BREAKDOWN = 2, PCGLOOP_NAN_RR = 3 };
 struct PcgLoopResult {
-    bool ran = false;   // false: no graph (the caller iterates from the host)
+    bool ran = false;   // false: no graph or no memory (the caller iterates from the host)
     int iters = 0, bad = PCGLOOP_OK;
     double rr = 0.0;    // <r, r> of the recursive residual
 };
 
+// Allocates the loop's scalars (assembly of a problem whose solves take it).
+template <typename R>
+int pcg_loop_reserve(const tfde_problem* P);
 // PCG on A x = b from the residual in v.r (p = P^{-1} r first) until <r, r> <=
 // thr or maxit iterations; x is updated in place.  One host read.
 template <typename R>

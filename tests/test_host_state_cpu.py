@@ -1,0 +1,31 @@
+"""The library's host-side bookkeeping without a GPU: its objects linked with a
+runtime whose device memory is host memory and whose kernels do nothing
+(native/fake_cudart.cpp), so that allocations can be counted and made to fail."""
+import glob
+import os
+import shutil
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+NATIVE = os.path.join(HERE, "native")
+
+
+def run_check(name, tmp_path):
+    if shutil.which("g++") is None:
+        pytest.skip("no host C++ compiler")
+    from paper_2511_21198_gb300 import build
+    build.build()
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc_path()))), "include")
+    exe = str(tmp_path / name)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-I", NATIVE, "-I", build.CSRC, "-I", os.path.join(ROOT, "include"),
+                    "-isystem", cuda, os.path.join(NATIVE, name + ".cpp"), os.path.join(NATIVE, "fake_cudart.cpp"),
+                    *sorted(glob.glob(os.path.join(build.BUILD_DIR, "*.o"))), "-o", exe], check=True)
+    out = subprocess.run([exe], capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stdout + out.stderr
+
+
+def test_loop_buffers(tmp_path):
+    run_check("loop_buffers_check", tmp_path)
