@@ -184,11 +184,12 @@ int validate_params(const tfde_params* p) {
     return TFDE_OK;
 }
 
-int mixed_init(tfde_problem* P, cudaStream_t s);   // tfde_mixed.cu
+int mixed_init(tfde_problem* P, cudaStream_t s, const int* bn);   // tfde_mixed.cu
 void mixed_free(tfde_problem* P);
 int destroy_problem(tfde_problem* P);
 
-int assemble_problem(const tfde_params* params, int precision, cudaStream_t s, tfde_problem** out) {
+// bn: lines per tile of the split contraction along each axis, or null
+int assemble_tiled(const tfde_params* params, int precision, const int* bn, cudaStream_t s, tfde_problem** out) {
     *out = nullptr;
     int st = validate_params(params);
     if (st) return st;
@@ -298,11 +299,15 @@ int assemble_problem(const tfde_params* params, int precision, cudaStream_t s, t
     if (precision == TFDE_MIXED) {
         // the tensor-core contraction where the grid suits it, else FP32 FFT
         // inner solves under the same FP64 refinement
-        if ((st = fmix_wanted(P) ? fmix_init(P, s) : mixed_init(P, s))) return fail(st);
+        if ((st = fmix_wanted(P) ? fmix_init(P, s) : mixed_init(P, s, bn))) return fail(st);
     }
     if (cudaStreamSynchronize(s) != cudaSuccess) return fail(set_error(TFDE_ECUDA, "assemble: stream sync failed"));
     *out = P;
     return TFDE_OK;
+}
+
+int assemble_problem(const tfde_params* params, int precision, cudaStream_t s, tfde_problem** out) {
+    return assemble_tiled(params, precision, nullptr, s, out);
 }
 
 int host_coefficients(const tfde_params* params, int axis, double* q, double* lam_tau, double* lam_mass,

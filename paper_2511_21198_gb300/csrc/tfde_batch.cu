@@ -25,7 +25,7 @@
 
 namespace tfde {
 
-int assemble_problem(const tfde_params* params, int precision, cudaStream_t s, tfde_problem** out);
+int assemble_tiled(const tfde_params* params, int precision, const int* bn, cudaStream_t s, tfde_problem** out);
 int destroy_problem(tfde_problem* P);
 int cn_prepare(tfde_problem* P, const double* u_prev, const double* F, const double* x0, double* u_next,
                cudaStream_t s, bool chained, bool* r_given, const double* guess, int* used_guess);
@@ -1291,9 +1291,16 @@ int batch_create(const tfde_params* params, int count, int restart, cudaStream_t
         free_batch(B);
         return set_error(TFDE_ENOMEM, "allocation of the batch error flag failed");
     }
+    // one tile width per axis for the grouped launches (and the problems' own)
+    for (int a = 0; a < 3; ++a) {
+        long long wide = 0;
+        for (int k = 0; k < count; ++k)
+            if (sz(k) > 0) wide += tc::wide_tiles(params[k].n, a);   // others are refused below
+        B->bn[a] = tc::tile_lines(wide);
+    }
     for (int k = 0; k < count; ++k) {
         tfde_problem* P = nullptr;
-        if ((st = assemble_problem(&params[idx[k]], TFDE_MIXED, s, &P))) {
+        if ((st = assemble_tiled(&params[idx[k]], TFDE_MIXED, B->bn, s, &P))) {
             free_batch(B);
             return st;
         }
@@ -1314,17 +1321,6 @@ int batch_create(const tfde_params* params, int count, int restart, cudaStream_t
         free_batch(B);
         return set_error(code, what);
     };
-    // one tile width per axis for the grouped launches (and the problems' own)
-    for (int a = 0; a < 3; ++a) {
-        long long wide = 0;
-        for (tfde_problem* P : B->P) wide += tc::wide_tiles(P->n, a);
-        B->bn[a] = tc::tile_lines(wide);
-    }
-    for (tfde_problem* P : B->P)
-        if ((st = mixed_set_tiles(P, B->bn))) {
-            free_batch(B);
-            return st;
-        }
     // grouped descriptors
     const size_t C = count, PS = sizeof(tc::Params);
     std::vector<tc::Params> mv(5 * C), pc(5 * C), pcl((size_t)(restart + 1) * C);

@@ -1277,22 +1277,6 @@ int spec_pass_descriptors(const tfde_problem* P, int kind, float* out_f32, tc::P
     return 3;
 }
 
-// The lines per tile along each axis, and the input maps whose boxes follow
-// them (before any pass or graph of the problem uses them).
-int mixed_set_tiles(const tfde_problem* P, const int bn[3]) {
-    MixedState* M = mixed(P);
-    for (int a = 0; a < 3; ++a) M->bn[a] = bn[a];
-    for (int pl = 0; pl < NPL; ++pl)
-        for (int a = 0; a < 3; ++a) {
-            int st = tc::make_map_B(&M->bmap_hi[pl][a], M->hi[pl], P->n, a, bn[a]);
-            if (!st) st = tc::make_map_B(&M->bmap_lo[pl][a], M->lo[pl], P->n, a, bn[a]);
-            if (st) return st;
-            M->bmap2_rank[pl][a] = tc::make_map_B_pair(&M->bmap2[pl][a], M->hi[pl], P->n, a, bn[a]);
-            M->bmap1_rank[pl][a] = tc::make_map_B_pair(&M->bmap1[pl][a], M->hi[pl], P->n, a, bn[a], 1);
-        }
-    return TFDE_OK;
-}
-
 int mixed_prepare_gmres(const tfde_problem* P, int restart) { return ensure_v32(P, restart); }
 
 namespace {
@@ -1323,7 +1307,10 @@ int upload_matrix(MixedState* M, int om, const std::vector<__nv_bfloat16>& h, in
 }
 }  // namespace
 
-int mixed_init(tfde_problem* P, cudaStream_t s) {
+// bn: the lines per tile along each axis (a batch's), or null for the problem's
+// own choice.  They are final here: the input maps' boxes, the grouped
+// descriptors and the graphs all follow them.
+int mixed_init(tfde_problem* P, cudaStream_t s, const int* bn) {
     for (int a = 0; a < 3; ++a)
     {
         if (P->n[a] % 8 != 0)
@@ -1415,6 +1402,7 @@ int mixed_init(tfde_problem* P, cudaStream_t s) {
         if (st) return st;
     }
     // workspace planes and their tensor maps
+    for (int a = 0; a < 3; ++a) M->bn[a] = bn ? bn[a] : tc::tile_lines(tc::wide_tiles(P->n, a));
     for (int pl = 0; pl < NPL; ++pl) {
         MX_TRY(cudaMalloc((void**)&M->hi[pl], 2 * N * sizeof(__nv_bfloat16)));
         M->lo[pl] = M->hi[pl] + N;
@@ -1422,14 +1410,13 @@ int mixed_init(tfde_problem* P, cudaStream_t s) {
         for (int a = 0; a < 3; ++a) {
             int st;
             if ((st = tc::make_out_map(&M->omap_hi[pl][a], M->hi[pl], P->n, a, false)) ||
-                (st = tc::make_out_map_pair(&M->omap_hl[pl][a], M->hi[pl], P->n, a)))
+                (st = tc::make_out_map_pair(&M->omap_hl[pl][a], M->hi[pl], P->n, a)) ||
+                (st = tc::make_map_B(&M->bmap_hi[pl][a], M->hi[pl], P->n, a, M->bn[a])) ||
+                (st = tc::make_map_B(&M->bmap_lo[pl][a], M->lo[pl], P->n, a, M->bn[a])))
                 return st;
+            M->bmap2_rank[pl][a] = tc::make_map_B_pair(&M->bmap2[pl][a], M->hi[pl], P->n, a, M->bn[a]);
+            M->bmap1_rank[pl][a] = tc::make_map_B_pair(&M->bmap1[pl][a], M->hi[pl], P->n, a, M->bn[a], 1);
         }
-    }
-    {
-        int bn[3];
-        for (int a = 0; a < 3; ++a) bn[a] = tc::tile_lines(tc::wide_tiles(P->n, a));
-        if (int st = mixed_set_tiles(P, bn)) return st;
     }
     for (int v = 0; v < NF; ++v) {
         MX_TRY(cudaMalloc((void**)&M->f[v], N * sizeof(float)));

@@ -241,7 +241,6 @@ int spec_pass_descriptors(const tfde_problem* P, int kind, float* out_f32, tc::P
                           double* flops, const float* dot_vec = nullptr, double* dot_out = nullptr);
 // Allocate the FP32 GMRES basis (restart + 1 vectors) and Hessenberg scratch.
 int mixed_prepare_gmres(const tfde_problem* P, int restart);
-int mixed_set_tiles(const tfde_problem* P, const int bn[3]);
 
 int oz_init(tfde_problem* P, const std::vector<double> etaB[3], cudaStream_t s);
 void oz_free(MixedState* M);

@@ -135,6 +135,7 @@ cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** fn, unsigned, u
 void** __cudaRegisterFatBinary(void*) { return reinterpret_cast<void**>(handle_storage); }
 void __cudaRegisterFatBinaryEnd(void**) {}
 void __cudaUnregisterFatBinary(void**) {}
+char __cudaInitModule(void**) { return 1; }
 void __cudaRegisterFunction(void**, const char*, char*, const char*, int, void*, void*, void*, void*, int*) {}
 void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
 cudaError_t __cudaGetKernel(cudaKernel_t* k, const void*) { return handle(k); }
