@@ -7,15 +7,17 @@
 // thread.  The other cost is the block reduction: FP64 adds issue at two lanes
 // per clock and SM, and a shuffle tree per result (40 warp-wide adds for eight)
 // took longer than the sweep at 128^3 (31 us per launch against 7).  The eight
-// results share one tree (9 warp-wide adds), and the compensated FP32 sums go
-// through it as pairs of FP32 values (two-sum, relative error 2^-45 per add):
-// their conversions to FP64 alone were 6000 lane operations per block.  The
-// partial sums over the blocks are added by the last block of the sweep, which
-// spares a launch each.  Both together: projection sweep of 64 uneven problems
-// 167 -> 84 us, at 128^3 14.6 -> 11.1 us.
+// results share one tree (9 warp-wide adds and 3 across the warps), and the
+// compensated FP32 sums go through it as three FP32 values (tfde_sum3.cuh, more
+// accurate than FP64): their conversions to FP64 alone were 6000 lane operations
+// per block.  The partial sums over the blocks are added by the last block of the
+// sweep, which spares a launch each.  Both together: projection sweep of 64 uneven
+// problems 167 -> 84 us, at 128^3 14.6 -> 11.1 us.
 #pragma once
 
 #include <cuda_runtime.h>
+
+#include "tfde_sum3.cuh"
 
 namespace tfde {
 namespace gs {
@@ -23,24 +25,15 @@ namespace gs {
 constexpr int kThreads = 256;
 constexpr int kWidth = 8;   // basis vectors per sweep
 
-// An unevaluated sum hi + lo of FP32 values, |lo| far below |hi|.
-struct Pair {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void operator+=(const Pair o) {
-        const float h = hi + o.hi, b = h - hi;   // Knuth's two-sum of the leading parts
-        lo += ((hi - (h - b)) + (o.hi - b)) + o.lo;
-        hi = h;
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-__device__ __forceinline__ Pair shfl_xor(const Pair v, int off) {
-    Pair o;
+__device__ __forceinline__ Sum3 shfl_xor(const Sum3 v, int off) {
+    Sum3 o;
     o.hi = __shfl_xor_sync(0xffffffffu, v.hi, off);
+    o.mid = __shfl_xor_sync(0xffffffffu, v.mid, off);
     o.lo = __shfl_xor_sync(0xffffffffu, v.lo, off);
     return o;
 }
 __device__ __forceinline__ double shfl_xor(double v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
-__device__ __forceinline__ double value_of(const Pair v) { return v.value(); }
+__device__ __forceinline__ double value_of(const Sum3 v) { return v.value(); }
 __device__ __forceinline__ double value_of(double v) { return v; }
 
 // Kahan-compensated FP32 accumulation.
@@ -53,11 +46,11 @@ struct KSum {
         s = t;
     }
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
-    __device__ __forceinline__ Pair pair() const {
-        Pair p;
-        p.hi = s;
-        p.lo = -c;
-        return p;
+    __device__ __forceinline__ Sum3 sum3() const {
+        Sum3 t;
+        t.hi = s;
+        t.mid = -c;
+        return t;
     }
 };
 __device__ __forceinline__ void add4(KSum& k, const float4 a, const float4 b) {
@@ -73,12 +66,13 @@ __device__ __forceinline__ void axpy4(float4& w, float h, const float4 v) {
     w.w = fmaf(-h, v.w, w.w);
 }
 
-// Block sums of eight values (double or Pair) per thread, result j < mc handed
+// Block sums of eight values (double or Sum3) per thread, result j < mc handed
 // to f(j, sum) by one thread.  Each exchange over the lanes halves the values a lane carries,
 // so the warp needs 4 + 2 + 1 + 1 + 1 adds; fixed order.  Every thread of the
 // (kThreads-wide) block calls it.
 template <typename T, typename F>
 __device__ __forceinline__ void block_sums8(T (&v)[kWidth], int mc, F f) {
+    static_assert(kThreads == 256 && kWidth == 8, "eight warps' sums of eight values");
     __shared__ T sh[kWidth][kThreads / 32 + 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -98,35 +92,36 @@ __device__ __forceinline__ void block_sums8(T (&v)[kWidth], int mc, F f) {
     __syncthreads();   // the previous call's reads of sh are done
     if ((lane & 3) == 0) sh[lane >> 2][warp] = v[0];   // lane bits 4..2 are the value's index
     __syncthreads();
-    if (threadIdx.x < mc) {
-        double t = 0.0;
-#pragma unroll
-        for (int w = 0; w < kThreads / 32; ++w) t += value_of(sh[threadIdx.x][w]);
-        f((int)threadIdx.x, t);
+    if (warp == 0) {   // four lanes per value, two warps' sums each
+        T t = sh[lane >> 2][lane & 3];
+        t += sh[lane >> 2][(lane & 3) + 4];
+        t += shfl_xor(t, 2);
+        t += shfl_xor(t, 1);
+        if ((lane & 3) == 0 && lane >> 2 < mc) f(lane >> 2, value_of(t));
     }
 }
 template <typename F>
 __device__ __forceinline__ void block_sums8(KSum (&k)[kWidth], int mc, F f) {
-    Pair v[kWidth];
+    Sum3 v[kWidth];
 #pragma unroll
-    for (int j = 0; j < kWidth; ++j) v[j] = k[j].pair();
+    for (int j = 0; j < kWidth; ++j) v[j] = k[j].sum3();
     block_sums8(v, mc, f);
 }
 // the same for one value per thread
 template <typename F>
 __device__ __forceinline__ void block_sum1(const KSum& k, F f) {
-    __shared__ Pair sh[kThreads / 32];
-    Pair v = k.pair();
+    __shared__ Sum3 sh[kThreads / 32];
+    Sum3 v = k.sum3();
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += shfl_xor(v, off);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
+    if (threadIdx.x < 32) {
+        v = sh[threadIdx.x & 7];
 #pragma unroll
-        for (int w = 0; w < kThreads / 32; ++w) t += sh[w].value();
-        f(t);
+        for (int off = 4; off > 0; off >>= 1) v += shfl_xor(v, off);
+        if (threadIdx.x == 0) f(v.value());
     }
 }
 
