@@ -21,6 +21,7 @@
 #include "tfde_mixed.h"
 #include "tfde_stats.h"
 #include "tfde_chain.cuh"
+#include "tfde_givens.h"
 #include "tfde_gs.cuh"
 
 namespace tfde {
@@ -552,10 +553,7 @@ __device__ __forceinline__ void givens_step(int i, int R, int j, double* __restr
         Rm[(q + 1) * R + j] = -sn[q] * Rm[q * R + j] + cs[q] * Rm[(q + 1) * R + j];
         Rm[q * R + j] = t;
     }
-    const double den = hypot(Rm[j * R + j], Rm[(j + 1) * R + j]);
-    cs[j] = den > 0.0 ? Rm[j * R + j] / den : 1.0;
-    sn[j] = den > 0.0 ? Rm[(j + 1) * R + j] / den : 0.0;
-    Rm[j * R + j] = den;
+    givens_rotation(Rm[j * R + j], Rm[(j + 1) * R + j], &cs[j], &sn[j], &Rm[j * R + j]);
     Rm[(j + 1) * R + j] = 0.0;
     g[j + 1] = -sn[j] * g[j];
     g[j] = cs[j] * g[j];

@@ -7,6 +7,7 @@
 
 #include "tfde_internal.h"
 #include "tfde_stats.h"
+#include "tfde_givens.h"
 #include "tfde_gs.cuh"
 #include "tfde_mixed.h"
 #include "tfde_pdl.cuh"
@@ -720,9 +721,8 @@ __global__ __launch_bounds__(kT) void gm_axpy_norm_kernel(long long N, const flo
             R[i] = cs[i] * r + sn[i] * next;
             r = -sn[i] * r + cs[i] * next;
         }
-        const double den = sqrt(fma(r, r, hn * hn)), inv = 1.0 / den;   // r, hn at most the unit vector's image
-        const double c = den > 0.0 ? r * inv : 1.0, q = den > 0.0 ? hn * inv : 0.0;
-        R[j] = den;
+        double c, q;
+        givens_rotation(r, hn, &c, &q, &R[j]);
         gs[GS_CS + j] = c;
         gs[GS_SN + j] = q;
         g[m] = -q * gj;
