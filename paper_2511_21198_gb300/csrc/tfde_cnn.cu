@@ -54,6 +54,7 @@
 
 #include "tfde_pdl.cuh"
 #include "tfde_pow2conv.cuh"
+#include "tfde_sum3.cuh"
 #include "tfde_internal.h"
 #include "tfde_stats.h"
 #include "tfde_tc.h"
@@ -78,8 +79,9 @@ constexpr int NUM_THREADS = 32 * (2 + EPI_WARPS);
 constexpr int MAX_SMEM = 232448;
 constexpr int CONV_FIXED_SMEM = 128 + W_BYTES + NUM_BARS * 8 + 16;
 constexpr int WG_ROWS = 9;         // weight gradient: one warp per (dz, dy) ...
-constexpr int WG_SETS = 2;         // ... and half of a tile's blocks of 128 slots
-constexpr int WG_WARPS = WG_ROWS * WG_SETS;
+constexpr int WG_HALVES = 2;       // ... and half of the input channels
+constexpr int WG_WARPS = WG_ROWS * WG_HALVES;
+constexpr int WG_CLOSE = 2;        // blocks of 128 slots that a warp sums in FP32
 constexpr int WG_THREADS = 32 * (WG_WARPS + 1);   // + the copy warp
 constexpr int WG_SMEM_FIXED = 128 + 2 * STAGES * 8 + 16;
 constexpr int GSZ = NTAP * 256 + CH;              // one partial: [tap][co][ci], then the bias
@@ -304,22 +306,17 @@ struct WgradParams {
     unsigned R;
     long long P, first;
     int ntiles;
-    float2* part;                  // [gridDim.x][GSZ]: sums as pairs of FP32 values
+    float* part;                   // [gridDim.x][3][GSZ]: the parts of the sums
     int* err;
 };
 
-// (hi, lo) += (v, w): Knuth's two-sum of the leading parts, its error and the
-// trailing parts collected in lo.  (FP64 converts and adds at two lanes per
-// clock and SM: closing the sums in FP64 took longer than forming them.)
-__device__ __forceinline__ void pair_add(float& hi, float& lo, float v, float w) {
-    const float h = hi + v, b = h - hi;
-    lo += ((hi - (h - b)) + (v - b)) + w;
-    hi = h;
-}
 __device__ __forceinline__ void ldsm_t4(uint32_t addr, uint32_t (&r)[4]) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(addr));
+}
+__device__ __forceinline__ void ldsm_t2(uint32_t addr, uint32_t (&r)[2]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
 }
 __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile(
@@ -330,13 +327,14 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4],
 
 // Partial sums over this CTA's tiles of dW[tap][co][ci] = sum_s dZ[s][co]
 // X[s + shift(tap)][ci] and db[co] = sum_s dZ[s][co] (dZ is zero on guard
-// slots).  A warp takes the three dx taps of one row (dz, dy) over every other
-// block of 128 slots: per 16 slots one transposed load of dZ (A, co x slots), three of X (B, slots x ci) and six
-// MMAs; the bias is a seventh MMA of row 4's warps against a matrix of ones.  Sums:
-// 16 slots in the tensor core, 128 slots in FP32, and those in pairs of FP32
-// values (two-sum), so that the error does not grow with the grid.  Bound: the
-// MMAs, one per 8.4 cycles and SM (nine warps 28.0, eighteen 26.5 us per layer
-// at 64^3; closing the sums in FP64 38.5 us).
+// slots).  A warp takes the three dx taps of one row (dz, dy) for eight of the 16
+// input channels: per 16 slots one transposed load of dZ (A, co x slots), two of
+// X (B, slots x ci) and three MMAs; the bias is one more MMA of a row 4 warp
+// against a matrix of ones.  Sums: 16 slots in the tensor core, WG_CLOSE blocks of
+// 128 slots in FP32, and those in three-part FP32 sums, so that the error does not
+// grow with the grid.  Bound: the MMAs, one per 8.4 cycles and SM.  One optimiser
+// step of eight 64^3 samples: 2.22 ms; 2.27 with warps that take all 16 channels of
+// every other block and sums in FP32 pairs, 2.72 with those sums in FP64.
 __global__ void __launch_bounds__(WG_THREADS, 1) wgrad_kernel(const __grid_constant__ WgradParams p) {
     using namespace tfde::tc;
     extern __shared__ uint8_t smem_raw[];
@@ -380,15 +378,26 @@ __global__ void __launch_bounds__(WG_THREADS, 1) wgrad_kernel(const __grid_const
         }
         return;
     }
-    const int row = warp % WG_ROWS, set = warp / WG_ROWS;
-    float hi[26], lo[26];   // 24 of the weights, 2 of the bias (every column the same)
+    const int row = warp % WG_ROWS, half = warp / WG_ROWS;
+    const bool bias = row == 4 && half == 0;
+    Sum3 acc[14];    // 12 of the weights, 2 of the bias (every column the same)
+    float sum[14];   // of the last blocks
+    int held = 0;
 #pragma unroll
-    for (int i = 0; i < 26; ++i) hi[i] = lo[i] = 0.f;
+    for (int i = 0; i < 14; ++i) sum[i] = 0.f;
+    auto close = [&]() {
+#pragma unroll
+        for (int i = 0; i < 14; ++i) {
+            acc[i].add(sum[i]);
+            sum[i] = 0.f;
+        }
+        held = 0;
+    };
     // A: matrices (slots 0-7, co 0-7), (0-7, 8-15), (8-15, 0-7), (8-15, 8-15);
-    // B: (slots 0-7, ci 0-7), (8-15, 0-7), (0-7, 8-15), (8-15, 8-15)
+    // B: slots 0-7 and 8-15 of dx = -1 and 0 (one load), then of dx = 1
     const int lr = lane & 7, lm = lane >> 3;
     const uint32_t aoff = (uint32_t)(2 * p.st.half_bytes + (lm & 1) * dz_half + ((lm >> 1) * 8 + lr) * 16);
-    const uint32_t boff = (uint32_t)((lm >> 1) * p.st.half_bytes + ((lm & 1) * 8 + lr + p.st.rowoff[row]) * 16);
+    const uint32_t boff = (uint32_t)(half * p.st.half_bytes + ((lane & 15) + (lane >> 4) + p.st.rowoff[row]) * 16);
     const uint32_t one2 = 0x3F803F80u;
     int s = 0;
     uint32_t ph = 0;
@@ -399,95 +408,81 @@ __global__ void __launch_bounds__(WG_THREADS, 1) wgrad_kernel(const __grid_const
         if (!ok) break;
         __syncwarp();
         const uint32_t base = smem_u32(stages + s * stage_bytes);
-        for (int k0 = set * TM; k0 < p.st.tile; k0 += WG_SETS * TM) {
-            float sum[26];
-#pragma unroll
-            for (int i = 0; i < 26; ++i) sum[i] = 0.f;
-#pragma unroll 1
+        for (int k0 = 0; k0 < p.st.tile; k0 += TM) {
+#pragma unroll 2
             for (int k = k0; k < k0 + TM; k += 16) {
-                uint32_t a[4];
+                uint32_t a[4], b[4], b1[2];
                 ldsm_t4(base + aoff + (uint32_t)k * 16u, a);
+                ldsm_t4(base + boff + (uint32_t)k * 16u, b);
+                ldsm_t2(base + boff + (uint32_t)(k + 2) * 16u, b1);
+                float c[3][4] = {};
+                mma_16816(c[0], a, b[0], b[1]);
+                mma_16816(c[1], a, b[2], b[3]);
+                mma_16816(c[2], a, b1[0], b1[1]);
 #pragma unroll
-                for (int dx = 0; dx < 3; ++dx) {
-                    uint32_t b[4];
-                    ldsm_t4(base + boff + (uint32_t)(k + dx) * 16u, b);
-                    float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
-                    mma_16816(c0, a, b[0], b[1]);
-                    mma_16816(c1, a, b[2], b[3]);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        sum[8 * dx + j] += c0[j];
-                        sum[8 * dx + 4 + j] += c1[j];
-                    }
-                }
-                if (row == 4) {
-                    float c[4] = {0.f, 0.f, 0.f, 0.f};
-                    mma_16816(c, a, one2, one2);
-                    sum[24] += c[0];
-                    sum[25] += c[2];
+                for (int i = 0; i < 12; ++i) sum[i] += c[i >> 2][i & 3];
+                if (bias) {
+                    float o[4] = {};
+                    mma_16816(o, a, one2, one2);
+                    sum[12] += o[0];
+                    sum[13] += o[2];
                 }
             }
-#pragma unroll
-            for (int i = 0; i < 26; ++i) pair_add(hi[i], lo[i], sum[i], 0.f);
+            if (++held == WG_CLOSE) close();
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[s]);
         if (++s == STAGES) { s = 0; ph ^= 1u; }
     }
-    // the second set's sums through shared memory (every copy has been read)
-    float* pass = reinterpret_cast<float*>(stages) + row * 32 + lane;
-    asm volatile("bar.sync 1, %0;" ::"n"(32 * WG_WARPS) : "memory");
-    if (set > 0) {
+    close();
+    // accumulator (co = lane / 4 (+ 8), ci = 2 (lane % 4) (+ 1) (+ 8)); the sums' three parts in planes
+    float* out = p.part + (size_t)blockIdx.x * 3 * GSZ;
+    auto put = [&](int at, const Sum3& v) {
+        out[at] = v.hi;
+        out[GSZ + at] = v.mid;
+        out[2 * GSZ + at] = v.lo;
+    };
 #pragma unroll
-        for (int i = 0; i < 26; ++i) {
-            pass[2 * i * 32 * WG_ROWS] = hi[i];
-            pass[(2 * i + 1) * 32 * WG_ROWS] = lo[i];
-        }
-    }
-    asm volatile("bar.sync 1, %0;" ::"n"(32 * WG_WARPS) : "memory");
-    if (set > 0) return;
-#pragma unroll
-    for (int i = 0; i < 26; ++i)
-        pair_add(hi[i], lo[i], pass[2 * i * 32 * WG_ROWS], pass[(2 * i + 1) * 32 * WG_ROWS]);
-    // accumulator (co = lane / 4 (+ 8), ci = 2 (lane % 4) (+ 1) (+ 8))
-    float2* out = p.part + (size_t)blockIdx.x * GSZ;
-#pragma unroll
-    for (int i = 0; i < 24; ++i) {
-        const int dx = i >> 3, half = (i >> 2) & 1, j = i & 3;
+    for (int i = 0; i < 12; ++i) {
+        const int dx = i >> 2, j = i & 3;
         const int co = (lane >> 2) + 8 * (j >> 1), ci = 8 * half + 2 * (lane & 3) + (j & 1);
-        out[(row * 3 + dx) * 256 + co * 16 + ci] = make_float2(hi[i], lo[i]);
+        put((row * 3 + dx) * 256 + co * 16 + ci, acc[i]);
     }
-    if (row == 4 && (lane & 3) == 0)
+    if (bias && (lane & 3) == 0)
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
-            out[NTAP * 256 + (lane >> 2) + 8 * j] = make_float2(hi[24 + j], lo[24 + j]);
+        for (int j = 0; j < 2; ++j) put(NTAP * 256 + (lane >> 2) + 8 * j, acc[12 + j]);
 }
 
 // grad[layer][W co][ci][tap] (and the bias) += the sum of the partials, all layers
-__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float2* __restrict__ part, int nparts,
+__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* __restrict__ part, int nparts,
                                                            float* __restrict__ grad) {
-    __shared__ float2 sh[8][33];
+    __shared__ Sum3 sh[8][33];
     const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
     const int idx = blockIdx.x * 32 + c;   // (tap, co, ci) or the bias
-    const float2* src = part + (size_t)blockIdx.y * nparts * GSZ;
-    float hi = 0.f, lo = 0.f;
+    const float* src = part + (size_t)blockIdx.y * nparts * 3 * GSZ;
+    Sum3 acc;
     if (idx < GSZ) {
 #pragma unroll 8
         for (int i = g; i < nparts; i += 8) {
-            const float2 v = src[(size_t)i * GSZ + idx];
-            pair_add(hi, lo, v.x, v.y);
+            const float* v = src + (size_t)i * 3 * GSZ + idx;
+            Sum3 t;
+            t.hi = v[0];
+            t.mid = v[GSZ];
+            t.lo = v[2 * GSZ];
+            acc += t;
         }
     }
-    sh[g][c] = make_float2(hi, lo);
+    sh[g][c] = acc;
     __syncthreads();
     if (g == 0 && idx < GSZ) {
-        for (int i = 1; i < 8; ++i) pair_add(hi, lo, sh[i][c].x, sh[i][c].y);
+        for (int i = 1; i < 8; ++i) acc += sh[i][c];
         float* gl = grad + (size_t)blockIdx.y * PSZ;
+        const float v = (float)acc.value();
         if (idx < NTAP * 256) {
             const int tap = idx / 256, co = (idx / 16) % 16, ci = idx % 16;
-            gl[(co * CH + ci) * NTAP + tap] += hi + lo;
+            gl[(co * CH + ci) * NTAP + tap] += v;
         } else {
-            gl[WSZ + idx - NTAP * 256] += hi + lo;
+            gl[WSZ + idx - NTAP * 256] += v;
         }
     }
 }
@@ -680,7 +675,7 @@ struct tfde_cnn {
     uint8_t* dz2 = nullptr;
     float* out = nullptr;      // network output, plain grid
     unsigned long long* scale = nullptr;   // max |u| (bits of a double; 0: no scaling)
-    float2* wpart = nullptr;    // weight-gradient partials [NL][wg_grid][GSZ]
+    float* wpart = nullptr;    // weight-gradient partials [NL][wg_grid][3][GSZ]
     double* lpart = nullptr;   // loss partials, then the error flag
     double* lpart_host = nullptr;
     int* err = nullptr;        // the word after lpart's partials
@@ -733,10 +728,7 @@ Staging staging(long long count, long long R, int limit, F smem) {
 // Two CTAs per SM share its 228 KB (1 KB of it reserved per CTA).
 constexpr int CONV_SMEM_LIMIT = 116736 - 1024;
 int conv_smem(const Staging& st) { return CONV_FIXED_SMEM + 16 + PLANES * 2 * st.plane_bytes; }
-constexpr int WG_PASS_BYTES = 2 * 26 * 32 * WG_ROWS * 4;   // one set's sums, in the place of the stages
-int wg_smem(const Staging& st) {
-    return WG_SMEM_FIXED + std::max(STAGES * (2 * st.half_bytes + 2 * st.tile * 16), WG_PASS_BYTES);
-}
+int wg_smem(const Staging& st) { return WG_SMEM_FIXED + STAGES * (2 * st.half_bytes + 2 * st.tile * 16); }
 
 int conv(tfde_cnn* C, const uint8_t* in, const __nv_bfloat16* w, const float* bias, int relu, const uint8_t* mask,
          uint8_t* out_act, float* out_f32, cudaStream_t s) {
@@ -785,7 +777,7 @@ int wgrad(tfde_cnn* C, int layer, const uint8_t* dz, cudaStream_t s) {
     p.P = C->P;
     p.first = C->first;
     p.ntiles = C->wg_tiles;
-    p.part = C->wpart + (size_t)layer * C->wg_grid * GSZ;
+    p.part = C->wpart + (size_t)layer * C->wg_grid * 3 * GSZ;
     p.err = C->err;
     stats_count_launch();
     CN_TRY(launch_pdl_smem(true, wgrad_kernel, C->wg_grid, WG_THREADS, wg_smem(p.st), s, p));
@@ -876,7 +868,7 @@ int cnn_create(const int n[3], tfde_cnn** out) {
               cudaMalloc((void**)&C->dz2, act_bytes) == cudaSuccess &&
               cudaMalloc((void**)&C->out, C->N * sizeof(float)) == cudaSuccess &&
               cudaMalloc((void**)&C->scale, sizeof(*C->scale)) == cudaSuccess &&
-              cudaMalloc((void**)&C->wpart, (size_t)NL * C->wg_grid * GSZ * sizeof(float2)) == cudaSuccess &&
+              cudaMalloc((void**)&C->wpart, (size_t)NL * C->wg_grid * 3 * GSZ * sizeof(float)) == cudaSuccess &&
               cudaMalloc((void**)&C->lpart, (LPART + 1) * sizeof(double)) == cudaSuccess &&
               cudaMallocHost((void**)&C->lpart_host, (LPART + 1) * sizeof(double)) == cudaSuccess;
     for (int l = 0; l < NL && ok; ++l) ok = cudaMalloc((void**)&C->act[l], act_bytes) == cudaSuccess;
