@@ -70,10 +70,11 @@ struct SegSpec {
 // (plane_seg hi + lo); *bytes / *flops receive its algorithmic traffic and
 // tensor-core work.
 void gemm_params(const tfde_problem* P, int axis, const SegSpec* segs, int nseg, int out_mode, float alpha,
-                 float* out_f32, int out_plane, bool lam_scale, tc::Params& prm, double* bytes, double* flops) {
+                 float* out_f32, int out_plane, bool lam_scale, tc::Params& prm, double* bytes, double* flops,
+                 int tiles = tc::TILES_SPLIT) {
     MixedState* M = mixed(P);
     std::memset(&prm, 0, sizeof(prm));
-    tc::set_geometry(prm, P->n, axis, M->bn[axis]);
+    tc::set_geometry(prm, P->n, axis, M->bn[tiles][axis]);
     // tensor maps: merged boxes where the allocation allows one copy per operand
     // (hi/lo operator pair; hi/lo plane pair with, on y/z, all line blocks)
     int na = 0, nb = 0;
@@ -96,15 +97,15 @@ void gemm_params(const tfde_problem* P, int axis, const SegSpec* segs, int nseg,
                 S.na = 2;
             }
         }
-        const int rank = M->bmap2_rank[segs[g].plane][axis];
-        if (rank > 0) {
-            prm.bmaps[nb] = M->bmap2[segs[g].plane][axis];
+        const MixedState::PlaneMaps& in = M->bmap[segs[g].plane][tiles][axis];
+        if (in.both_rank > 0) {
+            prm.bmaps[nb] = in.both;
             S.bmap2 = nb++;
-            prm.b_rank = rank;
+            prm.b_rank = in.both_rank;
         } else {
-            prm.bmaps[nb] = M->bmap_hi[segs[g].plane][axis];
+            prm.bmaps[nb] = in.hi;
             S.bmap[0] = nb++;
-            prm.bmaps[nb] = M->bmap_lo[segs[g].plane][axis];
+            prm.bmaps[nb] = in.lo;
             S.bmap[1] = nb++;
         }
         S.nb = 2;
@@ -231,7 +232,8 @@ int ensure_pairs(const tfde_problem* P, cudaStream_t s) {
         for (int i = 0; i < 2; ++i) {
             const Pass& q = ps[2 * g + i];
             double by, fl;
-            gemm_params(P, q.axis, q.seg, q.nseg, q.out_mode, 1.f, nullptr, q.out_plane, q.lam, prm[2 * g + i], &by, &fl);
+            gemm_params(P, q.axis, q.seg, q.nseg, q.out_mode, 1.f, nullptr, q.out_plane, q.lam, prm[2 * g + i], &by, &fl,
+                        tc::TILES_PAIR);
             gst[3 * g + i + 1] = gst[3 * g + i] + prm[2 * g + i].ntiles * prm[2 * g + i].mhalves;
             M->pair_bytes[g] += by;
             M->pair_flops[g] += fl;
@@ -257,7 +259,8 @@ int fast_matvec(const tfde_problem* P, int op, float* q32, cudaStream_t s, int o
     for (int g = 0; g < 2; ++g) {
         M->gemm_launches++;
         st = tc::launch_grouped(M->pair_d + 2 * g, M->pair_gstart + 3 * g, 2, M->pair_total[g], g == 0 ? 1 : 0,
-                                tc::OUT_HILO, 0, M->bn[g == 0 ? 0 : 1], nullptr, M->err, s, M->pair_bytes[g], M->pair_flops[g], skip);
+                                tc::OUT_HILO, 0, M->bn[tc::TILES_PAIR][g], nullptr, M->err, s, M->pair_bytes[g],
+                                M->pair_flops[g], skip);
         if (st) return st;
     }
     return run_passes(P, ps + 4, 1, q32, s, dot_vec, dot_out, skip);
@@ -286,16 +289,16 @@ int fast_precond_cg(const tfde_problem* P, float* p32, const float* p_old, doubl
         tc::Params prm;
         double bytes, flops;
         gemm_params(P, q.axis, q.seg, q.nseg, last ? tc::OUT_XPAY : tc::OUT_HI, 1.f, last ? p32 : nullptr,
-                    last ? PL_P : q.out_plane, q.lam, prm, &bytes, &flops);
+                    last ? PL_P : q.out_plane, q.lam, prm, &bytes, &flops, tc::TILES_HI);
         // one B plane (hi) and one product per pass
-        const int pl = q.seg[0].plane;
         tc::Segment& S = prm.seg[0];
+        const MixedState::PlaneMaps& in = M->bmap[q.seg[0].plane][tc::TILES_HI][q.axis];
         if (S.bmap2 >= 0) {
-            if (M->bmap1_rank[pl][q.axis] > 0) {
-                prm.bmaps[S.bmap2] = M->bmap1[pl][q.axis];
-                prm.b_rank = M->bmap1_rank[pl][q.axis];
+            if (in.hi_merged_rank > 0) {
+                prm.bmaps[S.bmap2] = in.hi_merged;
+                prm.b_rank = in.hi_merged_rank;
             } else {   // the merged box would carry both planes: per-plane boxes, hi alone
-                prm.bmaps[S.bmap2] = M->bmap_hi[pl][q.axis];
+                prm.bmaps[S.bmap2] = in.hi;
                 S.bmap[0] = S.bmap2;
                 S.bmap2 = -1;
             }
@@ -1402,7 +1405,12 @@ int mixed_init(tfde_problem* P, cudaStream_t s, const int* bn) {
         if (st) return st;
     }
     // workspace planes and their tensor maps
-    for (int a = 0; a < 3; ++a) M->bn[a] = bn ? bn[a] : tc::tile_lines(tc::wide_tiles(P->n, a));
+    for (int a = 0; a < 3; ++a) {
+        const long long wide = tc::wide_tiles(P->n, a);
+        M->bn[tc::TILES_SPLIT][a] = bn ? bn[a] : tc::tile_lines(wide);
+        M->bn[tc::TILES_HI][a] = tc::tile_lines(wide, tc::TILES_HI);
+        M->bn[tc::TILES_PAIR][a] = tc::tile_lines(wide, tc::TILES_PAIR);
+    }
     for (int pl = 0; pl < NPL; ++pl) {
         MX_TRY(cudaMalloc((void**)&M->hi[pl], 2 * N * sizeof(__nv_bfloat16)));
         M->lo[pl] = M->hi[pl] + N;
@@ -1410,12 +1418,16 @@ int mixed_init(tfde_problem* P, cudaStream_t s, const int* bn) {
         for (int a = 0; a < 3; ++a) {
             int st;
             if ((st = tc::make_out_map(&M->omap_hi[pl][a], M->hi[pl], P->n, a, false)) ||
-                (st = tc::make_out_map_pair(&M->omap_hl[pl][a], M->hi[pl], P->n, a)) ||
-                (st = tc::make_map_B(&M->bmap_hi[pl][a], M->hi[pl], P->n, a, M->bn[a])) ||
-                (st = tc::make_map_B(&M->bmap_lo[pl][a], M->lo[pl], P->n, a, M->bn[a])))
+                (st = tc::make_out_map_pair(&M->omap_hl[pl][a], M->hi[pl], P->n, a)))
                 return st;
-            M->bmap2_rank[pl][a] = tc::make_map_B_pair(&M->bmap2[pl][a], M->hi[pl], P->n, a, M->bn[a]);
-            M->bmap1_rank[pl][a] = tc::make_map_B_pair(&M->bmap1[pl][a], M->hi[pl], P->n, a, M->bn[a], 1);
+            for (int t = 0; t < tc::TILES_KINDS; ++t) {
+                MixedState::PlaneMaps& in = M->bmap[pl][t][a];
+                if ((st = tc::make_map_B(&in.hi, M->hi[pl], P->n, a, M->bn[t][a])) ||
+                    (st = tc::make_map_B(&in.lo, M->lo[pl], P->n, a, M->bn[t][a])))
+                    return st;
+                in.both_rank = tc::make_map_B_pair(&in.both, M->hi[pl], P->n, a, M->bn[t][a]);
+                in.hi_merged_rank = tc::make_map_B_pair(&in.hi_merged, M->hi[pl], P->n, a, M->bn[t][a], 1);
+            }
         }
     }
     for (int v = 0; v < NF; ++v) {

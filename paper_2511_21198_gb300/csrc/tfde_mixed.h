@@ -142,13 +142,15 @@ struct MixedState {
     bool has_amap2[NOM] = {};
     __nv_bfloat16* hi[NPL] = {};   // one allocation per plane pair: lo = hi + N
     __nv_bfloat16* lo[NPL] = {};
-    CUtensorMap bmap_hi[NPL][3];
-    CUtensorMap bmap_lo[NPL][3];
-    int bn[3] = {256, 256, 256};   // lines per tile of the passes along each axis (the planes' boxes)
-    CUtensorMap bmap2[NPL][3];     // both planes (and on y/z all four 64-line blocks) in one box
-    int bmap2_rank[NPL][3] = {};   // 3 (x), 5 (y/z), 0 = not available
-    CUtensorMap bmap1[NPL][3];     // the hi plane alone, same box otherwise
-    int bmap1_rank[NPL][3] = {};
+    // the planes as input, boxes for each tile width
+    struct PlaneMaps {
+        CUtensorMap hi, lo;
+        CUtensorMap both;       // both planes (and on y/z all 64-line blocks) in one box
+        CUtensorMap hi_merged;  // the hi plane alone, same box otherwise
+        int both_rank = 0, hi_merged_rank = 0;   // 3 (x), 5 (y/z), 0 = not available
+    };
+    PlaneMaps bmap[NPL][tc::TILES_KINDS][3];
+    int bn[tc::TILES_KINDS][3] = {};             // lines per tile of the passes along each axis
     CUtensorMap omap_hi[NPL][3];   // the planes as outputs of the epilogue's tensor stores
     CUtensorMap omap_hl[NPL][3];   // hi and lo as one tensor (lo = hi + N): one store per chunk
     float* f[NF] = {};

@@ -234,14 +234,25 @@ long long wide_tiles(const int n[3], int axis) {
 // lines) 36.2 -> 33.2 ms per 10 steps (64 lines: 33.8), 256^3 (512 tiles in
 // 3.4 rounds; 128 lines) 56.1 -> 55.7; 192^3 (288 tiles; 256 lines stay) 19.4
 // against 19.6 ms with 128.
-int tile_lines(long long wide) {
+// The hi-only passes have a third of the products, so that a third of a tile
+// does not shrink with it (256^3: 19.8 us with 256 lines, 22.9 with 128).  A
+// pair's launch has twice the tiles, and from one 256-line tile per SM on nothing
+// is gained by narrower ones (an inner PCG in the grid basis with pairs of 256
+// against 128 lines: 104^3 2.26 / 2.28 ms, 128^3, a tile short of that, 2.40 /
+// 2.39, 144^3 4.10 / 4.16, 256^3 12.47 / 12.63; 12.84 with the eigenbasis' widths
+// in every pass).
+int tile_lines(long long wide, int kind) {
+    constexpr int kLines[3] = {256, 128, 64};
+    constexpr int kCost[3] = {40, 22, 13}, kCostHi[3] = {40, 26, 18};
     const long long sms = num_sms();
+    if (kind == TILES_PAIR && 2 * wide > sms) return 256;
     int best = 0;
     long long least = 0;
-    for (const int bn : {256, 128, 64}) {
-        const long long tiles = wide * (256 / bn), cost = (tiles + sms - 1) / sms * (bn == 256 ? 40 : (bn == 128 ? 22 : 13));
+    for (int i = 0; i < 3; ++i) {
+        const long long tiles = wide * (256 / kLines[i]);
+        const long long cost = (tiles + sms - 1) / sms * (kind == TILES_HI ? kCostHi[i] : kCost[i]);
         if (!best || cost < least) {
-            best = bn;
+            best = kLines[i];
             least = cost;
         }
     }

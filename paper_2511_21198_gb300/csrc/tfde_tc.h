@@ -31,10 +31,14 @@ int make_map_B_box(CUtensorMap* m, const __nv_bfloat16* base, const int n[3], in
 // planes: 2 (hi and lo in one box) or 1 (the hi plane alone)
 int make_map_B_pair(CUtensorMap* m, const __nv_bfloat16* base, const int n[3], int axis, int bn, int planes = 2);
 void set_geometry(Params& P, const int n[3], int axis, int bn);
-// Tiles of 256 lines of one launch over a grid along `axis`, and the lines per
-// tile for a launch of that many.
+// Tiles of 256 lines of one contraction over a grid along `axis`, and the lines
+// per tile for that many: of the passes with split input planes (grouped launches:
+// the sum over the group), of those of the inner PCG's preconditioner in the grid
+// basis, which read the hi plane alone, and of the grid basis operator's x and y
+// passes, two contractions of that many tiles per launch.
+enum { TILES_SPLIT = 0, TILES_HI, TILES_PAIR, TILES_KINDS };
 long long wide_tiles(const int n[3], int axis);
-int tile_lines(long long wide);
+int tile_lines(long long wide, int kind = TILES_SPLIT);
 int launch(const Params& P, cudaStream_t s, double bytes, double flops);
 // One persistent launch over the tiles of `ngroups` contractions along the same
 // axis (descriptors and tile offsets gstart[0..ngroups] in device memory,

@@ -13,7 +13,7 @@ ROOT = os.path.dirname(HERE)
 NATIVE = os.path.join(HERE, "native")
 
 
-def run_check(name, tmp_path):
+def run_check(name, tmp_path, *args):
     if shutil.which("g++") is None:
         pytest.skip("no host C++ compiler")
     from paper_2511_21198_gb300 import build
@@ -29,8 +29,9 @@ def run_check(name, tmp_path):
     subprocess.run(["g++", "-O1", "-std=c++17", "-I", NATIVE, "-I", build.CSRC, "-I", os.path.join(ROOT, "include"),
                     "-isystem", cuda, src, os.path.join(NATIVE, "fake_cudart.cpp"),
                     *sorted(glob.glob(os.path.join(build.BUILD_DIR, "*.o"))), "-o", exe], check=True)
-    out = subprocess.run([exe], capture_output=True, text=True, timeout=300)
+    out = subprocess.run([exe, *map(str, args)], capture_output=True, text=True, timeout=300)
     assert out.returncode == 0, out.stdout + out.stderr
+    return out.stdout
 
 
 def test_loop_buffers(tmp_path):
@@ -39,3 +40,12 @@ def test_loop_buffers(tmp_path):
 
 def test_batch_tile_widths(tmp_path):
     run_check("batch_tiles_check", tmp_path)
+
+
+def test_tile_widths(tmp_path):
+    from test_gpu_widths import WIDTHS
+    out = run_check("tile_widths_check", tmp_path, *(v for n in WIDTHS for v in n))
+    got = [[int(v) for v in line.split()] for line in out.splitlines()]
+    assert got == [sum(map(list, w), []) for w in WIDTHS.values()]
+    for kind in range(3):   # every width of each rule occurs
+        assert {v for w in WIDTHS.values() for v in w[kind]} == {64, 128, 256}
