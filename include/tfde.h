@@ -248,17 +248,17 @@ int tfde_cn_advance_guess(const tfde_problem* prob, double* u, const double* F_h
 int tfde_set_guess_order(tfde_problem* prob, int order);
 
 /*
- * tfde_set_device_loop -- how the inner PCG of a TFDE_MIXED problem runs its
- * iterations (Sec. 3.1; no effect on TFDE_FP64 problems or on PGMRES).
+ * tfde_set_device_loop -- how the inner PCG and PGMRES of a TFDE_MIXED problem
+ * run their iterations (Sec. 3.1-3.2; no effect on TFDE_FP64 problems).
  *   enable != 0 (default): each refinement sweep's inner iterations run as one
  *   CUDA graph launch, a device-side while loop whose stop test (the inner
  *   residual norm against the sweep's target) is taken on the device; the host
  *   reads the iteration count and residual once per sweep.  enable = 0: the
  *   host takes the stop test after every iteration (one blocking read each).
- *   Both give the same iterates.  While tfde_stats_reset(1) times every
- *   tensor-core launch, the host-driven loop is used.  The graph is built on
- *   the problem's first sweep and captures its workspace pointers; it is
- *   released with the problem.  Errors: TFDE_EINVAL for a NULL problem.
+ *   Both give the same iterates up to the order of sums.  While
+ *   tfde_stats_reset(1) times every tensor-core launch, the host-driven loop is
+ *   used.  The graph is built on the problem's first sweep and captures its
+ *   workspace pointers; it is released with the problem.  Errors: TFDE_EINVAL for a NULL problem.
  */
 int tfde_set_device_loop(tfde_problem* prob, int enable);
 

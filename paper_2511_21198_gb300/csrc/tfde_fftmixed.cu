@@ -14,7 +14,7 @@
 // 1e-5.  Inner products accumulate in FP64.  The inner iterations run as one
 // CUDA graph per sweep with the stop test on the device (PCG: tfde_pcgloop.cu;
 // GMRES: build_cycle below, restart lengths up to GS_MAXM); with per-launch
-// timing on, or without such a graph, the host drives them and reads one scalar
+// timing on, tfde_set_device_loop(.., 0) or without such a graph, the host drives them and reads one scalar
 // per PCG iteration and two projections per Arnoldi step.
 #include <chrono>
 #include <cmath>
@@ -353,7 +353,7 @@ int inner_gmres(const tfde_problem* P, int m, double theta, int maxit, int* iter
     int st;
     *iters = 0;
     *est_ratio = 1.0;
-    if (!stats_timing() && maxit > 0) {
+    if (P->device_loop && !stats_timing() && maxit > 0) {
         if ((st = build_cycle(P, m, s))) return st;
         if (F->gm_exec && F->gm_restart == m) return inner_gmres_loop(P, m, theta, maxit, iters, est_ratio, s);
     }

@@ -148,6 +148,7 @@ struct tfde_problem {
     void* fft = nullptr;    // FFT tables of the FFT-embedded passes (tfde_fft.h), null: dense FP64
     mutable void* pcg_loop[2] = {nullptr, nullptr};   // device-side PCG loops, FP64 and FP32 (tfde_pcgloop.cu)
     void* fmix = nullptr;   // mixed-precision state on the FFT passes (tfde_fftmixed.cu)
+    bool device_loop = true;   // tfde_set_device_loop (TFDE_MIXED)
 
     // host copies of a tfde_cn_advance_host step (out == null otherwise): the
     // input goes host -> dev on `stream` while the step starts its work that

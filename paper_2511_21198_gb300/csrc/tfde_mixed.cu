@@ -394,7 +394,7 @@ int inner_pcg(const tfde_problem* P, double theta, int maxit, int* iters, PcgPen
     if (reached) *reached = 0.0;
     if (!(rr0 > 0.0) || !std::isfinite(rr0)) return rr0 == 0.0 ? TFDE_OK : set_error(TFDE_ENAN, "non-finite inner residual");
     // device-side loop unless every launch is to be timed on its own
-    if (M->device_loop && !stats_timing() && maxit > 0) {
+    if (P->device_loop && !stats_timing() && maxit > 0) {
         if ((st = build_pcg_graph(P, s))) return st;
         if (M->pcg_exec) return inner_pcg_graph(P, theta, maxit, iters, pend, s, reached, rr0);
     }
@@ -662,7 +662,7 @@ int inner_pcg_spec(const tfde_problem* P, double theta, int maxit, int* iters, P
     if (!(rr0 > 0.0) || !std::isfinite(rr0)) return rr0 == 0.0 ? TFDE_OK : set_error(TFDE_ENAN, "non-finite inner residual");
     auto pbuf = [&](int j) { return M->pring + (size_t)(j % kPRing) * N; };
     if ((st = spec_transform(P, PL_R, PL_T1, PL_T2, r, s))) return st;   // r~ = S_N r
-    if (M->device_loop && !stats_timing() && maxit > 0) {
+    if (P->device_loop && !stats_timing() && maxit > 0) {
         if ((st = build_pcg_graph_spec(P, s))) return st;
         if (M->spec_exec) return inner_pcg_spec_graph(P, theta, maxit, iters, pend, s, reached, rr0);
     }
@@ -922,10 +922,10 @@ int inner_gmres_spec(const tfde_problem* P, int restart, double ptheta, int maxi
         return st;
     MX_TRY(cudaMemsetAsync(M->f[F_X], 0, N * sizeof(float), s));
     int k = 0;
-    if (M->device_loop && !stats_timing() && maxit > 0 && restart <= GS_MAXM) {
+    if (P->device_loop && !stats_timing() && maxit > 0 && restart <= GS_MAXM) {
         if ((st = build_gmres_graph_spec(P, restart, s))) return st;
     }
-    if (M->device_loop && !stats_timing() && maxit > 0 && M->gms_exec && M->gms_graph_restart == restart) {
+    if (P->device_loop && !stats_timing() && maxit > 0 && M->gms_exec && M->gms_graph_restart == restart) {
         MX_TRY(cudaMemsetAsync(M->gm_ctl, 0, 4 * sizeof(int), s));
         const int maxsteps = restart < maxit ? restart : maxit;
         launch_gm_start(N, M->f[F_Z], P->red, P->nblk, M->gm_state, M->gm_ctl, maxsteps, ptheta, V,
@@ -1166,7 +1166,7 @@ int inner_gmres_graph(const tfde_problem* P, int restart, double ptheta, int max
 int inner_gmres(const tfde_problem* P, int restart, double ptheta, int maxit, int* iters, double* est_ratio,
                 cudaStream_t s) {
     MixedState* M = mixed(P);
-    if (M->device_loop && !stats_timing() && maxit > 0 && restart <= GS_MAXM) {
+    if (P->device_loop && !stats_timing() && maxit > 0 && restart <= GS_MAXM) {
         if (int st = build_gmres_graph(P, restart, s)) return st;
         if (M->gm_exec) return inner_gmres_graph(P, restart, ptheta, maxit, iters, est_ratio, s);
     }
@@ -1808,8 +1808,7 @@ long long mixed_graph_launches(const tfde_problem* P) {
 }
 
 int mixed_set_device_loop(tfde_problem* P, int enable) {
-    MixedState* M = mixed(P);
-    if (M) M->device_loop = enable != 0;
+    if (P->prec == TFDE_MIXED) P->device_loop = enable != 0;
     return TFDE_OK;
 }
 

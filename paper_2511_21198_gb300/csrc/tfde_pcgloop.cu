@@ -318,7 +318,7 @@ template <typename R>
 int pcg_loop(const tfde_problem* P, const PcgLoopVectors<R>& v, R* x, double thr, int maxit, PcgLoopResult* res,
              cudaStream_t s) {
     res->ran = false;
-    if (!P->fft || stats_timing() || maxit < 1) return TFDE_OK;
+    if (!P->fft || !P->device_loop || stats_timing() || maxit < 1) return TFDE_OK;
     Loop* L = loop_of<R>(P);   // there since assembly, but for a mixed solve's FP64 fallback
     if (!L) return TFDE_OK;
     if (int st = build<R>(P, L, v, s)) return st;

@@ -16,7 +16,7 @@ struct PcgLoopVectors {
 // updated) or not positive (nothing updated), <r, r> not finite
 enum { PCGLOOP_OK = 0, PCGLOOP_NAN_PAP = 1, PCGLOOP_BREAKDOWN = 2, PCGLOOP_NAN_RR = 3 };
 struct PcgLoopResult {
-    bool ran = false;   // false: no graph or no memory (the caller iterates from the host)
+    bool ran = false;   // false: switched off, no graph or no memory (the caller iterates from the host)
     int iters = 0, bad = PCGLOOP_OK;
     double rr = 0.0;    // <r, r> of the recursive residual
 };
