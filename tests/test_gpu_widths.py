@@ -71,3 +71,34 @@ def test_widths_match_fp64(T, n, sym):
             assert info.relres <= 1e-12 and not info.fallback and rel(x, ref) < 1e-10
     finally:
         T.tfde_destroy(h)
+
+
+def test_batch_of_256_line_tiles(T):
+    """Four 128^3 problems: 256 wide tiles per axis, for which the rule takes 256 lines."""
+    import torch
+    prm, us = [], []
+    for i in range(4):
+        km = (1.0, 1.2, 0.8) if i % 2 else (0.5, 0.6, 0.7)
+        prm.append(T.make_params((128,) * 3, (0.3, 0.5, 0.7), (1.0, 1.2, 0.8), km, 0.05))
+        us.append(to_dev(inp.smoothed_uniform((128,) * 3, i)))
+    ref = [u.clone() for u in us]
+    B = T.tfde_batch_create(prm, 20)
+    try:
+        for spectral in (1, 0):   # eigenbasis, then the grouped operator and preconditioner
+            T.tfde_batch_set_spectral_inner(B, spectral)
+            for u, w in zip(us, ref):
+                u.copy_(w)
+            for m in range(2):
+                infos = T.tfde_batch_cn_advance(B, us, None, m == 0, 1e-11)
+                assert all(i.relres <= 1e-11 and not i.fallback for i in infos)
+            for i, p in enumerate(prm):
+                h = T.tfde_assemble(p, T.TFDE_FP64)
+                try:
+                    w = ref[i].clone()
+                    for m in range(2):
+                        T.tfde_cn_advance(h, w, None, m == 0, 1e-12)
+                finally:
+                    T.tfde_destroy(h)
+                assert rel(us[i], w) < 1e-9
+    finally:
+        T.tfde_batch_destroy(B)
