@@ -447,11 +447,13 @@ int tfde_batch_cn_advance(tfde_batch* batch, double* const* u, const double* con
  * Autotuner of the tensor-core contraction's launch parameters (no
  * counterpart in the paper): the number of persistent CTAs (the SM count,
  * the count that deals the tiles evenly over the same number of waves, 7/8
- * and 3/4 of the SMs) and the depth of the operand ring (2 .. 4 stages of
- * 48 KB, or 2 of 96 KB), per launch class.  A class is the kernel instance
- * (grouped, operand layout, output mode), the stage size, the rows n of the
- * contraction (0 for grouped launches) and the number of tiles (128 rows x 256,
- * 128 or 64 lines, by the size of the launch).
+ * and 3/4 of the SMs) and the depth of the operand ring (2 .. 4 stages of 24 to
+ * 96 KB, as many as fit 192 KB), per launch class.  A class is what the table's
+ * key fields hold: grouped or not, operand layout, output mode, the stage size,
+ * the rows n of the contraction (0 for grouped launches) and the number of tiles
+ * (128 rows x 256, 128 or 64 lines, by the size of the launch).  Launches of one
+ * class share a choice, the one that suits the first of them recorded; they may
+ * differ in what the eigenbasis' y and z passes do besides the addend.
  *
  * tfde_tune records the launches of one operator and one preconditioner
  * application of a TFDE_MIXED problem on the tensor-core path, times each
@@ -473,7 +475,8 @@ int tfde_batch_cn_advance(tfde_batch* batch, double* const* u, const double* con
 typedef struct {
     int grouped;      /* 1: one launch over the tiles of several contractions   */
     int kmajor;       /* operand layout: 1 for x-axis contractions              */
-    int out_mode;     /* 0 FP32, 1 split planes, 2 direction update, 3 hi plane */
+    int out_mode;     /* 0 FP32, 1 split planes, 2 direction update, 3 hi plane,
+                         4 eigenbasis passes                                     */
     int stage_bytes;  /* ring stage size of the class                            */
     int n;            /* rows of the contraction (0 for grouped launches)        */
     long long tiles;  /* tiles of the launch                                      */

@@ -39,7 +39,7 @@
 // Weight gradients: per tap a 16 x 16 matrix summed over all slots, on
 // mma.sync m16n8k16 (tcgen05's smallest M of 64 would leave three quarters of
 // the rows empty); the same staged runs as the convolution serve all 27 taps.
-// One optimiser step of eight 64^3 samples: 2.3 ms, against 25.7 ms with the
+// One optimiser step of eight 64^3 samples: 2.2 ms, against 25.7 ms with the
 // nine-copy convolution, a CUDA-core weight gradient per tap and 256-slot
 // chunk (477 us per layer, 160 us for the sum of its partials), a one-block
 // max |u| (183 us) and a 16-block bias sum (41 us).

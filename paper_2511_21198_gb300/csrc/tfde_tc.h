@@ -56,9 +56,10 @@ int sum_part(const Params& P);
 
 // Launch parameters chosen by the autotuner (tfde_tune, tfde_batch_tune):
 // the number of persistent CTAs and of ring stages, per launch class.  A
-// class is the kernel instance (grouped, operand layout, output mode), the
-// stage size, the rows n of the contraction (0 for grouped launches) and the
-// number of tiles of the launch (128 rows x 256, 128 or 64 lines).
+// class is grouped or not, the operand layout and output mode, the stage size,
+// the rows n of the contraction (0 for grouped launches) and the number of tiles
+// of the launch (128 rows x 256, 128 or 64 lines).  The instances of an output
+// mode (EP_DOT, EP_DIV) share a class: the choice is the first recorded one's.
 struct TuneKey {
     int grouped, kmajor, out_mode, stage_bytes, n;
     long long tiles;
