@@ -291,7 +291,7 @@ long long tfde_device_loop_launches(const tfde_problem* prob);
  *   enable = 0: the grid basis (operator in 3 and preconditioner in 6 split
  *   passes per iteration).
  * The refinement's FP64 residual, and so the result's accuracy, are the same
- * either way.  The batched solver always iterates in the grid basis.
+ * either way.  A batch has its own switch (tfde_batch_set_spectral_inner).
  * Errors: TFDE_EINVAL for a NULL problem; TFDE_EUNSUPPORTED when enable != 0
  * for a TFDE_FP64 problem or a TFDE_MIXED problem on the FFT passes (enable =
  * 0 is accepted and has no effect there).

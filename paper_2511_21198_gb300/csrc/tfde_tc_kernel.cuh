@@ -13,19 +13,19 @@
 // 64 lines where 256 would leave SMs without a tile, Params::bn):
 //   warps 0..2  TMA producers: A tiles [128 x 64] (K-major, 128B swizzle; the
 //               hi and lo terms of a split operator in one 3-D box) and B
-//               tiles [64 x 256] (x axis: K-major 128B swizzle; y/z axes:
-//               MN-major 128B swizzle, 4 line blocks of 64 in one box with
-//               both planes) into a ring of 192 KB: 2 stages of 96 KB when a
-//               segment carries two operator terms and two planes, 4 stages
-//               of 48 KB for one term and one plane.  A stage moves 48-96 KB
+//               tiles [64 x lines] (x axis: K-major 128B swizzle; y/z axes:
+//               MN-major 128B swizzle, the line blocks of 64 in one box with
+//               both planes) into a ring of 192 KB: with 256 lines 2 stages of
+//               96 KB when a segment carries two operator terms and two planes, 4
+//               stages of 48 KB for one term and one plane.  A stage moves 24-96 KB
 //               in two copies: the issue cost of a copy (~0.2-0.4 us, measured
 //               by an in-kernel timeline) is paid per copy, not per byte, so
 //               64-wide k-blocks halve it against 32-wide ones.  The boxes of
 //               a stage are dealt round-robin to the issuing threads.
 //   warp 3      allocates TMEM (2 x 256 FP32 columns) and issues tcgen05.mma
-//               (M=128, N=256, K=16, BF16 in, FP32 accumulate) from one thread
+//               (M=128, N=lines, K=16, BF16 in, FP32 accumulate) from one thread
 //   warps 4..11 epilogue, two warps per TMEM lane quadrant (one per half of the
-//               256 columns), per 32 x 32 chunk: tcgen05.ld, scale, optional
+//               tile's columns), per 32 x 32 chunk: tcgen05.ld, scale, optional
 //               Lambda^{-1}, direction update and fused inner products, the
 //               chunk written to a swizzled shared-memory slot and sent to
 //               global memory by one TMA tensor store per output plane (the
